@@ -56,6 +56,10 @@ cudaError_t launch_linear_simt(const void* q, const void* k, const void* v, void
                                int dtype, Strides st, int h_begin, int h_count, float* S_io, float* z_io,
                                bool zero_init, cudaStream_t stream, bool global_sum = false,
                                const void* W = nullptr /* [h_count, d, d] storage dtype: positive random features */);
+// The causal heads with phi = elu + 1: register-tiled blocks of 32 tokens (launch_linear_simt comes here by itself).
+cudaError_t launch_linear_tiled(const void* q, const void* k, const void* v, void* o, int B, int N, int d, int dtype,
+                                Strides st, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
+                                cudaStream_t stream);
 cudaError_t launch_export_ring(const void* k, const void* v, void* k_cache, void* v_cache, int B, int N, int d,
                                int w, int dtype, Strides st, int h_sparse, cudaStream_t stream);
 // t_seq == nullptr: every sequence is at position t; else sequence b is at t_seq[b] (device array,
@@ -134,7 +138,7 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
   return __float2bfloat16_rn(x);
 }
 
-// phi(x) = elu(x) + 1 (Sec. II-B).
-__device__ __forceinline__ float phi_elu1(float x) { return x > 0.f ? x + 1.f : expf(x); }
+// phi(x) = elu(x) + 1 (Sec. II-B), without a branch: max(x, 0) + exp(min(x, 0)).
+__device__ __forceinline__ float phi_elu1(float x) { return fmaxf(x, 0.f) + expf(fminf(x, 0.f)); }
 
 }  // namespace gf

@@ -1,9 +1,8 @@
 // CUDA-core (fp32 arithmetic) kernels of libgformer.
 //
-// They serve every request the tensor-core kernels do not take: fp32 storage, windows
-// that are not a multiple of 64, and the memory-bound decode step / ring export, which
-// have no dense contraction worth a tensor core.  All of them are plain data-parallel
-// kernels: no inter-CTA communication, no spin waits.
+// The linear heads of fp32 tensors where neither the tensor-core kernels nor the register-tiled ones apply (the
+// bidirectional layer's sums, positive random features), and the memory-bound decode step and ring export, which have
+// no dense contraction worth a tensor core.  Plain data-parallel kernels: no inter-CTA communication, no spin waits.
 #include "common.cuh"
 
 namespace gf {
@@ -31,94 +30,6 @@ template <> struct Vec4<__nv_bfloat16> {
     *reinterpret_cast<uint2*>(p) = raw;
   }
 };
-
-// ------------------------------------------------------------------------------------
-// Windowed softmax attention (Eq. 1 + causal mask + left window of w keys).
-// One CTA = 32 query rows of one head, 4 threads per row, each owning d/4 of the head
-// dimension; keys/values pass through shared memory 32 rows at a time; online softmax.
-// ------------------------------------------------------------------------------------
-template <typename T, int D>
-__global__ void __launch_bounds__(128)
-window_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                   T* __restrict__ o, int N, int w, int fwd, float scale, Strides st, int h_begin) {
-  // fwd: keys after the query that it may see (0: the causal window; w - 1: the two-sided one)
-  constexpr int CH = D / 16;  // float4 chunks per thread
-  __shared__ __align__(16) float Ks[32][D];
-  __shared__ __align__(16) float Vs[32][D];
-
-  const int b = blockIdx.z, h = h_begin + blockIdx.y;
-  const long long base = (long long)b * st.b + (long long)h * st.h;
-  const int i0 = blockIdx.x * 32;
-  const int row = threadIdx.x >> 2, sub = threadIdx.x & 3;
-  const int i = i0 + row;
-
-  float4 qv[CH], ov[CH];
-#pragma unroll
-  for (int c = 0; c < CH; ++c) {
-    ov[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-    qv[c] = (i < N) ? Vec4<T>::load(q + base + (long long)i * st.n + 4 * (sub + 4 * c))
-                    : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  float m = -INFINITY, l = 0.f;
-
-  int jlo = i0 - w + 1;
-  if (jlo < 0) jlo = 0;
-  int jhi = i0 + 31 + fwd;
-  if (jhi > N - 1) jhi = N - 1;
-
-  for (int j0 = jlo; j0 <= jhi; j0 += 32) {
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < 32 * (D / 4); idx += 128) {
-      const int r = idx / (D / 4), c4 = idx % (D / 4);
-      const int j = j0 + r;
-      float4 kk = make_float4(0.f, 0.f, 0.f, 0.f), vv = kk;
-      if (j < N) {
-        kk = Vec4<T>::load(k + base + (long long)j * st.n + 4 * c4);
-        vv = Vec4<T>::load(v + base + (long long)j * st.n + 4 * c4);
-      }
-      *reinterpret_cast<float4*>(&Ks[r][4 * c4]) = kk;
-      *reinterpret_cast<float4*>(&Vs[r][4 * c4]) = vv;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int jj = 0; jj < 32; ++jj) {
-      const int j = j0 + jj;
-      float s = 0.f;
-#pragma unroll
-      for (int c = 0; c < CH; ++c) {
-        const float4 kk = *reinterpret_cast<const float4*>(&Ks[jj][4 * (sub + 4 * c)]);
-        s += qv[c].x * kk.x + qv[c].y * kk.y + qv[c].z * kk.z + qv[c].w * kk.w;
-      }
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      s += __shfl_xor_sync(0xffffffffu, s, 2);
-      const bool valid = (i < N) && (j <= i + fwd) && (j > i - w) && (j < N);
-      if (valid) {
-        s *= scale;
-        const float m_new = fmaxf(m, s);
-        const float corr = expf(m - m_new);
-        const float p = expf(s - m_new);
-        l = l * corr + p;
-#pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          const float4 vv = *reinterpret_cast<const float4*>(&Vs[jj][4 * (sub + 4 * c)]);
-          ov[c].x = ov[c].x * corr + p * vv.x;
-          ov[c].y = ov[c].y * corr + p * vv.y;
-          ov[c].z = ov[c].z * corr + p * vv.z;
-          ov[c].w = ov[c].w * corr + p * vv.w;
-        }
-        m = m_new;
-      }
-    }
-  }
-  if (i < N) {
-    const float inv = 1.f / l;
-#pragma unroll
-    for (int c = 0; c < CH; ++c) {
-      float4 r = make_float4(ov[c].x * inv, ov[c].y * inv, ov[c].z * inv, ov[c].w * inv);
-      Vec4<T>::store(o + base + (long long)i * st.n + 4 * (sub + 4 * c), r);
-    }
-  }
-}
 
 // ------------------------------------------------------------------------------------
 // Causal linear attention, Algorithm 1 token by token.
@@ -572,20 +483,6 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
 }
 
 template <typename T>
-cudaError_t window_dispatch(const void* q, const void* k, const void* v, void* o, int B, int N, int d, int w,
-                            int fwd, float scale, Strides st, int h_begin, int h_count, cudaStream_t stream) {
-  dim3 grid((N + 31) / 32, h_count, B);
-  if (d == 64)
-    window_simt_kernel<T, 64><<<grid, 128, 0, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, N, w, fwd,
-                                                        scale, st, h_begin);
-  else
-    window_simt_kernel<T, 128><<<grid, 128, 0, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, N, w, fwd,
-                                                         scale, st, h_begin);
-  note_launch();
-  return cudaGetLastError();
-}
-
-template <typename T>
 cudaError_t linear_dispatch(const void* q, const void* k, const void* v, void* o, int B, int N, int d,
                             Strides st, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
                             bool global_sum, cudaStream_t stream, const void* W) {
@@ -631,19 +528,12 @@ cudaError_t decode_dispatch(const void* q, const void* k, const void* v, void* o
 
 }  // namespace
 
-cudaError_t launch_window_simt(const void* q, const void* k, const void* v, void* o, int B, int N, int d, int w,
-                               int fwd, float scale, int dtype, Strides st, int h_begin, int h_count,
-                               cudaStream_t stream) {
-  if (h_count <= 0 || B <= 0) return cudaSuccess;
-  if (dtype == GF_F32)
-    return window_dispatch<float>(q, k, v, o, B, N, d, w, fwd, scale, st, h_begin, h_count, stream);
-  return window_dispatch<__nv_bfloat16>(q, k, v, o, B, N, d, w, fwd, scale, st, h_begin, h_count, stream);
-}
-
 cudaError_t launch_linear_simt(const void* q, const void* k, const void* v, void* o, int B, int N, int d,
                                int dtype, Strides st, int h_begin, int h_count, float* S_io, float* z_io,
                                bool zero_init, cudaStream_t stream, bool global_sum, const void* W) {
   if (h_count <= 0 || B <= 0) return cudaSuccess;
+  if (!global_sum && W == nullptr)
+    return launch_linear_tiled(q, k, v, o, B, N, d, dtype, st, h_begin, h_count, S_io, z_io, zero_init, stream);
   if (dtype == GF_F32)
     return linear_dispatch<float>(q, k, v, o, B, N, d, st, h_begin, h_count, S_io, z_io, zero_init, global_sum,
                                   stream, W);

@@ -1148,3 +1148,30 @@ def test_favor_is_not_elu_and_needs_its_projection():
                                              B, H, N, d, gf.GF_PHI_FAVOR_POS, 0, None, None, gf.GF_BF16, gf.GF_BHND,
                                              gf.Workspace(1 << 20).ptr, 1 << 20, None)
     assert rc == gf.GF_ERR_INVALID_ARG
+
+
+# ------------------------------------------------------------------ fp32 linear heads, tiled and cut
+@pytest.mark.parametrize("bnhd", [False, True])
+@pytest.mark.parametrize("N,d", [(31, 64), (33, 128), (225, 64), (225, 128), (352, 64), (353, 64), (385, 128), (384, 64),
+                                 (2017, 128), (2048, 64), (1999, 64)])
+def test_linear_f32_blocks_and_segments(N, d, bnhd):
+    """Edges of the 32-token blocks, the first lengths that are cut into segments (the states then wait in the
+    output rows), a last block of one token, with and without a state carried in and out."""
+    B, H = 2, 3
+    q, k, v = synth.qkv(B, H, N, d, "f32", seed=900 + N, gain=1.0)
+    g = torch.Generator().manual_seed(N)
+    S0 = torch.randn(B, H, d, d, generator=g)
+    z0 = 50.0 + torch.rand(B, H, d, generator=g)
+    S_ref, z_ref = f64(S0).copy(), f64(z0).copy()
+    ref = oracle.causal_linear_attn(f64(q), f64(k), f64(v), S_ref, z_ref)
+    layout = gf.GF_BNHD if bnhd else gf.GF_BHND
+    ins = [(t.permute(0, 2, 1, 3).contiguous() if bnhd else t).cuda() for t in (q, k, v)]
+    S, z = S0.cuda(), z0.cuda()
+    o = gf.causal_linear_attn(*ins, S, z, layout=layout)
+    # a row sums at most N + d products of features: an fp32 sum of n terms is off by about sqrt(n) 2^-24 < 3e-6
+    # of their size, below the fp32 gate
+    assert_parity(f64(o.permute(0, 2, 1, 3) if bnhd else o), ref, "f32", f"f32 linear N={N} d={d}")
+    assert errors(f64(S), S_ref)["rel_l2"] <= 1e-5 and errors(f64(z), z_ref)["rel_l2"] <= 1e-5
+    fresh = oracle.causal_linear_attn(f64(q), f64(k), f64(v))
+    o = gf.causal_linear_attn(*ins, layout=layout)
+    assert_parity(f64(o.permute(0, 2, 1, 3) if bnhd else o), fresh, "f32", f"f32 linear, no state, N={N} d={d}")
