@@ -76,6 +76,7 @@ constexpr int kWaitAttempts = 1000000;      // the clock limit (about two second
 // (status=1, where) in the two words at `status`.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned int* status,
                                           unsigned int where) {
+  if (mbar_test_wait(bar, parity)) return true;  // (try_wait is slower to say yes)
   if (mbar_try_wait(bar, parity, kWaitHintNs)) return true;
   // (only now, off the fast path, a look at global memory) status[3]: the limit in units of 1024
   // cycles when a test has shortened it, else 0

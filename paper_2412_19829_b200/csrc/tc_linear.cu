@@ -46,6 +46,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "linear_phi.cuh"
 #include "sm100.cuh"
 
 namespace gf {
@@ -55,7 +56,6 @@ using namespace sm100;
 
 constexpr int kThreads = 768;  // 24 warps, 80 registers each
 constexpr int kMaxL = 32;      // most chunks per segment of a cut chain
-constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kFlagStride = 32;  // one flag per 128-byte line
 
 template <int D>
@@ -200,56 +200,6 @@ __device__ __forceinline__ bool named_bar_or(int id, int n, bool pred) {
       : "r"((uint32_t)pred), "r"(id), "r"(n)
       : "memory");
   return r != 0;
-}
-
-// phi(x) = elu(x) + 1 = max(x, 0) + exp(min(x, 0)) on two packed bf16 values (branch free; the
-// result is needed in bf16 anyway).  log2(e) is split in two bf16 terms so that the exponent
-// argument carries only the rounding of one bf16 product.
-__device__ __forceinline__ uint32_t phi_bf16x2(uint32_t w) {
-  const __nv_bfloat162 x = *reinterpret_cast<const __nv_bfloat162*>(&w);
-  const __nv_bfloat162 zero = __float2bfloat162_rn(0.f);
-  const __nv_bfloat162 l2e_hi = __float2bfloat162_rn(1.4453125f);
-  const __nv_bfloat162 l2e_lo = __float2bfloat162_rn(kLog2e - 1.4453125f);
-  const __nv_bfloat162 t = __hmin2(__hfma2(x, l2e_lo, __hmul2(x, l2e_hi)), zero);
-  uint32_t e;  // native packed exponential (the header's h2exp2 goes through two fp32 ex2 + converts)
-  asm("ex2.approx.ftz.bf16x2 %0, %1;" : "=r"(e) : "r"(*reinterpret_cast<const uint32_t*>(&t)));
-  const __nv_bfloat162 f = __hadd2(__hmax2(x, zero), *reinterpret_cast<const __nv_bfloat162*>(&e));
-  return *reinterpret_cast<const uint32_t*>(&f);
-}
-
-// kId: the tensors the kernel reads as Q and K already hold features (positive random features
-// computed by a kernel of their own): the feature map here is the identity.
-template <bool kId>
-__device__ __forceinline__ uint32_t phi_sel(uint32_t w) {
-  if constexpr (kId) return w;
-  else return phi_bf16x2(w);
-}
-
-// phi on 64 rows (four groups of 16 from k8_begin on) x one 16-byte column chunk of a K tile, in
-// place in shared memory (128B swizzle); rows past the end of the sequence become zero.
-template <bool kId>
-__device__ __forceinline__ void transform_k_rows(uint8_t* kb, int cin, int lane16, int k8_begin, int n_valid) {
-  uint4 rawv[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int row = lane16 + 16 * (k8_begin + k);
-    rawv[k] = *reinterpret_cast<const uint4*>(kb + row * 128 + ((cin ^ (row & 7)) << 4));
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int row = lane16 + 16 * (k8_begin + k);
-    const uint32_t keep = (row < n_valid) ? 0xffffffffu : 0u;
-    rawv[k].x = phi_sel<kId>(rawv[k].x) & keep;
-    rawv[k].y = phi_sel<kId>(rawv[k].y) & keep;
-    rawv[k].z = phi_sel<kId>(rawv[k].z) & keep;
-    rawv[k].w = phi_sel<kId>(rawv[k].w) & keep;
-  }
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int row = lane16 + 16 * (k8_begin + k);
-    *reinterpret_cast<uint4*>(kb + row * 128 + ((cin ^ (row & 7)) << 4)) = rawv[k];
-  }
-  fence_proxy_async_smem();
 }
 
 // Critical path of the segment hand-over, run by the 16 phi warps (4 per TMEM lane quarter, each
@@ -730,7 +680,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     // Pass A and the hand-over of S are common to the two groups (one copy of the code); in pass
     // C the Q group applies phi to Q and the K group masks P.
     const bool kgrp = warp >= 14;
-    const int tt = kgrp ? tid - 14 * 32 : tid - 6 * 32;  // 0..255 within the group
+    const int tt = kgrp ? tid - 14 * 32 : 256 + tid - 6 * 32;  // number among the threads that transform K tiles
     const int quarter = warp & 3;                        // TMEM lane quarter of this warp
     const int half = ((warp - 6) >> 2) & 1;  // Q group: half of the head dimension; K group: half of the key columns
     const int colh = half;
@@ -779,22 +729,16 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       auto transform_direct = [&](uint32_t idx, int jrow) {
         const uint32_t sl = idx % KS;
         ok = ok && mbar_wait(&bar.k_full[sl], (idx / KS) & 1, p.status, 430);
-        const int cc = tt >> 4;
-        if (ok && tt < 2 * D)
-          transform_k_rows<kId>(sK + sl * C::kTile + (cc >> 3) * C::kBoxBytes, cc & 7, tt & 15, kgrp ? 0 : 4,
-                           p.N - (it.c_begin + jrow) * 128);
+        if (ok) transform_k_tile<D, kId, 512>(sK + sl * C::kTile, tt, p.N - (it.c_begin + jrow) * 128);
         __syncwarp();
         if (ok && lane == 0) mbar_arrive(&bar.kd_phi[sl]);
       };
       if (kDirect) transform_direct(nq, 0);
-      // ---- pass A: the K group takes rows 0..63 (by sixteens) of every K tile, the Q group rows 64..127
+      // ---- pass A: the two groups take half of every K tile each
       for (int j = 0; j < (kDirect ? 0 : it.nC); ++j) {
         const uint32_t sk = ta % KA;
         ok = ok && mbar_wait(&bar.ka_full[sk], (ta / KA) & 1, p.status, 410);
-        const int cc = tt >> 4;  // logical 16-byte column chunk 0 .. D/8-1
-        if (ok && tt < 2 * D)
-          transform_k_rows<kId>(a_kslot(sk) + (cc >> 3) * C::kBoxBytes, cc & 7, tt & 15, kgrp ? 0 : 4,
-                           p.N - (it.c_begin + j) * 128);
+        if (ok) transform_k_tile<D, kId, 512>(a_kslot(sk), tt, p.N - (it.c_begin + j) * 128);
         __syncwarp();
         if (ok && lane == 0) mbar_arrive(&bar.kphi_full[sk]);  // the tile may go to the tensor core and be parked
         ++ta;
@@ -811,8 +755,6 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         // ---- pass C: causal mask inside the chunk, bf16 back into TMEM.
         //      This warp owns rows [32 q, 32 q + 32) x key columns [64 colh, 64 colh + 64).
         for (int j = 0; j < it.nC; ++j) {
-          // kDirect: this group's half of the next chunk's K tile, while the tensor core forms P
-          if (kDirect && j + 1 < it.nC) transform_direct(nq + 1, j + 1);
           if (!ok || !mbar_wait(&bar.p_full, nq & 1, p.status, 301)) { ok = false; break; }
           tc_fence_after_sync();
 #pragma unroll 1
@@ -843,6 +785,11 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           tmem_wait_st();
           tc_fence_before_sync();
           mbar_arrive(&bar.pm_full);
+          // kDirect: this group's half of the next chunk's K tile, between the mask, which the tensor core waits for,
+          // and the state, which waits for the tensor core (before the mask it held that back until the tile had
+          // landed: 26 chains of 32K tokens, d = 128, 669 -> 642 us; 80 x 2048, d = 64, 40 -> 38 us)
+          if (kDirect && j + 1 < it.nC) transform_direct(nq + 1, j + 1);
+          if (!ok) break;
           // ---- S: the fp32 master stays in TMEM; once this chunk's readout has consumed the old
           //      bf16 copy, stream the new one (and z) into shared memory for the next chunk.
           //      This warp: rows [32 q, 32 q + 32) x columns [colh D/2, colh D/2 + D/2).
