@@ -13,6 +13,9 @@
 //            then per chunk: Q tile by TMA, phi(Q) into TMEM (8 warps), one product with
 //            N = D + 16 leaves the numerators and, in columns D and D + 1, the denominator split
 //            in two; 4 epilogue warps divide, pack and stage the tile for a TMA store.
+// At D = 64, where shared memory has room for both halves, and with chains enough for the SMs (or chains that are
+// short), one launch does it all:
+//   whole    a CTA takes whole chains; it sums chain c + 1 while it reads out chain c
 // Every wait is bounded; on expiry the kernel records a status word and drains.
 #include "common.cuh"
 #include "linear_phi.cuh"
@@ -498,6 +501,337 @@ linear_self_readout_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
   if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
+// ------------------------------------------------------------------------------------ whole
+// Both halves in one CTA, D = 64: the sums of a chain never leave the SM.  Warps: 0 K/V producer, 1 issuer of the
+// sums, 2-5 epilogue, 6-13 phi(Q), 14-21 phi(K), 22 Q producer, 23 issuer of the readout, 24-25 totals from TMEM into
+// the bf16 B operand (D = 64 feature rows: TMEM lane quarters 0 and 1), 26 output stores.  Accumulators, totals, Q,
+// phi(Q), O and staging are all double-buffered, so the two halves run side by side, a chain apart.
+// What bounds it is the memory system, as in the kernels above, but a chain's start-up and its totals are hidden
+// behind the chain before: 640 chains of 197 tokens take 20.5 us, in three launches 46.5 (16, 6 and 24: the totals of
+// an item are loaded when it begins, which for items of two chunks is most of their time).
+struct WholeCfg {
+  static constexpr int D = 64, kTile = 128 * D * 2;
+  static constexpr int kVSlots = 4, kKSlots = 3;  // V0 V1 V2 V3 ONES, as in RedCfg<64>
+  static constexpr int kOnes = 4 * kBox, kK = 5 * kBox, kQ = kK + kKSlots * kTile;
+  static constexpr int kSb = kQ + 2 * kTile;      // two times [64 rows][64 columns] of totals + the box of hi(z), lo(z)
+  static constexpr int kSbBox = D * 128, kSbSlot = 2 * kSbBox;
+  static constexpr int kStage = kSb + 2 * kSbSlot;
+  static constexpr int kBytes = kStage + 2 * kTile + 1024;
+  static constexpr int kAcc = D + 16;
+  static constexpr uint32_t tAcc = 0, tQ = 2 * kAcc, tO = tQ + D;  // two accumulators, two phi(Q), two O
+  static constexpr int kThreads = 27 * 32;
+};
+
+template <bool kId>
+__global__ void __launch_bounds__(WholeCfg::kThreads, 1)
+linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
+                         const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtensorMap mo,
+                         const SelfParams p) {
+  using C = WholeCfg;
+  constexpr int D = C::D, VS = C::kVSlots, KS = C::kKSlots;
+  extern __shared__ uint8_t raw_smem[];
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw_smem) + 1023) & ~(uintptr_t)1023);
+  __shared__ __align__(8) uint64_t k_full[KS], kphi[KS], k_free[KS], v_full[VS], v_free[VS], acc_done[2], acc_free[2],
+      q_full[2], q_free[2], qphi_full[2], tq_free[2], o_full[2], o_free[2], sb_ready[2], sb_free[2], o_staged[2],
+      stage_free[2];
+  __shared__ uint32_t tmem_base_s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+  if (tid == 0) {
+    atomicAdd(&p.status[5], 1u);  // WsHeader::placed: this CTA has an SM
+    for (int i = 0; i < KS; ++i) {
+      mbar_init(&k_full[i], 1);
+      mbar_init(&kphi[i], 8);
+      mbar_init(&k_free[i], 1);
+    }
+    for (int i = 0; i < VS; ++i) {
+      mbar_init(&v_full[i], 1);
+      mbar_init(&v_free[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&acc_done[i], 1);
+      mbar_init(&acc_free[i], 2);
+      mbar_init(&q_full[i], 1);
+      mbar_init(&q_free[i], 8);
+      mbar_init(&qphi_full[i], 8);
+      mbar_init(&tq_free[i], 1);
+      mbar_init(&o_full[i], 1);
+      mbar_init(&o_free[i], 128);
+      mbar_init(&sb_ready[i], 64);
+      mbar_init(&sb_free[i], 1);
+      mbar_init(&o_staged[i], 128);
+      mbar_init(&stage_free[i], 1);
+    }
+    mbar_fence_init();
+    tma_prefetch_desc(&mq);
+    tma_prefetch_desc(&mk);
+    tma_prefetch_desc(&mv);
+    tma_prefetch_desc(&mo);
+  }
+  if (warp == 1) {
+    tmem_alloc(&tmem_base_s, 512);
+    tmem_relinquish();
+  } else if (warp >= 2) {
+    // constant ones box, as in the reduce kernel
+    for (int i = tid - 64; i < kBox / 4; i += C::kThreads - 64) {
+      const int row = i >> 5, w = i & 31;
+      reinterpret_cast<uint32_t*>(sm + C::kOnes)[i] = (w == ((row & 7) << 2)) ? 0x00003F80u : 0u;
+    }
+    fence_proxy_async_smem();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem = tmem_base_s;
+
+  // Every role walks the chains blockIdx.x, blockIdx.x + gridDim.x, ... (an item is a whole chain) and keeps the same
+  // running counters: n = chunks so far, c = chains so far.
+  if (warp == 0 || warp == 22) {
+    if (elect_one()) {
+      const bool kv = warp == 0;
+      const uint64_t pol = l2_policy_evict_first();
+      uint32_t n = 0;
+      bool ok = true;
+      for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+        const SelfItem it = self_item(p, item);
+        for (int j = 0; j < it.nC; ++j, ++n) {
+          if (kv) {
+            const uint32_t sk = n % KS, sv = n % VS;
+            if (n >= KS && !mbar_wait(&k_free[sk], ((n / KS) + 1) & 1, p.status, 900)) { ok = false; break; }
+            mbar_arrive_expect_tx(&k_full[sk], C::kTile);
+            tma_load_4d_hint(sm + C::kK + sk * C::kTile, &mk, &k_full[sk], 0, j * 128, it.h, it.b, pol);
+            if (n >= VS && !mbar_wait(&v_free[sv], ((n / VS) + 1) & 1, p.status, 901)) { ok = false; break; }
+            mbar_arrive_expect_tx(&v_full[sv], C::kTile);
+            tma_load_4d_hint(sm + sv * kBox, &mv, &v_full[sv], 0, j * 128, it.h, it.b, pol);
+          } else {
+            const uint32_t s = n & 1;
+            if (n >= 2 && !mbar_wait(&q_free[s], ((n >> 1) + 1) & 1, p.status, 902)) { ok = false; break; }
+            mbar_arrive_expect_tx(&q_full[s], C::kTile);
+            tma_load_4d_hint(sm + C::kQ + s * C::kTile, &mq, &q_full[s], 0, j * 128, it.h, it.b, pol);
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (elect_one()) {
+      constexpr uint32_t id_s = umma_idesc_bf16(128, C::kAcc, true, true);  // [S | z] += Kc^T [V | 1]
+      uint32_t n = 0, c = 0;
+      bool ok = true;
+      for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x, ++c) {
+        const SelfItem it = self_item(p, item);
+        const uint32_t acc = tmem + C::tAcc + (c & 1) * C::kAcc;
+        if (c >= 2 && !mbar_wait(&acc_free[c & 1], ((c >> 1) + 1) & 1, p.status, 910)) break;
+        for (int j = 0; j < it.nC; ++j, ++n) {
+          const uint32_t sk = n % KS, sv = n % VS;
+          if (!mbar_wait(&kphi[sk], (n / KS) & 1, p.status, 911) || !mbar_wait(&v_full[sv], (n / VS) & 1, p.status, 912)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after_sync();
+          const uint32_t kbase = smem_u32(sm) + C::kK + sk * C::kTile, vbase = smem_u32(sm) + sv * kBox;
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks)  // (rows 64..127 of the product mirror 0..63)
+            umma_ss(acc, umma_smem_desc(kbase + ks * 2048, 0, 1024),
+                    umma_smem_desc(vbase + ks * 2048, (4 - sv) * kBox, 1024), id_s, (j > 0) || (ks > 0));
+          umma_commit(&k_free[sk]);
+          umma_commit(&v_free[sv]);
+        }
+        if (!ok) break;
+        umma_commit(&acc_done[c & 1]);
+      }
+    }
+  } else if (warp == 23) {
+    if (elect_one()) {
+      constexpr uint32_t id_o = umma_idesc_bf16(128, C::kAcc, false, true);  // [O | den] = Qc [Sb | Zb]
+      uint32_t n = 0, c = 0;
+      bool ok = true;
+      for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x, ++c) {
+        const SelfItem it = self_item(p, item);
+        if (!mbar_wait(&sb_ready[c & 1], (c >> 1) & 1, p.status, 920)) break;
+        const uint32_t sb = smem_u32(sm) + C::kSb + (c & 1) * C::kSbSlot;
+        for (int j = 0; j < it.nC; ++j, ++n) {
+          const uint32_t s = n & 1;
+          if (!mbar_wait(&qphi_full[s], (n >> 1) & 1, p.status, 921) ||
+              (n >= 2 && !mbar_wait(&o_free[s], ((n >> 1) + 1) & 1, p.status, 922))) {
+            ok = false;
+            break;
+          }
+          tc_fence_after_sync();
+          const uint32_t tq = tmem + C::tQ + s * (D / 2), to = tmem + C::tO + s * C::kAcc;
+#pragma unroll
+          for (int ks = 0; ks < D / 16; ++ks)
+            umma_ts(to, tq + ks * 8, umma_smem_desc(sb + ks * 2048, C::kSbBox, 1024), id_o, ks > 0);
+          umma_commit(&o_full[s]);
+          umma_commit(&tq_free[s]);
+        }
+        if (!ok) break;
+        umma_commit(&sb_free[c & 1]);
+      }
+    }
+  } else if (warp < 6) {
+    // epilogue: one thread per row
+    const int quarter = warp & 3, r = quarter * 32 + lane;
+    const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
+    uint32_t n = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+      for (int j = 0; j < p.nch; ++j, ++n) {
+        const uint32_t s = n & 1;
+        if (!mbar_wait(&o_full[s], (n >> 1) & 1, p.status, 930) ||
+            (n >= 2 && !mbar_wait(&stage_free[s], ((n >> 1) + 1) & 1, p.status, 931))) {
+          ok = false;
+          break;
+        }
+        tc_fence_after_sync();
+        const uint32_t to = tmem + C::tO + s * C::kAcc + lane_off;
+        uint32_t den_hi, den_lo;
+        tmem_ld2(to + D, den_hi, den_lo);
+        tmem_wait_ld();
+        const float inv = 1.f / (__uint_as_float(den_hi) + __uint_as_float(den_lo));
+#pragma unroll 1
+        for (int cc = 0; cc < D / 32; ++cc) {
+          uint32_t v[32];
+          tmem_ld32(to + cc * 32, v);
+          tmem_wait_ld();
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            uint4 val;
+            val.x = pack_bf16(__uint_as_float(v[8 * g + 0]) * inv, __uint_as_float(v[8 * g + 1]) * inv);
+            val.y = pack_bf16(__uint_as_float(v[8 * g + 2]) * inv, __uint_as_float(v[8 * g + 3]) * inv);
+            val.z = pack_bf16(__uint_as_float(v[8 * g + 4]) * inv, __uint_as_float(v[8 * g + 5]) * inv);
+            val.w = pack_bf16(__uint_as_float(v[8 * g + 6]) * inv, __uint_as_float(v[8 * g + 7]) * inv);
+            *reinterpret_cast<uint4*>(sm + C::kStage + s * C::kTile + swz128_offset(r, cc * 32 + g * 8)) = val;
+          }
+        }
+        tc_fence_before_sync();
+        mbar_arrive(&o_free[s]);
+        fence_proxy_async_smem();
+        mbar_arrive(&o_staged[s]);
+      }
+    }
+  } else if (warp < 14) {
+    // phi(Q): thread = (row, half of the head dimension); the result is the A operand in TMEM
+    const int quarter = warp & 3, half = ((warp - 6) >> 2) & 1, r = quarter * 32 + lane;
+    const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
+    constexpr int kChunks = D / 16;  // 16-byte chunks of one row half
+    uint32_t n = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+      for (int j = 0; j < p.nch && ok; ++j, ++n) {
+        const uint32_t s = n & 1;
+        ok = mbar_wait(&q_full[s], (n >> 1) & 1, p.status, 940);
+        uint32_t pk[kChunks * 4];
+        if (ok) {
+#pragma unroll
+          for (int g = 0; g < kChunks; ++g) {
+            const int cin = half * kChunks + g;
+            const uint4 rawv =
+                *reinterpret_cast<const uint4*>(sm + C::kQ + s * C::kTile + r * 128 + ((cin ^ (r & 7)) << 4));
+            pk[g * 4 + 0] = rawv.x;
+            pk[g * 4 + 1] = rawv.y;
+            pk[g * 4 + 2] = rawv.z;
+            pk[g * 4 + 3] = rawv.w;
+          }
+        }
+        // the buffer goes back to the TMA engine: these reads (generic proxy) must be ordered before its
+        // next write (async proxy), which a barrier arrival alone does not do
+        __threadfence_block();
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (ok && lane == 0) mbar_arrive(&q_free[s]);
+        if (ok) {
+#pragma unroll
+          for (int w = 0; w < kChunks * 4; ++w) pk[w] = phi_sel<kId>(pk[w]);
+          if (n >= 2) ok = mbar_wait(&tq_free[s], ((n >> 1) + 1) & 1, p.status, 941);
+        }
+        tc_fence_after_sync();
+        if (ok) {
+          tmem_st16(tmem + C::tQ + s * (D / 2) + lane_off + half * 16, pk);
+          tmem_wait_st();
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&qphi_full[s]);
+        }
+        ok = !__any_sync(0xffffffffu, !ok);
+      }
+    }
+  } else if (warp < 22) {
+    uint32_t n = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+      for (int j = 0; j < p.nch; ++j, ++n) {
+        const uint32_t sk = n % KS;
+        ok = ok && mbar_wait(&k_full[sk], (n / KS) & 1, p.status, 950);
+        if (ok) transform_k_tile<D, kId, 256>(sm + C::kK + sk * C::kTile, tid - 14 * 32, p.N - j * 128);
+        __syncwarp();
+        if (ok && lane == 0) mbar_arrive(&kphi[sk]);
+      }
+    }
+  } else if (warp < 26) {
+    // totals: one thread per feature row
+    const int quarter = warp & 3, r = quarter * 32 + lane;  // 0..63
+    const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
+    uint32_t c = 0;
+    for (int item = blockIdx.x; item < p.nitems; item += gridDim.x, ++c) {
+      const uint32_t s = c & 1;
+      bool ok = mbar_wait(&acc_done[s], (c >> 1) & 1, p.status, 960) &&
+                (c < 2 || mbar_wait(&sb_free[s], ((c >> 1) + 1) & 1, p.status, 961));
+      if (__any_sync(0xffffffffu, !ok)) break;
+      tc_fence_after_sync();
+      const uint32_t acc = tmem + C::tAcc + s * C::kAcc + lane_off;
+      uint8_t* sb = sm + C::kSb + s * C::kSbSlot;
+#pragma unroll 1
+      for (int cc = 0; cc < D / 32; ++cc) {
+        uint32_t v[32];
+        tmem_ld32(acc + cc * 32, v);
+        tmem_wait_ld();
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          uint4 val;
+          val.x = pack_bf16(__uint_as_float(v[8 * g + 0]), __uint_as_float(v[8 * g + 1]));
+          val.y = pack_bf16(__uint_as_float(v[8 * g + 2]), __uint_as_float(v[8 * g + 3]));
+          val.z = pack_bf16(__uint_as_float(v[8 * g + 4]), __uint_as_float(v[8 * g + 5]));
+          val.w = pack_bf16(__uint_as_float(v[8 * g + 6]), __uint_as_float(v[8 * g + 7]));
+          *reinterpret_cast<uint4*>(sb + swz128_offset(r, cc * 32 + g * 8)) = val;
+        }
+      }
+      const float z = __uint_as_float(tmem_ld1(acc + D));
+      tmem_wait_ld();
+      const float hi = __bfloat162float(__float2bfloat16_rn(z));
+      // row r of the box behind: columns 0, 1 = hi(z), lo(z); the other 14 columns the product reads are zero
+      *reinterpret_cast<uint4*>(sb + C::kSbBox + swz128_offset(r, 0)) = make_uint4(pack_bf16(hi, z - hi), 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(sb + C::kSbBox + swz128_offset(r, 8)) = make_uint4(0u, 0u, 0u, 0u);
+      tc_fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&acc_free[s]);
+      fence_proxy_async_smem();
+      mbar_arrive(&sb_ready[s]);
+    }
+  } else {
+    // TMA stores of the staged output tiles
+    if (elect_one()) {
+      uint32_t n = 0;
+      bool ok = true;
+      const uint64_t pol = l2_policy_evict_first();
+      for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+        const SelfItem it = self_item(p, item);
+        for (int j = 0; j < it.nC; ++j, ++n) {
+          const uint32_t s = n & 1;
+          if (!mbar_wait(&o_staged[s], (n >> 1) & 1, p.status, 970)) { ok = false; break; }
+          tma_store_4d_hint(&mo, sm + C::kStage + s * C::kTile, 0, j * 128, it.h, it.b, pol);
+          tma_store_commit();
+          tma_store_wait_read<0>();
+          mbar_arrive(&stage_free[s]);
+        }
+      }
+      tma_store_wait_all<0>();
+    }
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 1) tmem_dealloc(tmem, 512);
+}
+
 // Segments per chain.  CTAs take items (segments) round-robin, so a launch lasts ceil(items / CTAs)
 // rounds of one item each: among the segment counts that keep segments at least four chunks long
 // (and the scratch within 64 slots per chain, more when the chains are few), take the one with the least rounds x (chunks of the
@@ -520,6 +854,16 @@ int self_segments(int nchains, int nch) {
     }
   }
   return best_g;
+}
+
+// Whether whole chains go through linear_self_whole_kernel: its ceil(chains / CTAs) rounds of a whole chain each against
+// the three launches, whose work is spread evenly but costs a sixth more per chunk (its two halves do not run side by
+// side) and about nine chunks' time in launches and start-up.  Measured, whole against three launches: 128 chains of
+// 1024 tokens 20.5 and 30.8 us, 256 of 4096 102 and 127, 160 of 4096 89.0 and 92.1 (three launches), 24 of 197 10.3 and 19.7.
+bool self_whole(int nchains, int nch, int d, int sms) {
+  if (d != WholeCfg::D) return false;
+  const double rounds = (double)((nchains + sms - 1) / sms) * nch;
+  return rounds <= 1.17 * nchains * nch / sms + 9.0;
 }
 
 }  // namespace
@@ -551,19 +895,27 @@ cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, v
   p.h_begin = h_begin;
   p.h_count = h_count;
   p.nchains = B * h_count;
-  p.G = self_segments(p.nchains, p.nch);
+  int dev = 0, sms = 0;
+  cudaError_t e;
+  if ((e = device_info(&dev, &sms)) != cudaSuccess) return e;
+  const bool whole = self_whole(p.nchains, p.nch, d, sms);
+  p.G = whole ? 1 : self_segments(p.nchains, p.nch);
   p.seg_base = p.nch / p.G;
   p.seg_rem = p.nch % p.G;
   p.nitems = p.nchains * p.G;
   const int state_floats = d * d + d;
   p.partial = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(ws) + scratch_offset);
-  p.total = p.partial + (size_t)p.nitems * state_floats;
+  p.total = p.G == 1 ? p.partial : p.partial + (size_t)p.nitems * state_floats;  // one segment: its sum is the total
   p.status = &ws->status;
-  int dev = 0, sms = 0;
-  cudaError_t e;
-  if ((e = device_info(&dev, &sms)) != cudaSuccess) return e;
   dim3 grid(p.nitems < sms ? p.nitems : sms);
   if (first_grid) *first_grid = (int)grid.x;
+  if (whole) {
+    auto kern = features ? linear_self_whole_kernel<true> : linear_self_whole_kernel<false>;
+    if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, WholeCfg::kBytes)) != cudaSuccess) return e;
+    kern<<<grid, WholeCfg::kThreads, WholeCfg::kBytes, stream>>>(mq, mk, mv, mo, p);
+    note_launch();
+    return cudaGetLastError();
+  }
   auto launch_red = [&](auto kern, int smem, int threads) -> cudaError_t {
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem);
     if (err != cudaSuccess) return err;
@@ -584,9 +936,11 @@ cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, v
                   : launch_red(linear_self_reduce_kernel<128, false>, RedCfg<128>::kBytes, RedCfg<128>::kThreads);
   if (e != cudaSuccess) return e;
   note_launch();
-  linear_self_sum_kernel<<<dim3((state_floats / 4 + 255) / 256, p.nchains), 256, 0, stream>>>(p.partial, p.total, p.G,
-                                                                                              state_floats);
-  note_launch();
+  if (p.G > 1) {
+    linear_self_sum_kernel<<<dim3((state_floats / 4 + 255) / 256, p.nchains), 256, 0, stream>>>(p.partial, p.total, p.G,
+                                                                                                state_floats);
+    note_launch();
+  }
   if (features)
     e = (d == 64) ? launch_out(linear_self_readout_kernel<64, true>, OutCfg<64>::kBytes, OutCfg<64>::kThreads)
                   : launch_out(linear_self_readout_kernel<128, true>, OutCfg<128>::kBytes, OutCfg<128>::kThreads);

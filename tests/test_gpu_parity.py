@@ -1175,3 +1175,23 @@ def test_linear_f32_blocks_and_segments(N, d, bnhd):
     fresh = oracle.causal_linear_attn(f64(q), f64(k), f64(v))
     o = gf.causal_linear_attn(*ins, layout=layout)
     assert_parity(f64(o.permute(0, 2, 1, 3) if bnhd else o), fresh, "f32", f"f32 linear, no state, N={N} d={d}")
+
+
+# ------------------------------------------------------------------ bidirectional linear heads, whole chains in one launch
+@pytest.mark.parametrize("favor", [False, True])
+@pytest.mark.parametrize("B,H,N,d", [(1, 1, 1, 64), (1, 3, 127, 64), (2, 2, 128, 64), (3, 150, 129, 64), (5, 100, 197, 64),
+                                     (2, 75, 700, 64), (1, 149, 1025, 64), (3, 150, 129, 128), (1, 5, 300, 128)])
+def test_self_linear_heads_whole_chains(B, H, N, d, favor):
+    """Chains of 1 to 9 chunks, one to several per CTA (every double buffer wraps), ragged ends; at d = 128 one segment
+    per chain, whose sum is the total.  Sampled heads against the oracle; the rest must be finite."""
+    gain = None if favor else 1.0
+    q, k, v = synth.qkv(B, H, N, d, "bf16", seed=950 + N + H, gain=gain)
+    W = _proj(H, d, "bf16", 3) if favor else None
+    ws = gf.Workspace.for_problem(B, H, N, d, 1, 0, phi=gf.GF_PHI_FAVOR_POS if favor else gf.GF_PHI_ELU1)
+    o = gf.hybrid_attn_self(*dev(q, k, v), 16, h_sparse=0, ws=ws, W=W.cuda() if favor else None).cpu()
+    assert ws.last_device_status() == gf.GF_OK
+    assert torch.isfinite(o.float()).all()
+    hs = sorted({0, H // 2, H - 1})
+    ref = oracle.hybrid_attn_self(f64(q[:, hs]), f64(k[:, hs]), f64(v[:, hs]), 16, h_sparse=0,
+                                  **({"W": f64(W[hs])} if favor else {}))
+    assert_parity(f64(o[:, hs]), ref, "bf16", f"whole chains B={B} H={H} N={N} d={d}")
