@@ -9,11 +9,14 @@
 // and their products with the state stay inside the range of fp32 however small the key features
 // are.  The key features (and with them the state S, z) are the definition's.
 //
-// One CTA = 128 tokens of one (batch, head) of Q or of K: the token tile X (128 x d) and the head's
-// projection W (d x d, row a = w_a) come by TMA; one tcgen05.mma group computes Y = X W^T
-// (M = 128, N = d, K = d, both operands K-major from shared memory) into TMEM; 128 threads, one per
-// token, add up |x|^2 from the tile in shared memory, take the exponentials and write the features
-// over the tile, which a TMA store ships (rows past the end of the sequence are clipped).
+// A CTA (two per SM) takes a run of consecutive 128-token tiles of Q, then of K, in (head, tile) order, so that a head's
+// projection W (d x d, row a = w_a) is loaded once for many tiles.  Per tile X (128 x d, by TMA into one of two
+// buffers): one tcgen05.mma group computes Y = X W^T (M = 128, N = d, K = d, both operands K-major from shared
+// memory) into one of two TMEM buffers; 128 threads, one per token (a group of four warps for each buffer), take
+// the exponentials and write the features over the tile, which a TMA store ships (rows past the end of the sequence
+// are clipped).  Bound by the memory system: X in and features out once each.  26 heads of 32K tokens, d = 128:
+// 156 us = 5.6 TB/s (L2 eviction hints on either side make it slower); one CTA per tile, which loaded W with every tile and did load, product,
+// exponentials and store one after the other, took 181.
 #include "common.cuh"
 #include "sm100.cuh"
 
@@ -22,108 +25,184 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kFavorThreads = 192;  // warp 0: TMA, warp 1: MMA, warps 2..5: one thread per token
+constexpr int kFavorThreads = 11 * 32;  // warps 0-7: two groups of one thread per token, 8: loads, 9: products, 10: stores
 constexpr float kLog2eF = 1.4426950408889634f;
 
 struct FavorParams {
   int h_begin, h_count;  // heads [h_begin, h_begin + h_count) of the input tensors
+  int ntile;             // 128-token tiles of a head
+  long long rows;        // (batch, head) pairs; tiles are numbered Q first, then K: 2 x rows x ntile
   unsigned int* status;
 };
 
 template <int D>
-__global__ void __launch_bounds__(kFavorThreads)
+struct FavorCfg {
+  static constexpr int kTile = 128 * D * 2, kW = D * D * 2;
+  static constexpr int kBytes = 2 * kTile + kW + 1024;
+};
+
+template <int D>
+__global__ void __launch_bounds__(kFavorThreads, 2)
 favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__ CUtensorMap mxk,
                 const __grid_constant__ CUtensorMap mw, const __grid_constant__ CUtensorMap mfq,
                 const __grid_constant__ CUtensorMap mfk, const FavorParams p) {
-  constexpr int kTile = 128 * D * 2, kW = D * D * 2;
+  using C = FavorCfg<D>;
   extern __shared__ __align__(1024) uint8_t raw_smem[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw_smem) + 1023) & ~(uintptr_t)1023);
-  uint8_t* sX = sm;
-  uint8_t* sW = sm + kTile;
-  __shared__ __align__(8) uint64_t full, done;
+  uint8_t* sW = sm + 2 * C::kTile;
+  __shared__ __align__(8) uint64_t x_full[2], x_free[2], w_full, w_free, y_full[2], y_free[2], staged[2];
   __shared__ uint32_t tmem_base_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // (the (batch, head) index is the x coordinate of the grid, which has the range for it)
-  const int i0 = blockIdx.y * 128;
-  const int hl = blockIdx.x % p.h_count, b = blockIdx.x / p.h_count;
-  const bool is_k = blockIdx.z != 0;
-  const CUtensorMap* mx = is_k ? &mxk : &mxq;
-  const CUtensorMap* mf = is_k ? &mfk : &mfq;
   if (tid == 0) {
-    mbar_init(&full, 1);
-    mbar_init(&done, 1);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&x_full[i], 1);
+      mbar_init(&x_free[i], 1);
+      mbar_init(&y_full[i], 1);
+      mbar_init(&y_free[i], 128);
+      mbar_init(&staged[i], 128);
+    }
+    mbar_init(&w_full, 1);
+    mbar_init(&w_free, 1);
     mbar_fence_init();
-    tma_prefetch_desc(mx);
+    tma_prefetch_desc(&mxq);
+    tma_prefetch_desc(&mxk);
     tma_prefetch_desc(&mw);
-    tma_prefetch_desc(mf);
+    tma_prefetch_desc(&mfq);
+    tma_prefetch_desc(&mfk);
   }
-  if (warp == 1) {
-    tmem_alloc(&tmem_base_s, D);
+  if (warp == 9) {
+    tmem_alloc(&tmem_base_s, 2 * D);
     tmem_relinquish();
   }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
-  if (warp == 0) {
+
+  // This CTA's tiles [t0, t1); tile number n of the CTA lives in buffers n & 1.
+  const long long total = 2 * p.rows * p.ntile;
+  const long long t0 = total * blockIdx.x / gridDim.x, t1 = total * (blockIdx.x + 1) / gridDim.x;
+  struct Tile {
+    bool is_k;
+    int row, hl, b, i0;  // row: (batch, head) pair; W changes with hl
+  };
+  auto tile_at = [&](long long t) {
+    Tile x;
+    const long long r = t / p.ntile;
+    x.is_k = r >= p.rows;
+    x.row = (int)(x.is_k ? r - p.rows : r);
+    x.hl = x.row % p.h_count;
+    x.b = x.row / p.h_count;
+    x.i0 = (int)(t - r * p.ntile) * 128;
+    return x;
+  };
+  if (warp == 8) {
     if (elect_one()) {
-      mbar_arrive_expect_tx(&full, kTile + kW);
-      for (int c = 0; c < D / 64; ++c) {
-        tma_load_4d(sX + c * 16384, mx, &full, c * 64, i0, p.h_begin + hl, b);
-        tma_load_4d(sW + c * (D * 128), &mw, &full, c * 64, 0, hl, 0);
+      int have = -1;       // head whose W is loaded
+      uint32_t loads = 0;  // of W
+      uint32_t n = 0;
+      for (long long t = t0; t < t1; ++t, ++n) {
+        const Tile x = tile_at(t);
+        const uint32_t s = n & 1;
+        if (n >= 2 && !mbar_wait(&x_free[s], ((n >> 1) + 1) & 1, p.status, 900)) break;
+        mbar_arrive_expect_tx(&x_full[s], C::kTile);
+        for (int c = 0; c < D / 64; ++c)
+          tma_load_4d(sm + s * C::kTile + c * 16384, x.is_k ? &mxk : &mxq, &x_full[s], c * 64, x.i0, p.h_begin + x.hl, x.b);
+        if (x.hl != have) {  // the products with the old one are done
+          if (loads >= 1 && !mbar_wait(&w_free, (loads - 1) & 1, p.status, 901)) break;
+          mbar_arrive_expect_tx(&w_full, C::kW);
+          for (int c = 0; c < D / 64; ++c) tma_load_4d(sW + c * (D * 128), &mw, &w_full, c * 64, 0, x.hl, 0);
+          have = x.hl;
+          ++loads;
+        }
       }
     }
-  } else if (warp == 1) {
+  } else if (warp == 9) {
     if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc_bf16(128, D, false, false);
-      if (mbar_wait(&full, 0, p.status, 900)) {
+      int have = -1;
+      uint32_t loads = 0, n = 0;
+      for (long long t = t0; t < t1; ++t, ++n) {
+        const int hl = tile_at(t).hl;
+        const uint32_t s = n & 1;
+        if (hl != have) {
+          if (!mbar_wait(&w_full, loads & 1, p.status, 902)) break;
+          have = hl;
+          ++loads;
+        }
+        if (!mbar_wait(&x_full[s], (n >> 1) & 1, p.status, 903)) break;
+        if (n >= 2 && !mbar_wait(&y_free[s], ((n >> 1) + 1) & 1, p.status, 904)) break;
         tc_fence_after_sync();
+        const uint32_t xb = smem_u32(sm) + s * C::kTile, wb = smem_u32(sW);
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          umma_ss(tmem, umma_smem_desc(smem_u32(sX) + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024),
-                  umma_smem_desc(smem_u32(sW) + (ks >> 2) * (D * 128) + (ks & 3) * 32, 16, 1024), idesc, ks > 0);
-        umma_commit(&done);
+          umma_ss(tmem + s * D, umma_smem_desc(xb + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024),
+                  umma_smem_desc(wb + (ks >> 2) * (D * 128) + (ks & 3) * 32, 16, 1024), idesc, ks > 0);
+        umma_commit(&y_full[s]);
+        if (t + 1 < t1 && tile_at(t + 1).hl != hl) umma_commit(&w_free);
       }
     }
+  } else if (warp == 10) {
+    if (elect_one()) {
+      uint32_t n = 0;
+      for (long long t = t0; t < t1; ++t, ++n) {
+        const Tile x = tile_at(t);
+        const uint32_t s = n & 1;
+        if (!mbar_wait(&staged[s], (n >> 1) & 1, p.status, 905)) break;
+        for (int c = 0; c < D / 64; ++c)
+          tma_store_4d(x.is_k ? &mfk : &mfq, sm + s * C::kTile + c * 16384, c * 64, x.i0, p.h_begin + x.hl, x.b);
+        tma_store_commit();
+        tma_store_wait_read<0>();
+        mbar_arrive(&x_free[s]);
+      }
+      tma_store_wait_all<0>();
+    }
   } else {
+    const uint32_t s = warp >> 2;  // this group's buffer: every second tile of the CTA
     const int quarter = warp & 3;  // TMEM lane quarter this warp may touch
     const int r = quarter * 32 + lane;
-    const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
-    const bool ok = mbar_wait(&done, 0, p.status, 901);  // the products are done: X is no longer read by the tensor core
-    tc_fence_after_sync();
-    if (ok) {
-      // |x|^2 of this thread's token from the tile (128-byte swizzle: 16-byte chunks)
-      float n2 = 0.f;
-#pragma unroll
-      for (int c8 = 0; c8 < D / 8; ++c8) {
-        const uint4 v4 = *reinterpret_cast<const uint4*>(sX + (c8 >> 3) * 16384 + swz128_offset(r, (c8 & 7) * 8));
-        const uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w4[e]));
-          n2 = fmaf(f.x, f.x, n2);
-          n2 = fmaf(f.y, f.y, n2);
-        }
-      }
-      // keys: exp(y - n2 / 2) / sqrt(d) = 2^((y - n2 / 2) log2(e) - log2(d) / 2);
+    const uint32_t ty = tmem + s * D + ((uint32_t)(quarter * 32) << 16);
+    uint8_t* sX = sm + s * C::kTile;
+    uint32_t round = 0;
+    for (long long t = t0 + s; t < t1; t += 2, ++round) {
+      const bool is_k = tile_at(t).is_k;
+      // the products are done: X is no longer read by the tensor core
+      const bool ok = mbar_wait(&y_full[s], round & 1, p.status, 906);
+      if (__any_sync(0xffffffffu, !ok)) break;
+      tc_fence_after_sync();
+      // keys: exp(y - |x|^2 / 2) / sqrt(d) = 2^((y - |x|^2 / 2) log2(e) - log2(d) / 2);
       // queries: exp(y - max_a y) (the row's factor cancels in the output)
-      float shift = -0.5f * n2 * kLog2eF - 0.5f * log2f((float)D);
-      if (!is_k) {
-        float mx = -INFINITY;
+      float shift;
+      if (is_k) {  // |x|^2 of this thread's token from the tile (128-byte swizzle: 16-byte chunks)
+        float n2[2] = {0.f, 0.f};
 #pragma unroll
+        for (int c8 = 0; c8 < D / 8; ++c8) {
+          const uint4 v4 = *reinterpret_cast<const uint4*>(sX + (c8 >> 3) * 16384 + swz128_offset(r, (c8 & 7) * 8));
+          const uint32_t w4[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w4[e]));
+            n2[0] = fmaf(f.x, f.x, n2[0]);
+            n2[1] = fmaf(f.y, f.y, n2[1]);
+          }
+        }
+        shift = -0.5f * (n2[0] + n2[1]) * kLog2eF - 0.5f * log2f((float)D);
+      } else {
+        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll 1
         for (int c = 0; c < D / 32; ++c) {
           uint32_t y[32];
-          tmem_ld32(tmem + lane_off + c * 32, y);
+          tmem_ld32(ty + c * 32, y);
           tmem_wait_ld();
 #pragma unroll
-          for (int e = 0; e < 32; ++e) mx = fmaxf(mx, __uint_as_float(y[e]));
+          for (int e = 0; e < 32; ++e) mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(y[e]));
         }
-        shift = -mx * kLog2eF;
+        shift = -fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * kLog2eF;
       }
-#pragma unroll
+#pragma unroll 1
       for (int c = 0; c < D / 32; ++c) {
         uint32_t y[32];
-        tmem_ld32(tmem + lane_off + c * 32, y);
+        tmem_ld32(ty + c * 32, y);
         tmem_wait_ld();
         uint8_t* box = sX + (c >> 1) * 16384;
 #pragma unroll
@@ -140,18 +219,14 @@ favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__
         }
       }
       tc_fence_before_sync();
+      mbar_arrive(&y_free[s]);
       fence_proxy_async_smem();
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    if (ok && warp == 2 && elect_one()) {
-      for (int c = 0; c < D / 64; ++c) tma_store_4d(mf, sX + c * 16384, c * 64, i0, p.h_begin + hl, b);
-      tma_store_commit();
-      tma_store_wait_all<0>();
+      mbar_arrive(&staged[s]);
     }
   }
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == 1) tmem_dealloc(tmem, D);
+  if (warp == 9) tmem_dealloc(tmem, 2 * D);
 }
 
 }  // namespace
@@ -170,20 +245,21 @@ cudaError_t launch_favor_features_tc(const void* q, const void* k, const void* W
   p.h_begin = h_begin;
   p.h_count = h_count;
   p.status = &ws->status;
-  const long long rows = (long long)B * h_count, tiles = ((long long)N + 127) / 128;
-  if (rows > 0x7fffffffLL || tiles > 65535) return cudaErrorInvalidValue;  // (tiles: more than 8 million tokens)
-  dim3 grid((unsigned)rows, (unsigned)tiles, 2);
+  p.rows = (long long)B * h_count;
+  p.ntile = (N + 127) / 128;
+  const long long total = 2 * p.rows * p.ntile;
+  if (p.rows > 0x7fffffffLL) return cudaErrorInvalidValue;
   auto launch = [&](auto kern, int smem) -> cudaError_t {
     int dev = 0, sms = 0;
     cudaError_t err = device_info(&dev, &sms);
     if (err == cudaSuccess) err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem);
     if (err != cudaSuccess) return err;
+    const unsigned grid = (unsigned)(total < 2LL * sms ? total : 2LL * sms);
     kern<<<grid, kFavorThreads, smem, stream>>>(mxq, mxk, mw, mfq, mfk, p);
     note_launch();
     return cudaGetLastError();
   };
-  return d == 64 ? launch(favor_tc_kernel<64>, 128 * 64 * 2 + 64 * 64 * 2 + 1024)
-                 : launch(favor_tc_kernel<128>, 128 * 128 * 2 + 128 * 128 * 2 + 1024);
+  return d == 64 ? launch(favor_tc_kernel<64>, FavorCfg<64>::kBytes) : launch(favor_tc_kernel<128>, FavorCfg<128>::kBytes);
 }
 
 }  // namespace gf
