@@ -210,8 +210,8 @@ __global__ void export_ring_kernel(const T* __restrict__ k, const T* __restrict_
 // ------------------------------------------------------------------------------------
 // Decode step: one CTA per (b, h).
 // ------------------------------------------------------------------------------------
-// A 16-byte load that stays where it is written: two of them in a row are both in flight before the
-// first use (left to itself the compiler, short of registers, pairs every load with its use).
+// A 16-byte load that stays where it is written: several in a row are all in flight before the first use (left to
+// itself the compiler, short of registers, pairs every load with its use).
 __device__ __forceinline__ uint4 ld16_in_order(const void* p) {
   uint4 r;
   asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p) : "memory");
@@ -281,27 +281,46 @@ __device__ __forceinline__ float block_reduce(float x, bool is_max, float* scrat
   return scratch[32];
 }
 
-// Seven CTAs per SM: one CTA per (batch, head) then fits a batch of 64 x 16 heads in a single wave.
-template <typename T, int D>
-__global__ void __launch_bounds__(256, 7)
+// One CTA per (batch, head).  What bounds a step is round trips to L2 or HBM, so a thread has as many loads in flight as
+// its registers hold: NW key pieces and the NW value pieces of the same slots (windowed heads), or four pieces of S, the
+// first of them asked for before q and k have arrived.
+//   windowed heads  a group of threads that share a slot keeps a running maximum, sum and output of its own over the
+//                   slots it meets; the groups are combined once at the end, so that no barrier stands between keys
+//                   and values.
+// CTAS per SM and NW go together (registers): four with NW = 4, six with NW = 2 (decode_dispatch says which when).
+// Measured at B = 64, H = 16, d = 64, w = 256: 8.3 us a step (two loads in flight, scores and values apart by two
+// block-wide reductions: 10.3); B = 8, H = 32, d = 128, w = 512: 12.3 (18.6); B = 128, H = 32, d = 128, w = 512: 98 us =
+// 5.8 TB/s (110).
+template <typename T, int D, int CTAS, int NW>
+__global__ void __launch_bounds__(256, CTAS)
 decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                    T* __restrict__ o, T* __restrict__ kc, T* __restrict__ vc, float* __restrict__ S,
                    float* __restrict__ z, long long t_all, long long* __restrict__ t_seq, int H, int w,
                    int h_sparse, float scale, const T* __restrict__ W /* [H - h_sparse, D, D] or null: elu + 1 */) {
+  constexpr int NB = 4;
   constexpr int D4 = D / 4;
   constexpr int G = 256 / D4;  // thread groups along the reduced dimension
-  // windowed heads: a ring row is read 16 bytes per thread (a slot's round trip to L2 is what a step
-  // waits for, so the fewer rounds the better): TPS threads per slot, GW slots per round
+  // windowed heads: a ring row is read 16 bytes per thread: TPS threads per slot (8, 16 or 32: a group never straddles
+  // a warp), GW slots at a time
   constexpr int EPT = Row16<T>::kElems, TPS = D / EPT, GW = 256 / TPS;
-  extern __shared__ __align__(16) float dyn[];  // window heads: w scores
   __shared__ __align__(16) float qs[D];
   __shared__ __align__(16) float ks[D];
   __shared__ float scratch[33];
+  __shared__ float gm[GW], gl[GW];
   __shared__ __align__(16) float part[GW][D];  // GW >= G
 
-  const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
+  // the windowed heads of the whole batch come first: they take longest, so none of them should start late
+  const int tid = threadIdx.x, id = blockIdx.x, n_win = (int)(gridDim.x / (unsigned)H) * h_sparse;
+  int h, b;
+  if (id < n_win) {
+    b = id / h_sparse;
+    h = id - b * h_sparse;
+  } else {
+    const int h_lin = H - h_sparse;
+    b = (id - n_win) / h_lin;
+    h = h_sparse + (id - n_win) - b * h_lin;
+  }
   const long long io = ((long long)b * H + h) * D;
-  const int c4 = tid % D4, grp = tid / D4;
   // Position of this sequence: the whole batch in lock step, or its own entry of t_seq (a negative
   // entry marks an idle slot of the batch: state untouched, output row zero).  The sequence's H
   // CTAs count their arrivals in bits 48..62 of the entry; the last one clears the count and moves
@@ -311,6 +330,11 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
   float qv = 0.f;
   T kin = from_f32<T>(0.f), vin = from_f32<T>(0.f);
   long long t = t_all;
+  if (tid < D) {
+    qv = to_f32(q[io + tid]);
+    kin = k[io + tid];
+    vin = v[io + tid];
+  }
   if (t_seq != nullptr) {
     __shared__ long long t_sh;
     if (tid == 255) {
@@ -323,17 +347,8 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
       }
       t_sh = cur;
     }
-    if (tid < D) {
-      qv = to_f32(q[io + tid]);
-      kin = k[io + tid];
-      vin = v[io + tid];
-    }
     __syncthreads();
     t = t_sh;
-  } else if (tid < D) {
-    qv = to_f32(q[io + tid]);
-    kin = k[io + tid];
-    vin = v[io + tid];
   }
   if (t < 0) {
     if (tid < D) o[io + tid] = from_f32<T>(0.f);
@@ -350,69 +365,79 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
       kcb[(long long)cur * D + tid] = kin;
       vcb[(long long)cur * D + tid] = vin;
     }
-    __syncthreads();
-    // scores: TPS threads per slot (a warp reads whole cache lines of the ring), partial dot products
-    // reduced over the group by shuffles; slot `cur` is read from the step input (same values).  TPS is
-    // 8, 16 or 32, so a group never straddles a warp.
+    // slot `cur` is read from the step input (same values)
     const int cw = tid % TPS, gw = tid / TPS;
-    float mloc = -INFINITY;
-    for (int s0 = 0; s0 < nvalid; s0 += 2 * GW) {  // uniform trip count: the shuffles below are warp-wide
-      const int sa = s0 + gw, sb = s0 + GW + gw;
-      uint4 ra = make_uint4(0u, 0u, 0u, 0u), rb = ra;
-      if (sa < nvalid) ra = ld16_in_order(((sa == cur) ? (k + io) : (kcb + (long long)sa * D)) + EPT * cw);
-      if (sb < nvalid) rb = ld16_in_order(((sb == cur) ? (k + io) : (kcb + (long long)sb * D)) + EPT * cw);
-      float acc_a = Row16<T>::dot(ra, &qs[EPT * cw]), acc_b = Row16<T>::dot(rb, &qs[EPT * cw]);
+    float m = -INFINITY, l = 0.f, acc[EPT];
 #pragma unroll
-      for (int off = TPS / 2; off > 0; off >>= 1) {
-        acc_a += __shfl_xor_sync(0xffffffffu, acc_a, off);
-        acc_b += __shfl_xor_sync(0xffffffffu, acc_b, off);
-      }
-      if (cw == 0) {
-        if (sa < nvalid) {
-          acc_a *= scale;
-          dyn[sa] = acc_a;
-          mloc = fmaxf(mloc, acc_a);
-        }
-        if (sb < nvalid) {
-          acc_b *= scale;
-          dyn[sb] = acc_b;
-          mloc = fmaxf(mloc, acc_b);
-        }
-      }
-    }
-    const float mx = block_reduce(mloc, true, scratch);
-    float lloc = 0.f;
-    for (int s = tid; s < nvalid; s += 256) {
-      const float p = expf(dyn[s] - mx);
-      dyn[s] = p;
-      lloc += p;
-    }
-    const float lsum = block_reduce(lloc, false, scratch);  // barriers inside publish dyn[]
-    float accv[EPT];
+    for (int e = 0; e < EPT; ++e) acc[e] = 0.f;
+    for (int s0 = 0; s0 < nvalid; s0 += NW * GW) {  // uniform trip count: the shuffles below are warp-wide
+      uint4 rk[NW], rv[NW];
 #pragma unroll
-    for (int e = 0; e < EPT; ++e) accv[e] = 0.f;
-    for (int sa = gw; sa < nvalid; sa += 2 * GW) {
-      const int sb = sa + GW;
-      uint4 ra = ld16_in_order(((sa == cur) ? (v + io) : (vcb + (long long)sa * D)) + EPT * cw), rb = make_uint4(0u, 0u, 0u, 0u);
-      if (sb < nvalid) rb = ld16_in_order(((sb == cur) ? (v + io) : (vcb + (long long)sb * D)) + EPT * cw);
-      Row16<T>::axpy(ra, dyn[sa], accv);
-      Row16<T>::axpy(rb, sb < nvalid ? dyn[sb] : 0.f, accv);
+      for (int i = 0; i < NW; ++i) {
+        const int sl = s0 + i * GW + gw;
+        rk[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (sl < nvalid) rk[i] = ld16_in_order(((sl == cur) ? (k + io) : (kcb + (long long)sl * D)) + EPT * cw);
+      }
+#pragma unroll
+      for (int i = 0; i < NW; ++i) {
+        const int sl = s0 + i * GW + gw;
+        rv[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (sl < nvalid) rv[i] = ld16_in_order(((sl == cur) ? (v + io) : (vcb + (long long)sl * D)) + EPT * cw);
+      }
+      if (s0 == 0) __syncthreads();  // qs
+      float s[NW], mx = m;
+#pragma unroll
+      for (int i = 0; i < NW; ++i) {
+        s[i] = Row16<T>::dot(rk[i], &qs[EPT * cw]);
+#pragma unroll
+        for (int off = TPS / 2; off > 0; off >>= 1) s[i] += __shfl_xor_sync(0xffffffffu, s[i], off);
+        s[i] = (s0 + i * GW + gw < nvalid) ? s[i] * scale : -INFINITY;
+        mx = fmaxf(mx, s[i]);
+      }
+      if (mx != -INFINITY) {  // (a group that has met no slot yet keeps l = 0)
+        const float corr = expf(m - mx);
+        m = mx;
+        l *= corr;
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) acc[e] *= corr;
+#pragma unroll
+        for (int i = 0; i < NW; ++i) {
+          const float p = expf(s[i] - mx);
+          l += p;
+          Row16<T>::axpy(rv[i], p, acc);
+        }
+      }
     }
 #pragma unroll
     for (int e = 0; e < EPT; e += 4)
-      *reinterpret_cast<float4*>(&part[gw][EPT * cw + e]) = make_float4(accv[e], accv[e + 1], accv[e + 2], accv[e + 3]);
+      *reinterpret_cast<float4*>(&part[gw][EPT * cw + e]) = make_float4(acc[e], acc[e + 1], acc[e + 2], acc[e + 3]);
+    if (cw == 0) {
+      gm[gw] = m;
+      gl[gw] = l;
+    }
     __syncthreads();
     if (tid < D) {
-      float sum = 0.f;
+      float mx = -INFINITY, sum = 0.f, lsum = 0.f;
 #pragma unroll
-      for (int gi = 0; gi < GW; ++gi) sum += part[gi][tid];
+      for (int gi = 0; gi < GW; ++gi) mx = fmaxf(mx, gm[gi]);
+#pragma unroll 8
+      for (int gi = 0; gi < GW; ++gi) {
+        const float f = expf(gm[gi] - mx);
+        sum = fmaf(f, part[gi][tid], sum);
+        lsum = fmaf(f, gl[gi], lsum);
+      }
       o[io + tid] = from_f32<T>(sum / lsum);
     }
   } else {
+    const int c4 = tid % D4, grp = tid / D4;
     const long long sidx = (long long)b * (H - h_sparse) + (h - h_sparse);
-    float* Sb = S + sidx * D * D;
+    float* Sb = S + sidx * D * D + 4 * c4;
     float* zb = z + sidx * D;
-    float denloc = 0.f;
+    uint4 raw[NB];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) raw[i] = ld16_in_order(Sb + (grp + i * G) * D);
+    const float4 vv = Vec4<T>::load(v + io + 4 * c4);
+    const float zin = tid < D ? zb[tid] : 0.f;
     if (W != nullptr) {
       // positive random features of q_t and k_t (Sec. III-A / III-C): exp(<w_a, x> - |x|^2 / 2) / sqrt(D)
       // for the key; for the query exp(<w_a, q> - max_a <w_a, q>) (a factor common to its features cancels
@@ -451,32 +476,45 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
       const float kp = W != nullptr ? ks[tid] : phi_elu1(to_f32(kin));
       qs[tid] = qp;
       ks[tid] = kp;
-      const float zn = zb[tid] + kp;
+      const float zn = zin + kp;
       zb[tid] = zn;
-      denloc = qp * zn;
+      float den = qp * zn;  // the denominator: D/32 partial sums, one per warp
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
+      if ((tid & 31) == 0) scratch[tid >> 5] = den;
     }
-    const float den = block_reduce(denloc, false, scratch);  // barriers inside publish qs/ks
-    const float4 vv = Vec4<T>::load(v + io + 4 * c4);
+    __syncthreads();
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int a = grp; a < D; a += G) {
-      float4 s4 = *reinterpret_cast<float4*>(Sb + (long long)a * D + 4 * c4);
-      const float kp = ks[a], qp = qs[a];
-      s4.x = fmaf(kp, vv.x, s4.x);
-      s4.y = fmaf(kp, vv.y, s4.y);
-      s4.z = fmaf(kp, vv.z, s4.z);
-      s4.w = fmaf(kp, vv.w, s4.w);
-      *reinterpret_cast<float4*>(Sb + (long long)a * D + 4 * c4) = s4;
-      acc.x = fmaf(qp, s4.x, acc.x);
-      acc.y = fmaf(qp, s4.y, acc.y);
-      acc.z = fmaf(qp, s4.z, acc.z);
-      acc.w = fmaf(qp, s4.w, acc.w);
+#pragma unroll 1
+    for (int a0 = grp; a0 < D; a0 += NB * G) {
+#pragma unroll
+      for (int i = 0; i < NB; ++i) {
+        const int a = a0 + i * G;
+        const float kp = ks[a], qp = qs[a];
+        float4 s4;
+        s4.x = fmaf(kp, vv.x, __uint_as_float(raw[i].x));
+        s4.y = fmaf(kp, vv.y, __uint_as_float(raw[i].y));
+        s4.z = fmaf(kp, vv.z, __uint_as_float(raw[i].z));
+        s4.w = fmaf(kp, vv.w, __uint_as_float(raw[i].w));
+        *reinterpret_cast<float4*>(Sb + a * D) = s4;
+        acc.x = fmaf(qp, s4.x, acc.x);
+        acc.y = fmaf(qp, s4.y, acc.y);
+        acc.z = fmaf(qp, s4.z, acc.z);
+        acc.w = fmaf(qp, s4.w, acc.w);
+      }
+      if (a0 + NB * G < D) {
+#pragma unroll
+        for (int i = 0; i < NB; ++i) raw[i] = ld16_in_order(Sb + (a0 + (NB + i) * G) * D);
+      }
     }
     *reinterpret_cast<float4*>(&part[grp][4 * c4]) = acc;
     __syncthreads();
     if (tid < D) {
-      float sum = 0.f;
+      float sum = 0.f, den = 0.f;
 #pragma unroll
       for (int gi = 0; gi < G; ++gi) sum += part[gi][tid];
+#pragma unroll
+      for (int i = 0; i < D / 32; ++i) den += scratch[i];
       o[io + tid] = from_f32<T>(sum / den);
     }
   }
@@ -503,25 +541,18 @@ template <typename T>
 cudaError_t decode_dispatch(const void* q, const void* k, const void* v, void* o, void* kc, void* vc, float* S,
                             float* z, long long t, long long* t_seq, int B, int H, int d, int w, int h_sparse,
                             float scale, cudaStream_t stream, const void* W) {
-  dim3 grid(H, B);
-  const size_t dyn = (size_t)w * sizeof(float);
-  if (d == 64) {
-    auto kern = decode_step_kernel<T, 64>;
-    if (dyn > 40 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-      if (e != cudaSuccess) return e;
-    }
-    kern<<<grid, 256, dyn, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, (T*)kc, (T*)vc, S, z, t, t_seq,
-                                     H, w, h_sparse, scale, (const T*)W);
-  } else {
-    auto kern = decode_step_kernel<T, 128>;
-    if (dyn > 40 * 1024) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
-      if (e != cudaSuccess) return e;
-    }
-    kern<<<grid, 256, dyn, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, (T*)kc, (T*)vc, S, z, t, t_seq,
-                                     H, w, h_sparse, scale, (const T*)W);
-  }
+  int dev = 0, sms = 0;
+  const cudaError_t e = device_info(&dev, &sms);
+  if (e != cudaSuccess) return e;
+  // Four CTAs per SM with twice the loads in flight, unless heads of d = 64 (16 KB of state, or 256 bytes per slot) are
+  // more than that makes one wave of: then six, 8.3 against 9.2 us at B = 64, H = 16 and 20.5 against 22.7 at 128 x 32.
+  // Few or large ones want the loads: 4.2 against 5.2 us at 1 x 12, 70 against 84 at 32 x 12 with w = 4096, and at d = 128
+  // 12.3 against 14.4 us at 8 x 32 (at 128 x 32, bound by HBM, there is no difference).
+  auto* kern = d == 128                          ? decode_step_kernel<T, 128, 4, 4>
+               : (long long)B * H <= 4LL * sms ? decode_step_kernel<T, 64, 4, 4>
+                                                 : decode_step_kernel<T, 64, 6, 2>;
+  kern<<<(unsigned)(B * H), 256, 0, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, (T*)kc, (T*)vc, S, z, t, t_seq,
+                                              H, w, h_sparse, scale, (const T*)W);
   note_launch();
   return cudaGetLastError();
 }

@@ -1195,3 +1195,37 @@ def test_self_linear_heads_whole_chains(B, H, N, d, favor):
     ref = oracle.hybrid_attn_self(f64(q[:, hs]), f64(k[:, hs]), f64(v[:, hs]), 16, h_sparse=0,
                                   **({"W": f64(W[hs])} if favor else {}))
     assert_parity(f64(o[:, hs]), ref, "bf16", f"whole chains B={B} H={H} N={N} d={d}")
+
+
+# ------------------------------------------------------------------ decode: both forms of the kernel, partial rounds of slots
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("B,H,d,w,h0,t0", [(1, 2, 64, 1, 1, 0), (1, 3, 128, 129, 2, 40), (2, 4, 64, 600, 2, 599), (2, 4, 64, 600, 2, 2000),
+                                           (300, 2, 64, 70, 1, 33), (300, 2, 64, 200, 1, 500), (1, 3, 128, 1000, 3, 5000)])
+def test_decode_rounds_of_slots_and_grid_sizes(dtype, B, H, d, w, h0, t0):
+    """Fewer slots than one round of the CTA, a last round that is partly empty, a ring that has wrapped; grids on both
+    sides of four CTAs per SM (300 x 2), one step against plain fp64 arithmetic on the same state."""
+    g = torch.Generator().manual_seed(B + w + t0)
+    T = torch.float32 if dtype == "f32" else torch.bfloat16
+    st = gf.DecodeState(B, H, d, w, h0, T)
+    rnd = lambda *s: torch.randn(*s, generator=g)  # noqa: E731
+    st.k_cache.copy_(rnd(*st.k_cache.shape)); st.v_cache.copy_(rnd(*st.v_cache.shape))
+    st.S.copy_(rnd(*st.S.shape)); st.z.copy_(20.0 + torch.rand(st.z.shape, generator=g))
+    st.t = t0
+    q, k, v = [rnd(B, H, d).to(T) for _ in range(3)]
+    kc, vc, S, z = [x.double().cpu() for x in (st.k_cache, st.v_cache, st.S, st.z)]
+    o = gf.decode_step(q.cuda(), k.cuda(), v.cuda(), st).double().cpu()
+    qd, kd, vd = q.double(), k.double(), v.double()
+    ref = torch.empty(B, H, d, dtype=torch.float64)
+    kc[:, :h0, t0 % w], vc[:, :h0, t0 % w] = kd[:, :h0], vd[:, :h0]
+    n = min(t0 + 1, w)
+    s = torch.einsum("bhd,bhnd->bhn", qd[:, :h0], kc[:, :h0, :n]) / d**0.5
+    ref[:, :h0] = torch.einsum("bhn,bhnd->bhd", torch.softmax(s, -1), vc[:, :h0, :n])
+    if h0 < H:
+        phi = lambda x: torch.where(x > 0, x + 1, torch.exp(x.clamp(max=0)))  # noqa: E731
+        fq, fk = phi(qd[:, h0:]), phi(kd[:, h0:])
+        S += fk[..., None] * vd[:, h0:, None, :]
+        z += fk
+        ref[:, h0:] = torch.einsum("bha,bhac->bhc", fq, S) / (fq * z).sum(-1, keepdim=True)
+        assert errors(f64(st.S), S.numpy())["rel_l2"] <= 1e-6 and errors(f64(st.z), z.numpy())["rel_l2"] <= 1e-6
+    assert torch.equal(st.k_cache.cpu().double()[:, :h0], kc[:, :h0]) and torch.equal(st.v_cache.cpu().double()[:, :h0], vc[:, :h0])
+    assert_parity(o.numpy(), ref.numpy(), kind_of(dtype), f"decode B={B} H={H} d={d} w={w} t={t0}")
