@@ -47,11 +47,15 @@ __device__ __forceinline__ void transform_k_tile(uint8_t* tile, int tt, int n_va
   }
 #pragma unroll
   for (int k = 0; k < kRows; ++k) {
-    const uint32_t keep = (row0 + 16 * k < n_valid) ? 0xffffffffu : 0u;
-    raw[k].x = phi_sel<kId>(raw[k].x) & keep;
-    raw[k].y = phi_sel<kId>(raw[k].y) & keep;
-    raw[k].z = phi_sel<kId>(raw[k].z) & keep;
-    raw[k].w = phi_sel<kId>(raw[k].w) & keep;
+    raw[k].x = phi_sel<kId>(raw[k].x);
+    raw[k].y = phi_sel<kId>(raw[k].y);
+    raw[k].z = phi_sel<kId>(raw[k].z);
+    raw[k].w = phi_sel<kId>(raw[k].w);
+  }
+  if (n_valid < 128) {
+#pragma unroll
+    for (int k = 0; k < kRows; ++k)
+      if (row0 + 16 * k >= n_valid) raw[k] = make_uint4(0u, 0u, 0u, 0u);
   }
 #pragma unroll
   for (int k = 0; k < kRows; ++k) {

@@ -770,13 +770,13 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
               uint32_t v[32];
               tmem_ld32(tmem + C::tP + lane_off + cc * 32, v);
               tmem_wait_ld();
-              const bool diag = (cc == quarter);
+              if (cc == quarter) {  // (a select per element off the diagonal too cost 3 % of the kernel at D = 64)
   #pragma unroll
-              for (int jj = 0; jj < 16; ++jj) {
-                const float p0 = (!diag || 2 * jj <= lane) ? __uint_as_float(v[2 * jj]) : 0.f;
-                const float p1 = (!diag || 2 * jj + 1 <= lane) ? __uint_as_float(v[2 * jj + 1]) : 0.f;
-                pk[jj] = pack_bf16(p0, p1);
+                for (int jj = 0; jj < 32; ++jj)
+                  if (jj > lane) v[jj] = 0u;
               }
+  #pragma unroll
+              for (int jj = 0; jj < 16; ++jj) pk[jj] = pack_bf16(__uint_as_float(v[2 * jj]), __uint_as_float(v[2 * jj + 1]));
             }
             // packed P stays inside this warp's own fp32 columns (keys 64h..64h+63 -> columns 64h..64h+31),
             // so the two warps of a lane quarter never touch each other's unread input
