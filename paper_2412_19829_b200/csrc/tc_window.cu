@@ -57,6 +57,7 @@ struct WinCtl {
   uint64_t s_full[2][2], p_full[2][2];             // per query tile of the pair and S buffer
   uint64_t pv_done[2], o_full[2], o_free[2];       // per query tile of the pair
   uint32_t front;  // ring number of the half tile stream 0's next S will read (stream 1 stays behind it)
+  uint32_t k_issued, v_issued;  // half tiles whose load the producer has issued (monotonic)
   uint32_t tmem_base;
   int units_posted;          // entries of unit_ring written so far (monotonic)
   int unit_ring[kUnitRing];  // the CTA's n-th work unit (-1: no more)
@@ -89,7 +90,8 @@ struct WinParams {
 };
 
 // A wait that first polls the barrier for a few microseconds (a thread parked in try_wait takes a
-// few hundred cycles to come back) and then falls back to the bounded parked wait.
+// few hundred cycles to come back) and then falls back to the bounded parked wait.  For a lone thread only: sixteen
+// polling warps take issue slots from the ones at work (2 to 3 % of the kernel).
 __device__ __forceinline__ bool mbar_wait_hot(uint64_t* bar, uint32_t parity, unsigned int* status,
                                               unsigned int where) {
 #pragma unroll 1
@@ -115,10 +117,18 @@ __device__ __forceinline__ bool win_wait_epoch(const int* counter, int target, u
   return true;
 }
 
+__device__ __forceinline__ void publish(uint32_t* counter, uint32_t value) {
+  __threadfence_block();
+  *reinterpret_cast<volatile uint32_t*>(counter) = value;
+}
+
 // A unit: query tiles qtA (and qtA + 1 when nt == 2); tile x walks the key tiles f[x] .. l[x].
 struct Unit {
   int h, b, qtA, nt;
   int f[2], l[2];
+  // half tiles of tile x: number `off` of the unit's half tiles on, n_sub of them
+  __device__ __forceinline__ int off(int x) const { return 2 * (f[x] - f[0]); }
+  __device__ __forceinline__ int n_sub(int x) const { return x < nt ? 2 * (l[x] - f[x] + 1) : 0; }
 };
 
 template <int D, bool kTwoSided>
@@ -163,7 +173,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       mbar_init(&ctl->o_free[i], 256);
     }
     ctl->unit_ring[0] = blockIdx.x;  // the grid never exceeds the number of units
-    ctl->front = 0;
+    ctl->front = ctl->k_issued = ctl->v_issued = 0;
     ctl->units_posted = 1;
     mbar_fence_init();
     tma_prefetch_desc(&mq);
@@ -215,16 +225,25 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         const unsigned int t_next = atomicAdd(p.ticket, 1u);
         int u_next = -1;
         const int g0 = x.f[0], g1 = x.nt == 2 ? x.l[1] : x.l[0];
+        // A slot is released by two arrivals.  For a stream that has no use for a half tile the producer arrives itself,
+        // so that the stream need not wait until it has landed.
+        const int off1 = x.off(1), n0 = x.n_sub(0), n1 = x.n_sub(1);
         for (int hg = 2 * g0; hg <= 2 * g1 + 1; ++hg, ++kt) {  // kt counts half tiles here
+          const int m = hg - 2 * g0;
+          const bool unused = m >= n0 || m < off1 || m >= off1 + n1;  // by one of the streams
           const uint32_t slot = kt % ST, use = kt / ST;
           if (use >= 1 && !mbar_wait(&ctl->k_empty[slot], (use - 1) & 1, p.status, 10)) { ok = false; break; }
           mbar_arrive_expect_tx(&ctl->k_full[slot], SM::kHalf);
           for (int c = 0; c < D / 64; ++c)
             tma_load_4d(sK + slot * SM::kHalf + c * 8192, &mk, &ctl->k_full[slot], c * 64, hg * 64, x.h, x.b);
+          if (unused) mbar_arrive(&ctl->k_empty[slot]);
+          publish(&ctl->k_issued, kt + 1);
           if (use >= 1 && !mbar_wait(&ctl->v_empty[slot], (use - 1) & 1, p.status, 11)) { ok = false; break; }
           mbar_arrive_expect_tx(&ctl->v_full[slot], SM::kHalf);
           for (int c = 0; c < D / 64; ++c)
             tma_load_4d(sV + slot * SM::kHalf + c * 8192, &mv, &ctl->v_full[slot], c * 64, hg * 64, x.h, x.b);
+          if (unused) mbar_arrive(&ctl->v_empty[slot]);
+          publish(&ctl->v_issued, kt + 1);
           if (hg == 2 * g0) {  // the other roles learn of the next unit early (its Q is requested ahead)
             u_next = (t_next < (unsigned int)(p.total - (int)gridDim.x)) ? (int)(gridDim.x + t_next) : -1;
             ctl->unit_ring[(nu + 1) % kUnitRing] = u_next;
@@ -284,9 +303,9 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     // S(0), S(1), then P V(j) followed by S(j + 2): S buffer j & 1 is free again once P V(j) has been
     // issued, because the tensor core runs one thread's products in issue order.  The two streams
     // meet only in the ring: a half tile goes back to the producer when both streams are done
-    // with it, and stream 1, whose window starts one key tile later, does not overtake stream 0,
-    // so that the two read the same half tile at about the same time and the rest of the ring
-    // holds loads in flight.
+    // with it (or the producer has arrived for a stream that has no use for it), and stream 1, whose window starts one key
+    // tile later, does not overtake stream 0, so that the two read the same half tile at about the same time and the rest
+    // of the ring holds loads in flight.
     if (elect_one()) {
       constexpr uint32_t idesc_qk = umma_idesc_bf16(128, 64, false, false);
       constexpr uint32_t idesc_pv = umma_idesc_bf16(128, D, false, true);
@@ -295,89 +314,74 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         constexpr int t = decltype(T)::value;
         const uint32_t tSt = tmem + t * 128, tO = tmem + 256 + t * D;
         volatile uint32_t* front = &ctl->front;
-        uint32_t kt = 0, qn = 0, sub = 0, ntile = 0;  // key tiles, query tiles (both streams), own sub-tiles and tiles so far
+        uint32_t kt = 0, qn = 0, sub = 0, ntile = 0;  // half tiles, query tiles (both streams), own half tiles and tiles so far
+        // Half tile number n of the CTA has landed.  A parity wait tells a barrier's current phase only from the one before
+        // it, and the stream has not waited for the slot's uses that it had no use for; but once the producer has issued a
+        // load into the slot, all uses before it are over.
+        auto landed = [&](uint32_t* issued, uint64_t* full, uint32_t n, unsigned int where) -> bool {
+          return win_wait_epoch(reinterpret_cast<const int*>(issued), (int)n + 1, p.status, where) &&
+                 mbar_wait(&full[n % ST], (n / ST) & 1, p.status, where);
+        };
         for (uint32_t nu = 0;; ++nu) {
           const int u = unit_at(nu);
           if (u < 0) break;
           const Unit x = decode(u);
-          const int g0 = x.f[0];
-          const int n_key = (x.nt == 2 ? x.l[1] : x.l[0]) - g0 + 1;
-          // The stream walks every half tile of the unit in ring order, for S and (two steps behind)
-          // for P V.  Half tiles outside its own key range it only hands on: it waits until they
-          // have landed and arrives on their release barrier.  That way every thread that waits on
-          // a slot sees each of its phases exactly once, in order (a parity wait tells a barrier's
-          // current phase only from the one before it), and a slot is released by exactly two
-          // arrivals whoever reads it.
-          const bool mine = t < x.nt;
-          const int off = mine ? 2 * (x.f[t] - g0) : 0;  // own sub-tile j is half tile off + j of the unit
-          const int n_sub = mine ? 2 * (x.l[t] - x.f[t] + 1) : 0;
-          const uint32_t rbase = 2 * kt;  // ring number of the unit's first half tile
+          const uint32_t n_half = 2 * (uint32_t)((x.nt == 2 ? x.l[1] : x.l[0]) - x.f[0] + 1);
+          const int n_sub = x.n_sub(t);
+          const uint32_t rbase = kt + (t ? (uint32_t)x.off(1) : 0u);  // ring number of the stream's first half tile
           const uint32_t qbuf = (qn + t) % 3;
           const uint32_t qa = aX + qbuf * SM::kTile;
-          for (int m = 0; m < 2 * n_key + 2; ++m) {
-            if (m >= 2) {
-              const int jj = m - 2 - off;
-              const uint32_t n = rbase + (uint32_t)(m - 2), slot = n % ST;
-              if (!mbar_wait(&ctl->v_full[slot], (n / ST) & 1, p.status, 23)) return;
-              if (jj >= 0 && jj < n_sub) {  // O += P V of sub-tile jj
-                const int half = jj & 1;
-                if (!mbar_wait_hot(&ctl->p_full[t][half], ((sub + jj) >> 1) & 1, p.status, 22)) return;
-                // the first product of a tile overwrites O: the previous tile's epilogue has read it
-                if (jj == 0 && ntile >= 1 && !mbar_wait(&ctl->o_free[t], (ntile - 1) & 1, p.status, 24)) return;
-                tc_fence_after_sync();
-                const uint32_t va = aV + slot * SM::kHalf, tP = tSt + half * 64;
+          for (int m = 0; m < n_sub + 2 && n_sub > 0; ++m) {
+            if (m >= 2) {  // O += P V of half tile jj
+              const int jj = m - 2, half = jj & 1;
+              const uint32_t n = rbase + (uint32_t)jj, slot = n % ST;
+              if (!landed(&ctl->v_issued, ctl->v_full, n, 23)) return;
+              if (!mbar_wait_hot(&ctl->p_full[t][half], ((sub + jj) >> 1) & 1, p.status, 22)) return;
+              // the first product of a tile overwrites O: the previous tile's epilogue has read it
+              if (jj == 0 && ntile >= 1 && !mbar_wait(&ctl->o_free[t], (ntile - 1) & 1, p.status, 24)) return;
+              tc_fence_after_sync();
+              const uint32_t va = aV + slot * SM::kHalf, tP = tSt + half * 64;
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks)
-                  umma_ts(tO, tP + (ks >> 1) * 32 + (ks & 1) * 8, umma_smem_desc(va + ks * 2048, 8192, 1024), idesc_pv,
-                          (jj > 0) || (ks > 0));
-                umma_commit(&ctl->v_empty[slot]);
-                umma_commit(&ctl->pv_done[t]);
-                if (jj == n_sub - 1) umma_commit(&ctl->o_full[t]);
-              } else {
-                mbar_arrive(&ctl->v_empty[slot]);
-              }
+              for (int ks = 0; ks < 4; ++ks)
+                umma_ts(tO, tP + (ks >> 1) * 32 + (ks & 1) * 8, umma_smem_desc(va + ks * 2048, 8192, 1024), idesc_pv,
+                        (jj > 0) || (ks > 0));
+              umma_commit(&ctl->v_empty[slot]);
+              umma_commit(&ctl->pv_done[t]);
+              if (jj == n_sub - 1) umma_commit(&ctl->o_full[t]);
             }
-            if (m < 2 * n_key) {
-              const int j = m - off;
+            if (m < n_sub) {  // S of half tile m into S buffer m & 1
+              const int half = m & 1;
               const uint32_t n = rbase + (uint32_t)m, slot = n % ST;
-              if (j >= 0 && j < n_sub) {  // S of sub-tile j into S buffer j & 1
-                const int half = j & 1;
-                if (t == 1) {  // bounded: stream 0's next S must lie behind this half tile
-                  if (*front <= n) {
-                    const long long t0 = clock64(), limit = wait_limit_cycles(p.status);
-                    while (*front <= n) {
-                      if (clock64() - t0 > limit) {
-                        if (atomicCAS(p.status, 0u, 1u) == 0u) p.status[1] = 26;
-                        return;
-                      }
-                      __nanosleep(20);
+              if (t == 1) {  // bounded: stream 0's next S must lie behind this half tile
+                if (*front <= n) {
+                  const long long t0 = clock64(), limit = wait_limit_cycles(p.status);
+                  while (*front <= n) {
+                    if (clock64() - t0 > limit) {
+                      if (atomicCAS(p.status, 0u, 1u) == 0u) p.status[1] = 26;
+                      return;
                     }
+                    __nanosleep(20);
                   }
                 }
-                if (j == 0 && !mbar_wait(&ctl->q_full[qbuf], ((qn + t) / 3) & 1, p.status, 20)) return;
-                if (!mbar_wait(&ctl->k_full[slot], (n / ST) & 1, p.status, 21)) return;
-                tc_fence_after_sync();
-                const uint32_t ka = aK + slot * SM::kHalf;
-#pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks)
-                  umma_ss(tSt + half * 64, umma_smem_desc(qa + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024),
-                          umma_smem_desc(ka + (ks >> 2) * 8192 + (ks & 3) * 32, 16, 1024), idesc_qk, ks > 0);
-                umma_commit(&ctl->s_full[t][half]);
-                umma_commit(&ctl->k_empty[slot]);
-                // stream 0 tells where its next S will read: the next half tile of this query tile,
-                // or the first one of the next unit
-                if (t == 0) *front = (j + 1 < n_sub) ? n + 1 : 2 * (kt + (uint32_t)n_key);
-              } else {
-                if (!mbar_wait(&ctl->k_full[slot], (n / ST) & 1, p.status, 21)) return;
-                mbar_arrive(&ctl->k_empty[slot]);
               }
+              if (m == 0 && !mbar_wait(&ctl->q_full[qbuf], ((qn + t) / 3) & 1, p.status, 20)) return;
+              if (!landed(&ctl->k_issued, ctl->k_full, n, 21)) return;
+              tc_fence_after_sync();
+              const uint32_t ka = aK + slot * SM::kHalf;
+#pragma unroll
+              for (int ks = 0; ks < D / 16; ++ks)
+                umma_ss(tSt + half * 64, umma_smem_desc(qa + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024),
+                        umma_smem_desc(ka + (ks >> 2) * 8192 + (ks & 3) * 32, 16, 1024), idesc_qk, ks > 0);
+              umma_commit(&ctl->s_full[t][half]);
+              umma_commit(&ctl->k_empty[slot]);
+              // stream 0 tells where its next S will read: the next half tile of this query tile,
+              // or the first one of the next unit
+              if (t == 0) *front = (m + 1 < n_sub) ? n + 1 : kt + n_half;
             }
           }
-          if (mine) {
-            sub += (uint32_t)n_sub;
-            ++ntile;
-          }
-          kt += (uint32_t)n_key;
+          sub += (uint32_t)n_sub;
+          ntile += n_sub > 0;
+          kt += n_half;
           qn += (uint32_t)x.nt;
         }
         if (t == 0) *front = 0xffffffffu;
@@ -428,7 +432,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         const int hi_last = kTwoSided ? min(i_first + 31 + p.fwd, p.N - 1) - j0 : hi_first + 31;  // ... of its last row
         const bool none = (31 < lo_first || 0 > hi_last);
         const bool inside = (0 >= lo_first + 31) && (31 <= hi_first);
-        if (!mbar_wait_hot(&ctl->s_full[t][half], (sub >> 1) & 1, p.status, 30)) { ok = false; break; }
+        if (!mbar_wait(&ctl->s_full[t][half], (sub >> 1) & 1, p.status, 30)) { ok = false; break; }
         tc_fence_after_sync();
         // the block's 32 scores stay in registers from the maximum to the exponentials
         uint32_t sa[32];
@@ -507,8 +511,8 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       if (!ok) break;
       // epilogue: O / l -> bf16 -> shared (swizzled; the tile's Q buffer is dead once its last product
       // is done) -> TMA store by the store warp; this warp takes its half of the output columns
-      ok = mbar_wait(&ctl->o_full[t], ntile & 1, p.status, 32);
-      if (!ok) break;
+      const bool done = mbar_wait(&ctl->o_full[t], ntile & 1, p.status, 32);
+      if (__any_sync(0xffffffffu, !done)) break;
       tc_fence_after_sync();
       uint8_t* stage = sX + buf * SM::kTile;
       // the two halves of a row add their sums through bytes of the staging buffer that the
