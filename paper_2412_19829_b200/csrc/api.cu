@@ -37,8 +37,8 @@ Tuning tuning_now() {
 constexpr int kMaxDevices = 64;
 constexpr unsigned int kPlacedWaitNs = 20000;  // longest the windowed heads are held back for the linear kernel's CTAs
 struct Fork {
-  cudaStream_t side = nullptr, first = nullptr;  // lowest / highest stream priority
-  cudaEvent_t fork = nullptr, join = nullptr, join_first = nullptr;
+  cudaStream_t side = nullptr, first = nullptr, aux = nullptr;  // lowest / highest / lowest stream priority
+  cudaEvent_t fork = nullptr, join = nullptr, join_first = nullptr, join_aux = nullptr;
   bool ready = false;
   // held while a call enqueues its fork .. join section: the events are shared by every call on
   // the device, and a record from another host thread between this call's record and its waits
@@ -48,8 +48,8 @@ struct Fork {
 Fork g_fork[kMaxDevices];
 std::mutex g_fork_mutex;
 
-// Side stream + two events per device, created on first use; lets the two head groups of the
-// hybrid layer run concurrently while the caller sees a single-stream call.
+// Streams and events per device, created on first use; they let the two head groups of the hybrid layer (and the export
+// of the ring) run concurrently while the caller sees a single-stream call.
 Fork* get_fork() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
@@ -62,6 +62,8 @@ Fork* get_fork() {
     if (cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest) != cudaSuccess) return nullptr;
     if (cudaStreamCreateWithPriority(&f.side, cudaStreamNonBlocking, prio_least) != cudaSuccess) return nullptr;
     if (cudaStreamCreateWithPriority(&f.first, cudaStreamNonBlocking, prio_greatest) != cudaSuccess) return nullptr;
+    if (cudaStreamCreateWithPriority(&f.aux, cudaStreamNonBlocking, prio_least) != cudaSuccess) return nullptr;
+    if (cudaEventCreateWithFlags(&f.join_aux, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     if (cudaEventCreateWithFlags(&f.join_first, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     if (cudaEventCreateWithFlags(&f.fork, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     if (cudaEventCreateWithFlags(&f.join, cudaEventDisableTiming) != cudaSuccess) return nullptr;
@@ -117,10 +119,11 @@ int run_window(const Tuning& tn, const void* q, const void* k, const void* v, vo
 
 // Feature map of the linear heads of one call: elu + 1 (W null), or positive random features under
 // the projections W [h_count, d, d].  On the tensor-core path those are computed first, into the two
-// feature tensors at the end of the workspace (feat_offset bytes in).
+// feature tensors at the end of the workspace (feat_offset bytes in): fq, fk once run_features has launched that.
 struct Phi {
   const void* W = nullptr;
   size_t feat_offset = 0;
+  void *fq = nullptr, *fk = nullptr;
 };
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -132,21 +135,26 @@ int check_phi(int phi, const void* W) {
   return GF_ERR_UNSUPPORTED;
 }
 
+// The pre-pass of the positive random features.  It goes to the caller's stream, ahead of the fork of the two head groups:
+// windowed-heads CTAs that were already waiting for SMs when it ends would take them before the linear kernel's CTAs,
+// which wait for one another (42 chains of 3217 tokens beside 14 windowed heads: 97 or 110 us, as it fell, and 101;
+// 2 x 8 heads of 19 271 tokens 187.6 -> 182.0; 4 x 16 bidirectional heads of 2000 tokens 59.4 -> 51.8).
+int run_features(const Tuning& tn, const void* q, const void* k, int B, int H, int N, int d, int dtype, int layout,
+                 int h_begin, int h_count, WsHeader* ws, cudaStream_t stream, Phi* phi) {
+  if (h_count <= 0 || phi->W == nullptr || tn.force_simt || !gf::tc_linear_supported(N, d, dtype)) return GF_OK;
+  phi->fq = reinterpret_cast<uint8_t*>(ws) + phi->feat_offset;
+  phi->fk = reinterpret_cast<uint8_t*>(phi->fq) + feature_bytes(B, h_count, N, d);
+  return cuda_status(gf::launch_favor_features_tc(q, k, phi->W, phi->fq, phi->fk, B, H, N, d, layout, h_begin, h_count, ws,
+                                                  stream));
+}
+
 int run_linear(const Tuning& tn, const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d, int dtype,
                int layout, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init, int max_ctas,
                WsHeader* ws, cudaStream_t stream, bool shared = false, const Phi& phi = Phi(), int* first_grid = nullptr) {
   if (h_count <= 0) return GF_OK;
   if (!tn.force_simt && gf::tc_linear_supported(N, d, dtype)) {
-    void *fq = nullptr, *fk = nullptr;
-    if (phi.W != nullptr) {
-      fq = reinterpret_cast<uint8_t*>(ws) + phi.feat_offset;
-      fk = reinterpret_cast<uint8_t*>(fq) + feature_bytes(B, h_count, N, d);
-      const int rc = cuda_status(gf::launch_favor_features_tc(q, k, phi.W, fq, fk, B, H, N, d, layout, h_begin,
-                                                              h_count, ws, stream));
-      if (rc != GF_OK) return rc;
-    }
     return cuda_status(gf::launch_linear_tc(q, k, v, o, B, H, N, d, layout, h_begin, h_count, S_io, z_io,
-                                            zero_init, tn.linear_split, max_ctas, ws, stream, shared, fq, fk, first_grid));
+                                            zero_init, tn.linear_split, max_ctas, ws, stream, shared, phi.fq, phi.fk, first_grid));
   }
   return cuda_status(gf::launch_linear_simt(q, k, v, o, B, N, d, dtype, gf::make_strides(layout, H, N, d),
                                             h_begin, h_count, S_io, z_io, zero_init, stream, false, phi.W));
@@ -341,13 +349,11 @@ int gformer_hybrid_attn_self_w(const void* q, const void* k, const void* v, void
   rc = clear_ws(tn, ws, stream);
   if (rc != GF_OK) return rc;
   const bool tc_linear = !tn.force_simt && gf::tc_linear_supported(N, d, dtype);
-  // positive random features: computed first (on the stream the linear kernels run on), then read in
-  // place of Q and K
-  void *fq = nullptr, *fk = nullptr;
-  if (W != nullptr && tc_linear && h_sparse < H) {
-    fq = reinterpret_cast<uint8_t*>(ws) + feat_offset;
-    fk = reinterpret_cast<uint8_t*>(fq) + feature_bytes(B, H - h_sparse, N, d);
-  }
+  Phi fm;
+  fm.W = W;
+  fm.feat_offset = feat_offset;
+  if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, h_sparse, H - h_sparse, (WsHeader*)ws, stream, &fm)) != GF_OK)
+    return rc;
   if (h_sparse > 0 && h_sparse < H && tc_linear) {
     // Both head groups on tensor-core kernels: the three launches of the linear heads go to the
     // library's high-priority stream, the windowed heads to its side stream a few microseconds
@@ -359,13 +365,9 @@ int gformer_hybrid_attn_self_w(const void* q, const void* k, const void* v, void
     if (cudaEventRecord(f->fork, stream) != cudaSuccess) return GF_ERR_CUDA;
     if (cudaStreamWaitEvent(f->side, f->fork, 0) != cudaSuccess) return GF_ERR_CUDA;
     if (cudaStreamWaitEvent(f->first, f->fork, 0) != cudaSuccess) return GF_ERR_CUDA;
-    if (fq != nullptr)
-      rc = cuda_status(gf::launch_favor_features_tc(q, k, W, fq, fk, B, H, N, d, layout, h_sparse, H - h_sparse,
-                                                    (WsHeader*)ws, f->first));
     int lin_grid = 0;
-    if (rc == GF_OK)
-      rc = cuda_status(gf::launch_linear_self_tc(q, k, v, o, B, H, N, d, layout, h_sparse, H - h_sparse, (WsHeader*)ws,
-                                                 sizeof(WsHeader), f->first, fq, fk, &lin_grid));
+    rc = cuda_status(gf::launch_linear_self_tc(q, k, v, o, B, H, N, d, layout, h_sparse, H - h_sparse, (WsHeader*)ws,
+                                               sizeof(WsHeader), f->first, fm.fq, fm.fk, &lin_grid));
     if (cudaEventRecord(f->join_first, f->first) != cudaSuccess) return GF_ERR_CUDA;
     if (cudaStreamWaitEvent(stream, f->join_first, 0) != cudaSuccess) return GF_ERR_CUDA;
     // the windowed heads start once the CTAs of the first linear kernel have all started
@@ -381,15 +383,9 @@ int gformer_hybrid_attn_self_w(const void* q, const void* k, const void* v, void
   rc = run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, stream, true);
   if (rc != GF_OK) return rc;
   if (h_sparse == H) return GF_OK;
-  if (tc_linear) {
-    if (fq != nullptr) {
-      rc = cuda_status(gf::launch_favor_features_tc(q, k, W, fq, fk, B, H, N, d, layout, h_sparse, H - h_sparse,
-                                                    (WsHeader*)ws, stream));
-      if (rc != GF_OK) return rc;
-    }
+  if (tc_linear)
     return cuda_status(gf::launch_linear_self_tc(q, k, v, o, B, H, N, d, layout, h_sparse, H - h_sparse, (WsHeader*)ws,
-                                                 sizeof(WsHeader), stream, fq, fk));
-  }
+                                                 sizeof(WsHeader), stream, fm.fq, fm.fk));
   // fp32 storage (or the CUDA-core knob): token by token, a summing sweep and a readout sweep
   return cuda_status(gf::launch_linear_simt(q, k, v, o, B, N, d, dtype, gf::make_strides(layout, H, N, d), h_sparse,
                                             H - h_sparse, nullptr, nullptr, true, stream, true, W));
@@ -420,6 +416,7 @@ int gformer_causal_linear_attn_w(const void* q, const void* k, const void* v, vo
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   rc = clear_ws(tn, ws, stream, B * H, N, d, dtype);
   if (rc != GF_OK) return rc;
+  if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, 0, H, (WsHeader*)ws, stream, &fm)) != GF_OK) return rc;
   return run_linear(tn, q, k, v, o, B, H, N, d, dtype, layout, 0, H, S_io, z_io, false, 0, (WsHeader*)ws, stream, false,
                     fm);
 }
@@ -460,6 +457,7 @@ int gformer_hybrid_attn_w(const void* q, const void* k, const void* v, void* o, 
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   rc = clear_ws(tn, ws, stream, B * h_lin, N, d, dtype);
   if (rc != GF_OK) return rc;
+  if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, h_sparse, h_lin, (WsHeader*)ws, stream, &fm)) != GF_OK) return rc;
 
   float* S_out = state_out ? state_out->S : nullptr;
   float* z_out = state_out ? state_out->z : nullptr;
@@ -509,9 +507,18 @@ int gformer_hybrid_attn_w(const void* q, const void* k, const void* v, void* o, 
       cuda_status(gf::launch_wait_placed((WsHeader*)ws, (unsigned int)lin_grid, kPlacedWaitNs, wstream)) != GF_OK)
     return GF_ERR_CUDA;
   int rc2 = run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, wstream);
-  if (rc2 == GF_OK && state_out && h_sparse > 0)
+  // The ring only needs K and V.  Where the linear heads fill the device the windowed ones end last, and behind them the
+  // 3 to 9 us of the export would add to the call; on a stream of its own it fills gaps (14 x 4 heads of 3217 tokens 76.1
+  // -> 73.1 us).  A small call is bound by the host, which the two extra event calls would cost 1 us (18.7 -> 19.8).
+  if (rc2 == GF_OK && state_out && h_sparse > 0) {
+    cudaStream_t estream = lin_first ? f->aux : wstream;
+    if (lin_first && cudaStreamWaitEvent(f->aux, f->fork, 0) != cudaSuccess) return GF_ERR_CUDA;
     rc2 = cuda_status(gf::launch_export_ring(k, v, state_out->k_cache, state_out->v_cache, B, N, d, w, dtype,
-                                             gf::make_strides(layout, H, N, d), h_sparse, wstream));
+                                             gf::make_strides(layout, H, N, d), h_sparse, estream));
+    if (lin_first && (cudaEventRecord(f->join_aux, f->aux) != cudaSuccess ||
+                 cudaStreamWaitEvent(stream, f->join_aux, 0) != cudaSuccess))
+      return GF_ERR_CUDA;
+  }
   if (both) {
     if (cudaEventRecord(f->join, f->side) != cudaSuccess) return GF_ERR_CUDA;
     if (cudaStreamWaitEvent(stream, f->join, 0) != cudaSuccess) return GF_ERR_CUDA;
