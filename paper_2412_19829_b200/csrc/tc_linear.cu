@@ -20,7 +20,10 @@
 //       in L2 when pass C reads them back) and accumulates the segment's own state contribution
 //       dS | dz = sum Kc^T [V | 1] (not for a chain's last segment, whose contribution nobody needs),
 //   (B) waits for the inclusive state of the previous segment in global scratch (one bounded
-//       poller per CTA), publishes its own inclusive state = previous + dS and raises its flag,
+//       poller per CTA), publishes its own inclusive state = previous + dS and raises its flag;
+//       when every CTA has one segment (kSum) all publish dS at once instead and each adds up
+//       those before it, which takes the chain of hand-overs out of the call (about 2.8 us per
+//       segment at D = 128: 24 chains of 4798 tokens 50.6 -> 42.1 us, one of 32 768 107 -> 66),
 //   (C) walks its chunks with the full pipeline starting from the previous segment's state,
 //       reading phi(K) back instead of K, so every exponential of the layer is computed once.
 // Warp roles:
@@ -143,6 +146,7 @@ struct LinBarriers {
   uint64_t qphi_full[2], qphi_free[2];
   uint64_t p_full, s_full, o_full, mma2_done, a_done, pub_done, park_done, sb_idle, sb_parked;
   uint64_t pm_full, s_loaded, sb_full, s_final, o_free, o_staged[4][2];  // o_staged[V slot][box]
+  uint64_t st_done;    // kSum: the state before the segment is in TMEM and Sb
   uint64_t kd_phi[4];  // kDirect: a K tile of the chunk pipeline has been transformed in place
 };
 
@@ -262,7 +266,95 @@ __device__ __forceinline__ bool publish_inclusive(const LinParams& p, const LinI
   return ok;
 }
 
-template <int D, bool kDirect, bool kId>
+// The state before a segment when every CTA has one item (kSum): the caller's initial state plus the contributions of all
+// segments before it, added by the 16 phi warps (each thread one row x a quarter of the columns) in the order in which the
+// inclusive states of a chain would have been.  Every segment publishes its own contribution as soon as its first pass is
+// over, so no segment waits for the one before it to have waited.
+template <int D>
+__device__ __forceinline__ bool sum_states(const LinParams& p, const LinItem& it, LinBarriers& bar, uint8_t* sSb,
+                                           uint32_t tmem, int warp, int lane, const int* prev_epoch) {
+  using C = LinCfg<D>;
+  const int quarter = warp & 3, colq = (warp - 6) >> 2;
+  const int r = quarter * 32 + lane;
+  constexpr int W = D / 4;  // columns per thread
+  const uint32_t tS = tmem + C::tS + ((uint32_t)(quarter * 32) << 16) + colq * W;
+  float* slot0 = p.prefix + (long long)it.chain * p.G * C::kStateFloats + ((long long)(colq * (W / 4)) * 128 + r) * 4;
+  // (the caller's state is read before this segment's flag is raised: the chain's last segment, which waits for all
+  // flags, may then overwrite it)
+  const bool from_caller = p.S_io != nullptr && !p.zero_init && r < D;
+  const float* Sc = p.S_io + (((long long)it.b * p.h_count + it.hl) * D + r) * D + colq * W;
+  float4 acc[W / 4];
+#pragma unroll
+  for (int j = 0; j < W / 4; ++j)
+    acc[j] = from_caller ? __ldcg(reinterpret_cast<const float4*>(Sc) + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+  bool ok = true;
+  if (it.need_dS) {
+    ok = mbar_wait(&bar.a_done, 0, p.status, 600);
+    if (__any_sync(0xffffffffu, !ok)) return false;
+    tc_fence_after_sync();
+    uint32_t ds[W];
+    if constexpr (D == 128) tmem_ld32(tS, *reinterpret_cast<uint32_t(*)[32]>(ds));
+    else tmem_ld16(tS, ds);
+    tmem_wait_ld();
+    if (r < D) {
+      float4* out = reinterpret_cast<float4*>(slot0 + (long long)it.g * C::kStateFloats);
+#pragma unroll
+      for (int j = 0; j < W / 4; ++j)
+        __stcg(out + j * 128, make_float4(__uint_as_float(ds[4 * j]), __uint_as_float(ds[4 * j + 1]),
+                                          __uint_as_float(ds[4 * j + 2]), __uint_as_float(ds[4 * j + 3])));
+    }
+    tc_fence_before_sync();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&bar.pub_done);  // (released to the flag warp, as in publish_inclusive)
+  }
+  if (lane == 0) ok = wait_epoch(prev_epoch, 1, p.status, 601);
+  if (__any_sync(0xffffffffu, !ok)) return false;
+  if (r < D) {
+#pragma unroll 1
+    for (int g = 0; g < it.g; ++g) {
+      const float4* src = reinterpret_cast<const float4*>(slot0 + (long long)g * C::kStateFloats);
+      float4 in[W / 4];
+#pragma unroll
+      for (int j = 0; j < W / 4; ++j) in[j] = __ldcg(src + j * 128);
+#pragma unroll
+      for (int j = 0; j < W / 4; ++j) {
+        acc[j].x += in[j].x;
+        acc[j].y += in[j].y;
+        acc[j].z += in[j].z;
+        acc[j].w += in[j].w;
+      }
+    }
+  }
+  ok = mbar_wait(&bar.sb_parked, 0, p.status, 602);  // Sb held K tiles in pass A
+  if (__any_sync(0xffffffffu, !ok)) return false;
+  tc_fence_after_sync();
+  uint32_t v[W];
+#pragma unroll
+  for (int j = 0; j < W / 4; ++j) {
+    v[4 * j] = __float_as_uint(acc[j].x);
+    v[4 * j + 1] = __float_as_uint(acc[j].y);
+    v[4 * j + 2] = __float_as_uint(acc[j].z);
+    v[4 * j + 3] = __float_as_uint(acc[j].w);
+  }
+  if constexpr (D == 128) tmem_st32(tS, *reinterpret_cast<uint32_t(*)[32]>(v));
+  else tmem_st16(tS, v);
+  if (r < D) {
+    const int col0 = colq * W;
+#pragma unroll
+    for (int g = 0; g < W / 8; ++g)
+      *reinterpret_cast<uint4*>(sSb + (col0 >> 6) * C::kSbBox + swz128_offset(r, (col0 & 63) + g * 8)) =
+          make_uint4(pack_bf16(acc[2 * g].x, acc[2 * g].y), pack_bf16(acc[2 * g].z, acc[2 * g].w),
+                     pack_bf16(acc[2 * g + 1].x, acc[2 * g + 1].y), pack_bf16(acc[2 * g + 1].z, acc[2 * g + 1].w));
+  }
+  tmem_wait_st();
+  fence_proxy_async_smem();
+  tc_fence_before_sync();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(&bar.st_done);
+  return true;
+}
+
+template <int D, bool kDirect, bool kId, bool kSum = false>
 __global__ void __launch_bounds__(kThreads, 1)
 linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
                  const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtensorMap mo,
@@ -320,6 +412,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     mbar_init(&bar.a_done, 1);
     mbar_init(&bar.pub_done, 20);  // 16 phi warps + 4 P-group warps
     mbar_init(&bar.park_done, 1);
+    mbar_init(&bar.st_done, 16);
     mbar_init(&bar.pm_full, 256);
     mbar_init(&bar.s_loaded, 256);
     mbar_init(&bar.sb_full, 256);
@@ -553,6 +646,39 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       const LinItem it = decode_item(p, item);
       const long long sidx = (long long)it.b * p.h_count + it.hl;
       const long long slot = (long long)it.chain * p.G + it.g;
+      if constexpr (kSum) {
+        // ---- z as the phi warps do S (sum_states); the segment may start once both are in place
+        float z0 = (p.z_io != nullptr && !p.zero_init && s_row) ? __ldcg(p.z_io + sidx * D + r) : 0.f;
+        float* zslot = p.prefix + (slot - it.g) * C::kStateFloats + C::kStateZ + r;
+        if (it.need_dS) {
+          ok = mbar_wait(&bar.a_done, 0, p.status, 311);
+          if (named_bar_or(1, 128, !ok)) break;
+          tc_fence_after_sync();
+          const float dz = __uint_as_float(tmem_ld1(tmem + C::tSz + lane_off));
+          tmem_wait_ld();
+          if (s_row) __stcg(zslot + (long long)it.g * C::kStateFloats, dz);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bar.pub_done);
+          nv += it.nC;
+        }
+        ok = wait_epoch(&prev_epoch, 1, p.status, 312);
+        if (ok && s_row)
+          for (int g = 0; g < it.g; ++g) z0 += __ldcg(zslot + (long long)g * C::kStateFloats);
+        ok = ok && mbar_wait(&bar.st_done, 0, p.status, 313);
+        if (named_bar_or(1, 128, !ok)) break;
+        tc_fence_after_sync();
+        uint32_t zc[16];
+#pragma unroll
+        for (int jj = 1; jj < 16; ++jj) zc[jj] = 0u;
+        zc[0] = __float_as_uint(z0);
+        tmem_st16(tmem + C::tSz + lane_off, zc);
+        if (s_row) put_z(z0);
+        tmem_wait_st();
+        fence_proxy_async_smem();
+        tc_fence_before_sync();
+        mbar_arrive_cnt(&bar.s_loaded, 2);  // these barriers count the K group's 256 threads
+        mbar_arrive_cnt(&bar.sb_full, 2);
+      } else {
       // ---- hand-over of z (column 0 of tSz, one feature per thread): this segment's own sum is
       //      there after pass A; previous segment's inclusive z in, this segment's inclusive z out
       if (it.need_dS) ok = mbar_wait(&bar.a_done, n_a & 1, p.status, 311);
@@ -632,6 +758,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         tc_fence_before_sync();
         mbar_arrive_cnt(&bar.s_loaded, 2);  // these barriers count the K group's 256 threads
         mbar_arrive_cnt(&bar.sb_full, 2);
+      }
       }
       // ---- pass C
       for (int j = 0; j < it.nC; ++j) {
@@ -745,7 +872,9 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       }
 
       // ---- hand-over of S: the two groups publish the inclusive state (column quarters 0, 1 / 2, 3)
-      if (it.need_dS) {
+      if constexpr (kSum) {
+        ok = ok && sum_states<D>(p, it, bar, sSb, tmem, warp, lane, &prev_epoch);
+      } else if (it.need_dS) {
         ok = publish_inclusive<D>(p, it, bar, tmem, warp, lane, n_a & 1, &prev_epoch, (int)n_items);
         ++n_a;
       }
@@ -993,6 +1122,21 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       for (int item = blockIdx.x; item < p.nitems; item += gridDim.x, ++n_items) {
         const LinItem it = decode_item(p, item);
         const long long slot = (long long)it.chain * p.G + it.g;
+        if constexpr (kSum) {  // own contribution out, then everybody's before it in
+          if (it.need_dS) {
+            if (!mbar_wait(&bar.pub_done, 0, p.status, 510)) break;
+            if (reinterpret_cast<const volatile unsigned int*>(p.status)[4] != (unsigned int)slot + 1u) {
+              const unsigned int one = 1u;
+              asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.flags + slot * kFlagStride), "r"(one) : "memory");
+            }
+          }
+          bool seen = true;
+          for (int g = 0; g < it.g && seen; ++g) seen = wait_flag(p.flags + (slot - it.g + g) * kFlagStride, p.status, 511);
+          if (!seen) break;
+          __threadfence_block();
+          *reinterpret_cast<volatile int*>(&prev_epoch) = 1;
+          break;
+        }
         // one poller per CTA: hundreds of threads spinning on a handful of L2 lines slow the whole chain
         if (it.g > 0 && !wait_flag(p.flags + (slot - 1) * kFlagStride, p.status, 511)) break;
         __threadfence_block();
@@ -1097,6 +1241,18 @@ double best_cut(int nchains, int nch, int d, int kPlanSMs, int* G_out) {
       if (cost < best * (1.0 - 1e-9)) {
         best = cost;
         G = g;
+      }
+    }
+    // Segments that fit one round need no chain of hand-overs (sum_states): the round costs about its chunks and hardly
+    // more when a chain has many segments.  Measured, one round against the best of several (us): d = 128, 24 chains of
+    // 6000 tokens 48.5 and 65.4, 42 x 3217 47.1 and 52.6, 26 x 16384 128 and 130, 52 x 6000 102 and 97; d = 64, 16 x 12000
+    // 40.0 and 56.9, 30 x 6000 38.5 and 46.0, 42 x 8192 59 and 60, 52 x 6000 61.6 and 56.5.
+    const int g1 = kPlanSMs / nchains;
+    if ((long long)nchains * G > kPlanSMs && g1 >= 2 && g1 >= g_min && g1 <= g_max) {
+      const double one_round = 0.2 + (d == 128 ? 0.95 : 1.05) * ((nch + g1 - 1) / g1) + 0.12 * g1;
+      if (one_round < best) {
+        best = one_round;
+        G = g1;
       }
     }
     *G_out = G;
@@ -1287,6 +1443,14 @@ cudaError_t launch_linear_tc(const void* q, const void* k, const void* v, void* 
     p.seg_base = p.nch / g;
     p.seg_rem = p.nch % g;
     p.nitems = count * g;
+    // every CTA one segment: the states are sums of the contributions before a segment
+    if (!direct && p.nitems <= sms) {
+      if (features)
+        return d == 64 ? launch(linear_tc_kernel<64, false, true, true>, LinCfg<64>::kBytes)
+                       : launch(linear_tc_kernel<128, false, true, true>, LinCfg<128>::kBytes);
+      return d == 64 ? launch(linear_tc_kernel<64, false, false, true>, LinCfg<64>::kBytes)
+                     : launch(linear_tc_kernel<128, false, false, true>, LinCfg<128>::kBytes);
+    }
     if (features) {
       if (d == 64)
         return direct ? launch(linear_tc_kernel<64, true, true>, LinCfg<64>::kBytes)

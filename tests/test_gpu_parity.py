@@ -1229,3 +1229,30 @@ def test_decode_rounds_of_slots_and_grid_sizes(dtype, B, H, d, w, h0, t0):
         assert errors(f64(st.S), S.numpy())["rel_l2"] <= 1e-6 and errors(f64(st.z), z.numpy())["rel_l2"] <= 1e-6
     assert torch.equal(st.k_cache.cpu().double()[:, :h0], kc[:, :h0]) and torch.equal(st.v_cache.cpu().double()[:, :h0], vc[:, :h0])
     assert_parity(o.numpy(), ref.numpy(), kind_of(dtype), f"decode B={B} H={H} d={d} w={w} t={t0}")
+
+
+# ------------------------------------------------------------------ cut chains whose segments fit one round of the CTAs
+@pytest.mark.parametrize("favor,bnhd", [(False, False), (True, False), (False, True)])
+@pytest.mark.parametrize("H,N,d", [(1, 8193, 128), (3, 1100, 64), (24, 6000, 128), (37, 1025, 64), (5, 4001, 128)])
+def test_linear_segments_in_one_round(H, N, d, favor, bnhd):
+    """Every CTA has one segment: the states are sums of the contributions before it.  With a state carried in, which
+    all segments read and the last one overwrites; ragged last chunk."""
+    segments = gf.linear_plan(H, N, d)[0]
+    assert 1 < segments and segments * H <= 148
+    q, k, v = synth.qkv(1, H, N, d, "bf16", seed=970 + N, gain=None if favor else 1.0)
+    W = _proj(H, d, "bf16", 5) if favor else None
+    g = torch.Generator().manual_seed(H)
+    S0, z0 = torch.rand(1, H, d, d, generator=g), 30.0 + torch.rand(1, H, d, generator=g)
+    hs = sorted({0, H // 2, H - 1})
+    S_ref, z_ref = f64(S0[:, hs]).copy(), f64(z0[:, hs]).copy()
+    ref = oracle.causal_linear_attn(f64(q[:, hs]), f64(k[:, hs]), f64(v[:, hs]), S_ref, z_ref, **({"W": f64(W[hs])} if favor else {}))
+    layout = gf.GF_BNHD if bnhd else gf.GF_BHND
+    ins = [(t.permute(0, 2, 1, 3).contiguous() if bnhd else t).cuda() for t in (q, k, v)]
+    S, z = S0.cuda(), z0.cuda()
+    ws = gf.Workspace.for_problem(1, H, N, d, phi=gf.GF_PHI_FAVOR_POS if favor else gf.GF_PHI_ELU1)
+    o = gf.causal_linear_attn(*ins, S, z, layout=layout, ws=ws, W=W.cuda() if favor else None).cpu()
+    assert ws.last_device_status() == gf.GF_OK
+    o = o.permute(0, 2, 1, 3) if bnhd else o
+    assert torch.isfinite(o.float()).all()
+    assert_parity_by_scale(f64(o[:, hs]), ref, "bf16", f"one round H={H} N={N} d={d}")
+    assert errors(f64(S[:, hs].cpu()), S_ref)["rel_l2"] <= 1e-2 and errors(f64(z[:, hs].cpu()), z_ref)["rel_l2"] <= 1e-2
