@@ -9,8 +9,10 @@
 // What bounds both is shared memory: for these tiles the 16-byte loads take 1.5 to 3 times the cycles of the
 // multiply-adds (ncu at 8 x 12 heads x 2048 tokens, d = 64, w = 128: shared-memory pipe 60-75 % busy, FMA pipe 40-49 %).
 // Larger tiles (64 threads, 4 x 8, 4 x 4 and 8 x 8) need a third fewer loads but leave 8 warps per SM: no faster there
-// (245 us for the layer either way) and slower on few chains (56 against 39 us at 2 heads x 256 tokens).  The
-// token-by-token kernels that these replaced took 756 and 57 us: a block-wide reduction per 16 tokens, no reuse of K.
+// (244 us for the layer either way).  Token by token, with a block-wide reduction per 16 tokens and no reuse of K, it took
+// 756 us, and 2 heads of 256 tokens 57 us, now 17.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 
 namespace gf {
@@ -232,13 +234,16 @@ window_tiled_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
 // A CTA owns 64 value columns of a chain; S lives in its registers (a thread: D/8 features x 4 columns) with a copy
 // in shared memory for the readout.
 //
-// With few chains a chain is cut into G segments of a little more than D tokens, so that every SM has work:
+// With few chains a chain is cut into G segments, so that every SM has work.  Up to kMaxCluster of them are a cluster of
+// CTAs in one launch (kCluster): each sums its own segment, then adds up the sums of those before it from their shared
+// memory, then walks.  Longer chains in smaller numbers take three launches, with segments of a little more than D tokens:
 //   contribution   the sums of every segment but the last, each alone
 //   prefix         running sums over the segments of a chain
 //   walk           the segments' outputs, each from its own starting state
 // The states wait in the rows of the OUTPUT tensor that their own segment will later overwrite (row a of S in the
 // row of token a of the segment, z in the next row or two, one per 64 columns): no workspace, and a CTA of the walk
 // reads only rows and columns that itself will write.
+constexpr int kMaxCluster = 8;
 template <int D> struct LinT {
   static constexpr int LD = D + 4;
   static constexpr int ZROWS = D / 64;  // rows z takes behind S
@@ -288,6 +293,26 @@ __device__ __forceinline__ float column_sum(const float* col) {
   return (s[0] + s[1]) + (s[2] + s[3]);
 }
 
+// Adds tokens [n_begin, n_end) to S and z (thread tid < D: feature tid).
+template <typename T, int D>
+__device__ __forceinline__ void sum_segment(const T* k, const T* v, long long stride, int n_begin, int n_end, float* Ks,
+                                            float* Vs, int tid, int ag, int cg, float4 (&S)[D / 8], float& z) {
+  BlockRegs<T, D> rk;
+  BlockRegs<T, kW> rv;
+  rk.load(k, stride, n_begin, n_end, tid);
+  rv.load(v, stride, n_begin, n_end, tid);
+  for (int n0 = n_begin; n0 < n_end; n0 += kC) {
+    rk.store_phi(Ks, D + 4, n0, n_end, tid);
+    rv.store(Vs, kW, tid);
+    __syncthreads();
+    rk.load(k, stride, n0 + kC, n_end, tid);
+    rv.load(v, stride, n0 + kC, n_end, tid);
+    add_outer<D>(Ks, Vs, ag, cg, S);
+    if (tid < D) z += column_sum<D>(Ks + tid);
+    __syncthreads();
+  }
+}
+
 template <int D>
 __global__ void __launch_bounds__(kNT)
 linear_contribution_kernel(const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o, Segs sg,
@@ -301,20 +326,7 @@ linear_contribution_kernel(const float* __restrict__ k, const float* __restrict_
   for_state<D>(ag, S, [](int, float4& x) { x = make_float4(0.f, 0.f, 0.f, 0.f); });
   float z = 0.f;
   const int n_end = sg.begin(g + 1);
-  BlockRegs<float, D> rk;
-  BlockRegs<float, kW> rv;
-  rk.load(k + base, st.n, sg.begin(g), n_end, tid);
-  rv.load(v + base + col0, st.n, sg.begin(g), n_end, tid);
-  for (int n0 = sg.begin(g); n0 < n_end; n0 += kC) {
-    rk.store_phi(Ks, D + 4, n0, n_end, tid);
-    rv.store(Vs, kW, tid);
-    __syncthreads();
-    rk.load(k + base, st.n, n0 + kC, n_end, tid);
-    rv.load(v + base + col0, st.n, n0 + kC, n_end, tid);
-    add_outer<D>(Ks, Vs, ag, cg, S);
-    if (tid < D) z += column_sum<D>(Ks + tid);
-    __syncthreads();
-  }
+  sum_segment<float, D>(k + base, v + base + col0, st.n, sg.begin(g), n_end, Ks, Vs, tid, ag, cg, S, z);
   float* slot = o + base + (long long)n_end * st.n + col0;  // the state before segment g + 1, once summed
   for_state<D>(ag, S, [&](int a, float4& x) { store4(slot + (long long)a * st.n + 4 * cg, x); });
   if (tid < D) slot[(long long)(D + tid / kW) * st.n + tid % kW] = z;
@@ -354,8 +366,8 @@ __global__ void linear_prefix_kernel(float* __restrict__ o, Segs sg, Strides st,
 }
 
 // Without cuts (G == 1) the state before token 0 comes from S_io; with cuts from the segment's slot (segment 0 has
-// one only when there is an initial state).
-template <typename T, int D>
+// one only when there is an initial state), or, kCluster, from S_io and the cluster's CTAs before this one.
+template <typename T, int D, bool kCluster>
 __global__ void __launch_bounds__(kNT)
 linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* o, Segs sg, Strides st,
                    int h_begin, int h_count, float* S_io, float* z_io, int zero_init) {
@@ -363,7 +375,9 @@ linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
   extern __shared__ __align__(16) float sm[];
   float *Qs = sm, *Ks = Qs + kC * LD, *Vs = Ks + kC * LD, *Ss = Vs + kC * kW, *Ps = Ss + D * kW, *zs = Ps + kC * kLdP,
         *inv_s = zs + D;
-  const int g = blockIdx.x / (D / kW), col0 = (blockIdx.x % (D / kW)) * kW;
+  // (a cluster's CTAs are neighbours in x: segments of one slice)
+  const int g = kCluster ? blockIdx.x % sg.G : blockIdx.x / (D / kW);
+  const int col0 = (kCluster ? blockIdx.x / sg.G : blockIdx.x % (D / kW)) * kW;
   const long long base = (long long)blockIdx.z * st.b + (long long)(h_begin + blockIdx.y) * st.h;
   const long long sidx = (long long)blockIdx.z * h_count + blockIdx.y;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -371,7 +385,36 @@ linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
   const int n_begin = sg.begin(g), n_end = sg.begin(g + 1);
 
   float4 S[D / 8];
-  {
+  if constexpr (kCluster) {
+    auto cluster = cooperative_groups::this_cluster();
+    for_state<D>(i, S, [](int, float4& x) { x = make_float4(0.f, 0.f, 0.f, 0.f); });
+    float z = 0.f;
+    if (g < sg.G - 1) {  // nobody needs the last segment's sum
+      sum_segment<T, D>(k + base, v + base + col0, st.n, n_begin, n_end, Ks, Vs, tid, i, cg, S, z);
+      for_state<D>(i, S, [&](int a, float4& x) { *reinterpret_cast<float4*>(Ss + s_off(a, 4 * cg)) = x; });
+      if (tid < D) zs[tid] = z;
+    }
+    const bool from_caller = S_io != nullptr && !zero_init;
+    for_state<D>(i, S, [&](int a, float4& x) {
+      x = from_caller ? load4<float>(S_io + (sidx * D + a) * D + col0 + 4 * cg) : make_float4(0.f, 0.f, 0.f, 0.f);
+    });
+    z = (from_caller && tid < D) ? z_io[sidx * D + tid] : 0.f;
+    cluster.sync();
+    for (int gg = 0; gg < g; ++gg) {
+      const float* Sr = cluster.map_shared_rank(Ss, gg);
+      for_state<D>(i, S, [&](int a, float4& x) {
+        const float4 y = lds4(Sr + s_off(a, 4 * cg));
+        x.x += y.x;
+        x.y += y.y;
+        x.z += y.z;
+        x.w += y.w;
+      });
+      if (tid < D) z += *cluster.map_shared_rank(zs + tid, gg);
+    }
+    cluster.sync();  // everybody has read what is overwritten now (and the caller's state, which the last CTA will)
+    for_state<D>(i, S, [&](int a, float4& x) { *reinterpret_cast<float4*>(Ss + s_off(a, 4 * cg)) = x; });
+    if (tid < D) zs[tid] = z;
+  } else {
     const float* Sp = nullptr;  // row a of the starting state at Sp + a * stride
     long long stride = D;
     const float* zp = nullptr;
@@ -475,20 +518,21 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
   int dev = 0, sms = 0;
   cudaError_t e = device_info(&dev, &sms);
   if (e != cudaSuccess) return e;
-  // Cut the chains when they alone do not give every SM four CTAs and are long enough for the two extra launches to
-  // pay: 8 blocks of one chain take 39 us cut in two and 55 us whole.  bf16 outputs have no room for fp32 states,
-  // their chains stay whole.
+  // Clusters as large as one wave allows (three CTAs per SM at d = 64, two at 128, by registers), unless three launches
+  // can cut a chain into clearly more segments.  Measured (us, clusters of 8 | of 4 | three launches): 1 chain of 256
+  // tokens 17 | 21 | 39, 8 of 300 24.6 | 28.7 | 39, 6 of 1000 (d = 128) 74 | 107 | 100, 80 of 500 93 | 70.5 | 71, 80 of
+  // 2048 267 | 248 | 244, 1 of 2048 (d = 128) 113 | 203 | 99.  Clusters of 16 are no faster, and with 80 KB of shared
+  // memory per CTA slower (6 of 1000: 135).
   const int blocks = (N + kC - 1) / kC;
-  const long long ctas = (long long)B * h_count * (D / kW);
-  int G = 1;
-  if (sizeof(T) == 4 && blocks >= 8 && ctas < 4LL * sms) {
-    const long long want = (8LL * sms + ctas - 1) / ctas;
-    const int most = N / C::kMinSeg;
-    G = (int)(want < most ? want : most);
-  }
-  const Segs sg = {N, G, blocks / G, blocks % G};
-  if (G > 1) {
-    if constexpr (sizeof(T) == 4) {
+  const long long ctas = (long long)B * h_count * (D / kW), wave = (D == 64 ? 3LL : 2LL) * sms;
+  int cluster = 1;
+  while (2 * cluster <= kMaxCluster && 2 * cluster <= blocks && 2 * cluster * ctas <= wave) cluster *= 2;
+  if constexpr (sizeof(T) == 4) {
+    long long G3 = ctas < 4LL * sms ? (8LL * sms + ctas - 1) / ctas : 1;
+    if (G3 > N / C::kMinSeg) G3 = N / C::kMinSeg;
+    if (5 * G3 > 6 * cluster) {
+      const int G = (int)G3;
+      const Segs sg = {N, G, blocks / G, blocks % G};
       auto sum = linear_contribution_kernel<D>;
       if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(sum), dev, C::kSmemSum)) != cudaSuccess) return e;
       sum<<<dim3((G - 1) * (D / kW), h_count, B), kNT, C::kSmemSum, stream>>>((const float*)k, (const float*)v, (float*)o, sg,
@@ -496,14 +540,33 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
       constexpr int kItems = (D + C::ZROWS) * (D / 4);
       linear_prefix_kernel<D><<<dim3((kItems + 127) / 128, h_count, B), 128, 0, stream>>>(
           (float*)o, sg, st, h_begin, h_count, zero_init ? nullptr : S_io, z_io);
-      note_launch(2);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      auto walk = linear_walk_kernel<float, D, false>;
+      if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, C::kSmem)) != cudaSuccess) return e;
+      walk<<<dim3(G * (D / kW), h_count, B), kNT, C::kSmem, stream>>>((const float*)q, (const float*)k, (const float*)v,
+                                                                      (float*)o, sg, st, h_begin, h_count, S_io, z_io,
+                                                                      zero_init ? 1 : 0);
+      note_launch(3);
+      return cudaGetLastError();
     }
   }
-  auto walk = linear_walk_kernel<T, D>;
+  const Segs sg = {N, cluster, blocks / cluster, blocks % cluster};
+  auto walk = cluster > 1 ? linear_walk_kernel<T, D, true> : linear_walk_kernel<T, D, false>;
   if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, C::kSmem)) != cudaSuccess) return e;
-  walk<<<dim3(G * (D / kW), h_count, B), kNT, C::kSmem, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, sg, st,
-                                                                  h_begin, h_count, S_io, z_io, zero_init ? 1 : 0);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(cluster * (D / kW), h_count, B);
+  cfg.blockDim = dim3(kNT);
+  cfg.dynamicSmemBytes = C::kSmem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = cluster;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  if ((e = cudaLaunchKernelEx(&cfg, walk, (const T*)q, (const T*)k, (const T*)v, (T*)o, sg, st, h_begin, h_count, S_io, z_io,
+                              zero_init ? 1 : 0)) != cudaSuccess)
+    return e;
   note_launch();
   return cudaGetLastError();
 }
