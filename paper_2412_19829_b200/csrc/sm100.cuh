@@ -251,6 +251,11 @@ __device__ __forceinline__ uint64_t umma_smem_desc(uint32_t saddr, uint32_t lbo_
   return d;
 }
 
+// The descriptor `bytes` further on (the address field is the low one, in units of 16 bytes, and shared memory ends far
+// below its range).  A lone issuing thread that builds every descriptor from scratch needs about 60 cycles per product,
+// as long as the tensor core.
+__device__ __forceinline__ uint64_t umma_desc_add(uint64_t desc, uint32_t bytes) { return desc + (bytes >> 4); }
+
 // Instruction descriptor for kind::f16 with bf16 operands and fp32 accumulation.
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N, bool a_mn_major, bool b_mn_major) {
   return (1u << 4)                        // D format: f32

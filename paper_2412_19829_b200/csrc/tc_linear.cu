@@ -532,6 +532,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       constexpr uint32_t id_o = umma_idesc_bf16(128, C::kNExt, false, true);  // [O | den] = Qc [Sb | Zb], += Pm [V | 1]
       constexpr uint32_t kLboA = (D == 128) ? C::kBoxBytes : 0;           // D=64: rows 64..127 of S mirror 0..63
       constexpr int QS = C::kQSlots;
+      const uint64_t dsb = umma_smem_desc(smem_u32(sSb), C::kSbBox, 1024);
       uint32_t ta = 0, nv = 0, nq = 0, n_sl = 0, n_sb = 0, n_of = 0, n_pm = 0;
       bool ok = true, first_item = true;
       [[maybe_unused]] uint32_t n_items = 0;
@@ -555,10 +556,10 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
             const uint32_t vlbo = C::v_lbo(sv);
             if (!mbar_wait(&bar.v_full[sv], (nv / VS) & 1, p.status, 221)) { ok = false; break; }
             tc_fence_after_sync();
+            const uint64_t dk = umma_smem_desc(kbase, kLboA, 1024), dv = umma_smem_desc(vbase, vlbo, 1024);
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks)
-              umma_ss(tmem + C::tS, umma_smem_desc(kbase + ks * 2048, kLboA, 1024),
-                      umma_smem_desc(vbase + ks * 2048, vlbo, 1024), id_s, (j > 0) || (ks > 0));
+              umma_ss(tmem + C::tS, umma_desc_add(dk, ks * 2048), umma_desc_add(dv, ks * 2048), id_s, (j > 0) || (ks > 0));
             umma_commit(&bar.ka_free[sa]);  // second arrival: the store warp, once the tile is parked
             umma_commit(&bar.v_free[sv]);
             ++nv;
@@ -582,10 +583,11 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
             break;
           }
           tc_fence_after_sync();
-#pragma unroll 2
+          const uint64_t dkp = umma_smem_desc(kbase, 16, 1024), dks = umma_smem_desc(kbase, kLboA, 1024),
+                         dv = umma_smem_desc(vbase, vlbo, 1024);
+#pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            umma_ts(tmem + C::tP, tq + ks * 8,
-                    umma_smem_desc(kbase + (ks >> 2) * C::kBoxBytes + (ks & 3) * 32, 16, 1024), id_p, ks > 0);
+            umma_ts(tmem + C::tP, tq + ks * 8, umma_desc_add(dkp, (ks >> 2) * C::kBoxBytes + (ks & 3) * 32), id_p, ks > 0);
           umma_commit(&bar.p_full);
           if (!mbar_wait(&bar.v_full[sv], (nv / VS) & 1, p.status, 202) ||
               !mbar_wait(&bar.s_loaded, n_sl & 1, p.status, 203)) {
@@ -594,10 +596,9 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           }
           ++n_sl;
           tc_fence_after_sync();
-#pragma unroll 2
+#pragma unroll
           for (int ks = 0; ks < 8; ++ks)
-            umma_ss(tmem + C::tS, umma_smem_desc(kbase + ks * 2048, kLboA, 1024),
-                    umma_smem_desc(vbase + ks * 2048, vlbo, 1024), id_s, true);
+            umma_ss(tmem + C::tS, umma_desc_add(dks, ks * 2048), umma_desc_add(dv, ks * 2048), id_s, true);
           umma_commit(&bar.s_full);
           umma_commit(&bar.k_free[sk]);
           if (!mbar_wait(&bar.sb_full, n_sb & 1, p.status, 204)) { ok = false; break; }
@@ -607,21 +608,18 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
             ++n_of;
           }
           tc_fence_after_sync();
-#pragma unroll 2
+#pragma unroll
           for (int ks = 0; ks < D / 16; ++ks)
-            umma_ts(tmem + C::tO, tq + ks * 8, umma_smem_desc(smem_u32(sSb) + ks * 2048, C::kSbBox, 1024), id_o,
-                    ks > 0);
+            umma_ts(tmem + C::tO, tq + ks * 8, umma_desc_add(dsb, ks * 2048), id_o, ks > 0);
           umma_commit(&bar.mma2_done);
           umma_commit(&bar.qphi_free[sq]);
           if (j == it.nC - 1) umma_commit(&bar.sb_idle);  // Sb may now take a K tile of the next pass A
           if (!mbar_wait(&bar.pm_full, n_pm & 1, p.status, 206)) { ok = false; break; }
           ++n_pm;
           tc_fence_after_sync();
-#pragma unroll 2
+#pragma unroll
           for (int ks = 0; ks < 8; ++ks)
-            umma_ts(tmem + C::tO, tmem + C::tP + (ks >> 2) * 64 + (ks & 3) * 8,
-                    umma_smem_desc(vbase + ks * 2048, vlbo, 1024),
-                    id_o, true);
+            umma_ts(tmem + C::tO, tmem + C::tP + (ks >> 2) * 64 + (ks & 3) * 8, umma_desc_add(dv, ks * 2048), id_o, true);
           umma_commit(&bar.o_full);
           ++nv;
           ++nq;

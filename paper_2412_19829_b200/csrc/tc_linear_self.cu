@@ -163,11 +163,11 @@ linear_self_reduce_kernel(const __grid_constant__ CUtensorMap mk, const __grid_c
             break;
           }
           tc_fence_after_sync();
-          const uint32_t kbase = smem_u32(sK) + sk * C::kTile, vbase = smem_u32(sm) + C::v_off(sv);
+          const uint64_t dk = umma_smem_desc(smem_u32(sK) + sk * C::kTile, kLboA, 1024),
+                         dv = umma_smem_desc(smem_u32(sm) + C::v_off(sv), C::v_lbo(sv), 1024);
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)
-            umma_ss(acc, umma_smem_desc(kbase + ks * 2048, kLboA, 1024),
-                    umma_smem_desc(vbase + ks * 2048, C::v_lbo(sv), 1024), id_s, (j > 0) || (ks > 0));
+            umma_ss(acc, umma_desc_add(dk, ks * 2048), umma_desc_add(dv, ks * 2048), id_s, (j > 0) || (ks > 0));
           umma_commit(&k_free[sk]);
           umma_commit(&v_free[sv]);
           ++nk;
@@ -628,11 +628,11 @@ linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_co
             break;
           }
           tc_fence_after_sync();
-          const uint32_t kbase = smem_u32(sm) + C::kK + sk * C::kTile, vbase = smem_u32(sm) + sv * kBox;
+          const uint64_t dk = umma_smem_desc(smem_u32(sm) + C::kK + sk * C::kTile, 0, 1024),
+                         dv = umma_smem_desc(smem_u32(sm) + sv * kBox, (4 - sv) * kBox, 1024);
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)  // (rows 64..127 of the product mirror 0..63)
-            umma_ss(acc, umma_smem_desc(kbase + ks * 2048, 0, 1024),
-                    umma_smem_desc(vbase + ks * 2048, (4 - sv) * kBox, 1024), id_s, (j > 0) || (ks > 0));
+            umma_ss(acc, umma_desc_add(dk, ks * 2048), umma_desc_add(dv, ks * 2048), id_s, (j > 0) || (ks > 0));
           umma_commit(&k_free[sk]);
           umma_commit(&v_free[sv]);
         }

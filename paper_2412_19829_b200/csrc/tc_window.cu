@@ -330,7 +330,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           const int n_sub = x.n_sub(t);
           const uint32_t rbase = kt + (t ? (uint32_t)x.off(1) : 0u);  // ring number of the stream's first half tile
           const uint32_t qbuf = (qn + t) % 3;
-          const uint32_t qa = aX + qbuf * SM::kTile;
+          const uint64_t dq = umma_smem_desc(aX + qbuf * SM::kTile, 16, 1024);
           for (int m = 0; m < n_sub + 2 && n_sub > 0; ++m) {
             if (m >= 2) {  // O += P V of half tile jj
               const int jj = m - 2, half = jj & 1;
@@ -340,11 +340,11 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
               // the first product of a tile overwrites O: the previous tile's epilogue has read it
               if (jj == 0 && ntile >= 1 && !mbar_wait(&ctl->o_free[t], (ntile - 1) & 1, p.status, 24)) return;
               tc_fence_after_sync();
-              const uint32_t va = aV + slot * SM::kHalf, tP = tSt + half * 64;
+              const uint64_t dv = umma_smem_desc(aV + slot * SM::kHalf, 8192, 1024);
+              const uint32_t tP = tSt + half * 64;
 #pragma unroll
               for (int ks = 0; ks < 4; ++ks)
-                umma_ts(tO, tP + (ks >> 1) * 32 + (ks & 1) * 8, umma_smem_desc(va + ks * 2048, 8192, 1024), idesc_pv,
-                        (jj > 0) || (ks > 0));
+                umma_ts(tO, tP + (ks >> 1) * 32 + (ks & 1) * 8, umma_desc_add(dv, ks * 2048), idesc_pv, (jj > 0) || (ks > 0));
               umma_commit(&ctl->v_empty[slot]);
               umma_commit(&ctl->pv_done[t]);
               if (jj == n_sub - 1) umma_commit(&ctl->o_full[t]);
@@ -367,11 +367,11 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
               if (m == 0 && !mbar_wait(&ctl->q_full[qbuf], ((qn + t) / 3) & 1, p.status, 20)) return;
               if (!landed(&ctl->k_issued, ctl->k_full, n, 21)) return;
               tc_fence_after_sync();
-              const uint32_t ka = aK + slot * SM::kHalf;
+              const uint64_t dk = umma_smem_desc(aK + slot * SM::kHalf, 16, 1024);
 #pragma unroll
               for (int ks = 0; ks < D / 16; ++ks)
-                umma_ss(tSt + half * 64, umma_smem_desc(qa + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024),
-                        umma_smem_desc(ka + (ks >> 2) * 8192 + (ks & 3) * 32, 16, 1024), idesc_qk, ks > 0);
+                umma_ss(tSt + half * 64, umma_desc_add(dq, (ks >> 2) * 16384 + (ks & 3) * 32),
+                        umma_desc_add(dk, (ks >> 2) * 8192 + (ks & 3) * 32), idesc_qk, ks > 0);
               umma_commit(&ctl->s_full[t][half]);
               umma_commit(&ctl->k_empty[slot]);
               // stream 0 tells where its next S will read: the next half tile of this query tile,
