@@ -60,7 +60,7 @@ struct WinCtl {
   uint32_t k_issued, v_issued;  // half tiles whose load the producer has issued (monotonic)
   uint32_t tmem_base;
   int units_posted;          // entries of unit_ring written so far (monotonic)
-  int unit_ring[kUnitRing];  // the CTA's n-th work unit (-1: no more)
+  int4 unit_ring[kUnitRing];  // the CTA's n-th work unit: pair of query tiles (-1: no more), head, sequence
 };
 
 template <int D>
@@ -77,7 +77,7 @@ struct WinSmem {
   static constexpr int kSlack = (D == 128) ? 0 : 1024;
   static constexpr int kBytes = kCtl + 640 + kSlack;
 };
-static_assert(sizeof(WinCtl) <= 640, "control block");
+static_assert(sizeof(WinCtl) <= 640 && alignof(WinCtl) <= 16, "control block");
 static_assert(WinSmem<128>::kBytes <= 227 * 1024, "shared memory of one SM");
 
 struct WinParams {
@@ -151,6 +151,11 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   WinCtl* ctl = reinterpret_cast<WinCtl*>(sm + SM::kCtl);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // (divisions once per unit, by the thread that draws it)
+  auto split = [&](int u) -> int4 {
+    const int bh = u / p.npair, b = bh / p.h_count;
+    return make_int4(u - bh * p.npair, p.h_begin + bh - b * p.h_count, b, 0);
+  };
 
   if (tid == 0) {
     for (int i = 0; i < 3; ++i) {
@@ -172,7 +177,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       mbar_init(&ctl->o_full[i], 1);
       mbar_init(&ctl->o_free[i], 256);
     }
-    ctl->unit_ring[0] = blockIdx.x;  // the grid never exceeds the number of units
+    ctl->unit_ring[0] = split(blockIdx.x);  // the grid never exceeds the number of units
     ctl->front = ctl->k_issued = ctl->v_issued = 0;
     ctl->units_posted = 1;
     mbar_fence_init();
@@ -190,13 +195,11 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   tc_fence_after_sync();
   const uint32_t tmem = ctl->tmem_base;
 
-  auto decode = [&](int u) {
+  auto decode = [&](int4 u) {
     Unit x;
-    const int pq = u % p.npair;
-    const int bh = u / p.npair;
-    x.h = p.h_begin + bh % p.h_count;
-    x.b = bh / p.h_count;
-    x.qtA = 2 * pq;
+    x.qtA = 2 * u.x;
+    x.h = u.y;
+    x.b = u.z;
     x.nt = (x.qtA + 1 < p.nqt) ? 2 : 1;
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
@@ -207,9 +210,9 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     }
     return x;
   };
-  auto unit_at = [&](uint32_t n) -> int {
-    if (!win_wait_epoch(&ctl->units_posted, (int)n + 1, p.status, 90)) return -1;
-    return reinterpret_cast<const volatile int*>(ctl->unit_ring)[n % kUnitRing];
+  auto unit_at = [&](uint32_t n) -> int4 {
+    if (!win_wait_epoch(&ctl->units_posted, (int)n + 1, p.status, 90)) return make_int4(-1, 0, 0, 0);
+    return ctl->unit_ring[n % kUnitRing];
   };
 
   // Every role walks the same list of units and keeps the same running counters (units, query
@@ -219,11 +222,11 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     if (elect_one()) {
       uint32_t nu = 0, kt = 0;
       bool ok = true;
-      for (int u = blockIdx.x; u >= 0 && ok;) {
+      for (int4 u = ctl->unit_ring[0]; u.x >= 0 && ok;) {
         const Unit x = decode(u);
         // draw the next ticket now; its value is needed once this unit's first loads are out
         const unsigned int t_next = atomicAdd(p.ticket, 1u);
-        int u_next = -1;
+        int4 u_next = make_int4(-1, 0, 0, 0);
         const int g0 = x.f[0], g1 = x.nt == 2 ? x.l[1] : x.l[0];
         // A slot is released by two arrivals.  For a stream that has no use for a half tile the producer arrives itself,
         // so that the stream need not wait until it has landed.
@@ -245,7 +248,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           if (unused) mbar_arrive(&ctl->v_empty[slot]);
           publish(&ctl->v_issued, kt + 1);
           if (hg == 2 * g0) {  // the other roles learn of the next unit early (its Q is requested ahead)
-            u_next = (t_next < (unsigned int)(p.total - (int)gridDim.x)) ? (int)(gridDim.x + t_next) : -1;
+            if (t_next < (unsigned int)(p.total - (int)gridDim.x)) u_next = split((int)(gridDim.x + t_next));
             ctl->unit_ring[(nu + 1) % kUnitRing] = u_next;
             __threadfence_block();
             *reinterpret_cast<volatile int*>(&ctl->units_posted) = (int)nu + 2;
@@ -266,8 +269,8 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       bool ld_end = false;
       auto load_next = [&]() {
         if (ld_end) return;
-        const int u = unit_at(ld_nu);
-        if (u < 0) { ld_end = true; return; }
+        const int4 u = unit_at(ld_nu);
+        if (u.x < 0) { ld_end = true; return; }
         const Unit x = decode(u);
         const uint32_t buf = ql % 3;
         mbar_arrive_expect_tx(&ctl->q_full[buf], SM::kTile);
@@ -281,8 +284,8 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       load_next();
       load_next();
       for (;;) {
-        const int u = unit_at(st_nu);
-        if (u < 0) break;
+        const int4 u = unit_at(st_nu);
+        if (u.x < 0) break;
         const Unit x = decode(u);
         const uint32_t buf = qs % 3;
         if (!mbar_wait(&ctl->stage_full[buf], (qs / 3) & 1, p.status, 40)) break;
@@ -323,8 +326,8 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
                  mbar_wait(&full[n % ST], (n / ST) & 1, p.status, where);
         };
         for (uint32_t nu = 0;; ++nu) {
-          const int u = unit_at(nu);
-          if (u < 0) break;
+          const int4 u = unit_at(nu);
+          if (u.x < 0) break;
           const Unit x = decode(u);
           const uint32_t n_half = 2 * (uint32_t)((x.nt == 2 ? x.l[1] : x.l[0]) - x.f[0] + 1);
           const int n_sub = x.n_sub(t);
@@ -405,8 +408,8 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     uint32_t nu = 0, sub = 0, ntile = 0, qn = 0;
     bool ok = true;
     for (; ok; ++nu) {
-      const int u = unit_at(nu);
-      if (u < 0) break;
+      const int4 u = unit_at(nu);
+      if (u.x < 0) break;
       const Unit x = decode(u);
       const uint32_t buf = (qn + t) % 3;
       qn += (uint32_t)x.nt;
