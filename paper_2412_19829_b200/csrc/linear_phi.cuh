@@ -34,7 +34,7 @@ __device__ __forceinline__ uint32_t phi_sel(uint32_t w) {
 // thread (number tt) takes one 16-byte column chunk of rows sixteen apart, so that the tile is spread over all of them
 // whatever D is (with four rows per thread half of 512 threads had nothing to do at D = 64: 832 chains of 4096 tokens
 // 388 -> 364 us).  Rows from n_valid on (past the end of the sequence) become zero.
-template <int D, bool kId, int NT>
+template <int D, int NT>
 __device__ __forceinline__ void transform_k_tile(uint8_t* tile, int tt, int n_valid) {
   constexpr int kBox = 16384, kChunks = D / 8, kRows = 8 * 16 * kChunks / NT;
   const int cc = (tt >> 4) % kChunks, row0 = (tt & 15) + 16 * kRows * ((tt >> 4) / kChunks), cin = cc & 7;
@@ -47,10 +47,10 @@ __device__ __forceinline__ void transform_k_tile(uint8_t* tile, int tt, int n_va
   }
 #pragma unroll
   for (int k = 0; k < kRows; ++k) {
-    raw[k].x = phi_sel<kId>(raw[k].x);
-    raw[k].y = phi_sel<kId>(raw[k].y);
-    raw[k].z = phi_sel<kId>(raw[k].z);
-    raw[k].w = phi_sel<kId>(raw[k].w);
+    raw[k].x = phi_bf16x2(raw[k].x);
+    raw[k].y = phi_bf16x2(raw[k].y);
+    raw[k].z = phi_bf16x2(raw[k].z);
+    raw[k].w = phi_bf16x2(raw[k].w);
   }
   if (n_valid < 128) {
 #pragma unroll

@@ -270,7 +270,7 @@ __device__ __forceinline__ bool publish_inclusive(const LinParams& p, const LinI
 // segments before it, added by the 16 phi warps (each thread one row x a quarter of the columns) in the order in which the
 // inclusive states of a chain would have been.  Every segment publishes its own contribution as soon as its first pass is
 // over, so no segment waits for the one before it to have waited.
-template <int D>
+template <int D, bool kPark>
 __device__ __forceinline__ bool sum_states(const LinParams& p, const LinItem& it, LinBarriers& bar, uint8_t* sSb,
                                            uint32_t tmem, int warp, int lane, const int* prev_epoch) {
   using C = LinCfg<D>;
@@ -325,7 +325,7 @@ __device__ __forceinline__ bool sum_states(const LinParams& p, const LinItem& it
       }
     }
   }
-  ok = mbar_wait(&bar.sb_parked, 0, p.status, 602);  // Sb held K tiles in pass A
+  if (kPark) ok = mbar_wait(&bar.sb_parked, 0, p.status, 602);  // Sb held K tiles in pass A
   if (__any_sync(0xffffffffu, !ok)) return false;
   tc_fence_after_sync();
   uint32_t v[W];
@@ -360,6 +360,11 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
                  const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtensorMap mo,
                  const LinParams p) {
   using C = LinCfg<D>;
+  // Features given (kId): a K tile is ready for the tensor core as it lands (rows past the end of the sequence are filled
+  // with zeros by the copy), so nobody transforms it, nothing is parked (pass C reads the feature tensor again) and a
+  // chain's last segment has no pass A (26 chains of 32K
+  // tokens, d = 128, in a layer of 32 heads: 454 -> 426 us).
+  constexpr bool kPark = !kDirect && !kId;
   extern __shared__ uint8_t raw_smem[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw_smem) + 1023) & ~(uintptr_t)1023);
   uint8_t* sK = sm + C::kK;
@@ -386,7 +391,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     for (int s = 0; s < 5; ++s) {
       mbar_init(&bar.ka_full[s], 1);
       mbar_init(&bar.kphi_full[s], 16);
-      mbar_init(&bar.ka_free[s], 2);  // the MMA issuer and the store warp
+      mbar_init(&bar.ka_free[s], kPark ? 2 : 1);  // the MMA issuer and the store warp
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&bar.k_full[s], 1);
@@ -474,8 +479,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       const uint64_t pol_stream = l2_policy_evict_first(), pol_keep = l2_policy_evict_last();
       for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
         const LinItem it = decode_item(p, item);
-        for (int pass = kDirect ? 1 : 0; pass < 2 && ok; ++pass) {
-          if (!kDirect && pass == 1 && !mbar_wait(&bar.park_done, n_items & 1, p.status, 103)) { ok = false; break; }
+        for (int pass = (kPark || it.need_dS) ? 0 : 1; pass < 2 && ok; ++pass) {
+          if (kPark && pass == 1 && !mbar_wait(&bar.park_done, n_items & 1, p.status, 103)) { ok = false; break; }
           for (int j = 0; j < it.nC; ++j) {
             const int n0 = (it.c_begin + j) * 128;
             if (pass == 0) {
@@ -495,7 +500,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
               mbar_arrive_expect_tx(&bar.ka_full[sa], C::kTile);
               for (int x = 0; x < D / 64; ++x)
                 tma_load_4d_hint(a_kslot(sa) + x * C::kBoxBytes, &mk, &bar.ka_full[sa], x * 64, n0, it.h, it.b,
-                                 pol_stream);
+                                 kPark ? pol_stream : pol_keep);
               ++iss_a[sa];
               ++ta;
             } else {
@@ -504,8 +509,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
                    (kDirect || drain(&bar.ka_free[sc], obs_a[sc], iss_a[sc], 101));
               if (!ok) break;
               mbar_arrive_expect_tx(&bar.k_full[sc], C::kTile);
-              for (int x = 0; x < D / 64; ++x)  // the phi(K) tile parked in the output rows (kDirect: raw K)
-                tma_load_4d_hint(sK + sc * C::kTile + x * C::kBoxBytes, kDirect ? &mk : &mo, &bar.k_full[sc], x * 64, n0,
+              for (int x = 0; x < D / 64; ++x)  // the phi(K) tile parked in the output rows, or K itself
+                tma_load_4d_hint(sK + sc * C::kTile + x * C::kBoxBytes, kPark ? &mo : &mk, &bar.k_full[sc], x * 64, n0,
                                  it.h, it.b, pol_stream);
               ++iss_c[sc];
               ++nq;
@@ -547,9 +552,10 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         }
         first_item = false;
         // ---- pass A: dS = sum Kc^T V over the segment, from zero (only if somebody needs it)
-        for (int j = 0; j < (kDirect ? 0 : it.nC); ++j) {
+        const int nA = (kPark || it.need_dS) ? it.nC : 0;  // K tiles of pass A
+        for (int j = 0; j < nA; ++j) {
           const uint32_t sa = ta % KA;
-          if (!mbar_wait(&bar.kphi_full[sa], (ta / KA) & 1, p.status, 220)) { ok = false; break; }
+          if (!mbar_wait(kId ? &bar.ka_full[sa] : &bar.kphi_full[sa], (ta / KA) & 1, p.status, 220)) { ok = false; break; }
           if (it.need_dS) {
             const int sv = nv % VS;
             const uint32_t kbase = smem_u32(a_kslot(sa)), vbase = smem_u32(v_box(sv, 0));
@@ -576,9 +582,9 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           const uint32_t kbase = smem_u32(sK) + sk * C::kTile, vbase = smem_u32(v_box(sv, 0));
           const uint32_t vlbo = C::v_lbo(sv);
           const uint32_t tq = tmem + C::tQ + sq * (D / 2);
-          // the chunk's phi(K) tile: read back from the park, or (kDirect) transformed in place
+          // the chunk's phi(K) tile: read back from the park or given, or (kDirect) transformed in place
           if (!mbar_wait(&bar.qphi_full[sq], (nq / QS) & 1, p.status, 200) ||
-              !mbar_wait(kDirect ? &bar.kd_phi[sk] : &bar.k_full[sk], (nq / KS) & 1, p.status, 201)) {
+              !mbar_wait(kDirect && !kId ? &bar.kd_phi[sk] : &bar.k_full[sk], (nq / KS) & 1, p.status, 201)) {
             ok = false;
             break;
           }
@@ -704,7 +710,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         nv += it.nC;
       }
       // Sb held K tiles in pass A: they have been parked (and, above, consumed by the tensor core)
-      if (!kDirect) ok = mbar_wait(&bar.sb_parked, n_items & 1, p.status, 314) && ok;
+      if (kPark) ok = mbar_wait(&bar.sb_parked, n_items & 1, p.status, 314) && ok;
       // the K group has read the previous item's last state out of TMEM
       if (n_items > 0) ok = mbar_wait(&bar.s_final, (n_items - 1) & 1, p.status, 315) && ok;
       tc_fence_after_sync();
@@ -854,16 +860,16 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       auto transform_direct = [&](uint32_t idx, int jrow) {
         const uint32_t sl = idx % KS;
         ok = ok && mbar_wait(&bar.k_full[sl], (idx / KS) & 1, p.status, 430);
-        if (ok) transform_k_tile<D, kId, 512>(sK + sl * C::kTile, tt, p.N - (it.c_begin + jrow) * 128);
+        if (ok) transform_k_tile<D, 512>(sK + sl * C::kTile, tt, p.N - (it.c_begin + jrow) * 128);
         __syncwarp();
         if (ok && lane == 0) mbar_arrive(&bar.kd_phi[sl]);
       };
-      if (kDirect) transform_direct(nq, 0);
+      if (kDirect && !kId) transform_direct(nq, 0);
       // ---- pass A: the two groups take half of every K tile each
-      for (int j = 0; j < (kDirect ? 0 : it.nC); ++j) {
+      for (int j = 0; j < (kPark ? it.nC : 0); ++j) {
         const uint32_t sk = ta % KA;
         ok = ok && mbar_wait(&bar.ka_full[sk], (ta / KA) & 1, p.status, 410);
-        if (ok) transform_k_tile<D, kId, 512>(a_kslot(sk), tt, p.N - (it.c_begin + j) * 128);
+        if (ok) transform_k_tile<D, 512>(a_kslot(sk), tt, p.N - (it.c_begin + j) * 128);
         __syncwarp();
         if (ok && lane == 0) mbar_arrive(&bar.kphi_full[sk]);  // the tile may go to the tensor core and be parked
         ++ta;
@@ -871,7 +877,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
 
       // ---- hand-over of S: the two groups publish the inclusive state (column quarters 0, 1 / 2, 3)
       if constexpr (kSum) {
-        ok = ok && sum_states<D>(p, it, bar, sSb, tmem, warp, lane, &prev_epoch);
+        ok = ok && sum_states<D, kPark>(p, it, bar, sSb, tmem, warp, lane, &prev_epoch);
       } else if (it.need_dS) {
         ok = publish_inclusive<D>(p, it, bar, tmem, warp, lane, n_a & 1, &prev_epoch, (int)n_items);
         ++n_a;
@@ -915,7 +921,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           // kDirect: this group's half of the next chunk's K tile, between the mask, which the tensor core waits for,
           // and the state, which waits for the tensor core (before the mask it held that back until the tile had
           // landed: 26 chains of 32K tokens, d = 128, 669 -> 642 us; 80 x 2048, d = 64, 40 -> 38 us)
-          if (kDirect && j + 1 < it.nC) transform_direct(nq + 1, j + 1);
+          if (kDirect && !kId && j + 1 < it.nC) transform_direct(nq + 1, j + 1);
           if (!ok) break;
           // ---- S: the fp32 master stays in TMEM; once this chunk's readout has consumed the old
           //      bf16 copy, stream the new one (and z) into shared memory for the next chunk.
@@ -1059,7 +1065,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
               if (lane == 0) mbar_arrive(&bar.qphi_full[sq]);
             }
           }
-          if (kDirect && ok && j + 1 < it.nC) transform_direct(nq + 1, j + 1);
+          if (kDirect && !kId && ok && j + 1 < it.nC) transform_direct(nq + 1, j + 1);
           ok = !__any_sync(0xffffffffu, !ok);
           ++nq;
         }
@@ -1078,7 +1084,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
         const LinItem it = decode_item(p, item);
         // ---- pass A: park phi(K) tiles in the output rows of their chunk
-        for (int j = 0; j < (kDirect ? 0 : it.nC); ++j) {
+        for (int j = 0; j < (kPark ? it.nC : 0); ++j) {
           const uint32_t sk = ta % KA;
           if (!mbar_wait(&bar.kphi_full[sk], (ta / KA) & 1, p.status, 520)) { ok = false; break; }
           for (int x = 0; x < D / 64; ++x)

@@ -157,7 +157,7 @@ linear_self_reduce_kernel(const __grid_constant__ CUtensorMap mk, const __grid_c
         if (na >= 2 && !mbar_wait(&acc_free[na & 1], ((na >> 1) + 1) & 1, p.status, 710)) break;
         for (int j = 0; j < it.nC; ++j) {
           const uint32_t sk = nk % KS, sv = nv % VS;
-          if (!mbar_wait(&kphi[sk], (nk / KS) & 1, p.status, 711) ||
+          if (!mbar_wait(kId ? &k_full[sk] : &kphi[sk], (nk / KS) & 1, p.status, 711) ||
               !mbar_wait(&v_full[sv], (nv / VS) & 1, p.status, 712)) {
             ok = false;
             break;
@@ -206,8 +206,9 @@ linear_self_reduce_kernel(const __grid_constant__ CUtensorMap mk, const __grid_c
       tc_fence_before_sync();
       mbar_arrive(&acc_free[na & 1]);
     }
-  } else {
-    // phi on the K tiles, in place, by 16 warps
+  } else if (!kId) {
+    // phi on the K tiles, in place, by 16 warps (features given: a tile is ready as it lands, rows past the end of the
+    // sequence filled with zeros by the copy)
     const int tt = tid - 6 * 32;
     uint32_t nk = 0;
     bool ok = true;
@@ -216,7 +217,7 @@ linear_self_reduce_kernel(const __grid_constant__ CUtensorMap mk, const __grid_c
       for (int j = 0; j < it.nC; ++j) {
         const uint32_t sk = nk % KS;
         ok = ok && mbar_wait(&k_full[sk], (nk / KS) & 1, p.status, 730);
-        if (ok) transform_k_tile<D, kId, 512>(sK + sk * C::kTile, tt, p.N - (it.c_begin + j) * 128);
+        if (ok) transform_k_tile<D, 512>(sK + sk * C::kTile, tt, p.N - (it.c_begin + j) * 128);
         __syncwarp();
         if (ok && lane == 0) mbar_arrive(&kphi[sk]);
         ++nk;
@@ -623,7 +624,8 @@ linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_co
         if (c >= 2 && !mbar_wait(&acc_free[c & 1], ((c >> 1) + 1) & 1, p.status, 910)) break;
         for (int j = 0; j < it.nC; ++j, ++n) {
           const uint32_t sk = n % KS, sv = n % VS;
-          if (!mbar_wait(&kphi[sk], (n / KS) & 1, p.status, 911) || !mbar_wait(&v_full[sv], (n / VS) & 1, p.status, 912)) {
+          if (!mbar_wait(kId ? &k_full[sk] : &kphi[sk], (n / KS) & 1, p.status, 911) ||
+              !mbar_wait(&v_full[sv], (n / VS) & 1, p.status, 912)) {
             ok = false;
             break;
           }
@@ -756,16 +758,18 @@ linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_co
       }
     }
   } else if (warp < 22) {
+    if constexpr (!kId) {  // phi on the K tiles, in place (features given: a tile is ready as it lands)
     uint32_t n = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
       for (int j = 0; j < p.nch; ++j, ++n) {
         const uint32_t sk = n % KS;
         ok = ok && mbar_wait(&k_full[sk], (n / KS) & 1, p.status, 950);
-        if (ok) transform_k_tile<D, kId, 256>(sm + C::kK + sk * C::kTile, tid - 14 * 32, p.N - j * 128);
+        if (ok) transform_k_tile<D, 256>(sm + C::kK + sk * C::kTile, tid - 14 * 32, p.N - j * 128);
         __syncwarp();
         if (ok && lane == 0) mbar_arrive(&kphi[sk]);
       }
+    }
     }
   } else if (warp < 26) {
     // totals: one thread per feature row

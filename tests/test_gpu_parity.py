@@ -1062,6 +1062,23 @@ def test_favor_causal_linear_both_forms_and_bnhd(split):
     assert_parity(f64(o.permute(0, 2, 1, 3)), ref, "bf16", f"favor linear bnhd split={split}")
 
 
+@pytest.mark.parametrize("H,N,d,split", [(100, 700, 64, 2), (100, 641, 128, 1), (60, 1153, 128, 3), (160, 383, 64, 3)])
+def test_favor_cut_chains_in_several_rounds(H, N, d, split):
+    """Features need no first pass in a chain's last segment: several items per CTA, of one to three chunks, the last
+    chunk ragged, with the state carried in and out.  Gates of the other feature tests."""
+    q, k, v = synth.qkv(1, H, N, d, "bf16", seed=870 + N)
+    W = _proj(H, d, "bf16", seed=871)
+    S, z = torch.rand(1, H, d, d, device="cuda"), 1.0 + torch.rand(1, H, d, device="cuda")
+    S_ref, z_ref = f64(S), f64(z)
+    ref = oracle.causal_linear_attn(f64(q), f64(k), f64(v), S_ref, z_ref, W=f64(W))
+    gf.set_tuning(gf.GF_TUNE_LINEAR_SPLIT, split)
+    ws = gf.Workspace.for_problem(1, H, N, d, 1, 0, phi=gf.GF_PHI_FAVOR_POS)
+    o = gf.causal_linear_attn(*dev(q, k, v), S, z, W=W.cuda(), ws=ws)
+    assert ws.last_device_status() == gf.GF_OK
+    assert_parity(f64(o), ref, "bf16", f"favor linear H={H} N={N} d={d} split={split}")
+    assert errors(f64(S), S_ref)["rel_l2"] <= 1e-2 and errors(f64(z), z_ref)["rel_l2"] <= 1e-2
+
+
 @pytest.mark.parametrize("dtype,force_simt", [("f32", 0), ("bf16", 1)])
 @pytest.mark.parametrize("N,d", [(1, 64), (130, 64), (300, 128)])
 def test_favor_causal_linear_cuda_core_path(dtype, force_simt, N, d):
