@@ -15,15 +15,18 @@
 // A (batch, head) chain is cut into segments of L chunks; a work item is one segment.  CTAs are
 // persistent and take items round-robin in an order in which a segment's predecessor always has
 // a smaller index, so the CTA that owns it is already running.  For an item the CTA
-//   (A) applies phi to the segment's K tiles once, parks the results in the rows of the OUTPUT
+//   (A) walks the segment's chunks from the last to the first (a sum has no order, and the tiles that pass C wants first
+//       are then the last to have been in L2: one round of segments of 47 chunks, 13 chains of 64K tokens, D = 64, 131 ->
+//       121 us), applies phi to the K tiles once, parks the results in the rows of the OUTPUT
 //       tensor that this segment will later overwrite (no extra scratch, and the lines are still
 //       in L2 when pass C reads them back) and accumulates the segment's own state contribution
 //       dS | dz = sum Kc^T [V | 1] (not for a chain's last segment, whose contribution nobody needs),
 //   (B) waits for the inclusive state of the previous segment in global scratch (one bounded
 //       poller per CTA), publishes its own inclusive state = previous + dS and raises its flag;
 //       when every CTA has one segment (kSum) all publish dS at once instead and each adds up
-//       those before it, which takes the chain of hand-overs out of the call (about 2.8 us per
-//       segment at D = 128: 24 chains of 4798 tokens 50.6 -> 42.1 us, one of 32 768 107 -> 66),
+//       those before it, a lane of its flag warp per flag, which takes the chain of hand-overs out of
+//       the call (about 2.8 us per segment at D = 128: 24 chains of 4798 tokens 50.6 -> 42.1 us, one of
+//       32 768 107 -> 64),
 //   (C) walks its chunks with the full pipeline starting from the previous segment's state,
 //       reading phi(K) back instead of K, so every exponential of the layer is computed once.
 // Warp roles:
@@ -190,6 +193,15 @@ __device__ __forceinline__ bool wait_flag(const unsigned int* flag, unsigned int
   }
 }
 
+
+// The segment's published state is complete: releases it to whoever waits for the flag (one thread, on behalf of the warps
+// that have arrived at pub_done).
+__device__ __forceinline__ void raise_flag(const LinParams& p, long long slot) {
+  // (status[4]: failure injection for tests -- that segment's flag is never raised)
+  if (reinterpret_cast<const volatile unsigned int*>(p.status)[4] == (unsigned int)slot + 1u) return;
+  const unsigned int one = 1u;
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.flags + slot * kFlagStride), "r"(one) : "memory");
+}
 
 // Named barrier over `n` threads that also ORs a predicate, so that a timed-out wait makes the
 // whole group leave its loop together (nobody is left behind at a barrier).
@@ -482,7 +494,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         for (int pass = (kPark || it.need_dS) ? 0 : 1; pass < 2 && ok; ++pass) {
           if (kPark && pass == 1 && !mbar_wait(&bar.park_done, n_items & 1, p.status, 103)) { ok = false; break; }
           for (int j = 0; j < it.nC; ++j) {
-            const int n0 = (it.c_begin + j) * 128;
+            const int n0 = (it.c_begin + (pass == 0 ? it.nC - 1 - j : j)) * 128;
             if (pass == 0) {
               const uint32_t sa = ta % KA;
               // the slot's earlier pass-A uses, and what shares the buffer in pass C: a K slot, or
@@ -869,7 +881,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       for (int j = 0; j < (kPark ? it.nC : 0); ++j) {
         const uint32_t sk = ta % KA;
         ok = ok && mbar_wait(&bar.ka_full[sk], (ta / KA) & 1, p.status, 410);
-        if (ok) transform_k_tile<D, 512>(a_kslot(sk), tt, p.N - (it.c_begin + j) * 128);
+        if (ok) transform_k_tile<D, 512>(a_kslot(sk), tt, p.N - (it.c_begin + it.nC - 1 - j) * 128);
         __syncwarp();
         if (ok && lane == 0) mbar_arrive(&bar.kphi_full[sk]);  // the tile may go to the tensor core and be parked
         ++ta;
@@ -1088,7 +1100,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           const uint32_t sk = ta % KA;
           if (!mbar_wait(&bar.kphi_full[sk], (ta / KA) & 1, p.status, 520)) { ok = false; break; }
           for (int x = 0; x < D / 64; ++x)
-            tma_store_4d_hint(&mo, a_kslot(sk) + x * C::kBoxBytes, x * 64, (it.c_begin + j) * 128, it.h, it.b,
+            tma_store_4d_hint(&mo, a_kslot(sk) + x * C::kBoxBytes, x * 64, (it.c_begin + it.nC - 1 - j) * 128, it.h, it.b,
                               pol_keep);
           tma_store_commit();
           tma_store_wait_read<0>();
@@ -1120,27 +1132,30 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     }
   } else {
     // ================================================================ flag warp
-    if (elect_one()) {
+    if constexpr (kSum) {  // own contribution out, then everybody's before it in: a flag per lane
+      const int item = blockIdx.x;
+      if (item < p.nitems) {
+        const LinItem it = decode_item(p, item);
+        const long long slot = (long long)it.chain * p.G + it.g;
+        bool ok = true;
+        if (it.need_dS && lane == 0) {
+          ok = mbar_wait(&bar.pub_done, 0, p.status, 510);
+          if (ok) raise_flag(p, slot);
+        }
+        for (int g = lane; g < it.g && ok; g += 32) ok = wait_flag(p.flags + (slot - it.g + g) * kFlagStride, p.status, 511);
+        ok = !__any_sync(0xffffffffu, !ok);
+        __syncwarp();
+        if (ok && lane == 0) {
+          __threadfence_block();
+          *reinterpret_cast<volatile int*>(&prev_epoch) = 1;
+        }
+      }
+    } else if (elect_one()) {
       uint32_t n_a = 0;
       int n_items = 0;
       for (int item = blockIdx.x; item < p.nitems; item += gridDim.x, ++n_items) {
         const LinItem it = decode_item(p, item);
         const long long slot = (long long)it.chain * p.G + it.g;
-        if constexpr (kSum) {  // own contribution out, then everybody's before it in
-          if (it.need_dS) {
-            if (!mbar_wait(&bar.pub_done, 0, p.status, 510)) break;
-            if (reinterpret_cast<const volatile unsigned int*>(p.status)[4] != (unsigned int)slot + 1u) {
-              const unsigned int one = 1u;
-              asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.flags + slot * kFlagStride), "r"(one) : "memory");
-            }
-          }
-          bool seen = true;
-          for (int g = 0; g < it.g && seen; ++g) seen = wait_flag(p.flags + (slot - it.g + g) * kFlagStride, p.status, 511);
-          if (!seen) break;
-          __threadfence_block();
-          *reinterpret_cast<volatile int*>(&prev_epoch) = 1;
-          break;
-        }
         // one poller per CTA: hundreds of threads spinning on a handful of L2 lines slow the whole chain
         if (it.g > 0 && !wait_flag(p.flags + (slot - 1) * kFlagStride, p.status, 511)) break;
         __threadfence_block();
@@ -1149,10 +1164,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           // every warp of the hand-over has written its part of the inclusive state
           if (!mbar_wait(&bar.pub_done, n_a & 1, p.status, 510)) break;
           ++n_a;
-          const unsigned int one = 1u;
-          // (status[4]: failure injection for tests -- that segment's flag is never raised)
-          if (reinterpret_cast<const volatile unsigned int*>(p.status)[4] != (unsigned int)slot + 1u)
-            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.flags + slot * kFlagStride), "r"(one) : "memory");
+          raise_flag(p, slot);
         }
       }
     }
@@ -1170,16 +1182,16 @@ bool tc_linear_supported(int N, int d, int dtype) {
   return dtype == GF_BF16 && (d == 64 || d == 128);
 }
 
-// Segmentation of the chains: G segments per chain, their lengths differing by one chunk at most
-// (the longest has *L_out chunks).  CTAs take items round-robin, so the kernel lasts about
-// ceil(items / CTAs) rounds of one item each, an item costing its chunks plus the fixed cost h of a
-// hand-over (about one chunk); but a chain is also a serial pipeline - first pass of a segment,
-// one hand-over link per segment (about 0.65 chunk each), second pass - which bounds the time
-// from below when there are few chains.  Among the segment counts allowed, take the one with the
-// least max(rounds x (L + h) x spill, L + 0.65 G).  Segments are between 4 and 32 chunks long;
-// spill > 1 charges segments too long for what the CTAs running at one time park (phi(K) and V of
-// their segments) to stay in L2.  The plan must not depend on the device that is current when the workspace size is asked
-// for, so without a CTA count it assumes the 148 SMs of a B200.
+// Segmentation of the chains: G segments per chain, their lengths differing by one chunk at most (the longest has *L_out
+// chunks).  Where the segments of all chains fit one round of the CTAs nothing is handed from one to the next (sum_states):
+// the call costs a start, a sum that grows with G and one segment's chunks.  Otherwise CTAs take items round-robin and the
+// kernel lasts about ceil(items / CTAs) rounds of one item each, an item costing its chunks plus the fixed cost h of a
+// hand-over (about one chunk), after a start in which the first hand-overs follow one another.  The segment count with the
+// least cost is taken.  Against rounds of several items one round measured (us): d = 64, 42 chains of 64 chunks 57 and 59,
+// 12 x 160 45 and 64, 60 x 64 79 and 81, but 50 x 64 (two thirds of the CTAs) 74 and 67; d = 128, 38 x 64 95 and 99, 18 x 160
+// 105 and 123, 50 x 64 129 and 119.  Segments are between 4 and 32 chunks long; spill > 1 charges segments too long for what
+// the CTAs running at one time park (phi(K) and V of their segments) to stay in L2.  The plan must not depend on the device
+// that is current when the workspace size is asked for, so without a CTA count it assumes the 148 SMs of a B200.
 namespace {
 constexpr int kPlanL8 = 8;  // segment length the scratch is sized for when chains are many
 // cost of a chunk of an uncut chain, in two-pass chunks
@@ -1187,9 +1199,18 @@ constexpr double direct_chunk_cost(int d) { return d == 128 ? 0.8 : 0.83; }
 // ... and in a round that only part of the CTAs take part in: at d = 128 a full round of uncut chains is bound by
 // HBM (3.3 us per chunk on a B200), a thin one by the CTA's own pipeline (2.4 us); at d = 64 the CTA's pipeline
 // bounds both
-constexpr double direct_chunk_floor(int d) { return d == 128 ? 0.59 : 0.83; }
+constexpr double direct_chunk_floor(int d) { return d == 128 ? 0.59 : 0.8; }
 // fixed cost of an item (hand-over, pipeline refill) in chunks: a chunk is cheaper at d = 64, the hand-over hardly
 constexpr double handover_cost(int d) { return d == 128 ? 1.1 : 1.6; }
+// start and end of a call, in chunks: cut chains in one round, whole chains, cut chains in several rounds
+constexpr double one_round_start(int d) { return d == 128 ? 2.9 : 5.3; }
+constexpr double kWholeStart = 3.0;
+constexpr double kRoundsStart = 1.3;
+// one link of the chain of hand-overs
+constexpr double kHandOver = 0.85;
+// In one round a chain of 300 chunks or less is cut into no more segments than this: a lone chain of 256 chunks would gain
+// another 6 to 12 % from twice as many, for twice the SMs, which the windowed heads of a layer can use.
+constexpr int kOneRoundMaxG = 22;
 // Range of segment counts the automatic plan chooses from.
 void plan_range(int nchains, int nch, int* g_min_out, int* g_max_out) {
   const int g_min8 = (nch + kPlanL8 - 1) / kPlanL8;
@@ -1232,40 +1253,37 @@ double best_cut(int nchains, int nch, int d, int kPlanSMs, int* G_out) {
     int G = 1;
     double best = 1e300;
     for (int g = g_min > 2 ? g_min : 2; g <= g_max; ++g) {
-      const long long items = (long long)nchains * g;
-      const long long rounds = (items + kPlanSMs - 1) / kPlanSMs;
+      const long long items = (long long)nchains * g, rounds = (items + kPlanSMs - 1) / kPlanSMs;
       const double L = (double)nch / g;
-      // What the running CTAs park at one time should stay in L2 (l2_park_bytes): of a
-      // longer segment the excess comes back from DRAM, up to 40 % more time per chunk when the
-      // rounds bound the time (when the serial chain does, DRAM has slack and nothing is charged).
-      const double l_cap = l2_park_bytes() / ((double)(items < kPlanSMs ? items : kPlanSMs) * 4.0 * 128.0 * d);
-      const double spill = L > l_cap ? 1.0 + 0.4 * (1.0 - l_cap / L) : 1.0;
-      const double by_rounds = (double)rounds * (L + handover_cost(d)) * spill, by_chain = L + 0.65 * g;
-      const double cost = by_rounds > by_chain ? by_rounds : by_chain;
+      // a chunk costs less while SMs are idle
+      const double chunk = 0.53 + 0.45 * items / (double)(rounds * kPlanSMs);
+      double cost;
+      if (rounds == 1) {
+        if (g > g_min && g > kOneRoundMaxG && g * g > 1.6 * nch) continue;
+        // a start, a sum over the segments and the longest segment's chunks
+        cost = one_round_start(d) + (d == 128 ? 0.12 : 0.085) * g + (d == 128 ? 1.04 : 0.98) * ((nch + g - 1) / g) * chunk;
+      } else {
+        // What the running CTAs park at one time should stay in L2 (l2_park_bytes): of a longer segment the excess comes
+        // back from DRAM, up to 40 % more time per chunk.
+        const double l_cap = l2_park_bytes() / (kPlanSMs * 4.0 * 128.0 * d);
+        const double spill = L > l_cap ? 1.0 + 0.4 * (1.0 - l_cap / L) : 1.0;
+        // A round lasts an item or, when a chain has many segments in it, that many hand-overs; the first round starts with
+        // them.
+        const double by_item = (1.02 * chunk * L + handover_cost(d)) * spill, links = kHandOver * kPlanSMs / nchains;
+        cost = kRoundsStart + (double)rounds * (by_item > links ? by_item : links) + links;
+      }
       if (cost < best * (1.0 - 1e-9)) {
         best = cost;
         G = g;
-      }
-    }
-    // Segments that fit one round need no chain of hand-overs (sum_states): the round costs about its chunks and hardly
-    // more when a chain has many segments.  Measured, one round against the best of several (us): d = 128, 24 chains of
-    // 6000 tokens 48.5 and 65.4, 42 x 3217 47.1 and 52.6, 26 x 16384 128 and 130, 52 x 6000 102 and 97; d = 64, 16 x 12000
-    // 40.0 and 56.9, 30 x 6000 38.5 and 46.0, 42 x 8192 59 and 60, 52 x 6000 61.6 and 56.5.
-    const int g1 = kPlanSMs / nchains;
-    if ((long long)nchains * G > kPlanSMs && g1 >= 2 && g1 >= g_min && g1 <= g_max) {
-      const double one_round = 0.2 + (d == 128 ? 0.95 : 1.05) * ((nch + g1 - 1) / g1) + 0.12 * g1;
-      if (one_round < best) {
-        best = one_round;
-        G = g1;
       }
     }
     *G_out = G;
     return best;
 }
 
-// Fixed cost, in two-pass chunks, of running the leftover chains as a launch of their own (the gap
-// between the launches, the second kernel's start-up and its uneven end: about 15 us).
-constexpr double kSecondLaunchCost = 6.0;
+// What running the leftover chains as a launch of their own costs beyond the start that best_cut counts (the gap between
+// the launches and the uneven end of the first).
+constexpr double kSecondLaunchCost = 1.0;
 }  // namespace
 
 // `*whole_out` leading chains are left whole (the one-pass form), the others are cut into *G_out
@@ -1299,8 +1317,9 @@ void linear_tc_plan_parts(int nchains, int N, int d, int split, int ctas, int* w
     // The same holds from half a round of chains on (measured at d = 64 with 78 to 104 chains: whole chains
     // 3-23 % faster than cut ones beside the windowed heads; with 65 chains the cut plan still wins).
     if (shared && (full > 0 || 2 * nchains >= kPlanSMs)) best = 1e300;
-    if (full_cost + (double)nch * last <= best) {
-      best = full_cost + (double)nch * last;
+    const double whole_cost = kWholeStart + full_cost + (double)nch * last;
+    if (whole_cost <= best) {
+      best = whole_cost;
       G = 1;
       whole = nchains;
     }
@@ -1310,7 +1329,7 @@ void linear_tc_plan_parts(int nchains, int N, int d, int split, int ctas, int* w
     // chains on 148 CTAs, a loss of 3 to 11 % from 34 on).
     if (full > 0 && rest > 0 && (!shared || 6 * rest <= kPlanSMs)) {
       int g_rest = 1;
-      const double mixed = full_cost + kSecondLaunchCost + best_cut(rest, nch, d, kPlanSMs, &g_rest);
+      const double mixed = kWholeStart + full_cost + kSecondLaunchCost + best_cut(rest, nch, d, kPlanSMs, &g_rest);
       if (g_rest > 1 && mixed < best) {
         G = g_rest;
         whole = full * kPlanSMs;
