@@ -9,14 +9,15 @@
 // and their products with the state stay inside the range of fp32 however small the key features
 // are.  The key features (and with them the state S, z) are the definition's.
 //
-// A CTA (two per SM) takes a run of consecutive 128-token tiles of Q, then of K, in (head, tile) order, so that a head's
-// projection W (d x d, row a = w_a) is loaded once for many tiles.  Per tile X (128 x d, by TMA into one of two
-// buffers): one tcgen05.mma group computes Y = X W^T (M = 128, N = d, K = d, both operands K-major from shared
-// memory) into one of two TMEM buffers; 128 threads, one per token (a group of four warps for each buffer), take
-// the exponentials and write the features over the tile, which a TMA store ships (rows past the end of the sequence
-// are clipped).  Bound by the memory system: X in and features out once each.  26 heads of 32K tokens, d = 128:
-// 156 us = 5.6 TB/s (L2 eviction hints on either side make it slower); one CTA per tile, which loaded W with every tile and did load, product,
-// exponentials and store one after the other, took 181.
+// A CTA (one per SM) takes a run of consecutive 128-token tiles of Q, then of K, in (head, tile) order, so that a head's
+// projection W (d x d, row a = w_a) is loaded once for many tiles.  Per tile X (128 x d, by TMA into a ring of 6 buffers, 12
+// at d = 64): one tcgen05.mma group computes Y = X W^T (M = 128, N = d, K = d, both operands K-major from shared memory) into
+// one of four TMEM buffers; 128 threads, one per token (a group of four warps for each of those), take the exponentials and
+// write the features over the tile, which a TMA store ships (rows past the end of the sequence are clipped).  Bound by the
+// memory system: X in and features out once each, 26 heads of 32K tokens, d = 128: 148 us = 5.9 TB/s.  A buffer is away for
+// about 7 us (load, product, exponentials, store), so what counts is how many there are: with two CTAs per SM of two
+// buffers and a copy of W each it took 156 us, and the layer of 16 heads x 4 x 2048 tokens 71 against 66; with one CTA per
+// tile, which did load, product, exponentials and store one after the other, 181.  L2 eviction hints make it slower.
 #include "common.cuh"
 #include "sm100.cuh"
 
@@ -25,7 +26,7 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kFavorThreads = 11 * 32;  // warps 0-7: two groups of one thread per token, 8: loads, 9: products, 10: stores
+constexpr int kFavorThreads = 19 * 32;  // warps 0-15: four groups of one thread per token, 16: loads, 17: products, 18: stores
 constexpr float kLog2eF = 1.4426950408889634f;
 
 struct FavorParams {
@@ -38,28 +39,32 @@ struct FavorParams {
 template <int D>
 struct FavorCfg {
   static constexpr int kTile = 128 * D * 2, kW = D * D * 2;
-  static constexpr int kBytes = 2 * kTile + kW + 1024;
+  static constexpr int kX = (D == 128) ? 6 : 12;  // tiles in shared memory
+  static constexpr int kBytes = kX * kTile + kW + 1024;
 };
 
 template <int D>
-__global__ void __launch_bounds__(kFavorThreads, 2)
+__global__ void __launch_bounds__(kFavorThreads, 1)
 favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__ CUtensorMap mxk,
                 const __grid_constant__ CUtensorMap mw, const __grid_constant__ CUtensorMap mfq,
                 const __grid_constant__ CUtensorMap mfk, const FavorParams p) {
   using C = FavorCfg<D>;
   extern __shared__ __align__(1024) uint8_t raw_smem[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw_smem) + 1023) & ~(uintptr_t)1023);
-  uint8_t* sW = sm + 2 * C::kTile;
-  __shared__ __align__(8) uint64_t x_full[2], x_free[2], w_full, w_free, y_full[2], y_free[2], staged[2];
+  constexpr int NX = C::kX;
+  uint8_t* sW = sm + NX * C::kTile;
+  __shared__ __align__(8) uint64_t x_full[NX], x_free[NX], staged[NX], w_full, w_free, y_full[4], y_free[4];
   __shared__ uint32_t tmem_base_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < NX; ++i) {
       mbar_init(&x_full[i], 1);
       mbar_init(&x_free[i], 1);
+      mbar_init(&staged[i], 128);
+    }
+    for (int i = 0; i < 4; ++i) {
       mbar_init(&y_full[i], 1);
       mbar_init(&y_free[i], 128);
-      mbar_init(&staged[i], 128);
     }
     mbar_init(&w_full, 1);
     mbar_init(&w_free, 1);
@@ -70,8 +75,8 @@ favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__
     tma_prefetch_desc(&mfq);
     tma_prefetch_desc(&mfk);
   }
-  if (warp == 9) {
-    tmem_alloc(&tmem_base_s, 2 * D);
+  if (warp == 17) {
+    tmem_alloc(&tmem_base_s, 4 * D);
     tmem_relinquish();
   }
   tc_fence_before_sync();
@@ -79,7 +84,7 @@ favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
 
-  // This CTA's tiles [t0, t1); tile number n of the CTA lives in buffers n & 1.
+  // This CTA's tiles [t0, t1); tile number n of the CTA lives in buffer n % NX of shared memory and n & 3 of TMEM.
   const long long total = 2 * p.rows * p.ntile;
   const long long t0 = total * blockIdx.x / gridDim.x, t1 = total * (blockIdx.x + 1) / gridDim.x;
   struct Tile {
@@ -96,15 +101,15 @@ favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__
     x.i0 = (int)(t - r * p.ntile) * 128;
     return x;
   };
-  if (warp == 8) {
+  if (warp == 16) {
     if (elect_one()) {
       int have = -1;       // head whose W is loaded
       uint32_t loads = 0;  // of W
       uint32_t n = 0;
       for (long long t = t0; t < t1; ++t, ++n) {
         const Tile x = tile_at(t);
-        const uint32_t s = n & 1;
-        if (n >= 2 && !mbar_wait(&x_free[s], ((n >> 1) + 1) & 1, p.status, 900)) break;
+        const uint32_t s = n % NX;
+        if (n >= NX && !mbar_wait(&x_free[s], (n / NX + 1) & 1, p.status, 900)) break;
         mbar_arrive_expect_tx(&x_full[s], C::kTile);
         for (int c = 0; c < D / 64; ++c)
           tma_load_4d(sm + s * C::kTile + c * 16384, x.is_k ? &mxk : &mxq, &x_full[s], c * 64, x.i0, p.h_begin + x.hl, x.b);
@@ -117,57 +122,57 @@ favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__
         }
       }
     }
-  } else if (warp == 9) {
+  } else if (warp == 17) {
     if (elect_one()) {
       constexpr uint32_t idesc = umma_idesc_bf16(128, D, false, false);
       int have = -1;
       uint32_t loads = 0, n = 0;
       for (long long t = t0; t < t1; ++t, ++n) {
         const int hl = tile_at(t).hl;
-        const uint32_t s = n & 1;
+        const uint32_t s = n % NX, sy = n & 3;
         if (hl != have) {
           if (!mbar_wait(&w_full, loads & 1, p.status, 902)) break;
           have = hl;
           ++loads;
         }
-        if (!mbar_wait(&x_full[s], (n >> 1) & 1, p.status, 903)) break;
-        if (n >= 2 && !mbar_wait(&y_free[s], ((n >> 1) + 1) & 1, p.status, 904)) break;
+        if (!mbar_wait(&x_full[s], (n / NX) & 1, p.status, 903)) break;
+        if (n >= 4 && !mbar_wait(&y_free[sy], ((n >> 2) + 1) & 1, p.status, 904)) break;
         tc_fence_after_sync();
-        const uint32_t xb = smem_u32(sm) + s * C::kTile, wb = smem_u32(sW);
+        const uint64_t dx = umma_smem_desc(smem_u32(sm) + s * C::kTile, 16, 1024), dw = umma_smem_desc(smem_u32(sW), 16, 1024);
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          umma_ss(tmem + s * D, umma_smem_desc(xb + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024),
-                  umma_smem_desc(wb + (ks >> 2) * (D * 128) + (ks & 3) * 32, 16, 1024), idesc, ks > 0);
-        umma_commit(&y_full[s]);
+          umma_ss(tmem + sy * D, umma_desc_add(dx, (ks >> 2) * 16384 + (ks & 3) * 32),
+                  umma_desc_add(dw, (ks >> 2) * (D * 128) + (ks & 3) * 32), idesc, ks > 0);
+        umma_commit(&y_full[sy]);
         if (t + 1 < t1 && tile_at(t + 1).hl != hl) umma_commit(&w_free);
       }
     }
-  } else if (warp == 10) {
+  } else if (warp == 18) {
     if (elect_one()) {
       uint32_t n = 0;
       for (long long t = t0; t < t1; ++t, ++n) {
         const Tile x = tile_at(t);
-        const uint32_t s = n & 1;
-        if (!mbar_wait(&staged[s], (n >> 1) & 1, p.status, 905)) break;
+        const uint32_t s = n % NX;
+        if (!mbar_wait(&staged[s], (n / NX) & 1, p.status, 905)) break;
         for (int c = 0; c < D / 64; ++c)
           tma_store_4d(x.is_k ? &mfk : &mfq, sm + s * C::kTile + c * 16384, c * 64, x.i0, p.h_begin + x.hl, x.b);
         tma_store_commit();
-        tma_store_wait_read<0>();
-        mbar_arrive(&x_free[s]);
+        tma_store_wait_read<1>();  // the one before has been read out
+        if (n >= 1) mbar_arrive(&x_free[(n - 1) % NX]);
       }
       tma_store_wait_all<0>();
     }
   } else {
-    const uint32_t s = warp >> 2;  // this group's buffer: every second tile of the CTA
+    const uint32_t sy = warp >> 2;  // this group's TMEM buffer: every fourth tile of the CTA
     const int quarter = warp & 3;  // TMEM lane quarter this warp may touch
     const int r = quarter * 32 + lane;
-    const uint32_t ty = tmem + s * D + ((uint32_t)(quarter * 32) << 16);
-    uint8_t* sX = sm + s * C::kTile;
-    uint32_t round = 0;
-    for (long long t = t0 + s; t < t1; t += 2, ++round) {
+    const uint32_t ty = tmem + sy * D + ((uint32_t)(quarter * 32) << 16);
+    uint32_t n = sy;
+    for (long long t = t0 + sy; t < t1; t += 4, n += 4) {
+      uint8_t* sX = sm + (n % NX) * C::kTile;
       const bool is_k = tile_at(t).is_k;
       // the products are done: X is no longer read by the tensor core
-      const bool ok = mbar_wait(&y_full[s], round & 1, p.status, 906);
+      const bool ok = mbar_wait(&y_full[sy], (n >> 2) & 1, p.status, 906);
       if (__any_sync(0xffffffffu, !ok)) break;
       tc_fence_after_sync();
       // keys: exp(y - |x|^2 / 2) / sqrt(d) = 2^((y - |x|^2 / 2) log2(e) - log2(d) / 2);
@@ -219,14 +224,14 @@ favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__
         }
       }
       tc_fence_before_sync();
-      mbar_arrive(&y_free[s]);
+      mbar_arrive(&y_free[sy]);
       fence_proxy_async_smem();
-      mbar_arrive(&staged[s]);
+      mbar_arrive(&staged[n % NX]);
     }
   }
   tc_fence_before_sync();
   __syncthreads();
-  if (warp == 9) tmem_dealloc(tmem, 2 * D);
+  if (warp == 17) tmem_dealloc(tmem, 4 * D);
 }
 
 }  // namespace
@@ -254,7 +259,7 @@ cudaError_t launch_favor_features_tc(const void* q, const void* k, const void* W
     cudaError_t err = device_info(&dev, &sms);
     if (err == cudaSuccess) err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem);
     if (err != cudaSuccess) return err;
-    const unsigned grid = (unsigned)(total < 2LL * sms ? total : 2LL * sms);
+    const unsigned grid = (unsigned)(total < sms ? total : sms);
     kern<<<grid, kFavorThreads, smem, stream>>>(mxq, mxk, mw, mfq, mfk, p);
     note_launch();
     return cudaGetLastError();

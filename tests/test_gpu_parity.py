@@ -1062,10 +1062,12 @@ def test_favor_causal_linear_both_forms_and_bnhd(split):
     assert_parity(f64(o.permute(0, 2, 1, 3)), ref, "bf16", f"favor linear bnhd split={split}")
 
 
-@pytest.mark.parametrize("H,N,d,split", [(100, 700, 64, 2), (100, 641, 128, 1), (60, 1153, 128, 3), (160, 383, 64, 3)])
+@pytest.mark.parametrize("H,N,d,split", [(100, 700, 64, 2), (100, 641, 128, 1), (60, 1153, 128, 3), (160, 383, 64, 3),
+                                          (150, 1000, 64, 2)])
 def test_favor_cut_chains_in_several_rounds(H, N, d, split):
     """Features need no first pass in a chain's last segment: several items per CTA, of one to three chunks, the last
-    chunk ragged, with the state carried in and out.  Gates of the other feature tests."""
+    chunk ragged, with the state carried in and out.  The pre-pass has 4 to 16 tiles per CTA, of one to three heads: fewer and
+    more than its 6 (d = 128) or 12 buffers.  Gates of the other feature tests."""
     q, k, v = synth.qkv(1, H, N, d, "bf16", seed=870 + N)
     W = _proj(H, d, "bf16", seed=871)
     S, z = torch.rand(1, H, d, d, device="cuda"), 1.0 + torch.rand(1, H, d, device="cuda")
