@@ -92,6 +92,8 @@ cudaError_t launch_window_tc(const void* q, const void* k, const void* v, void* 
 // Global (unmasked) linear attention of the bidirectional layer, heads [h_begin, h_begin + h_count):
 // three launches (segment sums, totals, readout); its scratch starts scratch_offset bytes into ws.
 size_t linear_self_workspace_bytes(int nchains, int N, int d);
+// work items of its first launch: one CTA each as far as there are SMs
+int linear_self_items(int nchains, int N, int d, int sms);
 cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                                   int layout, int h_begin, int h_count, WsHeader* ws, size_t scratch_offset,
                                   cudaStream_t stream, const void* fq = nullptr, const void* fk = nullptr,

@@ -878,6 +878,11 @@ size_t linear_self_workspace_bytes(int nchains, int N, int d) {
   return (size_t)nchains * (self_segments(nchains, nch) + 1) * state;
 }
 
+int linear_self_items(int nchains, int N, int d, int sms) {
+  const int nch = (N + 127) / 128;
+  return self_whole(nchains, nch, d, sms) ? nchains : nchains * self_segments(nchains, nch);
+}
+
 cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                                   int layout, int h_begin, int h_count, WsHeader* ws, size_t scratch_offset,
                                   cudaStream_t stream, const void* fq, const void* fk, int* first_grid) {

@@ -114,6 +114,19 @@ def test_self_layer_against_the_oracle(B, H, N, d, w, h0):
     assert_parity(f64(o[bs]), ref, "bf16", f"self layer B={B} H={H} N={N} d={d} w={w} h0={h0}")
 
 
+@pytest.mark.parametrize("B,H,N,d,h0", [(37, 4, 200, 64, 1), (38, 4, 200, 64, 1), (1, 4, 64, 128, 1), (1, 150, 64, 64, 2)])
+def test_self_layer_with_and_without_ordered_head_groups(B, H, N, d, h0):
+    # 148 and 152 CTAs of the two head groups together, and either side far from that; gates of the layer test above
+    q, k, v = synth.qkv(B, H, N, d, "bf16", seed=760 + B, gain=1.0)
+    ws = gf.Workspace.for_problem(B, H, N, d, 20, h0)
+    for _ in range(2):
+        o = gf.hybrid_attn_self(*dev(q, k, v), 20, h_sparse=h0, ws=ws).cpu()
+        assert ws.last_device_status() == gf.GF_OK
+    bs = sorted({0, B - 1})
+    ref = oracle.hybrid_attn_self(f64(q[bs]), f64(k[bs]), f64(v[bs]), 20, h_sparse=h0)
+    assert_parity(f64(o[bs]), ref, "bf16", f"self layer B={B} H={H} N={N} d={d} h0={h0}")
+
+
 @pytest.mark.parametrize("dtype,force_simt", [("f32", 0), ("bf16", 1)])
 @pytest.mark.parametrize("N,d,w,h0", [(1, 64, 1, 0), (100, 64, 7, 1), (300, 128, 40, 1), (1000, 64, 128, 2)])
 def test_self_layer_cuda_core_path(dtype, force_simt, N, d, w, h0):
