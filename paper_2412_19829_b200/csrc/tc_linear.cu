@@ -126,17 +126,22 @@ struct LinItem {
 };
 
 
+// kDirect: an item is a whole chain, said at compile time, so that less of the hand-over is left in that form's code, which
+// the instruction caches do not hold: 500 chains of 2000 tokens (d = 64) 118 -> 115 us, 444 of 700 (d = 128) 75 -> 70.  That
+// there is no later segment is left to run time at d = 64: without that dead code the compiler lays out the chunk loop in
+// a way that takes 3 % longer on long chains (148 of 8192 tokens 117.5 and 121.6).
+template <int D, bool kDirect>
 __device__ __forceinline__ LinItem decode_item(const LinParams& p, int item) {
   LinItem it;
-  it.g = item / p.nchains;
+  it.g = kDirect ? 0 : item / p.nchains;
   it.chain = item - it.g * p.nchains;
   const int call_chain = p.chain0 + it.chain;
   it.b = call_chain / p.h_count;
   it.hl = call_chain - it.b * p.h_count;
   it.h = p.h_begin + it.hl;
-  it.c_begin = it.g * p.seg_base + (it.g < p.seg_rem ? it.g : p.seg_rem);
-  it.nC = p.seg_base + (it.g < p.seg_rem ? 1 : 0);
-  it.last_seg = (it.g == p.G - 1);
+  it.c_begin = kDirect ? 0 : it.g * p.seg_base + (it.g < p.seg_rem ? it.g : p.seg_rem);
+  it.nC = kDirect ? p.nch : p.seg_base + (it.g < p.seg_rem ? 1 : 0);
+  it.last_seg = (kDirect && D == 128) || it.g == p.G - 1;
   it.need_dS = !it.last_seg;  // the last segment's contribution is needed by nobody
   return it;
 }
@@ -490,8 +495,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       // tiles) come back within the same item and should stay in L2 until then
       const uint64_t pol_stream = l2_policy_evict_first(), pol_keep = l2_policy_evict_last();
       for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
-        const LinItem it = decode_item(p, item);
-        for (int pass = (kPark || it.need_dS) ? 0 : 1; pass < 2 && ok; ++pass) {
+        const LinItem it = decode_item<D, kDirect>(p, item);
+        for (int pass = !kDirect && (kPark || it.need_dS) ? 0 : 1; pass < 2 && ok; ++pass) {
           if (kPark && pass == 1 && !mbar_wait(&bar.park_done, n_items & 1, p.status, 103)) { ok = false; break; }
           for (int j = 0; j < it.nC; ++j) {
             const int n0 = (it.c_begin + (pass == 0 ? it.nC - 1 - j : j)) * 128;
@@ -551,20 +556,14 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       constexpr int QS = C::kQSlots;
       const uint64_t dsb = umma_smem_desc(smem_u32(sSb), C::kSbBox, 1024);
       uint32_t ta = 0, nv = 0, nq = 0, n_sl = 0, n_sb = 0, n_of = 0, n_pm = 0;
-      bool ok = true, first_item = true;
+      bool ok = true;
       [[maybe_unused]] uint32_t n_items = 0;
       for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x, ++n_items) {
-        const LinItem it = decode_item(p, item);
-        if (!first_item) {
-          // the previous item's last S conversion has read TMEM and written Sb: consume its phases
-          ok = mbar_wait(&bar.s_loaded, n_sl & 1, p.status, 210) && mbar_wait(&bar.sb_full, n_sb & 1, p.status, 211);
-          ++n_sl;
-          ++n_sb;
-          if (!ok) break;
-        }
-        first_item = false;
+        const LinItem it = decode_item<D, kDirect>(p, item);
+        // the previous item's state has been read out of TMEM before pass A writes there (kDirect: the row group waits)
+        if (!kDirect && n_items > 0 && !mbar_wait(&bar.s_final, (n_items - 1) & 1, p.status, 210)) break;
         // ---- pass A: dS = sum Kc^T V over the segment, from zero (only if somebody needs it)
-        const int nA = (kPark || it.need_dS) ? it.nC : 0;  // K tiles of pass A
+        const int nA = !kDirect && (kPark || it.need_dS) ? it.nC : 0;  // K tiles of pass A
         for (int j = 0; j < nA; ++j) {
           const uint32_t sa = ta % KA;
           if (!mbar_wait(kId ? &bar.ka_full[sa] : &bar.kphi_full[sa], (ta / KA) & 1, p.status, 220)) { ok = false; break; }
@@ -659,7 +658,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     uint32_t nv = 0, nq = 0, n_a = 0, n_items = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < p.nitems; item += gridDim.x) {
-      const LinItem it = decode_item(p, item);
+      const LinItem it = decode_item<D, kDirect>(p, item);
       const long long sidx = (long long)it.b * p.h_count + it.hl;
       const long long slot = (long long)it.chain * p.G + it.g;
       if constexpr (kSum) {
@@ -839,7 +838,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       if (++w_j < w_it.nC) return true;
       w_item += gridDim.x;
       if (w_item >= p.nitems) return false;
-      w_it = decode_item(p, w_item);
+      w_it = decode_item<D, kDirect>(p, w_item);
       w_j = 0;
       return true;
     };
@@ -851,14 +850,14 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     };
     if (tid == 6 * 32 && (int)blockIdx.x < p.nitems) {
       if constexpr (QL == 1) {
-        const LinItem first = decode_item(p, blockIdx.x);
+        const LinItem first = decode_item<D, kDirect>(p, blockIdx.x);
         mbar_arrive_expect_tx(&bar.q_full[0], C::kTile);
         for (int x = 0; x < D / 64; ++x)
           tma_load_4d_hint(q_box(0, x), &mq, &bar.q_full[0], x * 64, first.c_begin * 128, first.h, first.b,
                            l2_policy_evict_first());
       } else {
         int w_item = blockIdx.x, w_j = 0;
-        LinItem w_it = decode_item(p, w_item);
+        LinItem w_it = decode_item<D, kDirect>(p, w_item);
         for (int slot = 0; slot < QL; ++slot) {
           request_q(slot, w_it, w_j);
           if (!step(w_item, w_j, w_it)) break;
@@ -866,7 +865,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       }
     }
     for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
-      const LinItem it = decode_item(p, item);
+      const LinItem it = decode_item<D, kDirect>(p, item);
       // kDirect: phi on this group's half of the K tile with running index idx (chunk jrow of the
       // item) of the chunk pipeline, in place
       auto transform_direct = [&](uint32_t idx, int jrow) {
@@ -989,11 +988,17 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
                                   __uint_as_float(v[jj + 3]));
               }
             }
+            // (an item's last chunk arrives on s_final alone: the phases of s_loaded and sb_full are those that the MMA issuer
+            // waits for, the row group's first.  With one more per item, which the issuer had to observe before the row
+            // group completed the next, it could miss it: the two were only some hundred cycles apart)
             tc_fence_before_sync();
-            mbar_arrive(&bar.s_loaded);
-            fence_proxy_async_smem();
-            mbar_arrive(&bar.sb_full);
-            if (last_chunk) mbar_arrive(&bar.s_final);
+            if (last_chunk) {
+              mbar_arrive(&bar.s_final);
+            } else {
+              mbar_arrive(&bar.s_loaded);
+              fence_proxy_async_smem();
+              mbar_arrive(&bar.sb_full);
+            }
           }
           ++nq;
         }
@@ -1033,7 +1038,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
                   if (j + 1 == it.nC) {
                     n_item = item + gridDim.x;
                     if (n_item < p.nitems) {
-                      nx = decode_item(p, n_item);
+                      nx = decode_item<D, kDirect>(p, n_item);
                       n_chunk = nx.c_begin;
                     }
                   }
@@ -1094,7 +1099,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       const uint64_t pol_keep = l2_policy_evict_last();  // parked phi(K) tiles are read back by pass C
       const uint64_t pol_out = l2_policy_evict_first();  // nobody reads O again: leave L2 to the tiles that come back
       for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
-        const LinItem it = decode_item(p, item);
+        const LinItem it = decode_item<D, kDirect>(p, item);
         // ---- pass A: park phi(K) tiles in the output rows of their chunk
         for (int j = 0; j < (kPark ? it.nC : 0); ++j) {
           const uint32_t sk = ta % KA;
@@ -1135,7 +1140,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     if constexpr (kSum) {  // own contribution out, then everybody's before it in: a flag per lane
       const int item = blockIdx.x;
       if (item < p.nitems) {
-        const LinItem it = decode_item(p, item);
+        const LinItem it = decode_item<D, kDirect>(p, item);
         const long long slot = (long long)it.chain * p.G + it.g;
         bool ok = true;
         if (it.need_dS && lane == 0) {
@@ -1154,7 +1159,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       uint32_t n_a = 0;
       int n_items = 0;
       for (int item = blockIdx.x; item < p.nitems; item += gridDim.x, ++n_items) {
-        const LinItem it = decode_item(p, item);
+        const LinItem it = decode_item<D, kDirect>(p, item);
         const long long slot = (long long)it.chain * p.G + it.g;
         // one poller per CTA: hundreds of threads spinning on a handful of L2 lines slow the whole chain
         if (it.g > 0 && !wait_flag(p.flags + (slot - 1) * kFlagStride, p.status, 511)) break;

@@ -296,6 +296,31 @@ def test_hybrid_with_whole_and_cut_linear_chains_and_state_export():
     assert errors(f64(st.z[:, idx].cpu()), zr)["rel_l2"] <= 1e-2
 
 
+@pytest.mark.parametrize("N,d", [(127, 64), (300, 64), (300, 128)])
+def test_whole_chains_in_several_rounds_exporting_their_state(N, d):
+    # 832 chains on 148 CTAs: the state of one chain leaves tensor memory while the next chain starts; every repetition
+    # must end with its status word clear and give the same bits
+    B, H, w, h0 = 64, 16, 33, 3
+    assert gf.linear_plan_parts(B * (H - h0), N, d)[:2] == (B * (H - h0), 1)
+    q, k, v = synth.qkv(B, H, N, d, "bf16", seed=940 + N, gain=1.0)
+    ins, st, first = dev(q, k, v), gf.DecodeState(B, H, d, w, h0), None
+    ws = gf.Workspace.for_problem(B, H, N, d, w, h0)
+    for _ in range(25):
+        o = gf.hybrid_attn(*ins, w, h_sparse=h0, state_out=st, ws=ws)
+        assert ws.last_device_status() == gf.GF_OK
+        got = [o.clone(), st.S.clone(), st.z.clone()]
+        first = first or got
+        assert all(torch.equal(a, b) for a, b in zip(first, got))
+    bs, hs = [0, 11, B - 1], [h0, H - 1]
+    sub = [f64(t[bs][:, hs]) for t in (q, k, v)]
+    Sr, zr = np.zeros((3, 2, d, d)), np.zeros((3, 2, d))
+    ref = oracle.causal_linear_attn(*sub, Sr, zr)
+    assert_parity(f64(o[bs][:, hs]), ref, "bf16", f"whole chains in rounds N={N} d={d}")
+    idx = [h - h0 for h in hs]
+    assert errors(f64(st.S[bs][:, idx].cpu()), Sr)["rel_l2"] <= 1e-2  # the gates of the state tests above
+    assert errors(f64(st.z[bs][:, idx].cpu()), zr)["rel_l2"] <= 1e-2
+
+
 def test_cut_chain_calls_from_two_streams_and_two_threads():
     """Calls whose chains are cut into segments (CTAs that wait for one another) issued at the same time from
     two host threads on two streams: the library runs such kernels one after the other on a device, so every
