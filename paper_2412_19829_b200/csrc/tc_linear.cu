@@ -50,6 +50,7 @@
 // the chunk pipeline (four K slots at D = 64).
 // Every wait is bounded; on expiry the kernel records a status word and drains.
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "linear_phi.cuh"
@@ -371,7 +372,9 @@ __device__ __forceinline__ bool sum_states(const LinParams& p, const LinItem& it
   return true;
 }
 
-template <int D, bool kDirect, bool kId, bool kSum = false>
+// kOne: no CTA has more than one item.  Said at compile time it leaves the loops over items and all that joins one to the next
+// out of the code: 26 chains of 3001 tokens (d = 128) 35.9 -> 34.1 us, one of 32 768 60 -> 57, 18 of 8192 (d = 64) 33.0 -> 31.8.
+template <int D, bool kDirect, bool kId, bool kOne>
 __global__ void __launch_bounds__(kThreads, 1)
 linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
                  const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtensorMap mo,
@@ -382,6 +385,11 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   // chain's last segment has no pass A (26 chains of 32K
   // tokens, d = 128, in a layer of 32 heads: 454 -> 426 us).
   constexpr bool kPark = !kDirect && !kId;
+  constexpr bool kSum = kOne && !kDirect;  // the states are sums of the contributions before a segment
+  auto next_item = [&](int i) -> int {
+    if constexpr (kOne) return p.nitems;
+    else return i + gridDim.x;
+  };
   extern __shared__ uint8_t raw_smem[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw_smem) + 1023) & ~(uintptr_t)1023);
   uint8_t* sK = sm + C::kK;
@@ -494,7 +502,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       // K, Q and the second read of V are streamed once; the first read of V (and the parked phi(K)
       // tiles) come back within the same item and should stay in L2 until then
       const uint64_t pol_stream = l2_policy_evict_first(), pol_keep = l2_policy_evict_last();
-      for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+      for (int item = blockIdx.x; item < p.nitems && ok; item = next_item(item)) {
         const LinItem it = decode_item<D, kDirect>(p, item);
         for (int pass = !kDirect && (kPark || it.need_dS) ? 0 : 1; pass < 2 && ok; ++pass) {
           if (kPark && pass == 1 && !mbar_wait(&bar.park_done, n_items & 1, p.status, 103)) { ok = false; break; }
@@ -558,7 +566,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       uint32_t ta = 0, nv = 0, nq = 0, n_sl = 0, n_sb = 0, n_of = 0, n_pm = 0;
       bool ok = true;
       [[maybe_unused]] uint32_t n_items = 0;
-      for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x, ++n_items) {
+      for (int item = blockIdx.x; item < p.nitems && ok; item = next_item(item), ++n_items) {
         const LinItem it = decode_item<D, kDirect>(p, item);
         // the previous item's state has been read out of TMEM before pass A writes there (kDirect: the row group waits)
         if (!kDirect && n_items > 0 && !mbar_wait(&bar.s_final, (n_items - 1) & 1, p.status, 210)) break;
@@ -657,7 +665,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     };
     uint32_t nv = 0, nq = 0, n_a = 0, n_items = 0;
     bool ok = true;
-    for (int item = blockIdx.x; item < p.nitems; item += gridDim.x) {
+    for (int item = blockIdx.x; item < p.nitems; item = next_item(item)) {
       const LinItem it = decode_item<D, kDirect>(p, item);
       const long long sidx = (long long)it.b * p.h_count + it.hl;
       const long long slot = (long long)it.chain * p.G + it.g;
@@ -837,7 +845,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     auto step = [&](int& w_item, int& w_j, LinItem& w_it) -> bool {
       if (++w_j < w_it.nC) return true;
       w_item += gridDim.x;
-      if (w_item >= p.nitems) return false;
+      if (kOne || w_item >= p.nitems) return false;
       w_it = decode_item<D, kDirect>(p, w_item);
       w_j = 0;
       return true;
@@ -864,7 +872,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         }
       }
     }
-    for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+    for (int item = blockIdx.x; item < p.nitems && ok; item = next_item(item)) {
       const LinItem it = decode_item<D, kDirect>(p, item);
       // kDirect: phi on this group's half of the K tile with running index idx (chunk jrow of the
       // item) of the chunk pipeline, in place
@@ -1036,7 +1044,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
                   int n_item = item, n_chunk = it.c_begin + j + 1;
                   LinItem nx = it;
                   if (j + 1 == it.nC) {
-                    n_item = item + gridDim.x;
+                    n_item = next_item(item);
                     if (n_item < p.nitems) {
                       nx = decode_item<D, kDirect>(p, n_item);
                       n_chunk = nx.c_begin;
@@ -1098,7 +1106,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       bool ok = true;
       const uint64_t pol_keep = l2_policy_evict_last();  // parked phi(K) tiles are read back by pass C
       const uint64_t pol_out = l2_policy_evict_first();  // nobody reads O again: leave L2 to the tiles that come back
-      for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x) {
+      for (int item = blockIdx.x; item < p.nitems && ok; item = next_item(item)) {
         const LinItem it = decode_item<D, kDirect>(p, item);
         // ---- pass A: park phi(K) tiles in the output rows of their chunk
         for (int j = 0; j < (kPark ? it.nC : 0); ++j) {
@@ -1158,7 +1166,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     } else if (elect_one()) {
       uint32_t n_a = 0;
       int n_items = 0;
-      for (int item = blockIdx.x; item < p.nitems; item += gridDim.x, ++n_items) {
+      for (int item = blockIdx.x; item < p.nitems; item = next_item(item), ++n_items) {
         const LinItem it = decode_item<D, kDirect>(p, item);
         const long long slot = (long long)it.chain * p.G + it.g;
         // one poller per CTA: hundreds of threads spinning on a handful of L2 lines slow the whole chain
@@ -1471,26 +1479,17 @@ cudaError_t launch_linear_tc(const void* q, const void* k, const void* v, void* 
     p.seg_base = p.nch / g;
     p.seg_rem = p.nch % g;
     p.nitems = count * g;
-    // every CTA one segment: the states are sums of the contributions before a segment
-    if (!direct && p.nitems <= sms) {
+    const bool one = p.nitems <= sms;
+    auto pick = [&](auto dd) -> cudaError_t {
+      constexpr int DD = decltype(dd)::value;
+      constexpr size_t smem = LinCfg<DD>::kBytes;
       if (features)
-        return d == 64 ? launch(linear_tc_kernel<64, false, true, true>, LinCfg<64>::kBytes)
-                       : launch(linear_tc_kernel<128, false, true, true>, LinCfg<128>::kBytes);
-      return d == 64 ? launch(linear_tc_kernel<64, false, false, true>, LinCfg<64>::kBytes)
-                     : launch(linear_tc_kernel<128, false, false, true>, LinCfg<128>::kBytes);
-    }
-    if (features) {
-      if (d == 64)
-        return direct ? launch(linear_tc_kernel<64, true, true>, LinCfg<64>::kBytes)
-                      : launch(linear_tc_kernel<64, false, true>, LinCfg<64>::kBytes);
-      return direct ? launch(linear_tc_kernel<128, true, true>, LinCfg<128>::kBytes)
-                    : launch(linear_tc_kernel<128, false, true>, LinCfg<128>::kBytes);
-    }
-    if (d == 64)
-      return direct ? launch(linear_tc_kernel<64, true, false>, LinCfg<64>::kBytes)
-                    : launch(linear_tc_kernel<64, false, false>, LinCfg<64>::kBytes);
-    return direct ? launch(linear_tc_kernel<128, true, false>, LinCfg<128>::kBytes)
-                  : launch(linear_tc_kernel<128, false, false>, LinCfg<128>::kBytes);
+        return direct ? (one ? launch(linear_tc_kernel<DD, true, true, true>, smem) : launch(linear_tc_kernel<DD, true, true, false>, smem))
+                      : (one ? launch(linear_tc_kernel<DD, false, true, true>, smem) : launch(linear_tc_kernel<DD, false, true, false>, smem));
+      return direct ? (one ? launch(linear_tc_kernel<DD, true, false, true>, smem) : launch(linear_tc_kernel<DD, true, false, false>, smem))
+                    : (one ? launch(linear_tc_kernel<DD, false, false, true>, smem) : launch(linear_tc_kernel<DD, false, false, false>, smem));
+    };
+    return d == 64 ? pick(std::integral_constant<int, 64>()) : pick(std::integral_constant<int, 128>());
   };
   // `whole` leading chains uncut (automatic plan only: a segment length asked for by the caller always takes
   // the two-pass form, also when it covers the whole chain), the others cut into G segments behind them
