@@ -179,7 +179,9 @@ favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__
       // queries: exp(y - max_a y) (the row's factor cancels in the output)
       float shift;
       if (is_k) {  // |x|^2 of this thread's token from the tile (128-byte swizzle: 16-byte chunks)
-        float n2[2] = {0.f, 0.f};
+        // One running sum in column order: the last bit of a bf16 feature depends on the order.  In two halves (even and
+        // odd columns) 3 of 1000 features were the neighbouring bf16 value, which moved the outputs by 1.4e-4.
+        float n2 = 0.f;
 #pragma unroll
         for (int c8 = 0; c8 < D / 8; ++c8) {
           const uint4 v4 = *reinterpret_cast<const uint4*>(sX + (c8 >> 3) * 16384 + swz128_offset(r, (c8 & 7) * 8));
@@ -187,11 +189,11 @@ favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w4[e]));
-            n2[0] = fmaf(f.x, f.x, n2[0]);
-            n2[1] = fmaf(f.y, f.y, n2[1]);
+            n2 = fmaf(f.x, f.x, n2);
+            n2 = fmaf(f.y, f.y, n2);
           }
         }
-        shift = -0.5f * (n2[0] + n2[1]) * kLog2eF - 0.5f * log2f((float)D);
+        shift = -0.5f * n2 * kLog2eF - 0.5f * log2f((float)D);
       } else {
         float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll 1

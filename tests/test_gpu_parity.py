@@ -1207,6 +1207,25 @@ def test_favor_is_not_elu_and_needs_its_projection():
     assert rc == gf.GF_ERR_INVALID_ARG
 
 
+def test_favor_key_features_sum_the_squares_in_column_order():
+    """With all projections zero a key's features are 2^(-|k|^2 / 2 log2(e) - log2(d) / 2), rounded to bf16, and one token
+    leaves them as they are in z.  The bits depend on the order of the sum |k|^2: one running fp32 sum over the columns.
+    exp2f is off by 2 of its 2^24 units at most, a bf16 value has 2^8: of 4096 keys 0.5 may round the other way."""
+    B, H, d = 4, 1024, 128
+    q, k, v = synth.qkv(B, H, 1, d, "bf16", seed=880, gain=1.0)
+    S, z = torch.zeros(B, H, d, d, device="cuda"), torch.zeros(B, H, d, device="cuda")
+    gf.causal_linear_attn(*dev(q, k, v), S, z, W=torch.zeros(H, d, d, dtype=torch.bfloat16, device="cuda"))
+    x = f64(k)[:, :, 0]
+    n2 = np.zeros((B, H))
+    for c in range(d):
+        n2 = (n2 + x[..., c] * x[..., c]).astype(np.float32).astype(np.float64)
+    shift = (-0.5 * n2 * np.float64(np.float32(np.log2(np.e))) - 0.5 * np.log2(d)).astype(np.float32)
+    want = torch.from_numpy(np.exp2(shift.astype(np.float64))).to(torch.bfloat16)
+    got = z.cpu()
+    assert torch.equal(got, got[..., :1].expand_as(got))
+    assert int((got[..., 0] != want.float()).sum()) <= 2
+
+
 # ------------------------------------------------------------------ fp32 linear heads, tiled and cut
 @pytest.mark.parametrize("bnhd", [False, True])
 @pytest.mark.parametrize("N,d", [(31, 64), (33, 128), (225, 64), (225, 128), (352, 64), (353, 64), (385, 128), (384, 64),
