@@ -1226,6 +1226,21 @@ def test_favor_key_features_sum_the_squares_in_column_order():
     assert int((got[..., 0] != want.float()).sum()) <= 2
 
 
+@pytest.mark.parametrize("d", [64, 128])
+def test_favor_segments_are_summed_in_token_order(d):
+    """The fp32 sum of a segment depends on its order: of +big, -big and small, chunk by chunk, small is left in token
+    order and lost from the back.  All features of a kind are the same 8-bit value, so the products and partial sums of big are exact."""
+    H, big, small = 2, 2.0**40, 2.0
+    q, k, v = (torch.zeros(1, H, 1024, d, dtype=torch.bfloat16, device="cuda") for _ in range(3))
+    v[:, :, 0:128], v[:, :, 128:256], v[:, :, 256:384] = big, -big, small
+    gf.set_tuning(gf.GF_TUNE_LINEAR_SPLIT, 4)
+    o = gf.causal_linear_attn(q, k, v, W=torch.zeros(H, d, d, dtype=torch.bfloat16, device="cuda"))
+    i = torch.arange(512, 1024, dtype=torch.float64)
+    want = (128 * small / (i + 1))[None, None, :, None].expand(1, H, 512, d)
+    # the readout's roundings to bf16: S, z (in two terms) and the output, 2^-9 each
+    assert errors(f64(o[:, :, 512:]), want.numpy())["rel_l2"] <= 3 * 2.0**-9
+
+
 # ------------------------------------------------------------------ fp32 linear heads, tiled and cut
 @pytest.mark.parametrize("bnhd", [False, True])
 @pytest.mark.parametrize("N,d", [(31, 64), (33, 128), (225, 64), (225, 128), (352, 64), (353, 64), (385, 128), (384, 64),
