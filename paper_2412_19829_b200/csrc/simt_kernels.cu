@@ -3,6 +3,8 @@
 // The linear heads of fp32 tensors where neither the tensor-core kernels nor the register-tiled ones apply (the
 // bidirectional layer's sums, positive random features), and the memory-bound decode step and ring export, which have
 // no dense contraction worth a tensor core.  Plain data-parallel kernels: no inter-CTA communication, no spin waits.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 
 namespace gf {
@@ -72,6 +74,8 @@ linear_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
       S[a] = S_io[(sidx * D + (g * AR + a)) * D + slice * 32 + c];
       zr[a] = z_io[sidx * D + g * AR + a];
     }
+    // the slices of a chain are one cluster: the one that overwrites z waits until all have read it
+    cooperative_groups::this_cluster().sync();
   }
 
   for (int sweep = global_sum ? 0 : 1; sweep < 2; ++sweep) {
@@ -524,15 +528,21 @@ template <typename T>
 cudaError_t linear_dispatch(const void* q, const void* k, const void* v, void* o, int B, int N, int d,
                             Strides st, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
                             bool global_sum, cudaStream_t stream, const void* W) {
-  dim3 grid(d / 32, h_count, B);
-  if (d == 64)
-    linear_simt_kernel<T, 64><<<grid, 256, 0, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, N, st, h_begin,
-                                                        h_count, S_io, z_io, zero_init ? 1 : 0, global_sum ? 1 : 0,
-                                                        (const T*)W);
-  else
-    linear_simt_kernel<T, 128><<<grid, 256, 0, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, N, st, h_begin,
-                                                         h_count, S_io, z_io, zero_init ? 1 : 0, global_sum ? 1 : 0,
-                                                         (const T*)W);
+  auto* kern = d == 64 ? linear_simt_kernel<T, 64> : linear_simt_kernel<T, 128>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(d / 32, h_count, B);
+  cfg.blockDim = dim3(256);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = d / 32;
+  attr.val.clusterDim.y = 1;
+  attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = (S_io != nullptr && !zero_init) ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, (const T*)q, (const T*)k, (const T*)v, (T*)o, N, st, h_begin, h_count,
+                                           S_io, z_io, zero_init ? 1 : 0, global_sum ? 1 : 0, (const T*)W);
+  if (e != cudaSuccess) return e;
   note_launch();
   return cudaGetLastError();
 }

@@ -236,7 +236,8 @@ window_tiled_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
 //
 // With few chains a chain is cut into G segments, so that every SM has work.  Up to kMaxCluster of them are a cluster of
 // CTAs in one launch (kCluster): each sums its own segment, then adds up the sums of those before it from their shared
-// memory, then walks.  Longer chains in smaller numbers take three launches, with segments of a little more than D tokens:
+// memory, then walks.  Where a chain has two CTAs per segment (D = 128) and brings a state, both are in the cluster: both read
+// the caller's z, and one of them overwrites it, which has to wait until the other has started.  Longer chains in smaller numbers take three launches, with segments of a little more than D tokens:
 //   contribution   the sums of every segment but the last, each alone
 //   prefix         running sums over the segments of a chain
 //   walk           the segments' outputs, each from its own starting state
@@ -366,7 +367,8 @@ __global__ void linear_prefix_kernel(float* __restrict__ o, Segs sg, Strides st,
 }
 
 // Without cuts (G == 1) the state before token 0 comes from S_io; with cuts from the segment's slot (segment 0 has
-// one only when there is an initial state), or, kCluster, from S_io and the cluster's CTAs before this one.
+// one only when there is an initial state), or, kCluster, from S_io and the cluster's CTAs before this one.  A chain that
+// brings a state and has several slices is one cluster (G x D / kW CTAs), also when it is not cut.
 template <typename T, int D, bool kCluster>
 __global__ void __launch_bounds__(kNT)
 linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* o, Segs sg, Strides st,
@@ -375,7 +377,7 @@ linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
   extern __shared__ __align__(16) float sm[];
   float *Qs = sm, *Ks = Qs + kC * LD, *Vs = Ks + kC * LD, *Ss = Vs + kC * kW, *Ps = Ss + D * kW, *zs = Ps + kC * kLdP,
         *inv_s = zs + D;
-  // (a cluster's CTAs are neighbours in x: segments of one slice)
+  // (a cluster's CTAs are neighbours in x: the segments of one slice, then those of the next)
   const int g = kCluster ? blockIdx.x % sg.G : blockIdx.x / (D / kW);
   const int col0 = (kCluster ? blockIdx.x / sg.G : blockIdx.x % (D / kW)) * kW;
   const long long base = (long long)blockIdx.z * st.b + (long long)(h_begin + blockIdx.y) * st.h;
@@ -400,8 +402,9 @@ linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
     });
     z = (from_caller && tid < D) ? z_io[sidx * D + tid] : 0.f;
     cluster.sync();
+    const int rank0 = (int)cluster.block_rank() - g;  // first segment of this slice
     for (int gg = 0; gg < g; ++gg) {
-      const float* Sr = cluster.map_shared_rank(Ss, gg);
+      const float* Sr = cluster.map_shared_rank(Ss, rank0 + gg);
       for_state<D>(i, S, [&](int a, float4& x) {
         const float4 y = lds4(Sr + s_off(a, 4 * cg));
         x.x += y.x;
@@ -409,9 +412,9 @@ linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
         x.z += y.z;
         x.w += y.w;
       });
-      if (tid < D) z += *cluster.map_shared_rank(zs + tid, gg);
+      if (tid < D) z += *cluster.map_shared_rank(zs + tid, rank0 + gg);
     }
-    cluster.sync();  // everybody has read what is overwritten now (and the caller's state, which the last CTA will)
+    cluster.sync();  // everybody has read what is overwritten now, and the caller's state, which the last CTAs will overwrite
     for_state<D>(i, S, [&](int a, float4& x) { *reinterpret_cast<float4*>(Ss + s_off(a, 4 * cg)) = x; });
     if (tid < D) zs[tid] = z;
   } else {
@@ -525,8 +528,12 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
   // memory per CTA slower (6 of 1000: 135).
   const int blocks = (N + kC - 1) / kC;
   const long long ctas = (long long)B * h_count * (D / kW), wave = (D == 64 ? 3LL : 2LL) * sms;
+  // (Of a chain that brings a state all slices are one cluster, which at d = 128 leaves room for four segments: 6 of 1000 then
+  // take the three launches, 76 -> 100 us, 17 of 1000 165 -> 134, 18 of 500 118 -> 91.  Clusters of 16 CTAs take 76 us for
+  // 6 of 1000 but 189 for 17.)
+  const int slices = (S_io != nullptr && !zero_init) ? D / kW : 1;
   int cluster = 1;
-  while (2 * cluster <= kMaxCluster && 2 * cluster <= blocks && 2 * cluster * ctas <= wave) cluster *= 2;
+  while (2 * cluster * slices <= kMaxCluster && 2 * cluster <= blocks && 2 * cluster * ctas <= wave) cluster *= 2;
   if constexpr (sizeof(T) == 4) {
     long long G3 = ctas < 4LL * sms ? (8LL * sms + ctas - 1) / ctas : 1;
     if (G3 > N / C::kMinSeg) G3 = N / C::kMinSeg;
@@ -550,7 +557,8 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
     }
   }
   const Segs sg = {N, cluster, blocks / cluster, blocks % cluster};
-  auto walk = cluster > 1 ? linear_walk_kernel<T, D, true> : linear_walk_kernel<T, D, false>;
+  const int cluster_ctas = cluster * slices;
+  auto walk = cluster_ctas > 1 ? linear_walk_kernel<T, D, true> : linear_walk_kernel<T, D, false>;
   if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, C::kSmem)) != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(cluster * (D / kW), h_count, B);
@@ -559,11 +567,11 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
   cfg.stream = stream;
   cudaLaunchAttribute attr = {};
   attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = cluster;
+  attr.val.clusterDim.x = cluster_ctas;
   attr.val.clusterDim.y = 1;
   attr.val.clusterDim.z = 1;
   cfg.attrs = &attr;
-  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  cfg.numAttrs = cluster_ctas > 1 ? 1 : 0;
   if ((e = cudaLaunchKernelEx(&cfg, walk, (const T*)q, (const T*)k, (const T*)v, (T*)o, sg, st, h_begin, h_count, S_io, z_io,
                               zero_init ? 1 : 0)) != cudaSuccess)
     return e;

@@ -1268,6 +1268,35 @@ def test_linear_f32_blocks_and_segments(N, d, bnhd):
     assert_parity(f64(o.permute(0, 2, 1, 3) if bnhd else o), fresh, "f32", f"f32 linear, no state, N={N} d={d}")
 
 
+@pytest.mark.parametrize("busy", [False, True])
+@pytest.mark.parametrize("H,N,d,favor", [(17, 300, 128, False), (18, 1900, 128, False), (1, 700, 128, False), (3, 65, 128, False),
+                                         (400, 1, 128, False), (400, 32, 128, False), (400, 225, 128, False), (400, 33, 64, False),
+                                         (200, 20, 64, True), (200, 20, 128, True)])
+def test_f32_carried_state_with_several_ctas_per_chain(H, N, d, favor, busy):
+    """All CTAs of a chain read the z carried in and one of them overwrites it: few chains in segments, more chains than
+    the device holds at a time, and with another stream's kernels on the SMs, so that the CTAs of a chain start apart.  Gates
+    of the fp32 layer."""
+    q, k, v = synth.qkv(1, H, N, d, "f32", seed=960 + N, gain=None if favor else 1.0)
+    W = _proj(H, d, "f32", 961) if favor else None
+    g = torch.Generator().manual_seed(H + N)
+    # (a z as large as the call's own sums: starting from the final z would be off by their size)
+    S0, z0 = torch.randn(1, H, d, d, generator=g), N * (0.5 + torch.rand(1, H, d, generator=g))
+    S_ref, z_ref = f64(S0).copy(), f64(z0).copy()
+    ref = oracle.causal_linear_attn(f64(q), f64(k), f64(v), S_ref, z_ref, **({"W": f64(W)} if favor else {}))
+    ins, Wd = dev(q, k, v), W.cuda() if favor else None
+    side, x = torch.cuda.Stream(), torch.ones(1 << 22, device="cuda")
+    for _ in range(3):
+        S, z = S0.cuda(), z0.cuda()
+        torch.cuda.synchronize()
+        if busy:
+            with torch.cuda.stream(side):
+                for _ in range(30):
+                    x.sin_()
+        o = gf.causal_linear_attn(*ins, S, z, W=Wd)
+        assert_parity(f64(o), ref, "f32", f"carried state H={H} N={N} d={d} busy={busy}")
+        assert errors(f64(S), S_ref)["rel_l2"] <= 1e-5 and errors(f64(z), z_ref)["rel_l2"] <= 1e-5
+
+
 # ------------------------------------------------------------------ bidirectional linear heads, whole chains in one launch
 @pytest.mark.parametrize("favor", [False, True])
 @pytest.mark.parametrize("B,H,N,d", [(1, 1, 1, 64), (1, 3, 127, 64), (2, 2, 128, 64), (3, 150, 129, 64), (5, 100, 197, 64),
