@@ -140,7 +140,8 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
   return __float2bfloat16_rn(x);
 }
 
-// phi(x) = elu(x) + 1 (Sec. II-B), without a branch: max(x, 0) + exp(min(x, 0)).
-__device__ __forceinline__ float phi_elu1(float x) { return fmaxf(x, 0.f) + expf(fminf(x, 0.f)); }
+// phi(x) = elu(x) + 1 (Sec. II-B), without a branch: max(x, 0) + exp(min(x, 0)), and NaN of a NaN (a selection, because
+// fminf drops it).
+__device__ __forceinline__ float phi_elu1(float x) { return fmaxf(x, 0.f) + expf(x > 0.f ? 0.f : x); }
 
 }  // namespace gf

@@ -1376,3 +1376,39 @@ def test_linear_segments_in_one_round(H, N, d, favor, bnhd):
     assert torch.isfinite(o.float()).all()
     assert_parity_by_scale(f64(o[:, hs]), ref, "bf16", f"one round H={H} N={N} d={d}")
     assert errors(f64(S[:, hs].cpu()), S_ref)["rel_l2"] <= 1e-2 and errors(f64(z[:, hs].cpu()), z_ref)["rel_l2"] <= 1e-2
+
+
+# ------------------------------------------------------------------ values that are not finite
+@pytest.mark.parametrize("N,j", [(40, 5), (40, 39), (700, 333)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_f32_layer_nan_in_q_or_k_reaches_the_rows_that_see_it(d, N, j):
+    """fp32 linear heads: a NaN feature of key j makes every later row NaN (causal) or every row (bidirectional), one of
+    query j that row; all other rows are those of the clean input, up to the order of the fp32 sums."""
+    B, H = 1, 2
+    q, k, v = dev(*synth.qkv(B, H, N, d, "f32", seed=990 + N, gain=1.0))
+    qn, kn = q.clone(), k.clone()
+    qn[0, 1, j, 3] = kn[0, 1, j, d - 2] = float("nan")
+    for layer, rows in ((lambda a, b: gf.causal_linear_attn(a, b, v), slice(j, N)),
+                        (lambda a, b: gf.hybrid_attn_self(a, b, v, 4, h_sparse=0), slice(0, N))):
+        clean = layer(q, k)
+        for a, b, bad in ((q, kn, rows), (qn, k, slice(j, j + 1))):
+            o = layer(a, b)
+            mask = torch.zeros(N, dtype=torch.bool, device="cuda")
+            mask[bad] = True
+            assert torch.isnan(o[0, 1, mask]).all()
+            assert torch.equal(o[0, 0], clean[0, 0]) and torch.equal(o[0, 1, ~mask], clean[0, 1, ~mask])
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_decode_nan_in_q_or_k_reaches_the_linear_heads(dtype):
+    B, H, d, w, h0 = 2, 3, 64, 8, 1
+    for which in (0, 1):
+        g = torch.Generator().manual_seed(5)
+        qkv = [torch.randn(B, H, d, generator=g).to(dtype).cuda() for _ in range(3)]
+        qkv[which][1, 2, 7] = float("nan")
+        st = gf.DecodeState(B, H, d, w, h0, dtype)
+        o = gf.decode_step(*qkv, st)
+        bad = torch.zeros(B, H, dtype=torch.bool, device="cuda")
+        bad[1, 2] = True
+        assert torch.isnan(o[bad]).all() and torch.isfinite(o[~bad]).all()
+        assert bool(torch.isnan(st.z[1, 1, 7])) == (which == 1)
