@@ -262,6 +262,13 @@ template <> struct Row16<__nv_bfloat16> {
   }
 };
 
+// fmaxf drops a NaN
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 __device__ __forceinline__ float block_reduce(float x, bool is_max, float* scratch /* 33 floats */) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
@@ -396,9 +403,9 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
 #pragma unroll
         for (int off = TPS / 2; off > 0; off >>= 1) s[i] += __shfl_xor_sync(0xffffffffu, s[i], off);
         s[i] = (s0 + i * GW + gw < nvalid) ? s[i] * scale : -INFINITY;
-        mx = fmaxf(mx, s[i]);
+        mx = max_nan(mx, s[i]);
       }
-      if (mx != -INFINITY) {  // (a group that has met no slot yet keeps l = 0)
+      if (mx != -INFINITY) {  // (a group that has met no slot yet keeps l = 0; a NaN goes on into l and the output)
         const float corr = expf(m - mx);
         m = mx;
         l *= corr;

@@ -1412,3 +1412,32 @@ def test_decode_nan_in_q_or_k_reaches_the_linear_heads(dtype):
         bad[1, 2] = True
         assert torch.isnan(o[bad]).all() and torch.isfinite(o[~bad]).all()
         assert bool(torch.isnan(st.z[1, 1, 7])) == (which == 1)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("B,d,w,t,slot", [(1, 64, 8, 4, 1), (1, 128, 300, 9, 3), (1, 64, 300, 250, 200), (1, 128, 8, 21, 5), (400, 64, 40, 33, 32)])
+def test_decode_nan_key_in_the_ring_reaches_the_windowed_heads(dtype, B, d, w, t, slot):
+    """Also where a group of threads meets no other key (short rings, the slot of this step's token); a score of -inf
+    (the key's largest finite value times the query's) is a key without weight."""
+    H = h0 = 2
+    g = torch.Generator().manual_seed(t)
+    q, k, v = [torch.randn(B, H, d, generator=g).to(dtype).cuda() for _ in range(3)]
+    st = gf.DecodeState(B, H, d, w, h0, dtype)
+    st.k_cache.copy_(torch.randn(st.k_cache.shape, generator=g))
+    st.v_cache.copy_(torch.randn(st.v_cache.shape, generator=g))
+    st.t = t
+    n = min(t + 1, w)
+    out = []
+    for value in (float("nan"), -torch.finfo(dtype).max):
+        q[0, 1, 0] = 8.0
+        st.k_cache[0, 1, slot, 0] = value
+        if t % w == slot:
+            k[0, 1, 0] = value
+        st.t = t
+        out.append(gf.decode_step(q, k, v, st).double())
+    bad = torch.zeros(B, H, dtype=torch.bool, device="cuda")
+    bad[0, 1] = True
+    assert torch.isnan(out[0][bad]).all() and torch.equal(out[0][~bad], out[1][~bad])
+    s = torch.einsum("bhd,bhnd->bhn", q.double(), st.k_cache[:, :, :n].double()) / d**0.5
+    ref = torch.einsum("bhn,bhnd->bhd", torch.softmax(s, -1), st.v_cache[:, :, :n].double())
+    assert_parity(out[1].cpu().numpy(), ref.cpu().numpy(), "f32" if dtype == torch.float32 else "bf16", "a key without weight")
