@@ -53,6 +53,12 @@ __device__ __forceinline__ float dot4(float4 a, float4 b, float acc) {
   return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
 }
 
+// (also of infinities of both signs)
+__device__ __forceinline__ bool has_nan(float4 x) {
+  const float s = (x.x + x.y) + (x.z + x.w);
+  return s != s;
+}
+
 // A block's rows on their way from global to shared memory: COLS columns of 32 tokens, all loads of a thread in
 // flight at once and issued a block ahead of their use.  Rows past the end are zero.
 template <typename T, int COLS>
@@ -123,8 +129,34 @@ __device__ __forceinline__ void product(float4 (&acc)[4][NG], const float* A, in
 template <int D>
 constexpr int window_smem() { return (2 * kC * (D + 4) + kC * D + kC * kLdP + kC) * 4; }
 
+// Masked keys have weight 0 in the products above, which is nothing unless their value is infinite or NaN (0 x inf = NaN):
+// the output row of query i once more, by the four threads that share it, over the keys it sees and no others.  m, l: its
+// final maximum and sum.
 template <typename T, int D>
-__global__ void __launch_bounds__(kNT)
+__device__ __forceinline__ void window_row(const T* q, const T* k, const T* v, T* o, int i, int j_begin, int j_end, float scale,
+                                        long long stride, int part, unsigned int quad, float m, float l) {
+  float4 acc[D / 16];
+#pragma unroll
+  for (int c = 0; c < D / 16; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+  for (int j = j_begin; j < j_end; ++j) {
+    float s = 0.f;
+#pragma unroll
+    for (int c = 0; c < D / 16; ++c)
+      s = dot4(load4<T>(q + i * stride + 4 * (part + 4 * c)), load4<T>(k + j * stride + 4 * (part + 4 * c)), s);
+    s += __shfl_xor_sync(quad, s, 1);
+    s += __shfl_xor_sync(quad, s, 2);
+    const float p = expf(s * scale - m);
+#pragma unroll
+    for (int c = 0; c < D / 16; ++c) axpy4(acc[c], p, load4<T>(v + j * stride + 4 * (part + 4 * c)));
+  }
+#pragma unroll
+  for (int c = 0; c < D / 16; ++c)
+    store4(o + i * stride + 4 * (part + 4 * c), make_float4(acc[c].x / l, acc[c].y / l, acc[c].z / l, acc[c].w / l));
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kNT, D == 64 ? 5 : 3)  // (else the rare path at the end takes registers from the rest)
 window_tiled_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ o,
                     int N, int w, int fwd, float scale, Strides st, int h_begin) {
   // fwd: keys after the query that it may see (0: the causal window; w - 1: the two-sided one)
@@ -213,18 +245,30 @@ window_tiled_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
     product<kC, NC>(acc, Ps, kLdP, i, [&](int j, int c) { return Vs + j * D + c * 64 + 4 * cg; });
     __syncthreads();
   }
-  if (part == 0) As[t] = 1.f / l;
+  if (part == 0) {
+    As[t] = 1.f / l;
+    Ps[t] = 0.f;  // 1: the row has a NaN
+  }
   __syncthreads();
+  bool any = false;
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int row = i + 8 * r;
     if (i0 + row >= N) continue;
     const float inv = As[row];
 #pragma unroll
-    for (int c = 0; c < NC; ++c)
+    for (int c = 0; c < NC; ++c) {
+      if (has_nan(acc[r][c])) {
+        Ps[row] = 1.f;
+        any = true;
+      }
       store4(o + base + (long long)(i0 + row) * st.n + c * 64 + 4 * cg,
              make_float4(acc[r][c].x * inv, acc[r][c].y * inv, acc[r][c].z * inv, acc[r][c].w * inv));
+    }
   }
+  if (__syncthreads_or(any) && Ps[t] != 0.f)
+    window_row<T, D>(q + base, k + base, v + base, o + base, i0 + t, max(i0 + t - w + 1, 0), min(i0 + t + fwd, N - 1) + 1, scale,
+                     st.n, part, 0xfu << (lane & 28), m, l);
 }
 
 // ------------------------------------------------------------------------------------ causal linear heads
@@ -479,7 +523,21 @@ linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
     product<kC, 1>(acc, Ps, kLdP, i, [&](int j, int) { return Vs + j * kW + 4 * cg; });
     const bool more = n0 + kC < n_end || (g == sg.G - 1 && S_io != nullptr);  // somebody wants the state after this block
     if (more) add_outer<D>(Ks, Vs, i, cg, S);
-    __syncthreads();
+    if (__syncthreads_or(has_nan(acc[0][0]) || has_nan(acc[1][0]) || has_nan(acc[2][0]) || has_nan(acc[3][0]))) {
+      // a masked weight is 0, which is nothing unless the value is infinite or NaN (0 x inf = NaN): the same sums without
+      // the masked ones, so that a row sees no later value
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int row = i + 8 * r;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        for (int a = 0; a < D; ++a) axpy4(x, Qs[row * LD + a], lds4(Ss + s_off(a, 4 * cg)));
+#pragma unroll 1
+        for (int j = 0; j <= row; ++j) axpy4(x, Ps[row * kLdP + j], lds4(Vs + j * kW + 4 * cg));
+        acc[r][0] = x;
+      }
+      __syncthreads();
+    }
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int row = i + 8 * r;

@@ -1441,3 +1441,27 @@ def test_decode_nan_key_in_the_ring_reaches_the_windowed_heads(dtype, B, d, w, t
     s = torch.einsum("bhd,bhnd->bhn", q.double(), st.k_cache[:, :, :n].double()) / d**0.5
     ref = torch.einsum("bhn,bhnd->bhd", torch.softmax(s, -1), st.v_cache[:, :, :n].double())
     assert_parity(out[1].cpu().numpy(), ref.cpu().numpy(), "f32" if dtype == torch.float32 else "bf16", "a key without weight")
+
+
+@pytest.mark.parametrize("dtype,force_simt", [("f32", 0), ("bf16", 1)])
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("N,j,value", [(40, 5, float("inf")), (70, 64, float("nan")), (700, 333, float("-inf")), (97, 96, float("inf"))])
+def test_cuda_core_values_that_are_not_finite_stay_with_the_rows_that_see_them(N, j, value, d, dtype, force_simt):
+    """v of token j infinite or NaN in one column: that column of the rows that see the token, and nothing else.  The
+    other rows are those of the clean input: the same sums in the linear heads, a sum of their own in the windowed ones,
+    where a row's keys are added one by one (2^-24 sqrt(2 w) of their size for fp32, one bf16 rounding for bf16)."""
+    gf.set_tuning(gf.GF_TUNE_FORCE_SIMT, force_simt)
+    B, H, w, c = 1, 2, 24, d - 3
+    q, k, v = dev(*synth.qkv(B, H, N, d, dtype, seed=1100 + N, gain=1.0))
+    vb = v.clone()
+    vb[0, 1, j, c] = value
+    tol = 1e-5 if dtype == "f32" else 2.0**-8
+    rows = torch.arange(N, device="cuda")
+    for layer, sees, same in ((lambda x: gf.causal_linear_attn(q, k, x), rows >= j, True),
+                              (lambda x: gf.window_attn(q, k, x, w), (rows >= j) & (rows < j + w), False),
+                              (lambda x: gf.window_attn_self(q, k, x, w), (rows - j).abs() < w, False)):
+        clean, o = layer(v), layer(vb)
+        assert not torch.isfinite(o[0, 1, sees, c]).any()
+        o[0, 1, sees, c] = clean[0, 1, sees, c]
+        assert torch.isfinite(o).all()
+        assert torch.equal(o, clean) if same else ((o - clean).abs() <= tol * clean.abs().clamp(min=0.1)).all()
