@@ -201,6 +201,18 @@ __device__ __forceinline__ bool wait_flag(const unsigned int* flag, unsigned int
 }
 
 
+// Loads that stay before the arrivals and flags behind them in the source (__ldcg promises no such thing).
+__device__ __forceinline__ float ld_cg_in_order(const float* p) {
+  float x;
+  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(x) : "l"(p) : "memory");
+  return x;
+}
+__device__ __forceinline__ float4 ld_cg4_in_order(const float* p) {
+  float4 x;
+  asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "l"(p) : "memory");
+  return x;
+}
+
 // The segment's published state is complete: releases it to whoever waits for the flag (one thread, on behalf of the warps
 // that have arrived at pub_done).
 __device__ __forceinline__ void raise_flag(const LinParams& p, long long slot) {
@@ -305,7 +317,7 @@ __device__ __forceinline__ bool sum_states(const LinParams& p, const LinItem& it
   float4 acc[W / 4];
 #pragma unroll
   for (int j = 0; j < W / 4; ++j)
-    acc[j] = from_caller ? __ldcg(reinterpret_cast<const float4*>(Sc) + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+    acc[j] = from_caller ? ld_cg4_in_order(Sc + 4 * j) : make_float4(0.f, 0.f, 0.f, 0.f);
   bool ok = true;
   if (it.need_dS) {
     ok = mbar_wait(&bar.a_done, 0, p.status, 600);
@@ -328,6 +340,7 @@ __device__ __forceinline__ bool sum_states(const LinParams& p, const LinItem& it
   }
   if (lane == 0) ok = wait_epoch(prev_epoch, 1, p.status, 601);
   if (__any_sync(0xffffffffu, !ok)) return false;
+  __syncwarp();  // (a vote orders no memory: what lane 0 has seen holds for the other lanes' reads from here on)
   if (r < D) {
 #pragma unroll 1
     for (int g = 0; g < it.g; ++g) {
@@ -672,7 +685,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       const long long slot = (long long)it.chain * p.G + it.g;
       if constexpr (kSum) {
         // ---- z as the phi warps do S (sum_states); the segment may start once both are in place
-        float z0 = (p.z_io != nullptr && !p.zero_init && s_row) ? __ldcg(p.z_io + sidx * D + r) : 0.f;
+        // (z read before this segment's flag is raised, as the caller's S is)
+        float z0 = (p.z_io != nullptr && !p.zero_init && s_row) ? ld_cg_in_order(p.z_io + sidx * D + r) : 0.f;
         float* zslot = p.prefix + (slot - it.g) * C::kStateFloats + C::kStateZ + r;
         if (it.need_dS) {
           ok = mbar_wait(&bar.a_done, 0, p.status, 311);
