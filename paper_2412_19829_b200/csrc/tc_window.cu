@@ -42,7 +42,8 @@ constexpr int kWarpLoad = 16, kWarpMma = 17, kWarpIo = 19;  // warps 0..15: soft
 constexpr int kThreads = 20 * 32;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kRescaleThreshold = 8.0f;  // log2 units
-constexpr int kUnitRing = 8;               // no role is ever this many units behind the producer
+constexpr int kUnitRing = 8;               // units posted ahead; an entry is rewritten when every reader has read it
+constexpr int kUnitReaders = 16 + 2 + 1;   // the softmax warps, the issuers of the products, the store warp
 
 __device__ __forceinline__ float ex2_approx(float x) {  // 2^x, flushes denormals, 2^-inf = 0
   float y;
@@ -56,6 +57,7 @@ struct WinCtl {
   uint64_t k_full[8], k_empty[8], v_full[8], v_empty[8];   // per ring slot
   uint64_t s_full[2][2], p_full[2][2];             // per query tile of the pair and S buffer
   uint64_t pv_done[2], o_full[2], o_free[2];       // per query tile of the pair
+  uint64_t unit_read[kUnitRing];                   // per entry of unit_ring
   uint32_t front;  // ring number of the half tile stream 0's next S will read (stream 1 stays behind it)
   uint32_t k_issued, v_issued;  // half tiles whose load the producer has issued (monotonic)
   uint32_t tmem_base;
@@ -177,6 +179,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       mbar_init(&ctl->o_full[i], 1);
       mbar_init(&ctl->o_free[i], 256);
     }
+    for (int i = 0; i < kUnitRing; ++i) mbar_init(&ctl->unit_read[i], kUnitReaders);
     ctl->unit_ring[0] = split(blockIdx.x);  // the grid never exceeds the number of units
     ctl->front = ctl->k_issued = ctl->v_issued = 0;
     ctl->units_posted = 1;
@@ -214,6 +217,8 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     if (!win_wait_epoch(&ctl->units_posted, (int)n + 1, p.status, 90)) return make_int4(-1, 0, 0, 0);
     return ctl->unit_ring[n % kUnitRing];
   };
+  // (each reader once per unit; nothing else bounds how far the roles of stream 1 fall behind in a run of single tiles)
+  auto unit_read = [&](uint32_t n) { mbar_arrive(&ctl->unit_read[n % kUnitRing]); };
 
   // Every role walks the same list of units and keeps the same running counters (units, query
   // tiles, key tiles), from which the ring slots and barrier phases follow.
@@ -249,6 +254,11 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           publish(&ctl->v_issued, kt + 1);
           if (hg == 2 * g0) {  // the other roles learn of the next unit early (its Q is requested ahead)
             if (t_next < (unsigned int)(p.total - (int)gridDim.x)) u_next = split((int)(gridDim.x + t_next));
+            const uint32_t use_next = (nu + 1) / kUnitRing;
+            if (use_next >= 1 && !mbar_wait(&ctl->unit_read[(nu + 1) % kUnitRing], (use_next - 1) & 1, p.status, 12)) {
+              ok = false;
+              break;
+            }
             ctl->unit_ring[(nu + 1) % kUnitRing] = u_next;
             __threadfence_block();
             *reinterpret_cast<volatile int*>(&ctl->units_posted) = (int)nu + 2;
@@ -295,7 +305,11 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         tma_store_commit();
         tma_store_wait_read<0>();
         ++qs;
-        if (++st_which == x.nt) { st_which = 0; ++st_nu; }
+        if (++st_which == x.nt) {
+          st_which = 0;
+          unit_read(st_nu);
+          ++st_nu;
+        }
         load_next();
       }
       tma_store_wait_all<0>();
@@ -328,6 +342,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         for (uint32_t nu = 0;; ++nu) {
           const int4 u = unit_at(nu);
           if (u.x < 0) break;
+          unit_read(nu);
           const Unit x = decode(u);
           const uint32_t n_half = 2 * (uint32_t)((x.nt == 2 ? x.l[1] : x.l[0]) - x.f[0] + 1);
           const int n_sub = x.n_sub(t);
@@ -410,6 +425,8 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     for (; ok; ++nu) {
       const int4 u = unit_at(nu);
       if (u.x < 0) break;
+      __syncwarp();
+      if (lane == 0) unit_read(nu);
       const Unit x = decode(u);
       const uint32_t buf = (qn + t) % 3;
       qn += (uint32_t)x.nt;

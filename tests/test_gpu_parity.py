@@ -85,6 +85,22 @@ def test_window_tensor_core(N, w, d, gain):
     assert_parity(f64(o), ref, "bf16", f"window tc N={N} w={w} d={d}")
 
 
+@pytest.mark.parametrize("two_sided", [False, True])
+@pytest.mark.parametrize("N,w,d", [(100, 16, 64), (1, 1, 128), (300, 40, 64), (300, 1, 128), (640, 128, 128)])
+def test_window_more_units_per_cta_than_the_unit_list_holds(N, w, d, two_sided):
+    """2000 heads: 13 to 40 units of one or two query tiles per CTA, whose list has 8 entries; all units of one tile
+    (stream 1 has nothing to do), or every second or third.  Sampled heads against the oracle, the rest finite."""
+    H = 2000
+    q, k, v = synth.qkv(1, H, N, d, "bf16", seed=260 + N, gain=1.0)
+    ws = gf.Workspace.for_problem(1, H, N, d, w, H)
+    o = (gf.window_attn_self if two_sided else gf.window_attn)(*dev(q, k, v), w, ws=ws).cpu()
+    assert ws.last_device_status() == gf.GF_OK
+    assert torch.isfinite(o.float()).all()
+    hs = sorted({0, 147, 148, 1000, H - 1})
+    ref = (oracle.window_attn_self if two_sided else oracle.window_attn)(f64(q[:, hs]), f64(k[:, hs]), f64(v[:, hs]), w)
+    assert_parity(f64(o[:, hs]), ref, "bf16", f"many units N={N} w={w} d={d} two_sided={two_sided}")
+
+
 @pytest.mark.parametrize("dtype,force_simt", [("f32", 0), ("bf16", 1), ("bf16", 0)])
 @pytest.mark.parametrize("N,w,d", [(1, 1, 64), (100, 1, 64), (128, 128, 128), (129, 2, 64), (300, 64, 128), (777, 129, 64),
                                    (1000, 128, 128), (1030, 300, 128), (640, 5000, 64), (2100, 513, 128)])
