@@ -135,10 +135,7 @@ int check_phi(int phi, const void* W) {
   return GF_ERR_UNSUPPORTED;
 }
 
-// The pre-pass of the positive random features.  It goes to the caller's stream, ahead of the fork of the two head groups:
-// windowed-heads CTAs that were already waiting for SMs when it ends would take them before the linear kernel's CTAs,
-// which wait for one another (42 chains of 3217 tokens beside 14 windowed heads: 97 or 110 us, as it fell, and 101;
-// 2 x 8 heads of 19 271 tokens 187.6 -> 182.0; 4 x 16 bidirectional heads of 2000 tokens 59.4 -> 51.8).
+// The pre-pass of the positive random features.
 int run_features(const Tuning& tn, const void* q, const void* k, int B, int H, int N, int d, int dtype, int layout,
                  int h_begin, int h_count, WsHeader* ws, cudaStream_t stream, Phi* phi) {
   if (h_count <= 0 || phi->W == nullptr || tn.force_simt || !gf::tc_linear_supported(N, d, dtype)) return GF_OK;
@@ -352,6 +349,8 @@ int gformer_hybrid_attn_self_w(const void* q, const void* k, const void* v, void
   Phi fm;
   fm.W = W;
   fm.feat_offset = feat_offset;
+  // (the pre-pass ahead of the fork: windowed-heads CTAs beside it would still hold SMs when the linear heads want them all;
+  // 4 x 16 heads of 2000 tokens, d = 128, 68.8 us and, behind the fork, 82.7; 64 x 12 of 197, d = 64, 50.3 and 63.6)
   if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, h_sparse, H - h_sparse, (WsHeader*)ws, stream, &fm)) != GF_OK)
     return rc;
   if (h_sparse > 0 && h_sparse < H && tc_linear) {
@@ -464,7 +463,6 @@ int gformer_hybrid_attn_w(const void* q, const void* k, const void* v, void* o, 
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   rc = clear_ws(tn, ws, stream, B * h_lin, N, d, dtype);
   if (rc != GF_OK) return rc;
-  if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, h_sparse, h_lin, (WsHeader*)ws, stream, &fm)) != GF_OK) return rc;
 
   float* S_out = state_out ? state_out->S : nullptr;
   float* z_out = state_out ? state_out->z : nullptr;
@@ -474,6 +472,7 @@ int gformer_hybrid_attn_w(const void* q, const void* k, const void* v, void* o, 
   // stream of the highest priority; the windowed heads' short-lived CTAs then fill the SMs that
   // linear CTAs leave at different times towards the end.
   const bool both = h_sparse > 0 && h_lin > 0;
+  bool rounds = false;  // of whole chains, more than one
   int lin_ctas = 0;
   if (both && !tn.force_simt && gf::tc_linear_supported(N, d, dtype)) {
     int L = 0, G = 0, whole = 0, dev = 0, sms = 0;
@@ -482,8 +481,17 @@ int gformer_hybrid_attn_w(const void* q, const void* k, const void* v, void* o, 
     if (gf::device_info(&dev, &sms) != cudaSuccess) return GF_ERR_CUDA;
     if ((long long)B * h_lin * G >= sms) {
       lin_ctas = (tn.linear_ctas > 0 && tn.linear_ctas < sms) ? tn.linear_ctas : sms;
+      rounds = whole > 0;
     }
   }
+  // The pre-pass of random features goes to the stream of the linear heads behind the fork, so that windowed heads run beside
+  // it and in its tail (us, ahead of the fork and behind it: 4 x 32 heads of 544 tokens, d = 64, 41.3 and 32.0; 8 x 8 of 3217
+  // 71.5 and 62.5; 32 of 32 768, d = 128, 454 and 444), but ahead of it where the linear heads fill the device for more than
+  // a round of whole chains (32 x 12 of 1024, d = 64, 91.4 and 102.4; 16 x 16 of 2048, d = 128, 190 and 198).
+  auto features = [&](cudaStream_t s) {
+    return run_features(tn, q, k, B, H, N, d, dtype, layout, h_sparse, h_lin, (WsHeader*)ws, s, &fm);
+  };
+  if (rounds && (rc = features(stream)) != GF_OK) return rc;
   Fork* f = both ? get_fork() : nullptr;
   if (both && f == nullptr) return GF_ERR_CUDA;
   std::unique_lock<std::mutex> enqueue_guard;
@@ -498,9 +506,12 @@ int gformer_hybrid_attn_w(const void* q, const void* k, const void* v, void* o, 
   // (the caller's stream may well have the lowest, like the side stream).
   const bool lin_first = both && lin_ctas > 0;
   if (lin_first && cudaStreamWaitEvent(f->first, f->fork, 0) != cudaSuccess) return GF_ERR_CUDA;
+  cudaStream_t lstream = lin_first ? f->first : stream;
   int lin_grid = 0;
-  rc = run_linear(tn, q, k, v, o, B, H, N, d, dtype, layout, h_sparse, h_lin, S_out, z_out, true, lin_ctas,
-                  (WsHeader*)ws, lin_first ? f->first : stream, both, fm, &lin_grid);
+  if (!rounds) rc = features(lstream);
+  if (rc == GF_OK)
+    rc = run_linear(tn, q, k, v, o, B, H, N, d, dtype, layout, h_sparse, h_lin, S_out, z_out, true, lin_ctas,
+                    (WsHeader*)ws, lstream, both, fm, &lin_grid);
   if (lin_first) {
     if (cudaEventRecord(f->join_first, f->first) != cudaSuccess) return GF_ERR_CUDA;
     if (cudaStreamWaitEvent(stream, f->join_first, 0) != cudaSuccess) return GF_ERR_CUDA;

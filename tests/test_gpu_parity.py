@@ -1167,6 +1167,23 @@ def test_favor_hybrid_layer_prefill_then_decode(B, H, N, d, w, h0):
         check(f64(ot), ref[:, :, t], "bf16", f"favor decode step {t - N}")
 
 
+@pytest.mark.parametrize("B,H,N,d,w,h0", [(10, 16, 300, 64, 32, 1), (2, 10, 300, 128, 32, 2), (1, 4, 5000, 64, 64, 1)])
+def test_favor_hybrid_layer_orders_of_the_pre_pass(B, H, N, d, w, h0):
+    """150 whole chains (features ahead of the fork of the head groups), 16 whole and 3 cut ones (behind it), a state
+    exported; sampled sequences against the oracle."""
+    q, k, v = synth.qkv(B, H, N, d, "bf16", seed=885 + N)
+    W = _proj(H - h0, d, "bf16", seed=886)
+    st = gf.DecodeState(B, H, d, w, h0)
+    ws = gf.Workspace.for_problem(B, H, N, d, w, h0, phi=gf.GF_PHI_FAVOR_POS)
+    o = gf.hybrid_attn(*dev(q, k, v), w, h_sparse=h0, state_out=st, W=W.cuda(), ws=ws).cpu()
+    assert ws.last_device_status() == gf.GF_OK
+    bs = sorted({0, B - 1})
+    ref = oracle.hybrid_attn(f64(q[bs]), f64(k[bs]), f64(v[bs]), w, h_sparse=h0, W=f64(W))
+    assert_parity(f64(o[bs]), ref, "bf16", f"favor hybrid B={B} H={H} N={N} d={d}")
+    slots = torch.arange(N - w, N) % w
+    assert torch.equal(st.k_cache[:, :h0, slots].cpu(), k[:, :h0, N - w:]) and torch.equal(st.v_cache[:, :h0, slots].cpu(), v[:, :h0, N - w:])
+
+
 def test_favor_ragged_decode_matches_every_sequence_alone():
     # three slots at different positions (one prefilled past the window, one from scratch, one idle) under the
     # positive random features: every sequence against the oracle's layer on that sequence alone
