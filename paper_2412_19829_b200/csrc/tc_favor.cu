@@ -255,7 +255,7 @@ cudaError_t launch_favor_features_tc(const void* q, const void* k, const void* W
   p.rows = (long long)B * h_count;
   p.ntile = (N + 127) / 128;
   const long long total = 2 * p.rows * p.ntile;
-  if (p.rows > 0x7fffffffLL) return cudaErrorInvalidValue;
+  if (p.rows > 0x7fffffffLL || p.ntile > 65535) return cudaErrorInvalidValue;  // (tiles: more than 8 million tokens)
   auto launch = [&](auto kern, int smem) -> cudaError_t {
     int dev = 0, sms = 0;
     cudaError_t err = device_info(&dev, &sms);

@@ -1184,6 +1184,18 @@ def test_favor_hybrid_layer_orders_of_the_pre_pass(B, H, N, d, w, h0):
     assert torch.equal(st.k_cache[:, :h0, slots].cpu(), k[:, :h0, N - w:]) and torch.equal(st.v_cache[:, :h0, slots].cpu(), v[:, :h0, N - w:])
 
 
+def test_favor_refuses_more_than_65535_tiles():
+    # the limit of the feature pre-pass: refused before anything but the workspace header is written
+    N, d = 65535 * 128 + 1, 64
+    q = torch.zeros(1, 1, N, d, dtype=torch.bfloat16, device="cuda")
+    o = torch.full_like(q, 7.0)
+    with pytest.raises(gf.GformerError) as e:
+        gf.causal_linear_attn(q, q, q, W=torch.zeros(1, d, d, dtype=torch.bfloat16, device="cuda"), out=o,
+                              ws=gf.Workspace.for_problem(1, 1, N, d, phi=gf.GF_PHI_FAVOR_POS))
+    assert e.value.status == gf.GF_ERR_CUDA
+    assert bool((o == 7.0).all())
+
+
 def test_favor_ragged_decode_matches_every_sequence_alone():
     # three slots at different positions (one prefilled past the window, one from scratch, one idle) under the
     # positive random features: every sequence against the oracle's layer on that sequence alone
