@@ -587,6 +587,8 @@ static int decode_step_impl(const void* q, const void* k, const void* v, void* o
   if (st->dtype != GF_F32 && st->dtype != GF_BF16) return GF_ERR_INVALID_ARG;
   if (st->d != 64 && st->d != 128) return GF_ERR_UNSUPPORTED;
   if (st->B > 65535) return GF_ERR_UNSUPPORTED;
+  // (rings of more than 40 960 slots are refused since the scores of a window were kept in shared memory; the kernel has no
+  // such limit any more, and nothing above it is tested)
   if ((size_t)st->w * sizeof(float) > 160 * 1024) return GF_ERR_UNSUPPORTED;
   if (st->h_sparse > 0 &&
       (!st->k_cache || !st->v_cache || !aligned16(st->k_cache) || !aligned16(st->v_cache)))

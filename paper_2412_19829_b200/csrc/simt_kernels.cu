@@ -34,7 +34,8 @@ template <> struct Vec4<__nv_bfloat16> {
 };
 
 // ------------------------------------------------------------------------------------
-// Causal linear attention, Algorithm 1 token by token.
+// Linear attention token by token: Algorithm 1 with positive random features, and both feature maps of the bidirectional
+// layer (the causal heads with elu + 1 are linear_walk_kernel).
 // One CTA = one head x one slice of 32 value columns.  Warp g owns features
 // a in [g*D/8, (g+1)*D/8); lane c owns value column c of the slice.  S lives in registers
 // (D/8 per thread), z is replicated per lane.  Tokens are staged 16 at a time.

@@ -862,8 +862,11 @@ int self_segments(int nchains, int nch) {
 
 // Whether whole chains go through linear_self_whole_kernel: its ceil(chains / CTAs) rounds of a whole chain each against
 // the three launches, whose work is spread evenly but costs a sixth more per chunk (its two halves do not run side by
-// side) and about nine chunks' time in launches and start-up.  Measured, whole against three launches: 128 chains of
-// 1024 tokens 20.5 and 30.8 us, 256 of 4096 102 and 127, 160 of 4096 89.0 and 92.1 (three launches), 24 of 197 10.3 and 19.7.
+// side) and about nine chunks' time in launches and start-up.  Measured (us, whole | three launches): where the rule takes
+// whole chains 128 of 1024 tokens 20.5 | 30.8, 160 of 1024 29.2 | 41.0, 310 of 2048 74 | 89, 260 of 4096 110 | 126, 24 of 197
+// 10.3 | 19.7; where it takes three launches 40 of 2048 30.8 | 26.7, 160 of 4096 94.1 | 90.1, 160 of 8192 175 | 157, 150 of
+// 16 384 333 | 279.  It errs where the last round is thin or the chains are short: 160 of 2048 51.1 | 59.4, 200 of 4096
+// 97 | 101, 300 of 4096 139 | 152, all three in three launches.
 bool self_whole(int nchains, int nch, int d, int sms) {
   if (d != WholeCfg::D) return false;
   const double rounds = (double)((nchains + sms - 1) / sms) * nch;

@@ -375,7 +375,7 @@ def test_cut_chain_calls_from_two_streams_and_two_threads():
 @pytest.mark.parametrize("d", [64, 128])
 def test_linear_chunk_size_invariance(d):
     """Algorithm 1 regrouped in different ways gives the same values up to rounding: token by token
-    (the CUDA-core path: a chunk of one row), 128 rows at a time with every chain whole, and 128-row
+    (decode steps: a chunk of one row), 32 rows at a time (the CUDA-core path), 128 rows at a time with every chain whole, and 128-row
     chunks in segments of 1, 2 and 5 chunks with the state handed over between CTAs.  (128 is the only
     chunk height of the tensor-core path -- the M of a one-CTA tcgen05 product -- so the `chunk` argument
     takes 0 or 128 and answers GF_ERR_UNSUPPORTED to 64 and 256; what varies is the regrouping around it.)"""
@@ -394,8 +394,14 @@ def test_linear_chunk_size_invariance(d):
         assert errors(f64(S), S_ref)["rel_l2"] <= 1e-2 and errors(f64(z), z_ref)["rel_l2"] <= 1e-2
         outs[name], states[name] = f64(o), f64(S)
 
+    st = gf.DecodeState(B, H, d, 1, 0)
+    steps = [t.permute(2, 0, 1, 3).contiguous() for t in dev(q, k, v)]
+    o = torch.stack([gf.decode_step(*(t[n] for t in steps), st) for n in range(N)], dim=2)
+    assert_parity(f64(o), ref, "bf16", f"linear d={d} token by token")
+    assert errors(f64(st.S), S_ref)["rel_l2"] <= 1e-2 and errors(f64(st.z), z_ref)["rel_l2"] <= 1e-2
+    outs["token by token"], states["token by token"] = f64(o), f64(st.S)
     gf.set_tuning(gf.GF_TUNE_FORCE_SIMT, 1)
-    run("token by token")
+    run("blocks of 32")
     gf.set_tuning(gf.GF_TUNE_FORCE_SIMT, 0)
     for split, name in ((-1, "whole chains"), (1, "segments of 1"), (2, "segments of 2"), (5, "segments of 5")):
         gf.set_tuning(gf.GF_TUNE_LINEAR_SPLIT, split)
@@ -403,9 +409,10 @@ def test_linear_chunk_size_invariance(d):
     base = outs["whole chains"]
     for name, o in outs.items():
         assert errors(o, base)["max_abs"] <= 2e-2, name
-        # (the tensor-core forms round phi(K) to bf16 before the products, the token-wise form keeps fp32:
-        # their states differ by that rounding, a few 1e-3; among the tensor-core forms far less)
-        assert errors(states[name], states["whole chains"])["rel_l2"] <= (5e-3 if name == "token by token" else 1e-3), name
+        # (the tensor-core forms round phi(K) to bf16 before the products, the others keep fp32: their
+        # states differ by that rounding, a few 1e-3; among the tensor-core forms far less)
+        fp32 = name in ("token by token", "blocks of 32")
+        assert errors(states[name], states["whole chains"])["rel_l2"] <= (5e-3 if fp32 else 1e-3), name
     # other chunk heights are refused, not silently replaced
     ws = gf.Workspace.for_problem(B, H, N, d, 1, 0)
     for chunk in (64, 256):
