@@ -19,8 +19,10 @@ runs only that head group's kernel a few times (a small driver for profilers).
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import os
+import re
 import subprocess
 import sys
 import tempfile
@@ -83,12 +85,25 @@ def measured_peaks():
     return 6650.0, "fallback"
 
 
+def kernel_sources_hash():
+    """Of the sources of the tensor-core kernels, without comments and white space: what a capture of them belongs to."""
+    csrc = os.path.join(ROOT, "paper_2412_19829_b200", "csrc")
+    h = hashlib.sha256()
+    for name in ("tc_linear.cu", "tc_linear_self.cu", "tc_window.cu", "linear_phi.cuh", "sm100.cuh"):
+        with open(os.path.join(csrc, name)) as f:
+            h.update("".join(re.sub(r"//.*", "", f.read()).split()).encode())
+    return h.hexdigest()[:16]
+
+
 def recorded_traffic(workload):
-    """DRAM bytes per launch of the workload's kernels ({kernel: bytes}) from the committed ncu captures, if recorded."""
+    """DRAM bytes per launch of the workload's kernels ({kernel: bytes}) from the committed ncu captures; None where there
+    is none or the kernels have changed since."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if os.path.exists(p):
         with open(p) as f:
-            return json.load(f).get(workload)
+            recorded = json.load(f)
+        if recorded.get("kernel_sources") == kernel_sources_hash():
+            return recorded.get(workload)
     return None
 
 
