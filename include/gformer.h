@@ -265,11 +265,11 @@ int gformer_noalloc_last_device_status(void* cuda_stream);
 /*
  * The hybrid layer (Sec. III-A): heads [0, h_sparse) as gformer_window_attn, heads
  * [h_sparse, H) as gformer_causal_linear_attn with a zero initial state; h_sparse < 0
- * selects gformer_default_h_sparse(H).  The two groups run side by side on the device (on two
- * streams of the library's own, forked from and joined back into `cuda_stream`, so the caller
- * sees a single-stream call that may also be captured into a CUDA graph).  Host threads may call
- * concurrently, each with its own workspace and stream; on one device their fork .. join sections
- * are enqueued one after the other.
+ * selects gformer_default_h_sparse(H).  The two groups run side by side on the device, as a chain
+ * of kernels in `cuda_stream` that start without waiting for one another's end; what follows the
+ * call in the stream waits for all of them, and the call may be captured into a CUDA graph.  Host
+ * threads may call concurrently, each with its own workspace and stream; on one device calls whose
+ * linear heads are cut into segments follow one another.
  * state_out (may be NULL): if given, its B, H, d, w, h_sparse, dtype must match the call
  * and its buffers receive the decode state after the N tokens: the last min(N, w) keys
  * and values of the windowed heads in ring slots j mod w, the final S and z of the linear

@@ -3,7 +3,6 @@
 #include <stdint.h>
 
 #include <atomic>
-#include <mutex>
 
 #include "common.cuh"
 
@@ -32,44 +31,6 @@ Tuning tuning_now() {
   t.wait_kcycles = g_wait_kcycles.load(std::memory_order_relaxed);
   t.drop_flag = g_drop_flag.load(std::memory_order_relaxed);
   return t;
-}
-
-constexpr int kMaxDevices = 64;
-constexpr unsigned int kPlacedWaitNs = 20000;  // longest the windowed heads are held back for the linear kernel's CTAs
-struct Fork {
-  cudaStream_t side = nullptr, first = nullptr, aux = nullptr;  // lowest / highest / lowest stream priority
-  cudaEvent_t fork = nullptr, join = nullptr, join_first = nullptr, join_aux = nullptr;
-  bool ready = false;
-  // held while a call enqueues its fork .. join section: the events are shared by every call on
-  // the device, and a record from another host thread between this call's record and its waits
-  // would make the side streams wait for the wrong point
-  std::mutex enqueue;
-};
-Fork g_fork[kMaxDevices];
-std::mutex g_fork_mutex;
-
-// Streams and events per device, created on first use; they let the two head groups of the hybrid layer (and the export
-// of the ring) run concurrently while the caller sees a single-stream call.
-Fork* get_fork() {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-  std::lock_guard<std::mutex> lock(g_fork_mutex);
-  Fork& f = g_fork[dev];
-  if (!f.ready) {
-    // lowest priority: where the two kernels compete for an SM, the persistent linear kernel
-    // (whose CTAs wait for one another) is placed first
-    int prio_least = 0, prio_greatest = 0;
-    if (cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest) != cudaSuccess) return nullptr;
-    if (cudaStreamCreateWithPriority(&f.side, cudaStreamNonBlocking, prio_least) != cudaSuccess) return nullptr;
-    if (cudaStreamCreateWithPriority(&f.first, cudaStreamNonBlocking, prio_greatest) != cudaSuccess) return nullptr;
-    if (cudaStreamCreateWithPriority(&f.aux, cudaStreamNonBlocking, prio_least) != cudaSuccess) return nullptr;
-    if (cudaEventCreateWithFlags(&f.join_aux, cudaEventDisableTiming) != cudaSuccess) return nullptr;
-    if (cudaEventCreateWithFlags(&f.join_first, cudaEventDisableTiming) != cudaSuccess) return nullptr;
-    if (cudaEventCreateWithFlags(&f.fork, cudaEventDisableTiming) != cudaSuccess) return nullptr;
-    if (cudaEventCreateWithFlags(&f.join, cudaEventDisableTiming) != cudaSuccess) return nullptr;
-    f.ready = true;
-  }
-  return &f;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -106,15 +67,15 @@ int cuda_status(cudaError_t e) { return e == cudaSuccess ? GF_OK : GF_ERR_CUDA; 
 // Window heads [h_begin, h_begin+h_count) on `stream`.
 int run_window(const Tuning& tn, const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d, int w,
                float scale, int dtype, int layout, int h_begin, int h_count, WsHeader* ws,
-               cudaStream_t stream, bool two_sided = false) {
+               cudaStream_t stream, gf::Link link, bool two_sided = false, bool hold = false) {
   if (h_count <= 0) return GF_OK;
   const int w_eff = w > N ? N : w;  // keys before token 0 (or after the last one) do not exist
   const int fwd = two_sided ? w_eff - 1 : 0;
   if (!tn.force_simt && gf::tc_window_supported(N, d, w_eff, dtype))
     return cuda_status(
-        gf::launch_window_tc(q, k, v, o, B, H, N, d, w_eff, fwd, scale, layout, h_begin, h_count, ws, stream));
+        gf::launch_window_tc(q, k, v, o, B, H, N, d, w_eff, fwd, scale, layout, h_begin, h_count, ws, stream, link, hold));
   return cuda_status(gf::launch_window_simt(q, k, v, o, B, N, d, w_eff, fwd, scale, dtype,
-                                            gf::make_strides(layout, H, N, d), h_begin, h_count, stream));
+                                            gf::make_strides(layout, H, N, d), h_begin, h_count, stream, gf::kBeside));
 }
 
 // Feature map of the linear heads of one call: elu + 1 (W null), or positive random features under
@@ -142,32 +103,50 @@ int run_features(const Tuning& tn, const void* q, const void* k, int B, int H, i
   phi->fq = reinterpret_cast<uint8_t*>(ws) + phi->feat_offset;
   phi->fk = reinterpret_cast<uint8_t*>(phi->fq) + feature_bytes(B, h_count, N, d);
   return cuda_status(gf::launch_favor_features_tc(q, k, phi->W, phi->fq, phi->fk, B, H, N, d, layout, h_begin, h_count, ws,
-                                                  stream));
+                                                  stream, gf::kAfter));
 }
 
 int run_linear(const Tuning& tn, const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d, int dtype,
                int layout, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init, int max_ctas,
-               WsHeader* ws, cudaStream_t stream, bool shared = false, const Phi& phi = Phi(), int* first_grid = nullptr) {
+               WsHeader* ws, cudaStream_t stream, gf::Link link, bool shared = false, const Phi& phi = Phi()) {
   if (h_count <= 0) return GF_OK;
   if (!tn.force_simt && gf::tc_linear_supported(N, d, dtype)) {
     return cuda_status(gf::launch_linear_tc(q, k, v, o, B, H, N, d, layout, h_begin, h_count, S_io, z_io,
-                                            zero_init, tn.linear_split, max_ctas, ws, stream, shared, phi.fq, phi.fk, first_grid));
+                                            zero_init, tn.linear_split, max_ctas, ws, stream, link, shared, phi.fq, phi.fk));
   }
   return cuda_status(gf::launch_linear_simt(q, k, v, o, B, N, d, dtype, gf::make_strides(layout, H, N, d),
-                                            h_begin, h_count, S_io, z_io, zero_init, stream, false, phi.W));
+                                            h_begin, h_count, S_io, z_io, zero_init, stream, gf::kBeside, false, phi.W));
 }
 
-// Zeroes the workspace header and, for a call that runs the tensor-core linear kernel on n_lin
-// chains, the hand-over flags behind it: one memset, ahead of everything the call launches.
-int clear_ws(const Tuning& tn, void* ws, cudaStream_t stream, int n_lin = 0, int N = 0, int d = 0, int dtype = GF_BF16) {
-  size_t bytes = sizeof(WsHeader);
-  if (n_lin > 0 && !tn.force_simt && gf::tc_linear_supported(N, d, dtype))
-    bytes += gf::linear_tc_flag_bytes(n_lin, N, tn.linear_split);
-  if (cudaMemsetAsync(ws, 0, bytes, stream) != cudaSuccess) return GF_ERR_CUDA;
-  // the two test knobs travel in the header (all zero otherwise: nothing more to do)
-  if (tn.wait_kcycles != 0 || tn.drop_flag != 0)
-    return cuda_status(gf::launch_set_header((WsHeader*)ws, (unsigned int)tn.wait_kcycles, (unsigned int)tn.drop_flag, stream));
-  return GF_OK;
+// The first launch of every call but a decode step: zeroes the workspace header and the flags or counters of a linear kernel
+// behind it.  What follows in the call's chain of kernels (launch_link)
+// runs kAfter it or, the kernels that use no workspace and those behind one that is kAfter it, kBeside it.
+// A memset and two streams with events for the two head groups, which this chain replaced, took 11 driver calls for a layer
+// instead of three and left the device idle for 2 to 4 us behind the memset and again at the end: 64 x 12 heads of 197 tokens
+// (d = 64, both directions) 33.0 -> 26.7 us, 8 x 12 of 2048 34.0 -> 32.7, 1 x 32 of 32 768 (d = 128, w = 512) 343 -> 336.
+int clear_ws(const Tuning& tn, void* ws, cudaStream_t stream, size_t flag_bytes = 0) {
+  return cuda_status(gf::launch_clear_ws(ws, sizeof(WsHeader) + flag_bytes, (unsigned int)tn.wait_kcycles,
+                                         (unsigned int)tn.drop_flag, stream));
+}
+
+// How the tensor-core kernel of the causal linear heads will run a call's chains: max_ctas as for launch_linear_tc, bytes of
+// flags, the order among cut-chain calls entered where there are any.
+int plan_linear(const Tuning& tn, int chains, int N, int d, int dtype, bool shared, cudaStream_t stream, int* max_ctas,
+                size_t* flag_bytes, gf::CutChainOrder* order) {
+  *max_ctas = 0;
+  *flag_bytes = 0;
+  if (chains <= 0 || tn.force_simt || !gf::tc_linear_supported(N, d, dtype)) return GF_OK;
+  int L = 0, G = 0, whole = 0, dev = 0, sms = 0;
+  if (gf::device_info(&dev, &sms) != cudaSuccess) return GF_ERR_CUDA;
+  if (shared && tn.linear_ctas > 0 && tn.linear_ctas < sms) {
+    gf::linear_tc_plan_parts(chains, N, d, tn.linear_split, 0, &whole, &L, &G, true);
+    // (leaving SMs to the windowed heads from the start only makes sense where there is work for every SM)
+    if ((long long)chains * (whole > 0 ? 1 : G) >= sms) *max_ctas = sms = tn.linear_ctas;
+  }
+  gf::linear_tc_plan_parts(chains, N, d, tn.linear_split, sms, &whole, &L, &G, shared);
+  if (whole == chains) return GF_OK;  // (whole chains hand nothing on)
+  *flag_bytes = gf::linear_tc_flag_bytes(chains, N, tn.linear_split);
+  return cuda_status(order->enter(dev, stream));
 }
 
 size_t workspace_bytes(const Tuning& tn, int B, int H, int N, int d, int h_sparse, int dtype, int phi = GF_PHI_ELU1,
@@ -301,7 +280,7 @@ int gformer_window_attn(const void* q, const void* k, const void* v, void* o, in
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   rc = clear_ws(tn, ws, stream);
   if (rc != GF_OK) return rc;
-  return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream);
+  return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream, gf::kAfter);
 }
 
 int gformer_window_attn_self(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
@@ -317,7 +296,7 @@ int gformer_window_attn_self(const void* q, const void* k, const void* v, void* 
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   rc = clear_ws(tn, ws, stream);
   if (rc != GF_OK) return rc;
-  return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream, true);
+  return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream, gf::kAfter, true);
 }
 
 int gformer_hybrid_attn_self(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
@@ -343,58 +322,32 @@ int gformer_hybrid_attn_self_w(const void* q, const void* k, const void* v, void
   if (rc != GF_OK) return rc;
   if (!(scale > 0.f)) scale = 1.0f / sqrtf((float)d);
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  rc = clear_ws(tn, ws, stream);
-  if (rc != GF_OK) return rc;
   const bool tc_linear = !tn.force_simt && gf::tc_linear_supported(N, d, dtype);
+  rc = clear_ws(tn, ws, stream, tc_linear ? gf::linear_self_count_bytes(B * (H - h_sparse)) : 0);
+  if (rc != GF_OK) return rc;
   Phi fm;
   fm.W = W;
   fm.feat_offset = feat_offset;
-  // (the pre-pass ahead of the fork: windowed-heads CTAs beside it would still hold SMs when the linear heads want them all;
-  // 4 x 16 heads of 2000 tokens, d = 128, 68.8 us and, behind the fork, 82.7; 64 x 12 of 197, d = 64, 50.3 and 63.6)
   if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, h_sparse, H - h_sparse, (WsHeader*)ws, stream, &fm)) != GF_OK)
     return rc;
-  if (h_sparse > 0 && h_sparse < H && tc_linear) {
-    // Both head groups on tensor-core kernels: the three launches of the linear heads go to the
-    // library's high-priority stream, the windowed heads to its side stream a few microseconds
-    // later; their CTAs run while the small totals kernel has the device and in the tails of the
-    // two big ones.  Forked from and joined back into the caller's stream.  Where all CTAs fit the device there is nothing to
-    // order: the linear heads stay on the caller's stream and the windowed ones start at once (a small call is bound by the
-    // host, and the stream, its events and the ordering kernel cost it 3.6 us: 16 heads of 700 tokens, d = 64, 20.2 -> 16.6).
-    Fork* f = get_fork();
-    int dev = 0, sms = 0;
-    if (f == nullptr || gf::device_info(&dev, &sms) != cudaSuccess) return GF_ERR_CUDA;
-    const long long win_units = (long long)B * h_sparse * ((N + 255) / 256);
-    const bool compete = gf::linear_self_items(B * (H - h_sparse), N, d, sms) + win_units > sms;
-    cudaStream_t lstream = compete ? f->first : stream;
-    std::unique_lock<std::mutex> enqueue_guard(f->enqueue);
-    if (cudaEventRecord(f->fork, stream) != cudaSuccess) return GF_ERR_CUDA;
-    if (cudaStreamWaitEvent(f->side, f->fork, 0) != cudaSuccess) return GF_ERR_CUDA;
-    if (compete && cudaStreamWaitEvent(f->first, f->fork, 0) != cudaSuccess) return GF_ERR_CUDA;
-    int lin_grid = 0;
+  if (h_sparse == H)
+    return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream, gf::kAfter, true);
+  int wrc = GF_OK;  // of the windowed heads: on the SMs that the linear heads leave idle, and between their kernels
+  auto window = [&]() -> cudaError_t {
+    wrc = run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, stream, gf::kBeside, true);
+    return wrc == GF_OK ? cudaSuccess : cudaErrorUnknown;
+  };
+  if (tc_linear) {
+    // (half tiles of 64 keys, 0.6 us each on an SM: tc_window.cu)
+    const double window_us = 0.5 * B * h_sparse * ((N + 127) / 128) * (4.0 * (((w < N ? w : N) + 126) / 128) + 2.0) / 148.0;
     rc = cuda_status(gf::launch_linear_self_tc(q, k, v, o, B, H, N, d, layout, h_sparse, H - h_sparse, (WsHeader*)ws,
-                                               sizeof(WsHeader), lstream, fm.fq, fm.fk, &lin_grid));
-    if (compete && (cudaEventRecord(f->join_first, f->first) != cudaSuccess ||
-                    cudaStreamWaitEvent(stream, f->join_first, 0) != cudaSuccess))
-      return GF_ERR_CUDA;
-    // the windowed heads start once the CTAs of the first linear kernel have all started
-    int rc2 = (rc == GF_OK && compete && lin_grid > 0)
-                  ? cuda_status(gf::launch_wait_placed((WsHeader*)ws, (unsigned int)lin_grid, kPlacedWaitNs, f->side))
-                  : GF_OK;
-    if (rc2 == GF_OK)
-      rc2 = run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, f->side, true);
-    if (cudaEventRecord(f->join, f->side) != cudaSuccess) return GF_ERR_CUDA;
-    if (cudaStreamWaitEvent(stream, f->join, 0) != cudaSuccess) return GF_ERR_CUDA;
-    return rc != GF_OK ? rc : rc2;
+                                               sizeof(WsHeader), stream, window, window_us, fm.fq, fm.fk));
+  } else {  // fp32 storage (or the CUDA-core knob): token by token, a summing sweep and a readout sweep
+    rc = cuda_status(gf::launch_linear_simt(q, k, v, o, B, N, d, dtype, gf::make_strides(layout, H, N, d), h_sparse,
+                                            H - h_sparse, nullptr, nullptr, true, stream, gf::kBeside, true, W));
+    if (rc == GF_OK) (void)window();
   }
-  rc = run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, stream, true);
-  if (rc != GF_OK) return rc;
-  if (h_sparse == H) return GF_OK;
-  if (tc_linear)
-    return cuda_status(gf::launch_linear_self_tc(q, k, v, o, B, H, N, d, layout, h_sparse, H - h_sparse, (WsHeader*)ws,
-                                                 sizeof(WsHeader), stream, fm.fq, fm.fk));
-  // fp32 storage (or the CUDA-core knob): token by token, a summing sweep and a readout sweep
-  return cuda_status(gf::launch_linear_simt(q, k, v, o, B, N, d, dtype, gf::make_strides(layout, H, N, d), h_sparse,
-                                            H - h_sparse, nullptr, nullptr, true, stream, true, W));
+  return wrc != GF_OK ? wrc : rc;
 }
 
 int gformer_causal_linear_attn(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
@@ -420,11 +373,16 @@ int gformer_causal_linear_attn_w(const void* q, const void* k, const void* v, vo
   rc = check_ws(ws, ws_bytes, workspace_bytes(tn, B, H, N, d, 0, dtype, phi, &fm.feat_offset));
   if (rc != GF_OK) return rc;
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  rc = clear_ws(tn, ws, stream, B * H, N, d, dtype);
-  if (rc != GF_OK) return rc;
+  gf::CutChainOrder order;
+  int max_ctas = 0;
+  size_t flags = 0;
+  if ((rc = plan_linear(tn, B * H, N, d, dtype, false, stream, &max_ctas, &flags, &order)) != GF_OK) return rc;
+  if ((rc = clear_ws(tn, ws, stream, flags)) != GF_OK) return rc;
   if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, 0, H, (WsHeader*)ws, stream, &fm)) != GF_OK) return rc;
-  return run_linear(tn, q, k, v, o, B, H, N, d, dtype, layout, 0, H, S_io, z_io, false, 0, (WsHeader*)ws, stream, false,
-                    fm);
+  if ((rc = run_linear(tn, q, k, v, o, B, H, N, d, dtype, layout, 0, H, S_io, z_io, false, max_ctas, (WsHeader*)ws, stream,
+                       gf::kAfter, false, fm)) != GF_OK)
+    return rc;
+  return cuda_status(order.leave());
 }
 
 int gformer_hybrid_attn(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d, int w,
@@ -461,88 +419,44 @@ int gformer_hybrid_attn_w(const void* q, const void* k, const void* v, void* o, 
   if (rc != GF_OK) return rc;
   if (!(scale > 0.f)) scale = 1.0f / sqrtf((float)d);
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  rc = clear_ws(tn, ws, stream, B * h_lin, N, d, dtype);
-  if (rc != GF_OK) return rc;
-
   float* S_out = state_out ? state_out->S : nullptr;
   float* z_out = state_out ? state_out->z : nullptr;
-  // The two head groups run side by side on two streams.  The persistent linear kernel holds one
-  // CTA per SM it uses.  When it has work for every SM it still takes them all (measured on a
-  // B200, leaving some to the windowed heads from the start was no faster and less steady), on a
-  // stream of the highest priority; the windowed heads' short-lived CTAs then fill the SMs that
-  // linear CTAs leave at different times towards the end.
+  // The two head groups run side by side.  The linear heads (long serial chains, one CTA per SM, which takes all of the
+  // SM's shared memory) come first and take every SM that they have work for (leaving some to the windowed heads from the start
+  // was no faster and less steady); the windowed heads' CTAs fill the SMs that are free or that linear CTAs leave at different
+  // times towards the end.  They are launched when all linear CTAs, which wait for one another, have started.  The export of the
+  // ring, which only needs K and V, runs beside the linear heads: its CTAs fit into what those leave of an SM.
   const bool both = h_sparse > 0 && h_lin > 0;
-  bool rounds = false;  // of whole chains, more than one
-  int lin_ctas = 0;
-  if (both && !tn.force_simt && gf::tc_linear_supported(N, d, dtype)) {
-    int L = 0, G = 0, whole = 0, dev = 0, sms = 0;
-    gf::linear_tc_plan_parts(B * h_lin, N, d, tn.linear_split, 0, &whole, &L, &G, true);
-    if (whole > 0) G = 1;  // items of the first launch: the chains left whole
-    if (gf::device_info(&dev, &sms) != cudaSuccess) return GF_ERR_CUDA;
-    if ((long long)B * h_lin * G >= sms) {
-      lin_ctas = (tn.linear_ctas > 0 && tn.linear_ctas < sms) ? tn.linear_ctas : sms;
-      rounds = whole > 0;
-    }
-  }
-  // The pre-pass of random features goes to the stream of the linear heads behind the fork, so that windowed heads run beside
-  // it and in its tail (us, ahead of the fork and behind it: 4 x 32 heads of 544 tokens, d = 64, 41.3 and 32.0; 8 x 8 of 3217
-  // 71.5 and 62.5; 32 of 32 768, d = 128, 454 and 444), but ahead of it where the linear heads fill the device for more than
-  // a round of whole chains (32 x 12 of 1024, d = 64, 91.4 and 102.4; 16 x 16 of 2048, d = 128, 190 and 198).
-  auto features = [&](cudaStream_t s) {
-    return run_features(tn, q, k, B, H, N, d, dtype, layout, h_sparse, h_lin, (WsHeader*)ws, s, &fm);
+  gf::CutChainOrder order;
+  int max_ctas = 0;
+  size_t flags = 0;
+  if ((rc = plan_linear(tn, B * h_lin, N, d, dtype, both, stream, &max_ctas, &flags, &order)) != GF_OK) return rc;
+  if ((rc = clear_ws(tn, ws, stream, flags)) != GF_OK) return rc;
+  if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, h_sparse, h_lin, (WsHeader*)ws, stream, &fm)) != GF_OK) return rc;
+  auto linear = [&](gf::Link link) {
+    return run_linear(tn, q, k, v, o, B, H, N, d, dtype, layout, h_sparse, h_lin, S_out, z_out, true, max_ctas, (WsHeader*)ws,
+                      stream, link, both, fm);
   };
-  if (rounds && (rc = features(stream)) != GF_OK) return rc;
-  Fork* f = both ? get_fork() : nullptr;
-  if (both && f == nullptr) return GF_ERR_CUDA;
-  std::unique_lock<std::mutex> enqueue_guard;
-  if (both) enqueue_guard = std::unique_lock<std::mutex>(f->enqueue);
-  if (both) {
-    // fork: the linear heads (the long serial chains) stay on the caller's stream, the
-    // windowed heads go to the side stream; join before returning control to the stream.
-    if (cudaEventRecord(f->fork, stream) != cudaSuccess) return GF_ERR_CUDA;
-    if (cudaStreamWaitEvent(f->side, f->fork, 0) != cudaSuccess) return GF_ERR_CUDA;
+  auto window = [&](gf::Link link, bool hold) {
+    return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, stream, link, false, hold);
+  };
+  // Behind a pre-pass of random features the windowed heads come first and fill its tail, and the linear heads theirs (us, after
+  // the linear heads and ahead of them: 32 heads of 32 768 tokens, d = 128, 461 and 444; 8 x 8 of 3217, d = 64, 62.0 and 57.9;
+  // 32 x 12 of 1024 87.8 and 86.1; without features ahead of them is slower, 8 x 12 of 2048 32.6 and 39.6).
+  const bool window_first = both && fm.fq != nullptr;
+  if (window_first) {
+    if ((rc = window(gf::kBeside, true)) != GF_OK) return rc;  // (it lets go of the linear heads when the features are complete)
+    if ((rc = linear(gf::kBeside)) != GF_OK) return rc;
+  } else if ((rc = linear(gf::kAfter)) != GF_OK) {
+    return rc;
   }
-  // When the two kernels compete for SMs the linear one goes to a stream of the highest priority
-  // (the caller's stream may well have the lowest, like the side stream).
-  const bool lin_first = both && lin_ctas > 0;
-  if (lin_first && cudaStreamWaitEvent(f->first, f->fork, 0) != cudaSuccess) return GF_ERR_CUDA;
-  cudaStream_t lstream = lin_first ? f->first : stream;
-  int lin_grid = 0;
-  if (!rounds) rc = features(lstream);
-  if (rc == GF_OK)
-    rc = run_linear(tn, q, k, v, o, B, H, N, d, dtype, layout, h_sparse, h_lin, S_out, z_out, true, lin_ctas,
-                    (WsHeader*)ws, lstream, both, fm, &lin_grid);
-  if (lin_first) {
-    if (cudaEventRecord(f->join_first, f->first) != cudaSuccess) return GF_ERR_CUDA;
-    if (cudaStreamWaitEvent(stream, f->join_first, 0) != cudaSuccess) return GF_ERR_CUDA;
-  }
-  cudaStream_t wstream = both ? f->side : stream;
-  // Both kernels become runnable at the fork.  CTAs of the persistent linear kernel wait for one
-  // another and want every SM from the start, while a windowed-heads CTA that got onto an SM first
-  // keeps it for many tiles: the side stream is held back until the linear kernel's CTAs have all
-  // started (they count themselves in the workspace header), 20 microseconds at most.
-  if (lin_first && rc == GF_OK && lin_grid > 0 &&
-      cuda_status(gf::launch_wait_placed((WsHeader*)ws, (unsigned int)lin_grid, kPlacedWaitNs, wstream)) != GF_OK)
-    return GF_ERR_CUDA;
-  int rc2 = run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, wstream);
-  // The ring only needs K and V.  Where the linear heads fill the device the windowed ones end last, and behind them the
-  // 3 to 9 us of the export would add to the call; on a stream of its own it fills gaps (14 x 4 heads of 3217 tokens 76.1
-  // -> 73.1 us).  A small call is bound by the host, which the two extra event calls would cost 1 us (18.7 -> 19.8).
-  if (rc2 == GF_OK && state_out && h_sparse > 0) {
-    cudaStream_t estream = lin_first ? f->aux : wstream;
-    if (lin_first && cudaStreamWaitEvent(f->aux, f->fork, 0) != cudaSuccess) return GF_ERR_CUDA;
-    rc2 = cuda_status(gf::launch_export_ring(k, v, state_out->k_cache, state_out->v_cache, B, N, d, w, dtype,
-                                             gf::make_strides(layout, H, N, d), h_sparse, estream));
-    if (lin_first && (cudaEventRecord(f->join_aux, f->aux) != cudaSuccess ||
-                 cudaStreamWaitEvent(stream, f->join_aux, 0) != cudaSuccess))
-      return GF_ERR_CUDA;
-  }
-  if (both) {
-    if (cudaEventRecord(f->join, f->side) != cudaSuccess) return GF_ERR_CUDA;
-    if (cudaStreamWaitEvent(stream, f->join, 0) != cudaSuccess) return GF_ERR_CUDA;
-  }
-  if (rc != GF_OK) return rc;
-  if (rc2 != GF_OK) return rc2;
+  if (state_out && (rc = cuda_status(gf::launch_export_ring(k, v, state_out->k_cache, state_out->v_cache, B, N, d, w, dtype,
+                                                            gf::make_strides(layout, H, N, d), h_sparse, stream,
+                                                            gf::kBeside))) != GF_OK)
+    return rc;
+  // (with windowed heads alone nothing before them has waited for the cleared header)
+  if (!window_first && (rc = window(h_lin > 0 ? gf::kBeside : gf::kAfter, false)) != GF_OK) return rc;
+  if ((rc = cuda_status(order.leave())) != GF_OK) return rc;
   if (state_out) state_out->t = N;
   return GF_OK;
 }

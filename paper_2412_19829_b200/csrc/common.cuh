@@ -6,6 +6,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
+#include <mutex>
+
 #include "gformer.h"
 
 namespace gf {
@@ -36,47 +39,81 @@ struct WsHeader {
   unsigned int ticket;   // work counter of the persistent kernels
   unsigned int wait_kcycles;  // limit of every bounded wait in units of 1024 cycles; 0 = default (about 2 s)
   unsigned int drop_flag;     // failure injection for tests: the linear kernel skips the flag of segment n - 1
-  unsigned int placed;        // CTAs of the call's linear-attention kernels that have started (see launch_wait_placed)
-  unsigned int pad[58];
+  unsigned int pad[59];
 };
 static_assert(sizeof(WsHeader) == 256, "workspace header is 256 bytes");
 
 // Counts kernel launches (reported by gformer_launch_count).
 void note_launch(int n = 1);
 
+// Zeroes the first `bytes` bytes (a multiple of 16) of a workspace and writes the two test knobs into its header.
+cudaError_t launch_clear_ws(void* ws, size_t bytes, unsigned int wait_kcycles, unsigned int drop_flag, cudaStream_t stream);
+
+// ---- The kernels of a call, in one stream, as a chain of programmatic dependent launches.
+//
+// A kernel of the chain is launched as soon as every CTA of the kernel before it has started and has called
+// grid_dep_launch(), and its CTAs are placed wherever an SM has room for them.  Two kinds of link:
+//   kAfter   the kernel reads what the one before it writes: its CTAs set themselves up, then grid_dep_wait()
+//   kBeside  it depends on nothing that the kernel before it does, only on what that one had itself waited for before it
+//            let go of its dependents.  It starts at once, on the SMs that are free or become so.  One of its CTAs waits
+//            before it ends (grid_dep_wait() returns when all kernels before it are complete), so that what follows the
+//            call in the stream follows all of its kernels.
+// The head of a chain is launched the ordinary way (kFirst): it starts when everything before it in the stream is complete.
+enum Link { kFirst = 0, kAfter = 1, kBeside = 2 };
+template <typename... P, typename... A>
+cudaError_t launch_link_clusters(Link link, int cluster /* CTAs along x; 1: none */, void (*kern)(P...), dim3 grid, dim3 block,
+                                 size_t smem, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2] = {};
+  if (link != kFirst) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = cluster;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+  if (e != cudaSuccess) return e;
+  note_launch();
+  return cudaGetLastError();
+}
+template <typename... P, typename... A>
+cudaError_t launch_link(Link link, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+  return launch_link_clusters(link, 1, kern, grid, block, smem, stream, args...);
+}
+
 // ---- SIMT (CUDA-core, fp32 arithmetic) path: any w, d in {64,128}, f32 or bf16 storage.
 // Heads [h_begin, h_begin + h_count) of the [B, H, N, d] tensors are processed.
 // fwd: keys after the query it may see: 0 = the causal window, w - 1 = the two-sided window |i - j| < w.
 cudaError_t launch_window_simt(const void* q, const void* k, const void* v, void* o, int B, int N, int d,
                                int w, int fwd, float scale, int dtype, Strides st, int h_begin, int h_count,
-                               cudaStream_t stream);
+                               cudaStream_t stream, Link link);
 // S_io/z_io: [B, h_count, d, d] / [B, h_count, d] or null.  zero_init: ignore their contents on entry.
 // global_sum: the unmasked linear attention of the bidirectional layer (sum over all tokens, then readout).
 cudaError_t launch_linear_simt(const void* q, const void* k, const void* v, void* o, int B, int N, int d,
                                int dtype, Strides st, int h_begin, int h_count, float* S_io, float* z_io,
-                               bool zero_init, cudaStream_t stream, bool global_sum = false,
+                               bool zero_init, cudaStream_t stream, Link link, bool global_sum = false,
                                const void* W = nullptr /* [h_count, d, d] storage dtype: positive random features */);
 // The causal heads with phi = elu + 1: register-tiled blocks of 32 tokens (launch_linear_simt comes here by itself).
 cudaError_t launch_linear_tiled(const void* q, const void* k, const void* v, void* o, int B, int N, int d, int dtype,
                                 Strides st, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
-                                cudaStream_t stream);
+                                cudaStream_t stream, Link link);
 cudaError_t launch_export_ring(const void* k, const void* v, void* k_cache, void* v_cache, int B, int N, int d,
-                               int w, int dtype, Strides st, int h_sparse, cudaStream_t stream);
+                               int w, int dtype, Strides st, int h_sparse, cudaStream_t stream, Link link);
 // t_seq == nullptr: every sequence is at position t; else sequence b is at t_seq[b] (device array,
 // negative = idle slot, otherwise below 2^48) and the kernel itself moves the positions on.
 cudaError_t launch_decode_step(const void* q, const void* k, const void* v, void* o, void* k_cache,
                                void* v_cache, float* S, float* z, long long t, long long* t_seq, int B, int H,
                                int d, int w, int h_sparse, float scale, int dtype, cudaStream_t stream,
                                const void* W = nullptr /* [H - h_sparse, d, d] storage dtype */);
-
-// Writes the two test knobs into a workspace header that has just been cleared.
-cudaError_t launch_set_header(WsHeader* ws, unsigned int wait_kcycles, unsigned int drop_flag, cudaStream_t stream);
-
-// One tiny CTA that returns once `target` CTAs of the call's linear-attention kernel have started
-// (WsHeader::placed), or after max_ns nanoseconds whichever comes first: holds back the work queued
-// behind it in its stream without occupying an SM's shared memory or tensor memory.  Never an error:
-// when the limit ends the wait, the work behind it simply starts.
-cudaError_t launch_wait_placed(WsHeader* ws, unsigned int target, unsigned int max_ns, cudaStream_t stream);
 
 // The current device and its SM count (asked of the driver once per device).
 cudaError_t device_info(int* dev, int* sms);
@@ -88,16 +125,19 @@ bool tc_window_supported(int N, int d, int w, int dtype);
 bool tc_linear_supported(int N, int d, int dtype);
 cudaError_t launch_window_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                              int w, int fwd, float scale, int layout, int h_begin, int h_count, WsHeader* ws,
-                             cudaStream_t stream);
-// Global (unmasked) linear attention of the bidirectional layer, heads [h_begin, h_begin + h_count):
-// three launches (segment sums, totals, readout); its scratch starts scratch_offset bytes into ws.
+                             cudaStream_t stream, Link link,
+                             bool hold = false /* what follows it kBeside needs what the kernel before it writes */);
+// Global (unmasked) linear attention of the bidirectional layer, heads [h_begin, h_begin + h_count): one launch, or three
+// (segment sums, totals, readout), kAfter the kernel before them; its scratch starts scratch_offset bytes into ws, with
+// linear_self_count_bytes that must be zero.  beside() launches, kBeside, what is to run between the first launch and
+// the others (the windowed heads), and takes about beside_us microseconds of the whole device.
+size_t linear_self_count_bytes(int nchains);
 size_t linear_self_workspace_bytes(int nchains, int N, int d);
-// work items of its first launch: one CTA each as far as there are SMs
-int linear_self_items(int nchains, int N, int d, int sms);
 cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                                   int layout, int h_begin, int h_count, WsHeader* ws, size_t scratch_offset,
-                                  cudaStream_t stream, const void* fq = nullptr, const void* fk = nullptr,
-                                  int* first_grid = nullptr /* CTAs of the first launch */);
+                                  cudaStream_t stream, const std::function<cudaError_t()>& beside, double beside_us,
+                                  const void* fq = nullptr,
+                                  const void* fk = nullptr);
 // Segmentation used by the tensor-core linear kernel (split: 0 = automatic, else chunks per segment;
 // ctas: CTAs the kernel will run with, 0 = one per SM of a B200) and the scratch it needs beyond
 // the workspace header (sized for the largest segment count the plan may pick for any ctas).
@@ -114,18 +154,38 @@ size_t linear_tc_workspace_bytes(int nchains, int N, int d, int split);
 size_t linear_tc_flag_bytes(int nchains, int N, int split);
 cudaError_t launch_linear_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                              int layout, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
-                             int split, int max_ctas, WsHeader* ws, cudaStream_t stream, bool shared = false,
-                             const void* fq = nullptr, const void* fk = nullptr,
-                             int* first_grid = nullptr /* CTAs of the first launch */);
+                             int split, int max_ctas, WsHeader* ws, cudaStream_t stream, Link link, bool shared = false,
+                             const void* fq = nullptr, const void* fk = nullptr);
+// The CTAs of a cut-chain launch wait for one another, so two such kernels must not share the SMs: each could hold some of
+// them while its own unplaced CTAs wait for the rest.  Per device the calls that have one are therefore chained by an event:
+// such a call starts only when the previous one, from whatever stream or host thread, has finished.  (Not inside a stream
+// capture, where an outside event cannot be waited for: there the order of the caller's graphs applies.)  Entered ahead
+// of the call's first launch and left behind its last one, because an event between two kernels would part their chain.
+class CutChainOrder {
+ public:
+  cudaError_t enter(int dev, cudaStream_t stream);
+  cudaError_t leave();  // records the event
+
+ private:
+  std::unique_lock<std::mutex> lock_;
+  int dev_ = 0;
+  cudaStream_t stream_ = nullptr;
+};
+
 // Positive random features phi_W of Q and K of heads [h_begin, h_begin + h_count) (bf16 storage) into the
 // contiguous bf16 tensors fq, fk [B, h_count, N, d]; W: [h_count, d, d] bf16, row a of a head's matrix is
 // its projection vector w_a.  With fq, fk given, the two linear-attention launchers read them in place
 // of Q and K and leave their own feature map out.
 cudaError_t launch_favor_features_tc(const void* q, const void* k, const void* W, void* fq, void* fk, int B, int H,
                                      int N, int d, int layout, int h_begin, int h_count, WsHeader* ws,
-                                     cudaStream_t stream);
+                                     cudaStream_t stream, Link link);
 
 // ---- device helpers
+// All kernels before this one in the stream are complete and what they wrote can be read.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The kernel that follows in the stream may be launched once every CTA of this one has said so.
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Cycles a bounded wait may take; `status` points at the first word of the workspace header.
 __device__ __forceinline__ long long wait_limit_cycles(const unsigned int* status) {
   const unsigned int kc = reinterpret_cast<const volatile unsigned int*>(status)[3];

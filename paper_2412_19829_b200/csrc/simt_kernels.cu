@@ -4,6 +4,7 @@
 // bidirectional layer's sums, positive random features), and the memory-bound decode step and ring export, which have
 // no dense contraction worth a tensor core.  Plain data-parallel kernels: no inter-CTA communication, no spin waits.
 #include <cooperative_groups.h>
+#include <stddef.h>
 
 #include "common.cuh"
 
@@ -57,6 +58,7 @@ linear_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
   __shared__ float red[TB][8][33];
   __shared__ float redden[TB][8];
 
+  grid_dep_launch();
   const int slice = blockIdx.x, hl = blockIdx.y, b = blockIdx.z;
   const int h = h_begin + hl;
   const long long base = (long long)b * st.b + (long long)h * st.h;
@@ -186,30 +188,38 @@ linear_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
 
 // ------------------------------------------------------------------------------------
 // Ring export: the last min(N, w) keys/values of the windowed heads into slot j mod w.
+// It runs beside the linear heads, whose kernel leaves 4096 registers of an SM: 128 threads of 32.  A thread moves two 16-byte
+// pieces of K and two of V, all four loads in flight at once.
 // ------------------------------------------------------------------------------------
-template <typename T>
-__global__ void export_ring_kernel(const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ kc,
-                                   T* __restrict__ vc, int N, int d, int w, int wn, Strides st,
-                                   int h_sparse, long long total4) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= total4) return;
-  const int d4 = d / 4;
-  const int c4 = (int)(idx % d4);
-  long long r = idx / d4;
-  const int jj = (int)(r % wn);
-  r /= wn;
-  const int h = (int)(r % h_sparse);
-  const int b = (int)(r / h_sparse);
-  const int j = N - wn + jj;
-  const long long src = (long long)b * st.b + (long long)h * st.h + (long long)j * st.n + 4 * c4;
-  const long long dst = (((long long)b * h_sparse + h) * w + (j % w)) * d + 4 * c4;
-  if (sizeof(T) == 4) {
-    *reinterpret_cast<float4*>(kc + dst) = *reinterpret_cast<const float4*>(k + src);
-    *reinterpret_cast<float4*>(vc + dst) = *reinterpret_cast<const float4*>(v + src);
-  } else {
-    *reinterpret_cast<uint2*>(kc + dst) = *reinterpret_cast<const uint2*>(k + src);
-    *reinterpret_cast<uint2*>(vc + dst) = *reinterpret_cast<const uint2*>(v + src);
+constexpr int kExportThreads = 128;
+__global__ void __launch_bounds__(kExportThreads, 16)
+export_ring_kernel(const uint4* __restrict__ k, const uint4* __restrict__ v, uint4* __restrict__ kc, uint4* __restrict__ vc,
+                   int N, int d16, int w, int wn, Strides st16, int h_sparse, unsigned int total) {
+  // d16, st16: row length and strides in 16-byte pieces
+  grid_dep_launch();
+  uint4 x[2], y[2];
+  long long dst[2];
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const unsigned int idx = (blockIdx.x * 2u + e) * kExportThreads + threadIdx.x;
+    dst[e] = -1;
+    if (idx < total) {
+      const unsigned int row = idx / (unsigned)d16, c = idx - row * d16;
+      const unsigned int bh = row / (unsigned)wn, b = bh / (unsigned)h_sparse;
+      const int j = N - wn + (int)(row - bh * wn);
+      const long long src = b * st16.b + (bh - b * h_sparse) * st16.h + j * st16.n + c;
+      x[e] = k[src];
+      y[e] = v[src];
+      dst[e] = ((long long)bh * w + j % w) * d16 + c;
+    }
   }
+#pragma unroll
+  for (int e = 0; e < 2; ++e)
+    if (dst[e] >= 0) {
+      kc[dst[e]] = x[e];
+      vc[dst[e]] = y[e];
+    }
+  if (blockIdx.x == 0) grid_dep_wait();
 }
 
 // ------------------------------------------------------------------------------------
@@ -535,24 +545,11 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
 template <typename T>
 cudaError_t linear_dispatch(const void* q, const void* k, const void* v, void* o, int B, int N, int d,
                             Strides st, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
-                            bool global_sum, cudaStream_t stream, const void* W) {
-  auto* kern = d == 64 ? linear_simt_kernel<T, 64> : linear_simt_kernel<T, 128>;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(d / 32, h_count, B);
-  cfg.blockDim = dim3(256);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = d / 32;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = (S_io != nullptr && !zero_init) ? 1 : 0;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, (const T*)q, (const T*)k, (const T*)v, (T*)o, N, st, h_begin, h_count,
-                                           S_io, z_io, zero_init ? 1 : 0, global_sum ? 1 : 0, (const T*)W);
-  if (e != cudaSuccess) return e;
-  note_launch();
-  return cudaGetLastError();
+                            bool global_sum, cudaStream_t stream, Link link, const void* W) {
+  return launch_link_clusters(link, S_io != nullptr && !zero_init ? d / 32 : 1,
+                              d == 64 ? linear_simt_kernel<T, 64> : linear_simt_kernel<T, 128>, dim3(d / 32, h_count, B),
+                              dim3(256), 0, stream, (const T*)q, (const T*)k, (const T*)v, (T*)o, N, st, h_begin, h_count, S_io,
+                              z_io, zero_init ? 1 : 0, global_sum ? 1 : 0, (const T*)W);
 }
 
 template <typename T>
@@ -579,65 +576,48 @@ cudaError_t decode_dispatch(const void* q, const void* k, const void* v, void* o
 
 cudaError_t launch_linear_simt(const void* q, const void* k, const void* v, void* o, int B, int N, int d,
                                int dtype, Strides st, int h_begin, int h_count, float* S_io, float* z_io,
-                               bool zero_init, cudaStream_t stream, bool global_sum, const void* W) {
+                               bool zero_init, cudaStream_t stream, Link link, bool global_sum, const void* W) {
   if (h_count <= 0 || B <= 0) return cudaSuccess;
   if (!global_sum && W == nullptr)
-    return launch_linear_tiled(q, k, v, o, B, N, d, dtype, st, h_begin, h_count, S_io, z_io, zero_init, stream);
+    return launch_linear_tiled(q, k, v, o, B, N, d, dtype, st, h_begin, h_count, S_io, z_io, zero_init, stream, link);
   if (dtype == GF_F32)
     return linear_dispatch<float>(q, k, v, o, B, N, d, st, h_begin, h_count, S_io, z_io, zero_init, global_sum,
-                                  stream, W);
+                                  stream, link, W);
   return linear_dispatch<__nv_bfloat16>(q, k, v, o, B, N, d, st, h_begin, h_count, S_io, z_io, zero_init, global_sum,
-                                        stream, W);
+                                        stream, link, W);
 }
 
 cudaError_t launch_export_ring(const void* k, const void* v, void* k_cache, void* v_cache, int B, int N, int d,
-                               int w, int dtype, Strides st, int h_sparse, cudaStream_t stream) {
+                               int w, int dtype, Strides st, int h_sparse, cudaStream_t stream, Link link) {
   if (h_sparse <= 0 || B <= 0) return cudaSuccess;
-  const int wn = N < w ? N : w;
-  const long long total4 = (long long)B * h_sparse * wn * (d / 4);
-  const int threads = 256;
-  const long long blocks = (total4 + threads - 1) / threads;
-  if (dtype == GF_F32)
-    export_ring_kernel<float><<<(unsigned)blocks, threads, 0, stream>>>(
-        (const float*)k, (const float*)v, (float*)k_cache, (float*)v_cache, N, d, w, wn, st, h_sparse, total4);
-  else
-    export_ring_kernel<__nv_bfloat16><<<(unsigned)blocks, threads, 0, stream>>>(
-        (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, N,
-        d, w, wn, st, h_sparse, total4);
-  note_launch();
-  return cudaGetLastError();
+  const int wn = N < w ? N : w, per16 = dtype == GF_F32 ? 4 : 8;  // elements of 16 bytes
+  const long long total = (long long)B * h_sparse * wn * (d / per16);
+  // (64 GB of keys)
+  if (total > 0xffffffffLL - 2 * kExportThreads) return cudaErrorInvalidValue;
+  const Strides st16 = {st.b / per16, st.h / per16, st.n / per16};
+  return launch_link(link, export_ring_kernel, dim3((unsigned)((total + 2 * kExportThreads - 1) / (2 * kExportThreads))),
+                     dim3(kExportThreads), 0, stream, (const uint4*)k, (const uint4*)v, (uint4*)k_cache, (uint4*)v_cache, N,
+                     d / per16, w, wn, st16, h_sparse, (unsigned)total);
 }
 
 namespace {
-__global__ void wait_placed_kernel(const unsigned int* placed, unsigned int target, unsigned int max_ns) {
-  unsigned long long t0, t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-  for (int i = 0; i < 100000; ++i) {  // bounded whatever the timer does
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(placed) : "memory");
-    if (v >= target) break;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    if (t - t0 >= max_ns) break;
-    __nanosleep(100);
-  }
+__global__ void clear_ws_kernel(uint4* ws, unsigned int n16, unsigned int wait_kcycles, unsigned int drop_flag) {
+  grid_dep_launch();
+  const unsigned int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n16) return;
+  uint4 x = make_uint4(0u, 0u, 0u, 0u);
+  if (i == 0) x.w = wait_kcycles;  // WsHeader::wait_kcycles
+  if (i == 1) x.x = drop_flag;     // WsHeader::drop_flag
+  ws[i] = x;
 }
+static_assert(offsetof(WsHeader, wait_kcycles) == 12 && offsetof(WsHeader, drop_flag) == 16, "what the kernel above writes");
 }  // namespace
 
-__global__ void set_header_kernel(WsHeader* ws, unsigned int wait_kcycles, unsigned int drop_flag) {
-  ws->wait_kcycles = wait_kcycles;
-  ws->drop_flag = drop_flag;
-}
-
-cudaError_t launch_set_header(WsHeader* ws, unsigned int wait_kcycles, unsigned int drop_flag, cudaStream_t stream) {
-  set_header_kernel<<<1, 1, 0, stream>>>(ws, wait_kcycles, drop_flag);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_wait_placed(WsHeader* ws, unsigned int target, unsigned int max_ns, cudaStream_t stream) {
-  wait_placed_kernel<<<1, 1, 0, stream>>>(&ws->placed, target, max_ns);
-  note_launch();
-  return cudaGetLastError();
+cudaError_t launch_clear_ws(void* ws, size_t bytes, unsigned int wait_kcycles, unsigned int drop_flag, cudaStream_t stream) {
+  const size_t n16 = bytes / 16;
+  if (n16 > 0x7fffffffu) return cudaErrorInvalidValue;
+  return launch_link(kFirst, clear_ws_kernel, dim3((unsigned)((n16 + 255) / 256)), dim3(256), 0, stream, (uint4*)ws,
+                     (unsigned)n16, wait_kcycles, drop_flag);
 }
 
 cudaError_t launch_decode_step(const void* q, const void* k, const void* v, void* o, void* k_cache,

@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(kNT, D == 64 ? 5 : 3)  // (else the rare path 
 window_tiled_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ o,
                     int N, int w, int fwd, float scale, Strides st, int h_begin) {
   // fwd: keys after the query that it may see (0: the causal window; w - 1: the two-sided one)
+  grid_dep_launch();
   constexpr int LD = D + 4, NC = D / 64;  // NC: groups of four output columns per thread, 64 apart
   extern __shared__ __align__(16) float sm[];
   float *Qs = sm, *Ks = Qs + kC * LD, *Vs = Ks + kC * LD, *Ps = Vs + kC * D, *As = Ps + kC * kLdP;
@@ -269,6 +270,7 @@ window_tiled_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
   if (__syncthreads_or(any) && Ps[t] != 0.f)
     window_row<T, D>(q + base, k + base, v + base, o + base, i0 + t, max(i0 + t - w + 1, 0), min(i0 + t + fwd, N - 1) + 1, scale,
                      st.n, part, 0xfu << (lane & 28), m, l);
+  if (blockIdx.x + blockIdx.y + blockIdx.z == 0) grid_dep_wait();
 }
 
 // ------------------------------------------------------------------------------------ causal linear heads
@@ -363,6 +365,7 @@ __global__ void __launch_bounds__(kNT)
 linear_contribution_kernel(const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o, Segs sg,
                            Strides st, int h_begin) {
   extern __shared__ __align__(16) float sm[];
+  grid_dep_launch();
   float *Ks = sm, *Vs = Ks + kC * (D + 4);
   const int g = blockIdx.x / (D / kW), col0 = (blockIdx.x % (D / kW)) * kW;
   const long long base = (long long)blockIdx.z * st.b + (long long)(h_begin + blockIdx.y) * st.h;
@@ -375,6 +378,7 @@ linear_contribution_kernel(const float* __restrict__ k, const float* __restrict_
   float* slot = o + base + (long long)n_end * st.n + col0;  // the state before segment g + 1, once summed
   for_state<D>(ag, S, [&](int a, float4& x) { store4(slot + (long long)a * st.n + 4 * cg, x); });
   if (tid < D) slot[(long long)(D + tid / kW) * st.n + tid % kW] = z;
+  if (blockIdx.x + blockIdx.y + blockIdx.z == 0) grid_dep_wait();
 }
 
 // The slots of segments 1 .. G - 1 hold contributions; turned into running sums from the caller's initial state
@@ -383,6 +387,8 @@ template <int D>
 __global__ void linear_prefix_kernel(float* __restrict__ o, Segs sg, Strides st, int h_begin, int h_count,
                                      const float* __restrict__ S_in, const float* __restrict__ z_in) {
   constexpr int D4 = D / 4, kRows = D + LinT<D>::ZROWS, kAhead = 8;
+  grid_dep_wait();
+  grid_dep_launch();
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= kRows * D4) return;
   const int row = idx / D4, c = 4 * (idx % D4);
@@ -416,8 +422,10 @@ __global__ void linear_prefix_kernel(float* __restrict__ o, Segs sg, Strides st,
 template <typename T, int D, bool kCluster>
 __global__ void __launch_bounds__(kNT)
 linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* o, Segs sg, Strides st,
-                   int h_begin, int h_count, float* S_io, float* z_io, int zero_init) {
+                   int h_begin, int h_count, float* S_io, float* z_io, int zero_init, int after) {
   constexpr int LD = LinT<D>::LD;
+  if (after) grid_dep_wait();  // the segments' starting states
+  grid_dep_launch();
   extern __shared__ __align__(16) float sm[];
   float *Qs = sm, *Ks = Qs + kC * LD, *Vs = Ks + kC * LD, *Ss = Vs + kC * kW, *Ps = Ss + D * kW, *zs = Ps + kC * kLdP,
         *inv_s = zs + D;
@@ -556,25 +564,24 @@ linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
     for_state<D>(i, S, [&](int a, float4& x) { store4(S_io + (sidx * D + a) * D + col0 + 4 * cg, x); });
     if (col0 == 0 && tid < D) z_io[sidx * D + tid] = zs[tid];
   }
+  if (blockIdx.x + blockIdx.y + blockIdx.z == 0) grid_dep_wait();
 }
 
 template <typename T, int D>
 cudaError_t window_launch(const void* q, const void* k, const void* v, void* o, int B, int N, int w, int fwd, float scale,
-                          Strides st, int h_begin, int h_count, cudaStream_t stream) {
+                          Strides st, int h_begin, int h_count, cudaStream_t stream, Link link) {
   int dev = 0, sms = 0;
   cudaError_t e = device_info(&dev, &sms);
   if (e != cudaSuccess) return e;
   auto kern = window_tiled_kernel<T, D>;
   if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, window_smem<D>())) != cudaSuccess) return e;
-  kern<<<dim3((N + kC - 1) / kC, h_count, B), kNT, window_smem<D>(), stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, N,
-                                                                               w, fwd, scale, st, h_begin);
-  note_launch();
-  return cudaGetLastError();
+  return launch_link(link, kern, dim3((N + kC - 1) / kC, h_count, B), dim3(kNT), window_smem<D>(), stream, (const T*)q,
+                     (const T*)k, (const T*)v, (T*)o, N, w, fwd, scale, st, h_begin);
 }
 
 template <typename T, int D>
 cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, int B, int N, Strides st, int h_begin,
-                          int h_count, float* S_io, float* z_io, bool zero_init, cudaStream_t stream) {
+                          int h_count, float* S_io, float* z_io, bool zero_init, cudaStream_t stream, Link link) {
   using C = LinT<D>;
   int dev = 0, sms = 0;
   cudaError_t e = device_info(&dev, &sms);
@@ -600,60 +607,46 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
       const Segs sg = {N, G, blocks / G, blocks % G};
       auto sum = linear_contribution_kernel<D>;
       if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(sum), dev, C::kSmemSum)) != cudaSuccess) return e;
-      sum<<<dim3((G - 1) * (D / kW), h_count, B), kNT, C::kSmemSum, stream>>>((const float*)k, (const float*)v, (float*)o, sg,
-                                                                              st, h_begin);
+      if ((e = launch_link(link, sum, dim3((G - 1) * (D / kW), h_count, B), dim3(kNT), C::kSmemSum, stream, (const float*)k,
+                           (const float*)v, (float*)o, sg, st, h_begin)) != cudaSuccess)
+        return e;
       constexpr int kItems = (D + C::ZROWS) * (D / 4);
-      linear_prefix_kernel<D><<<dim3((kItems + 127) / 128, h_count, B), 128, 0, stream>>>(
-          (float*)o, sg, st, h_begin, h_count, zero_init ? nullptr : S_io, z_io);
+      if ((e = launch_link(kAfter, linear_prefix_kernel<D>, dim3((kItems + 127) / 128, h_count, B), dim3(128), 0, stream,
+                           (float*)o, sg, st, h_begin, h_count, zero_init ? nullptr : S_io, z_io)) != cudaSuccess)
+        return e;
       auto walk = linear_walk_kernel<float, D, false>;
       if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, C::kSmem)) != cudaSuccess) return e;
-      walk<<<dim3(G * (D / kW), h_count, B), kNT, C::kSmem, stream>>>((const float*)q, (const float*)k, (const float*)v,
-                                                                      (float*)o, sg, st, h_begin, h_count, S_io, z_io,
-                                                                      zero_init ? 1 : 0);
-      note_launch(3);
-      return cudaGetLastError();
+      return launch_link(kAfter, walk, dim3(G * (D / kW), h_count, B), dim3(kNT), C::kSmem, stream, (const float*)q,
+                         (const float*)k, (const float*)v, (float*)o, sg, st, h_begin, h_count, S_io, z_io, zero_init ? 1 : 0, 1);
     }
   }
   const Segs sg = {N, cluster, blocks / cluster, blocks % cluster};
   const int cluster_ctas = cluster * slices;
   auto walk = cluster_ctas > 1 ? linear_walk_kernel<T, D, true> : linear_walk_kernel<T, D, false>;
   if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, C::kSmem)) != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cluster * (D / kW), h_count, B);
-  cfg.blockDim = dim3(kNT);
-  cfg.dynamicSmemBytes = C::kSmem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = cluster_ctas;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = cluster_ctas > 1 ? 1 : 0;
-  if ((e = cudaLaunchKernelEx(&cfg, walk, (const T*)q, (const T*)k, (const T*)v, (T*)o, sg, st, h_begin, h_count, S_io, z_io,
-                              zero_init ? 1 : 0)) != cudaSuccess)
-    return e;
-  note_launch();
-  return cudaGetLastError();
+  return launch_link_clusters(link, cluster_ctas, walk, dim3(cluster * (D / kW), h_count, B), dim3(kNT), C::kSmem, stream,
+                              (const T*)q, (const T*)k, (const T*)v, (T*)o, sg, st, h_begin, h_count, S_io, z_io,
+                              zero_init ? 1 : 0, 0);
 }
 
 }  // namespace
 
 cudaError_t launch_window_simt(const void* q, const void* k, const void* v, void* o, int B, int N, int d, int w, int fwd,
-                               float scale, int dtype, Strides st, int h_begin, int h_count, cudaStream_t stream) {
+                               float scale, int dtype, Strides st, int h_begin, int h_count, cudaStream_t stream,
+                               Link link) {
   if (h_count <= 0 || B <= 0) return cudaSuccess;
   auto* f = dtype == GF_F32 ? (d == 64 ? window_launch<float, 64> : window_launch<float, 128>)
                             : (d == 64 ? window_launch<__nv_bfloat16, 64> : window_launch<__nv_bfloat16, 128>);
-  return f(q, k, v, o, B, N, w, fwd, scale, st, h_begin, h_count, stream);
+  return f(q, k, v, o, B, N, w, fwd, scale, st, h_begin, h_count, stream, link);
 }
 
 cudaError_t launch_linear_tiled(const void* q, const void* k, const void* v, void* o, int B, int N, int d, int dtype,
                                 Strides st, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
-                                cudaStream_t stream) {
+                                cudaStream_t stream, Link link) {
   if (h_count <= 0 || B <= 0) return cudaSuccess;
   auto* f = dtype == GF_F32 ? (d == 64 ? linear_launch<float, 64> : linear_launch<float, 128>)
                             : (d == 64 ? linear_launch<__nv_bfloat16, 64> : linear_launch<__nv_bfloat16, 128>);
-  return f(q, k, v, o, B, N, st, h_begin, h_count, S_io, z_io, zero_init, stream);
+  return f(q, k, v, o, B, N, st, h_begin, h_count, S_io, z_io, zero_init, stream, link);
 }
 
 }  // namespace gf

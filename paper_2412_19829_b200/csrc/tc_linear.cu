@@ -117,6 +117,7 @@ struct LinParams {
   float* S_io;           // [B, h_count, D, D] or null
   float* z_io;           // [B, h_count, D] or null
   int zero_init;
+  int beside;            // the kernel before this one in the stream may still be running (Link::kBeside)
   unsigned int* status;  // two words: status, where
   unsigned int* flags;   // [nchains * G] x kFlagStride: 1 once the segment's inclusive state is in `prefix`
   float* prefix;         // [nchains * G][D*D + D]
@@ -424,7 +425,6 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) {
-    atomicAdd(&p.status[5], 1u);  // WsHeader::placed: this CTA has an SM
     mbar_init(&bar.q_full[0], 1);
     mbar_init(&bar.q_full[1], 1);
     for (int s = 0; s < 5; ++s) {
@@ -488,6 +488,8 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
+  if (!p.beside) grid_dep_wait();
+  grid_dep_launch();
 
   // Every role walks the same item list and keeps the same running counters: ta = K tiles of pass
   // A so far (slot = ta % KA, phase = ta / KA), nq = pass-C chunks so far (K slot = nq % KS, phase =
@@ -1200,6 +1202,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, C::kTmemCols);
+  if (blockIdx.x == 0 && p.beside) grid_dep_wait();
 }
 
 }  // namespace
@@ -1412,23 +1415,32 @@ size_t linear_tc_workspace_bytes(int nchains, int N, int d, int split) {
 }
 
 namespace {
-// The CTAs of a cut-chain launch wait for one another, so two such kernels must not share the SMs: each
-// could hold some of them while its own unplaced CTAs wait for the rest.  Per device the launches are
-// therefore chained by an event: a cut-chain kernel starts only when the previous one, from whatever
-// stream or host thread, has finished.  (Not inside a stream capture, where an outside event cannot be
-// waited for: there the order of the caller's graphs applies.)
-struct CutChainOrder {
-  std::mutex mu;
-  cudaEvent_t last[64] = {};
-};
-CutChainOrder g_cut_order;
+std::mutex g_cut_mutex;
+cudaEvent_t g_cut_last[64] = {};  // per device: behind the last call that has a cut-chain launch
 }  // namespace
+
+cudaError_t CutChainOrder::enter(int dev, cudaStream_t stream) {
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(stream, &capturing);
+  if (e != cudaSuccess || capturing != cudaStreamCaptureStatusNone) return e;
+  lock_ = std::unique_lock<std::mutex>(g_cut_mutex);
+  dev_ = dev;
+  stream_ = stream;
+  cudaEvent_t& ev = g_cut_last[dev];
+  return ev == nullptr ? cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) : cudaStreamWaitEvent(stream, ev, 0);
+}
+
+cudaError_t CutChainOrder::leave() {
+  if (!lock_.owns_lock()) return cudaSuccess;
+  const cudaError_t e = cudaEventRecord(g_cut_last[dev_], stream_);
+  lock_.unlock();
+  return e;
+}
 
 cudaError_t launch_linear_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                              int layout, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
-                             int split, int max_ctas, WsHeader* ws, cudaStream_t stream, bool shared,
-                             const void* fq, const void* fk, int* first_grid) {
-  if (first_grid) *first_grid = 0;
+                             int split, int max_ctas, WsHeader* ws, cudaStream_t stream, Link link, bool shared,
+                             const void* fq, const void* fk) {
   if (h_count <= 0) return cudaSuccess;
   // fq, fk: feature tensors [B, h_count, N, d] that stand in for Q and K (feature map: identity)
   const bool features = fq != nullptr;
@@ -1464,25 +1476,9 @@ cudaError_t launch_linear_tc(const void* q, const void* k, const void* v, void* 
   auto launch = [&](auto kern, size_t smem) -> cudaError_t {
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, (int)smem);
     if (err != cudaSuccess) return err;
-    dim3 grid(p.nitems < sms ? p.nitems : sms);
-    if (first_grid && *first_grid == 0) *first_grid = (int)grid.x;
-    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (p.G > 1 && (err = cudaStreamIsCapturing(stream, &capturing)) != cudaSuccess) return err;
-    const bool chained = p.G > 1 && capturing == cudaStreamCaptureStatusNone;
-    std::unique_lock<std::mutex> order;
-    if (chained) {
-      order = std::unique_lock<std::mutex>(g_cut_order.mu);
-      cudaEvent_t& ev = g_cut_order.last[dev];
-      if (ev == nullptr) {
-        if ((err = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) return err;
-      } else if ((err = cudaStreamWaitEvent(stream, ev, 0)) != cudaSuccess) {
-        return err;
-      }
-    }
-    kern<<<grid, kThreads, smem, stream>>>(mq, mk, mv, mo, p);
-    note_launch();
-    err = cudaGetLastError();
-    if (chained && err == cudaSuccess) err = cudaEventRecord(g_cut_order.last[dev], stream);
+    p.beside = link == kBeside;
+    err = launch_link(link, kern, dim3(p.nitems < sms ? p.nitems : sms), dim3(kThreads), smem, stream, mq, mk, mv, mo, p);
+    link = kBeside;  // a second launch depends on nothing that the first one does
     return err;
   };
   // Chains [chain0, chain0 + count) of the call in one launch: whole (the one-pass form of the kernel) or cut

@@ -34,7 +34,33 @@ struct SelfParams {
   float* partial;                    // [nitems][D*D + D]: a segment's sums (S row-major [feature][column], then z)
   float* total;                      // [nchains][D*D + D]
   unsigned int* status;
+  // What the launches hand on is counted per chain, because the windowed heads of a layer run between them: warps that have
+  // written their rows of a segment's sums (4 G), then blocks of the totals (sum_blocks, with more than one segment).
+  // Zero at launch.
+  unsigned int *summed, *totalled;
+  unsigned int sum_blocks;
+  int totals_of_one;  // the sums were formed in one segment per chain: no totals
 };
+constexpr int kSumThreads = 64;
+
+__device__ __forceinline__ void count_up(unsigned int* counter) {
+  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
+}
+// Bounded poll (acquire) until the counter has reached the target.
+__device__ __forceinline__ bool wait_count(const unsigned int* counter, unsigned int target, unsigned int* status,
+                                           unsigned int where) {
+  const long long t0 = clock64();
+  for (unsigned int n = 0;; ++n) {
+    unsigned int v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
+    if (v >= target) return true;
+    if (n > 0 && clock64() - t0 > wait_limit_cycles(status)) {
+      if (atomicCAS(status, 0u, 1u) == 0u) status[1] = where;
+      return false;
+    }
+    __nanosleep(100);
+  }
+}
 
 struct SelfItem {
   int chain, g, b, h, c_begin, nC;
@@ -84,7 +110,6 @@ linear_self_reduce_kernel(const __grid_constant__ CUtensorMap mk, const __grid_c
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) {
-    atomicAdd(&p.status[5], 1u);  // WsHeader::placed: this CTA has an SM
     for (int i = 0; i < KS; ++i) {
       mbar_init(&k_full[i], 1);
       mbar_init(&kphi[i], 16);
@@ -118,6 +143,8 @@ linear_self_reduce_kernel(const __grid_constant__ CUtensorMap mk, const __grid_c
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
+  grid_dep_wait();
+  grid_dep_launch();
 
   // Every role walks the same items and keeps the same running counters: nk = K tiles so far
   // (slot nk % KS, phase nk / KS), nv likewise for V, na = items so far (accumulator na & 1).
@@ -183,6 +210,7 @@ linear_self_reduce_kernel(const __grid_constant__ CUtensorMap mk, const __grid_c
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     uint32_t na = 0;
     for (int item = blockIdx.x; item < p.nitems; item += gridDim.x, ++na) {
+      const SelfItem it = self_item(p, item);
       if (!mbar_wait(&acc_done[na & 1], (na >> 1) & 1, p.status, 720)) break;
       tc_fence_after_sync();
       const uint32_t acc = tmem + (na & 1) * C::kAcc + lane_off;
@@ -205,6 +233,8 @@ linear_self_reduce_kernel(const __grid_constant__ CUtensorMap mk, const __grid_c
       if (r < D) dst[D * D + r] = __uint_as_float(zc);
       tc_fence_before_sync();
       mbar_arrive(&acc_free[na & 1]);
+      __syncwarp();
+      if (lane == 0) count_up(p.summed + it.chain);
     }
   } else if (!kId) {
     // phi on the K tiles, in place, by 16 warps (features given: a tile is ready as it lands, rows past the end of the
@@ -230,22 +260,40 @@ linear_self_reduce_kernel(const __grid_constant__ CUtensorMap mk, const __grid_c
 }
 
 // ------------------------------------------------------------------------------------ sum
-// total[chain] = sum over the chain's segments, in segment order (deterministic).
-__global__ void linear_self_sum_kernel(const float* __restrict__ partial, float* __restrict__ total, int G,
-                                       int state_floats) {
+// total[chain] = sum over the chain's segments, in segment order (deterministic).  It is launched behind the windowed heads
+// and runs beside them: they leave 4096 registers of an SM, room for one block of 64 threads.  Eight loads in flight per
+// thread (one after the other, and with the device to itself, it took 6 us for 26 chains of 11 segments at d = 128).
+__global__ void __launch_bounds__(kSumThreads, 16)
+linear_self_sum_kernel(const SelfParams p, int state_floats) {
+  constexpr int kAhead = 8;
+  grid_dep_launch();
+  __shared__ int ready;
   const int chain = blockIdx.y;
-  const int i = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
-  if (i >= state_floats) return;
-  const float* src = partial + (long long)chain * G * state_floats + i;
-  float4 acc = *reinterpret_cast<const float4*>(src);
-  for (int g = 1; g < G; ++g) {
-    const float4 x = *reinterpret_cast<const float4*>(src + (long long)g * state_floats);
-    acc.x += x.x;
-    acc.y += x.y;
-    acc.z += x.z;
-    acc.w += x.w;
+  if (threadIdx.x == 0) ready = wait_count(p.summed + chain, 4u * p.G, p.status, 790);
+  __syncthreads();
+  const int i = (blockIdx.x * kSumThreads + threadIdx.x) * 4;
+  if (ready && i < state_floats) {
+    const float* src = p.partial + (long long)chain * p.G * state_floats + i;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int g0 = 0; g0 < p.G; g0 += kAhead) {
+      float4 x[kAhead];
+#pragma unroll
+      for (int e = 0; e < kAhead; ++e)
+        x[e] = g0 + e < p.G ? __ldcg(reinterpret_cast<const float4*>(src + (long long)(g0 + e) * state_floats))
+                          : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int e = 0; e < kAhead; ++e) {
+        acc.x += x[e].x;
+        acc.y += x[e].y;
+        acc.z += x[e].z;
+        acc.w += x[e].w;
+      }
+    }
+    *reinterpret_cast<float4*>(p.total + (long long)chain * state_floats + i) = acc;
   }
-  *reinterpret_cast<float4*>(total + (long long)chain * state_floats + i) = acc;
+  __syncthreads();
+  if (threadIdx.x == 0 && ready) count_up(p.totalled + chain);
+  if (blockIdx.x + blockIdx.y == 0) grid_dep_wait();
 }
 
 // ------------------------------------------------------------------------------------ readout
@@ -305,6 +353,7 @@ linear_self_readout_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
+  grid_dep_launch();
 
   // Running counters shared by all roles: nq = chunks so far (Q slot, phi(Q) slot and O buffer
   // nq & 1, phase nq >> 1; staging buffer phase nq), ni = items so far.
@@ -360,6 +409,11 @@ linear_self_readout_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
     bool ok = true;
     for (int item = blockIdx.x; item < p.nitems && ok; item += gridDim.x, ++ni) {
       const SelfItem it = self_item(p, item);
+      if (lane == 0)
+        ok = p.totals_of_one ? wait_count(p.summed + it.chain, 4u, p.status, 823)
+                             : wait_count(p.totalled + it.chain, p.sum_blocks, p.status, 822);
+      if (__any_sync(0xffffffffu, !ok)) break;
+      __syncwarp();  // (a vote orders no memory)
       // (the previous item's last product has completed: its o_full was seen below)
       if (s_row) {
         const float* src = p.total + (long long)it.chain * (D * D + D);
@@ -500,6 +554,7 @@ linear_self_readout_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, 512);
+  if (blockIdx.x == 0) grid_dep_wait();
 }
 
 // ------------------------------------------------------------------------------------ whole
@@ -539,7 +594,6 @@ linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_co
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   if (tid == 0) {
-    atomicAdd(&p.status[5], 1u);  // WsHeader::placed: this CTA has an SM
     for (int i = 0; i < KS; ++i) {
       mbar_init(&k_full[i], 1);
       mbar_init(&kphi[i], 8);
@@ -584,6 +638,8 @@ linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_co
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
+  grid_dep_wait();
+  grid_dep_launch();
 
   // Every role walks the chains blockIdx.x, blockIdx.x + gridDim.x, ... (an item is a whole chain) and keeps the same
   // running counters: n = chunks so far, c = chains so far.
@@ -835,7 +891,6 @@ linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_co
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem, 512);
 }
-
 // Segments per chain.  CTAs take items (segments) round-robin, so a launch lasts ceil(items / CTAs)
 // rounds of one item each: among the segment counts that keep segments at least four chunks long
 // (and the scratch within 64 slots per chain, more when the chains are few), take the one with the least rounds x (chunks of the
@@ -860,6 +915,28 @@ int self_segments(int nchains, int nch) {
   return best_g;
 }
 
+// Segments that the sums are formed in, at most self_segments.  Where windowed heads run behind the first launch (beside_us)
+// they fill the SMs that it leaves idle, so that only what they do not fill counts, in microseconds, beside the work itself; more segments
+// are more slots to add up, beside the windowed heads at 0.7 TB/s.
+int self_sum_segments(int nchains, int nch, int d, double beside_us) {
+  const int g_max = self_segments(nchains, nch);
+  if (beside_us <= 0.0) return g_max;
+  const double chunk_us = d == 128 ? 1.5 : 0.8, state = ((double)d * d + d) * sizeof(float);
+  int best_g = 1;
+  double best = 1e300;
+  for (int g = 1; g <= g_max; ++g) {
+    const double rounds = (double)(((long long)nchains * g + 147) / 148);
+    const double work = nchains * (double)(nch + g) / 148 * chunk_us, span = rounds * ((nch + g - 1) / g + 1) * chunk_us;
+    const double idle = span - work - beside_us, sum = g > 1 ? 1.0 + nchains * g * state / 0.7e6 - 0.7 * beside_us : 0.0;
+    const double cost = work + (idle > 0.0 ? idle : 0.0) + (g > 1 ? (sum > 1.0 ? sum : 1.0) : 0.0);
+    if (cost < best) {
+      best = cost;
+      best_g = g;
+    }
+  }
+  return best_g;
+}
+
 // Whether whole chains go through linear_self_whole_kernel: its ceil(chains / CTAs) rounds of a whole chain each against
 // the three launches, whose work is spread evenly but costs a sixth more per chunk (its two halves do not run side by
 // side) and about nine chunks' time in launches and start-up.  Measured (us, whole | three launches): where the rule takes
@@ -875,22 +952,20 @@ bool self_whole(int nchains, int nch, int d, int sms) {
 
 }  // namespace
 
+// Counters at the start of the scratch, cleared by the caller with the workspace header.
+size_t linear_self_count_bytes(int nchains) { return ((size_t)nchains * 2 * sizeof(unsigned int) + 255) & ~(size_t)255; }
+
 size_t linear_self_workspace_bytes(int nchains, int N, int d) {
   const int nch = (N + 127) / 128;
   const size_t state = ((size_t)d * d + d) * sizeof(float);
-  return (size_t)nchains * (self_segments(nchains, nch) + 1) * state;
-}
-
-int linear_self_items(int nchains, int N, int d, int sms) {
-  const int nch = (N + 127) / 128;
-  return self_whole(nchains, nch, d, sms) ? nchains : nchains * self_segments(nchains, nch);
+  return linear_self_count_bytes(nchains) + (size_t)nchains * (self_segments(nchains, nch) + 1) * state;
 }
 
 cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                                   int layout, int h_begin, int h_count, WsHeader* ws, size_t scratch_offset,
-                                  cudaStream_t stream, const void* fq, const void* fk, int* first_grid) {
-  if (first_grid) *first_grid = 0;
-  if (h_count <= 0) return cudaSuccess;
+                                  cudaStream_t stream, const std::function<cudaError_t()>& beside, double beside_us, const void* fq,
+                                  const void* fk) {
+  if (h_count <= 0) return beside();
   // fq, fk: feature tensors [B, h_count, N, d] that stand in for Q and K (feature map: identity)
   const bool features = fq != nullptr;
   CUtensorMap mq, mk, mv, mo;
@@ -911,34 +986,37 @@ cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, v
   cudaError_t e;
   if ((e = device_info(&dev, &sms)) != cudaSuccess) return e;
   const bool whole = self_whole(p.nchains, p.nch, d, sms);
-  p.G = whole ? 1 : self_segments(p.nchains, p.nch);
-  p.seg_base = p.nch / p.G;
-  p.seg_rem = p.nch % p.G;
-  p.nitems = p.nchains * p.G;
+  auto cut = [&](int G) {
+    p.G = G;
+    p.seg_base = p.nch / G;
+    p.seg_rem = p.nch % G;
+    p.nitems = p.nchains * G;
+    return dim3(p.nitems < sms ? p.nitems : sms);
+  };
+  dim3 grid = cut(whole ? 1 : self_sum_segments(p.nchains, p.nch, d, beside_us));
   const int state_floats = d * d + d;
-  p.partial = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(ws) + scratch_offset);
+  uint8_t* scratch = reinterpret_cast<uint8_t*>(ws) + scratch_offset;
+  p.summed = reinterpret_cast<unsigned int*>(scratch);
+  p.totalled = p.summed + p.nchains;
+  p.sum_blocks = (unsigned)((state_floats / 4 + kSumThreads - 1) / kSumThreads);
+  p.partial = reinterpret_cast<float*>(scratch + linear_self_count_bytes(p.nchains));
   p.total = p.G == 1 ? p.partial : p.partial + (size_t)p.nitems * state_floats;  // one segment: its sum is the total
   p.status = &ws->status;
-  dim3 grid(p.nitems < sms ? p.nitems : sms);
-  if (first_grid) *first_grid = (int)grid.x;
   if (whole) {
     auto kern = features ? linear_self_whole_kernel<true> : linear_self_whole_kernel<false>;
     if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, WholeCfg::kBytes)) != cudaSuccess) return e;
-    kern<<<grid, WholeCfg::kThreads, WholeCfg::kBytes, stream>>>(mq, mk, mv, mo, p);
-    note_launch();
-    return cudaGetLastError();
+    e = launch_link(kAfter, kern, grid, dim3(WholeCfg::kThreads), WholeCfg::kBytes, stream, mq, mk, mv, mo, p);
+    return e == cudaSuccess ? beside() : e;
   }
   auto launch_red = [&](auto kern, int smem, int threads) -> cudaError_t {
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem);
     if (err != cudaSuccess) return err;
-    kern<<<grid, threads, smem, stream>>>(mk, mv, p);
-    return cudaSuccess;
+    return launch_link(kAfter, kern, grid, dim3(threads), smem, stream, mk, mv, p);
   };
   auto launch_out = [&](auto kern, int smem, int threads) -> cudaError_t {
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem);
     if (err != cudaSuccess) return err;
-    kern<<<grid, threads, smem, stream>>>(mq, mo, p);
-    return cudaSuccess;
+    return launch_link(kBeside, kern, grid, dim3(threads), smem, stream, mq, mo, p);
   };
   if (features)
     e = (d == 64) ? launch_red(linear_self_reduce_kernel<64, true>, RedCfg<64>::kBytes, RedCfg<64>::kThreads)
@@ -947,21 +1025,19 @@ cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, v
     e = (d == 64) ? launch_red(linear_self_reduce_kernel<64, false>, RedCfg<64>::kBytes, RedCfg<64>::kThreads)
                   : launch_red(linear_self_reduce_kernel<128, false>, RedCfg<128>::kBytes, RedCfg<128>::kThreads);
   if (e != cudaSuccess) return e;
-  note_launch();
-  if (p.G > 1) {
-    linear_self_sum_kernel<<<dim3((state_floats / 4 + 255) / 256, p.nchains), 256, 0, stream>>>(p.partial, p.total, p.G,
-                                                                                                state_floats);
-    note_launch();
-  }
+  // The windowed heads between the two: they start on the SMs that the first kernel leaves, and the readout on those that they
+  // leave.
+  if ((e = beside()) != cudaSuccess) return e;
+  if (p.G > 1 && (e = launch_link(kBeside, linear_self_sum_kernel, dim3(p.sum_blocks, p.nchains), dim3(kSumThreads), 0, stream, p,
+                                  state_floats)) != cudaSuccess)
+    return e;
+  p.totals_of_one = p.G == 1;
+  grid = cut(self_segments(p.nchains, p.nch));  // (the readout goes by the segments that fill the device best by themselves)
   if (features)
-    e = (d == 64) ? launch_out(linear_self_readout_kernel<64, true>, OutCfg<64>::kBytes, OutCfg<64>::kThreads)
-                  : launch_out(linear_self_readout_kernel<128, true>, OutCfg<128>::kBytes, OutCfg<128>::kThreads);
-  else
-    e = (d == 64) ? launch_out(linear_self_readout_kernel<64, false>, OutCfg<64>::kBytes, OutCfg<64>::kThreads)
-                  : launch_out(linear_self_readout_kernel<128, false>, OutCfg<128>::kBytes, OutCfg<128>::kThreads);
-  if (e != cudaSuccess) return e;
-  note_launch();
-  return cudaGetLastError();
+    return (d == 64) ? launch_out(linear_self_readout_kernel<64, true>, OutCfg<64>::kBytes, OutCfg<64>::kThreads)
+                     : launch_out(linear_self_readout_kernel<128, true>, OutCfg<128>::kBytes, OutCfg<128>::kThreads);
+  return (d == 64) ? launch_out(linear_self_readout_kernel<64, false>, OutCfg<64>::kBytes, OutCfg<64>::kThreads)
+                   : launch_out(linear_self_readout_kernel<128, false>, OutCfg<128>::kBytes, OutCfg<128>::kThreads);
 }
 
 }  // namespace gf

@@ -89,6 +89,8 @@ struct WinParams {
   int h_begin, h_count, nqt, npair, total;  // work units: (batch, head, pair of query tiles), pair fastest
   unsigned int* status;
   unsigned int* ticket;  // zero at launch; units beyond the first one of every CTA come from here
+  int beside;            // the kernel before this one in the stream may still be running (Link::kBeside)
+  int hold;              // the next kernel may only start when the one before this is complete
 };
 
 // A wait that first polls the barrier for a few microseconds (a thread parked in try_wait takes a
@@ -197,6 +199,8 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = ctl->tmem_base;
+  if (!p.beside) grid_dep_wait();
+  if (!p.hold) grid_dep_launch();
 
   auto decode = [&](int4 u) {
     Unit x;
@@ -293,6 +297,10 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       load_next();
       load_next();
       load_next();
+      if (p.hold) {
+        grid_dep_wait();
+        grid_dep_launch();
+      }
       for (;;) {
         const int4 u = unit_at(st_nu);
         if (u.x < 0) break;
@@ -584,6 +592,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   tc_fence_before_sync();
   __syncthreads();
   if (warp == kWarpMma) tmem_dealloc(tmem, 512);
+  if (blockIdx.x == 0) grid_dep_wait();
 }
 
 }  // namespace
@@ -596,7 +605,7 @@ bool tc_window_supported(int N, int d, int w, int dtype) {
 
 cudaError_t launch_window_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                              int w, int fwd, float scale, int layout, int h_begin, int h_count, WsHeader* ws,
-                             cudaStream_t stream) {
+                             cudaStream_t stream, Link link, bool hold) {
   if (h_count <= 0) return cudaSuccess;
   CUtensorMap mq, mk, mv, mo;
   if (!make_qkv_tensor_map(&mq, q, B, H, N, d, layout, 128) || !make_qkv_tensor_map(&mk, k, B, H, N, d, layout, 64) ||
@@ -618,6 +627,8 @@ cudaError_t launch_window_tc(const void* q, const void* k, const void* v, void* 
   p.total = (int)total;
   p.status = &ws->status;
   p.ticket = &ws->ticket;  // zeroed with the workspace header by the caller
+  p.beside = link == kBeside;
+  p.hold = hold;
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = device_info(&dev, &sms)) != cudaSuccess) return e;
@@ -627,17 +638,13 @@ cudaError_t launch_window_tc(const void* q, const void* k, const void* v, void* 
   auto launch = [&](auto kern, int smem) -> cudaError_t {
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem);
     if (err != cudaSuccess) return err;
-    kern<<<grid, kThreads, smem, stream>>>(mq, mk, mv, mo, p);
-    return cudaSuccess;
+    return launch_link(link, kern, grid, dim3(kThreads), smem, stream, mq, mk, mv, mo, p);
   };
   if (d == 64)
-    e = fwd > 0 ? launch(window_tc_kernel<64, true>, WinSmem<64>::kBytes) : launch(window_tc_kernel<64, false>, WinSmem<64>::kBytes);
-  else
-    e = fwd > 0 ? launch(window_tc_kernel<128, true>, WinSmem<128>::kBytes)
-                : launch(window_tc_kernel<128, false>, WinSmem<128>::kBytes);
-  if (e != cudaSuccess) return e;
-  note_launch();
-  return cudaGetLastError();
+    return fwd > 0 ? launch(window_tc_kernel<64, true>, WinSmem<64>::kBytes)
+                   : launch(window_tc_kernel<64, false>, WinSmem<64>::kBytes);
+  return fwd > 0 ? launch(window_tc_kernel<128, true>, WinSmem<128>::kBytes)
+                 : launch(window_tc_kernel<128, false>, WinSmem<128>::kBytes);
 }
 
 }  // namespace gf

@@ -973,6 +973,47 @@ def test_hybrid_layer_called_from_two_host_threads():
         assert j["bad"] == [] and j["ws"].last_device_status() == gf.GF_OK
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,H,N,d,w,h0", [
+    (1, 6, 5000, 128, 512, 3),    # few chains, long windows: sums of fewer segments than the readout's
+    (1, 9, 1500, 128, 1, 1),      # hardly any windowed work: as many
+    (40, 4, 300, 128, 64, 1),     # a segment per chain: no totals
+    (2, 6, 3000, 64, 700, 2),
+])
+def test_self_layer_sums_and_readout_cut_differently(B, H, N, d, w, h0):
+    q, k, v = synth.qkv(B, H, N, d, "bf16", seed=81)
+    qd, kd, vd = dev(q, k, v)
+    ws = gf.Workspace.for_problem(B, H, N, d, w, h0)
+    ws.buf.fill_(0xff)  # counters and header are cleared by the call
+    o = gf.hybrid_attn_self(qd, kd, vd, w, h_sparse=h0, ws=ws)
+    again = gf.hybrid_attn_self(qd, kd, vd, w, h_sparse=h0, ws=ws)
+    assert ws.last_device_status() == gf.GF_OK and torch.equal(o, again)
+    b = B - 1
+    ref = oracle.hybrid_attn_self(f64(q[b:]), f64(k[b:]), f64(v[b:]), w, h_sparse=h0)
+    assert_parity(f64(o[b:]), ref, "bf16", "self layer")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("N,w", [(1, 3), (37, 64), (64, 64), (333, 100)])
+def test_what_follows_a_layer_in_its_stream_follows_all_of_its_kernels(dtype, N, w):
+    """Outputs, ring and state read by the next operation of the stream, many calls in a row without a synchronisation."""
+    B, H, d, h0 = 3, 5, 64, 2
+    sets = [dev(*synth.qkv(B, H, N, d, dtype, seed=s)) for s in range(3)]
+    st = gf.DecodeState(B, H, d, w, h0, torch.float32 if dtype == "f32" else torch.bfloat16)
+    got = []
+    for i in range(12):
+        o = gf.hybrid_attn(*sets[i % 3], w, h_sparse=h0, state_out=st)
+        got.append([x.clone() for x in (o, st.k_cache, st.v_cache, st.S, st.z)])
+    torch.cuda.synchronize()
+    n = min(N, w)
+    for i in range(12):
+        assert all(torch.equal(a, b) for a, b in zip(got[i], got[i % 3]))
+        for ring, x in ((got[i][1], sets[i % 3][1]), (got[i][2], sets[i % 3][2])):
+            for j in range(N - n, N):
+                assert torch.equal(ring[:, :, j % w], x[:, :h0, j])
+
+
 # ----------------------------------------------------------------------------- head partition (Algorithm 2)
 @pytest.mark.gpu
 def test_measured_partition_balances_the_two_head_kinds():
