@@ -76,7 +76,7 @@ typedef enum { GF_PHI_ELU1 = 0, GF_PHI_FAVOR_POS = 1 } gf_phi;
 
 /* Process-wide knobs for tests and benchmarks (gformer_set_tuning). */
 typedef enum {
-  GF_TUNE_FORCE_SIMT = 0, /* 1: never take the tensor-core kernels (default 0)              */
+  GF_TUNE_FORCE_SIMT = 0, /* 1: always the fp32-arithmetic kernels, not the tcgen05 ones (default 0) */
   GF_TUNE_LINEAR_SPLIT = 1, /* 128-row chunks per sequence segment of a linear chain: 0 = auto,
                                -1 = never cut a chain (the one-pass form of the kernel)          */
   GF_TUNE_LINEAR_CTAS = 2,  /* gformer_hybrid_attn: CTAs of the persistent linear-attention kernel
@@ -286,7 +286,7 @@ int gformer_hybrid_attn(const void* q, const void* k, const void* v, void* o,
  * heads [0, h_sparse) as gformer_window_attn_self, heads [h_sparse, H) global linear attention,
  *   S = sum_j phi(k_j) v_j^T,  z = sum_j phi(k_j)  over all j,   o_i = phi(q_i)^T S / (phi(q_i) . z)
  * (Sec. II-B, rows normalised as in Algorithm 1).  bf16 storage takes the tensor-core kernels,
- * fp32 storage (or GF_TUNE_FORCE_SIMT) CUDA-core kernels in fp32 arithmetic, as in the causal
+ * fp32 storage (or GF_TUNE_FORCE_SIMT) kernels in fp32 arithmetic, as in the causal
  * layer.  Streams, graph capture and host threads as for gformer_hybrid_attn.  Workspace:
  * gformer_workspace_bytes.
  */

@@ -1,17 +1,21 @@
-// Attention in fp32 arithmetic on the CUDA cores, as register-tiled products: the windowed heads and the causal
-// linear heads of fp32 tensors (and of bf16 ones when the tensor-core kernels are switched off).
+// Attention in fp32 arithmetic: the windowed heads and the causal linear heads of fp32 tensors (and of bf16 ones when the
+// tcgen05 kernels are switched off).
 //
-// Both kernels walk 32-token blocks with 128 threads.  A thread's tile of a product is 4 rows x 4 columns (4 x 2 of a
-// score block, D/8 x 4 of the state).  Rows are i + 8 r of a block, so that the eight row groups of a warp read eight
-// different padded rows of shared memory without bank conflicts; operands are read 16 bytes at a time, along the
-// contracted dimension for A and along the columns for B.  The next block's rows are loaded into registers while one
-// is worked on: loaded when they are needed, a block waited about 5 us for them.
-// What bounds both is shared memory: for these tiles the 16-byte loads take 1.5 to 3 times the cycles of the
-// multiply-adds (ncu at 8 x 12 heads x 2048 tokens, d = 64, w = 128: shared-memory pipe 60-75 % busy, FMA pipe 40-49 %).
-// Larger tiles (64 threads, 4 x 8, 4 x 4 and 8 x 8) need a third fewer loads but leave 8 warps per SM: no faster there
-// (244 us for the layer either way).  Token by token, with a block-wide reduction per 16 tokens and no reuse of K, it took
-// 756 us, and 2 heads of 256 tokens 57 us, now 17.
+// The products run on the tensor cores as mma.sync with tf32 operands, each operand split in two (x = hi + lo, hi rounded to
+// tf32's 11 bits, lo the exact rest, of which at most the last bit is dropped): hi hi + hi lo + lo hi, what is left out is
+// 2^-24 of a product.  The tensor core rounds towards zero when it adds to an accumulator, so no sum runs through it: the 8 products of
+// an instruction (windowed heads: of two) start from zero and are added to the running sum on the CUDA cores, rounded to
+// nearest.  Against 64 bits (2 x 12 heads of 2048 tokens, d = 64, w = 128; relative error, windowed and linear heads) that is
+// 2.0e-7 and 1.1e-7, all sums in the accumulators 1.2e-6 and 1.1e-6, FFMA products 3.1e-7 and 1.5e-7.  (tcgen05.mma, four times
+// as fast, could only add up in its accumulators.)
+// Register-tiled FFMA products, which this replaced, were bound by shared memory (us, before and now): 8 x 12 heads of 2048
+// tokens, d = 64, windowed (w = 128) 296 and 214, linear 240 and 173; d = 128 548 and 469, 843 and 698; the layer with 2
+// windowed heads 246 and 181.  What bounds these is the issue of instructions and their latency: 1600 a warp for a block of 32
+// tokens, a quarter of them splitting operands, at 55 % of the issue slots; tensor pipe 38 %.  Not faster: operands split once
+// and kept as pairs in shared memory (10 to 25 % slower), cvt.rna (8 %), the three products of a split apart (3 %).
 #include <cooperative_groups.h>
+
+#include <atomic>
 
 #include "common.cuh"
 
@@ -19,9 +23,11 @@ namespace gf {
 namespace {
 
 constexpr int kC = 32;    // tokens per block
-constexpr int kNT = 128;  // threads per CTA
+constexpr int kLinThreads = 256;
 constexpr int kW = 64;    // value columns per CTA of the linear heads
-constexpr int kLdP = kC + 4;
+// Row strides in shared memory: the fragments are read 8 bytes (rows g, columns 2 t) or 4 bytes (rows t, columns g) per lane,
+// both without bank conflicts when the stride is 8 mod 32; rows 2 t and 2 t + 1, or rows g and columns t, when it is 4.
+constexpr int kLdV = kW + 8, kLdP = kC + 4;
 
 template <typename T> __device__ __forceinline__ float4 load4(const T* p);
 template <> __device__ __forceinline__ float4 load4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
@@ -38,7 +44,12 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, float4 x) {
   raw.y = *reinterpret_cast<const uint32_t*>(&b);
   *reinterpret_cast<uint2*>(p) = raw;
 }
+__device__ __forceinline__ void store2(float* p, float x, float y) { *reinterpret_cast<float2*>(p) = make_float2(x, y); }
+__device__ __forceinline__ void store2(__nv_bfloat16* p, float x, float y) {
+  *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(x, y);
+}
 __device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float2 lds2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 __device__ __forceinline__ float4 phi4(float4 x) {
   return make_float4(phi_elu1(x.x), phi_elu1(x.y), phi_elu1(x.z), phi_elu1(x.w));
 }
@@ -52,18 +63,66 @@ __device__ __forceinline__ void axpy4(float4& acc, float a, float4 b) {
 __device__ __forceinline__ float dot4(float4 a, float4 b, float acc) {
   return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
 }
+__device__ __forceinline__ bool is_nan(float x) { return x != x; }
+__device__ __forceinline__ bool is_finite(float x) { return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u; }
 
-// (also of infinities of both signs)
-__device__ __forceinline__ bool has_nan(float4 x) {
-  const float s = (x.x + x.y) + (x.z + x.w);
-  return s != s;
+// ------------------------------------------------------------------------------------ products
+struct Split {
+  uint32_t hi, lo;
+};
+__device__ __forceinline__ Split split(float x) {
+  const uint32_t hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+  return {hi, __float_as_uint(x - __uint_as_float(hi))};
+}
+// Lane (g, t) = (lane / 4, lane % 4) of an m16n8k8 product holds A[g | g + 8][t | t + 4], B[t | t + 4][g] and
+// C[g | g + 8][2 t | 2 t + 1].  The order of the contracted index is free as long as A and B agree.
+__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t a0, const uint32_t a1, const uint32_t a2, const uint32_t a3,
+                                         const uint32_t b0, const uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// d += the 8 (or, small: the corrections of the 8) products of an element
+__device__ __forceinline__ void product_small(float (&d)[4], const Split (&a)[4], const Split b0, const Split b1) {
+  mma_tf32(d, a[0].lo, a[1].lo, a[2].lo, a[3].lo, b0.hi, b1.hi);
+  mma_tf32(d, a[0].hi, a[1].hi, a[2].hi, a[3].hi, b0.lo, b1.lo);
+}
+__device__ __forceinline__ void product_big(float (&d)[4], const Split (&a)[4], const Split b0, const Split b1) {
+  mma_tf32(d, a[0].hi, a[1].hi, a[2].hi, a[3].hi, b0.hi, b1.hi);
+}
+// acc += A B over 8 contracted elements, or 16
+__device__ __forceinline__ void product8(float (&acc)[4], const Split (&a)[4], const Split b0, const Split b1) {
+  float d[4] = {0.f, 0.f, 0.f, 0.f};
+  product_small(d, a, b0, b1);
+  product_big(d, a, b0, b1);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) acc[e] += d[e];
+}
+__device__ __forceinline__ void product16(float (&acc)[4], const Split (&a)[2][4], const Split (&b)[2][2]) {
+  float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int x = 0; x < 2; ++x) product_small(d, a[x], b[x][0], b[x][1]);
+#pragma unroll
+  for (int x = 0; x < 2; ++x) product_big(d, a[x], b[x][0], b[x][1]);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) acc[e] += d[e];
+}
+__device__ __forceinline__ void lds_split2(Split& x, Split& y, const float* p) {
+  const float2 v = lds2(p);
+  x = split(v.x);
+  y = split(v.y);
+}
+// A from rows row, row + 8 of a row-major array (a pair of columns per lane)
+__device__ __forceinline__ void rows_a(Split (&a)[4], const float* p, int ld8) {
+  lds_split2(a[0], a[2], p);
+  lds_split2(a[1], a[3], p + ld8);
 }
 
 // A block's rows on their way from global to shared memory: COLS columns of 32 tokens, all loads of a thread in
 // flight at once and issued a block ahead of their use.  Rows past the end are zero.
-template <typename T, int COLS>
+template <typename T, int COLS, int THREADS>
 struct BlockRegs {
-  static constexpr int C4 = COLS / 4, kN = kC * C4 / kNT, kStep = kNT / C4;
+  static constexpr int C4 = COLS / 4, kN = kC * C4 / THREADS, kStep = THREADS / C4;
   float4 x[kN];
   __device__ __forceinline__ void load(const T* p, long long stride, int n0, int n_end, int tid) {
     const T* src = p + (long long)(n0 + tid / C4) * stride + 4 * (tid % C4);
@@ -84,69 +143,41 @@ struct BlockRegs {
   }
 };
 
-// Scores of a 32 x 32 block: rows i + 8 r of A against rows jg + 16 s of B, both [32][D + 4].
-template <int D>
-__device__ __forceinline__ void score_block(const float* A, const float* B, int i, int jg, float (&acc)[4][2]) {
-  constexpr int LD = D + 4;
-#pragma unroll
-  for (int r = 0; r < 4; ++r) acc[r][0] = acc[r][1] = 0.f;
-#pragma unroll 4
-  for (int a = 0; a < D; a += 4) {
-    const float4 b0 = lds4(B + jg * LD + a), b1 = lds4(B + (jg + 16) * LD + a);
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const float4 x = lds4(A + (i + 8 * r) * LD + a);
-      acc[r][0] = dot4(x, b0, acc[r][0]);
-      acc[r][1] = dot4(x, b1, acc[r][1]);
-    }
-  }
-}
-// acc[r][c] += rows i + 8 r of A (K entries each, row stride lda) times B, four columns at col(k, c)
-template <int K, int NG, typename Col>
-__device__ __forceinline__ void product(float4 (&acc)[4][NG], const float* A, int lda, int i, Col col) {
-#pragma unroll 2
-  for (int k = 0; k < K; k += 4) {
-    float4 x[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) x[r] = lds4(A + (i + 8 * r) * lda + k);
-#pragma unroll
-    for (int c = 0; c < NG; ++c) {
-      const float4 b0 = lds4(col(k, c)), b1 = lds4(col(k + 1, c)), b2 = lds4(col(k + 2, c)), b3 = lds4(col(k + 3, c));
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        axpy4(acc[r][c], x[r].x, b0);
-        axpy4(acc[r][c], x[r].y, b1);
-        axpy4(acc[r][c], x[r].z, b2);
-        axpy4(acc[r][c], x[r].w, b3);
-      }
-    }
-  }
-}
-
 // ------------------------------------------------------------------------------------ windowed heads
-// One CTA = 32 query rows of one head; keys and values pass through shared memory 32 at a time; online softmax
-// with the running maximum and sum of a row kept by the four threads that share it.
+// One CTA = 64 query rows of one head, 16 per warp, as two groups of four warps that take every other block of 32 keys and
+// values; online softmax in registers, a row shared by four lanes.  Weights go from the scores' accumulators to the operand
+// of the second product as they are (its contracted index in the accumulators' order).  The groups' sums meet at the end.
+// (One group: 12 heads of 100 tokens, w = 512, 16.4 us against 12.3, 8 of 1000, d = 128, w = 64, 25.0 and 18.5.)
+constexpr int kWinRows = 64, kWinGroup = 128, kWinThreads = 2 * kWinGroup;
 template <int D>
-constexpr int window_smem() { return (2 * kC * (D + 4) + kC * D + kC * kLdP + kC) * 4; }
+constexpr int window_smem() { return (kWinRows * (D + 8) + 2 * kC * (D + 8) + 2 * kC * (D + 4)) * 4; }
 
-// Masked keys have weight 0 in the products above, which is nothing unless their value is infinite or NaN (0 x inf = NaN):
-// the output row of query i once more, by the four threads that share it, over the keys it sees and no others.  m, l: its
-// final maximum and sum.
+// Masked keys have weight 0 in the products above, which is nothing unless their value is infinite or NaN (0 x inf = NaN), and
+// an infinite operand's rest is NaN: the output row of query i once more, by the four lanes that share it, over the keys it
+// sees and no others.
 template <typename T, int D>
-__device__ __forceinline__ void window_row(const T* q, const T* k, const T* v, T* o, int i, int j_begin, int j_end, float scale,
-                                        long long stride, int part, unsigned int quad, float m, float l) {
+__device__ __noinline__ void window_row(const T* q, const T* k, const T* v, T* o, int i, int j_begin, int j_end, float scale,
+                                        long long stride, int part, unsigned int quad) {
+  auto score = [&](int j) {
+    float s = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < D / 16; ++c)
+      s = dot4(load4<T>(q + i * stride + 4 * (part + 4 * c)), load4<T>(k + j * stride + 4 * (part + 4 * c)), s);
+    s += __shfl_xor_sync(quad, s, 1);
+    s += __shfl_xor_sync(quad, s, 2);
+    return s * scale;
+  };
+  float m = -INFINITY, l = 0.f;
+#pragma unroll 1
+  for (int j = j_begin; j < j_end; ++j) m = fmaxf(m, score(j));
+  const float ref = m == -INFINITY ? 0.f : m;
   float4 acc[D / 16];
 #pragma unroll
   for (int c = 0; c < D / 16; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
   for (int j = j_begin; j < j_end; ++j) {
-    float s = 0.f;
-#pragma unroll
-    for (int c = 0; c < D / 16; ++c)
-      s = dot4(load4<T>(q + i * stride + 4 * (part + 4 * c)), load4<T>(k + j * stride + 4 * (part + 4 * c)), s);
-    s += __shfl_xor_sync(quad, s, 1);
-    s += __shfl_xor_sync(quad, s, 2);
-    const float p = expf(s * scale - m);
+    const float p = expf(score(j) - ref);
+    l += p;
 #pragma unroll
     for (int c = 0; c < D / 16; ++c) axpy4(acc[c], p, load4<T>(v + j * stride + 4 * (part + 4 * c)));
   }
@@ -155,121 +186,188 @@ __device__ __forceinline__ void window_row(const T* q, const T* k, const T* v, T
     store4(o + i * stride + 4 * (part + 4 * c), make_float4(acc[c].x / l, acc[c].y / l, acc[c].z / l, acc[c].w / l));
 }
 
+template <typename T>
+struct WindowArgs {
+  const T *q, *k, *v;
+  T* o;
+  int N, w, fwd;  // fwd: keys after the query that it may see (0: the causal window; w - 1: the two-sided one)
+  float scale;
+  Strides st;
+  int h_begin;
+};
+
 template <typename T, int D>
-__global__ void __launch_bounds__(kNT, D == 64 ? 5 : 3)  // (else the rare path at the end takes registers from the rest)
-window_tiled_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* __restrict__ o,
-                    int N, int w, int fwd, float scale, Strides st, int h_begin) {
-  // fwd: keys after the query that it may see (0: the causal window; w - 1: the two-sided one)
-  grid_dep_launch();
-  constexpr int LD = D + 4, NC = D / 64;  // NC: groups of four output columns per thread, 64 apart
-  extern __shared__ __align__(16) float sm[];
-  float *Qs = sm, *Ks = Qs + kC * LD, *Vs = Ks + kC * LD, *Ps = Vs + kC * D, *As = Ps + kC * kLdP;
+__device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, int head, int b, float* sm) {
+  constexpr int LD = D + 8, LDV = D + 4, NT = D / 8;
+  const int group = threadIdx.x / kWinGroup, tid = threadIdx.x % kWinGroup, lane = tid & 31, warp = tid >> 5;
+  float *Qs = sm, *Ks = Qs + kWinRows * LD + group * kC * (LD + LDV), *Vs = Ks + kC * LD;
+  const int N = p.N;
+  const long long base = (long long)b * p.st.b + (long long)(p.h_begin + head) * p.st.h;
+  const int i0 = tile * kWinRows;
+  const int g = lane >> 2, t = lane & 3;
+  const int iw = i0 + 16 * warp;  // the warp's first row
+  auto sync_group = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kWinGroup) : "memory"); };
 
-  const long long base = (long long)blockIdx.z * st.b + (long long)(h_begin + blockIdx.y) * st.h;
-  const int i0 = blockIdx.x * kC, tid = threadIdx.x, lane = tid & 31;
-  const int i = lane & 7, cg = (tid >> 5) * 4 + (lane >> 3);  // row group, column group of the products
-  const int t = tid >> 2, part = tid & 3;                     // row and quarter of it in the softmax
-
-  const int jlo = max(i0 - w + 1, 0), jhi = min(i0 + kC - 1 + fwd, N - 1);
-  BlockRegs<T, D> rk, rv;
-  rk.load(q + base, st.n, i0, N, tid);
-  rk.store(Qs, LD, tid);
-  rk.load(k + base, st.n, jlo, N, tid);
-  rv.load(v + base, st.n, jlo, N, tid);
-  float4 acc[4][NC];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < NC; ++c) acc[r][c] = make_float4(0.f, 0.f, 0.f, 0.f);
-  float m = -INFINITY, l = 0.f;
-
-  for (int j0 = jlo; j0 <= jhi; j0 += kC) {
-    rk.store(Ks, LD, tid);
-    rv.store(Vs, D, tid);
-    __syncthreads();
-    if (j0 + kC <= jhi) {
-      rk.load(k + base, st.n, j0 + kC, N, tid);
-      rv.load(v + base, st.n, j0 + kC, N, tid);
-    }
-    {
-      float s[4][2];
-      score_block<D>(Qs, Ks, i, cg, s);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        Ps[(i + 8 * r) * kLdP + cg] = s[r][0];
-        Ps[(i + 8 * r) * kLdP + cg + 16] = s[r][1];
-      }
-    }
-    __syncthreads();
-    {
-      float* row = Ps + t * kLdP + part * 8;
-      const float4 x0 = lds4(row), x1 = lds4(row + 4);
-      float s[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-      const int lo = i0 + t - w - (j0 + part * 8), hi = min(i0 + t + fwd, N - 1) - (j0 + part * 8);  // lo < e <= hi
-      float mx = -INFINITY;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        s[e] = (e > lo && e <= hi) ? s[e] * scale : -INFINITY;
-        mx = fmaxf(mx, s[e]);
-      }
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-      const float m_new = fmaxf(m, mx);
-      const float ref = (m_new == -INFINITY) ? 0.f : m_new;  // a row that has seen no key yet
-      const float corr = expf(m - ref);
-      float sum = 0.f;
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        s[e] = expf(s[e] - ref);
-        sum += s[e];
-      }
-      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-      l = l * corr + sum;
-      m = m_new;
-      *reinterpret_cast<float4*>(row) = make_float4(s[0], s[1], s[2], s[3]);
-      *reinterpret_cast<float4*>(row + 4) = make_float4(s[4], s[5], s[6], s[7]);
-      if (part == 0) As[t] = corr;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const float corr = As[i + 8 * r];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        acc[r][c].x *= corr;
-        acc[r][c].y *= corr;
-        acc[r][c].z *= corr;
-        acc[r][c].w *= corr;
-      }
-    }
-    product<kC, NC>(acc, Ps, kLdP, i, [&](int j, int c) { return Vs + j * D + c * 64 + 4 * cg; });
-    __syncthreads();
-  }
-  if (part == 0) {
-    As[t] = 1.f / l;
-    Ps[t] = 0.f;  // 1: the row has a NaN
+  const int jlo = max(i0 - p.w + 1, 0) + kC * group, jhi = min(min(i0 + kWinRows, N) - 1 + p.fwd, N - 1);
+  BlockRegs<T, D, kWinGroup> rk, rv;
+  {
+    BlockRegs<T, D, kWinGroup> rq;
+    rq.load(p.q + base, p.st.n, i0 + kC * group, N, tid);
+    rk.load(p.k + base, p.st.n, jlo, N, tid);
+    rv.load(p.v + base, p.st.n, jlo, N, tid);
+    rq.store(Qs + kC * group * LD, LD, tid);
   }
   __syncthreads();
-  bool any = false;
+  float acc[NT][4];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int row = i + 8 * r;
-    if (i0 + row >= N) continue;
-    const float inv = As[row];
+  for (int n = 0; n < NT; ++n)
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      if (has_nan(acc[r][c])) {
-        Ps[row] = 1.f;
-        any = true;
+    for (int e = 0; e < 4; ++e) acc[n][e] = 0.f;
+  float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};  // rows iw + g, iw + g + 8
+
+  for (int j0 = jlo; j0 <= jhi; j0 += 2 * kC) {
+    rk.store(Ks, LD, tid);
+    rv.store(Vs, LDV, tid);
+    sync_group();
+    if (j0 + 2 * kC <= jhi) {
+      rk.load(p.k + base, p.st.n, j0 + 2 * kC, N, tid);
+      rv.load(p.v + base, p.st.n, j0 + 2 * kC, N, tid);
+    }
+    // keys that a row of the warp can see
+    if (iw < N && j0 <= iw + 15 + p.fwd && j0 + kC - 1 >= iw - p.w + 1) {
+      float s[4][4];
+#pragma unroll
+      for (int n = 0; n < 4; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[n][e] = 0.f;
+#pragma unroll 1
+      for (int kk = 0; kk < NT; kk += 2) {
+        Split a[2][4];
+        rows_a(a[0], Qs + (16 * warp + g) * LD + 8 * kk + 2 * t, 8 * LD);
+        rows_a(a[1], Qs + (16 * warp + g) * LD + 8 * kk + 8 + 2 * t, 8 * LD);
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+          Split k2[2][2];
+          lds_split2(k2[0][0], k2[0][1], Ks + (8 * n + g) * LD + 8 * kk + 2 * t);
+          lds_split2(k2[1][0], k2[1][1], Ks + (8 * n + g) * LD + 8 * kk + 8 + 2 * t);
+          product16(s[n], a, k2);
+        }
       }
-      store4(o + base + (long long)(i0 + row) * st.n + c * 64 + 4 * cg,
-             make_float4(acc[r][c].x * inv, acc[r][c].y * inv, acc[r][c].z * inv, acc[r][c].w * inv));
+      // some row does not see some key of the block
+      const bool edge = j0 <= iw + 15 - p.w || j0 + kC - 1 > min(iw + p.fwd, N - 1);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const int i = iw + g + 8 * r;
+        if (edge) {
+          const int lo = i - p.w - j0 - 2 * t, hi = min(i + p.fwd, N - 1) - j0 - 2 * t;  // lo < 8 n + e <= hi
+#pragma unroll
+          for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+              if (!(8 * n + e > lo && 8 * n + e <= hi)) s[n][2 * r + e] = -INFINITY;
+        }
+        float mx = -INFINITY;
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            float& x = s[n][2 * r + e];
+            x *= p.scale;
+            mx = fmaxf(mx, x);
+          }
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        const float m_new = fmaxf(m[r], mx);
+        const float ref = (m_new == -INFINITY) ? 0.f : m_new;  // a row that has seen no key yet
+        const float corr = expf(m[r] - ref);
+        float sum = 0.f;
+#pragma unroll
+        for (int n = 0; n < 4; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            float& x = s[n][2 * r + e];
+            x = expf(x - ref);
+            sum += x;
+          }
+        l[r] = l[r] * corr + sum;  // (of this lane's keys)
+        m[r] = m_new;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          acc[n][2 * r] *= corr;
+          acc[n][2 * r + 1] *= corr;
+        }
+      }
+#pragma unroll
+      for (int kk = 0; kk < 4; kk += 2) {
+        const Split a[2][4] = {{split(s[kk][0]), split(s[kk][2]), split(s[kk][1]), split(s[kk][3])},
+                               {split(s[kk + 1][0]), split(s[kk + 1][2]), split(s[kk + 1][1]), split(s[kk + 1][3])}};
+        const float* vp = Vs + (8 * kk + 2 * t) * LDV + g;
+#pragma unroll
+        for (int n = 0; n < NT; ++n) {
+          const Split v2[2][2] = {{split(vp[8 * n]), split(vp[8 * n + LDV])},
+                                  {split(vp[8 * n + 8 * LDV]), split(vp[8 * n + 9 * LDV])}};
+          product16(acc[n], a, v2);
+        }
+      }
+    }
+    sync_group();
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    l[r] += __shfl_xor_sync(0xffffffffu, l[r], 1);
+    l[r] += __shfl_xor_sync(0xffffffffu, l[r], 2);
+  }
+  // the second group's sums, element by element of a lane, through the room of the keys and values
+  static_assert((NT * 4 + 4) * kWinGroup <= 2 * kC * (LD + LDV), "room of the sums");
+  float* part = Qs + kWinRows * LD + tid;
+  __syncthreads();
+  if (group == 1) {
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) part[(4 * n + e) * kWinGroup] = acc[n][e];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      part[(4 * NT + r) * kWinGroup] = m[r];
+      part[(4 * NT + 2 + r) * kWinGroup] = l[r];
     }
   }
-  if (__syncthreads_or(any) && Ps[t] != 0.f)
-    window_row<T, D>(q + base, k + base, v + base, o + base, i0 + t, max(i0 + t - w + 1, 0), min(i0 + t + fwd, N - 1) + 1, scale,
-                     st.n, part, 0xfu << (lane & 28), m, l);
+  __syncthreads();
+  if (group == 1) return;
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int i = iw + g + 8 * r;
+    const float m1 = part[(4 * NT + r) * kWinGroup], mx = fmaxf(m[r], m1), ref = mx == -INFINITY ? 0.f : mx;
+    const float f0 = expf(m[r] - ref), f1 = expf(m1 - ref);
+    const float inv = 1.f / (l[r] * f0 + part[(4 * NT + 2 + r) * kWinGroup] * f1);
+#pragma unroll
+    for (int n = 0; n < NT; ++n)
+#pragma unroll
+      for (int e = 0; e < 2; ++e)
+        acc[n][2 * r + e] = acc[n][2 * r + e] * f0 + part[(4 * n + 2 * r + e) * kWinGroup] * f1;
+    bool bad = false;
+#pragma unroll
+    for (int n = 0; n < NT; ++n) {
+      bad |= is_nan(acc[n][2 * r]) || is_nan(acc[n][2 * r + 1]);
+      if (i < N)
+        store2(p.o + base + (long long)i * p.st.n + 8 * n + 2 * t, acc[n][2 * r] * inv, acc[n][2 * r + 1] * inv);
+    }
+    const unsigned int quad = 0xfu << (lane & 28);
+    if ((__ballot_sync(0xffffffffu, bad) & quad) != 0u && i < N) {
+      __syncwarp(quad);  // (the row's stores above come first)
+      window_row<T, D>(p.q + base, p.k + base, p.v + base, p.o + base, i, max(i - p.w + 1, 0), min(i + p.fwd, N - 1) + 1, p.scale,
+                       p.st.n, t, quad);
+    }
+    __syncwarp();
+  }
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(kWinThreads, D == 64 ? 2 : 1)
+window_tiled_kernel(const WindowArgs<T> p) {
+  extern __shared__ __align__(16) float sm[];
+  grid_dep_launch();
+  window_tile<T, D>(p, blockIdx.x, blockIdx.y, blockIdx.z, sm);
   if (blockIdx.x + blockIdx.y + blockIdx.z == 0) grid_dep_wait();
 }
 
@@ -277,13 +375,17 @@ window_tiled_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
 // Algorithm 1 regrouped in blocks of 32 tokens (exactly equal by associativity): with S, z the sums before a block,
 //   P = phi(Q) phi(K)^T masked to j <= i,   O = (P V + phi(Q) S) / (rowsum(P) + phi(Q) z),
 //   S += phi(K)^T V,   z += colsum(phi(K)).
-// A CTA owns 64 value columns of a chain; S lives in its registers (a thread: D/8 features x 4 columns) with a copy
-// in shared memory for the readout.
+// A CTA owns 64 value columns of a chain, a warp 16 of them and half of the features.  S lives in the warps' registers as the
+// accumulators of S^T += V^T phi(K) (a lane: columns g, g + 8, features 8 n + 2 t, + 1 of its half), which are at the same
+// time its operand in phi(Q) S; the two halves of O meet in shared memory.  (Four warps with all features each need 168
+// registers a lane, three CTAs per SM, and take 5.2 us for a block when alone on one, eight 3.6.)
 //
 // With few chains a chain is cut into G segments, so that every SM has work.  Up to kMaxCluster of them are a cluster of
-// CTAs in one launch (kCluster): each sums its own segment, then adds up the sums of those before it from their shared
-// memory, then walks.  Where a chain has two CTAs per segment (D = 128) and brings a state, both are in the cluster: both read
-// the caller's z, and one of them overwrites it, which has to wait until the other has started.  Longer chains in smaller numbers take three launches, with segments of a little more than D tokens:
+// CTAs in one launch (kCluster): each sums its own segment; every CTA then turns its share of the elements, read from all
+// CTAs' shared memory at once, into running sums and puts those back; then they walk.  Where a chain has two CTAs per segment
+// (D = 128) and brings a state, both are in the cluster: both read the caller's z, and one of them overwrites it, which has
+// to wait until the other has started.  Longer chains in smaller numbers take three launches, with segments of a little
+// more than D tokens:
 //   contribution   the sums of every segment but the last, each alone
 //   prefix         running sums over the segments of a chain
 //   walk           the segments' outputs, each from its own starting state
@@ -292,91 +394,186 @@ window_tiled_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
 // reads only rows and columns that itself will write.
 constexpr int kMaxCluster = 8;
 template <int D> struct LinT {
-  static constexpr int LD = D + 4;
+  static constexpr int LD = D + 8;
   static constexpr int ZROWS = D / 64;  // rows z takes behind S
   // shortest segment: D + ZROWS rows, also when the last segment's last block is a single token
   static constexpr int kMinSeg = D + 32 * ZROWS;
-  static constexpr int kSmem = (2 * kC * LD + kC * kW + D * kW + kC * kLdP + D + kC) * 4;
-  static constexpr int kSmemSum = (kC * LD + kC * kW) * 4;
+  static constexpr int kSmem = (2 * kC * LD + kC * kLdV + kC * kLdP + D * kW + kC * kW + D + 2 * kC) * 4;
+  static constexpr int kSmemSum = (kC * LD + kC * kLdV) * 4;
 };
 struct Segs {  // tokens [begin(g), begin(g + 1)) of segment g, whole blocks but for the last
   int N, G, base, rem;  // blocks per segment: base, one more for the first rem
   __host__ __device__ int begin(int g) const { return g >= G ? N : kC * (g * base + (g < rem ? g : rem)); }
 };
 
-// The 16-byte column groups of row a of the shared copy of S are swizzled, so that the eight feature groups of a warp
-// store without bank conflicts.
-__device__ __forceinline__ int s_off(int a, int col) { return a * kW + (col ^ (a & 28)); }
-
-// S += phi(K)^T V: features 4 ag .. 4 ag + 3 of every 32, columns 4 cg .. 4 cg + 3
-template <int D>
-__device__ __forceinline__ void add_outer(const float* Ks, const float* Vs, int ag, int cg, float4 (&S)[D / 8]) {
-#pragma unroll 2
-  for (int j = 0; j < kC; ++j) {
-    const float4 vv = lds4(Vs + j * kW + 4 * cg);
+// The lane's share of S: S[n][0 | 1] column g, S[n][2 | 3] column g + 8 of the warp's 16; features 8 n + 2 t, + 1 of its half.
+template <int D> using State = float[D / 16][4];
+struct Lane {
+  int g, t, c0, half;  // c0: the warp's first column
+};
+__device__ __forceinline__ Lane lane_of() {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  return {lane >> 2, lane & 3, 16 * (warp & 3), warp >> 2};
+}
+// f(feature, column of the CTA's 64, element)
+template <int D, typename F>
+__device__ __forceinline__ void for_state(State<D>& S, F f) {
+  const Lane l = lane_of();
 #pragma unroll
-    for (int e = 0; e < D / 32; ++e) {
-      const float4 kk = lds4(Ks + j * (D + 4) + 32 * e + 4 * ag);
-      axpy4(S[4 * e + 0], kk.x, vv);
-      axpy4(S[4 * e + 1], kk.y, vv);
-      axpy4(S[4 * e + 2], kk.z, vv);
-      axpy4(S[4 * e + 3], kk.w, vv);
+  for (int n = 0; n < D / 16; ++n)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) f(l.half * (D / 2) + 8 * n + 2 * l.t + (e & 1), l.c0 + l.g + 8 * (e >> 1), S[n][e]);
+}
+// kSane: values that are not finite count as 0
+template <bool kSane>
+__device__ __forceinline__ Split split_value(float v) { return split(kSane && !is_finite(v) ? 0.f : v); }
+
+// S += phi(K)^T V
+template <int D, bool kSane>
+__device__ __forceinline__ void add_outer(const float* Ks, const float* Vs, State<D>& S) {
+  constexpr int LD = LinT<D>::LD;
+  const Lane l = lane_of();
+#pragma unroll 2
+  for (int kk = 0; kk < kC / 8; ++kk) {
+    const float *v = Vs + (8 * kk + l.t) * kLdV + l.c0 + l.g, *k = Ks + (8 * kk + l.t) * LD + l.half * (D / 2) + l.g;
+    const Split a[4] = {split_value<kSane>(v[0]), split_value<kSane>(v[8]), split_value<kSane>(v[4 * kLdV]),
+                        split_value<kSane>(v[4 * kLdV + 8])};
+#pragma unroll
+    for (int n = 0; n < D / 16; ++n) product8(S[n], a, split(k[8 * n]), split(k[8 * n + 4 * LD]));
+  }
+}
+// This half's part of phi(Q) S + P V (its features; half of the keys): rows 16 m + g | + 8, columns 8 n + 2 t | + 1 of the warp's
+template <int D, bool kSane>
+__device__ __forceinline__ void readout(const float* Qs, const float* Vs, const float* Ps, const State<D>& S, float (&acc)[2][2][4]) {
+  constexpr int LD = LinT<D>::LD;
+  const Lane l = lane_of();
+#pragma unroll
+  for (int m = 0; m < 2; ++m)
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.f;
+#pragma unroll
+  for (int kk = 0; kk < D / 16; ++kk) {
+    const Split b[4] = {split(S[kk][0]), split(S[kk][1]), split(S[kk][2]), split(S[kk][3])};
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      Split a[4];
+      rows_a(a, Qs + (16 * m + l.g) * LD + l.half * (D / 2) + 8 * kk + 2 * l.t, 8 * LD);
+      product8(acc[m][0], a, b[0], b[1]);
+      product8(acc[m][1], a, b[2], b[3]);
+    }
+  }
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const int key = 8 * (2 * l.half + x) + l.t;
+    const float* v = Vs + key * kLdV + l.c0 + l.g;
+    const Split b[4] = {split_value<kSane>(v[0]), split_value<kSane>(v[4 * kLdV]), split_value<kSane>(v[8]),
+                        split_value<kSane>(v[4 * kLdV + 8])};
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      if (m == 0 && l.half == 1) continue;  // masked
+      const float* p = Ps + (16 * m + l.g) * kLdP + key;
+      const Split a[4] = {split(p[0]), split(p[8 * kLdP]), split(p[4]), split(p[8 * kLdP + 4])};
+      product8(acc[m][0], a, b[0], b[1]);
+      product8(acc[m][1], a, b[2], b[3]);
     }
   }
 }
-// f(feature, element) for the thread's 4-column pieces of S
-template <int D, typename F>
-__device__ __forceinline__ void for_state(int ag, float4 (&S)[D / 8], F f) {
+// The six tiles of P that are not all masked, 16 rows x 8 keys each, by six warps; phi(Q) z by the other two.
+template <int D>
+__device__ __forceinline__ void score_block(const float* Qs, const float* Ks, const float* zs, float* Ps, float* qz_s) {
+  constexpr int LD = LinT<D>::LD;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, warp = threadIdx.x >> 5;
+  if (warp < 6) {
+    const int m = warp < 2 ? 0 : 1, n = warp < 2 ? warp : warp - 2;
+    float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};  // (two sums: half the chain)
+#pragma unroll 4
+    for (int kk = 0; kk < D / 8; ++kk) {
+      Split a[4], b0, b1;
+      lds_split2(b0, b1, Ks + (8 * n + g) * LD + 8 * kk + 2 * t);
+      rows_a(a, Qs + (16 * m + g) * LD + 8 * kk + 2 * t, 8 * LD);
+      product8(s[kk & 1], a, b0, b1);
+    }
 #pragma unroll
-  for (int e = 0; e < D / 32; ++e)
-#pragma unroll
-    for (int x = 0; x < 4; ++x) f(32 * e + 4 * ag + x, S[4 * e + x]);
+    for (int r = 0; r < 2; ++r) {
+      const int row = 16 * m + g + 8 * r, key = 8 * n + 2 * t;
+      store2(Ps + row * kLdP + key, key <= row ? s[0][2 * r] + s[1][2 * r] : 0.f,
+             key + 1 <= row ? s[0][2 * r + 1] + s[1][2 * r + 1] : 0.f);
+    }
+  } else {
+    const int row = (threadIdx.x - 192) >> 1, part = threadIdx.x & 1;
+    float d[2] = {0.f, 0.f};
+#pragma unroll 4
+    for (int a = 0; a < D; a += 8)
+      d[(a >> 3) & 1] = dot4(lds4(Qs + row * LD + a + 4 * part), lds4(zs + a + 4 * part), d[(a >> 3) & 1]);
+    float q = d[0] + d[1];
+    q += __shfl_xor_sync(0xffffffffu, q, 1);
+    if (part == 0) qz_s[row] = q;
+  }
 }
 template <int D>
 __device__ __forceinline__ float column_sum(const float* col) {
   float s[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int j = 0; j < kC; ++j) s[j & 3] += col[j * (D + 4)];
+#pragma unroll 8
+  for (int j = 0; j < kC; ++j) s[j & 3] += (col[j * LinT<D>::LD]);
   return (s[0] + s[1]) + (s[2] + s[3]);
 }
 
-// Adds tokens [n_begin, n_end) to S and z (thread tid < D: feature tid).
+// Adds tokens [n_begin, n_end) to S = 0 and z = 0 (thread tid < D: feature tid).
 template <typename T, int D>
 __device__ __forceinline__ void sum_segment(const T* k, const T* v, long long stride, int n_begin, int n_end, float* Ks,
-                                            float* Vs, int tid, int ag, int cg, float4 (&S)[D / 8], float& z) {
-  BlockRegs<T, D> rk;
-  BlockRegs<T, kW> rv;
+                                            float* Vs, int tid, State<D>& S, float& z) {
+  BlockRegs<T, D, kLinThreads> rk;
+  BlockRegs<T, kW, kLinThreads> rv;
   rk.load(k, stride, n_begin, n_end, tid);
   rv.load(v, stride, n_begin, n_end, tid);
   for (int n0 = n_begin; n0 < n_end; n0 += kC) {
-    rk.store_phi(Ks, D + 4, n0, n_end, tid);
-    rv.store(Vs, kW, tid);
+    rk.store_phi(Ks, LinT<D>::LD, n0, n_end, tid);
+    rv.store(Vs, kLdV, tid);
     __syncthreads();
     rk.load(k, stride, n0 + kC, n_end, tid);
     rv.load(v, stride, n0 + kC, n_end, tid);
-    add_outer<D>(Ks, Vs, ag, cg, S);
+    add_outer<D, false>(Ks, Vs, S);
     if (tid < D) z += column_sum<D>(Ks + tid);
     __syncthreads();
+  }
+  // (an infinite operand's rest is NaN)
+  bool bad = false;
+  for_state<D>(S, [&](int, int, float& x) { bad |= is_nan(x); });
+  if (bad) {
+    const Lane l = lane_of();
+    for (int n = 0; n < D / 16; ++n)
+      for (int e = 0; e < 4; ++e) {
+        const int a = l.half * (D / 2) + 8 * n + 2 * l.t + (e & 1), c = l.c0 + l.g + 8 * (e >> 1);
+        float x = 0.f;
+        for (int j = n_begin; j < n_end; ++j) x = fmaf(phi_elu1(to_f32(k[j * stride + a])), to_f32(v[j * stride + c]), x);
+#pragma unroll
+        for (int n1 = 0; n1 < D / 16; ++n1)
+#pragma unroll
+          for (int e1 = 0; e1 < 4; ++e1)
+            if (n1 == n && e1 == e && is_nan(S[n1][e1])) S[n1][e1] = x;
+      }
   }
 }
 
 template <int D>
-__global__ void __launch_bounds__(kNT)
+__global__ void __launch_bounds__(kLinThreads, 2)
 linear_contribution_kernel(const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o, Segs sg,
                            Strides st, int h_begin) {
   extern __shared__ __align__(16) float sm[];
   grid_dep_launch();
-  float *Ks = sm, *Vs = Ks + kC * (D + 4);
+  float *Ks = sm, *Vs = Ks + kC * LinT<D>::LD;
   const int g = blockIdx.x / (D / kW), col0 = (blockIdx.x % (D / kW)) * kW;
   const long long base = (long long)blockIdx.z * st.b + (long long)(h_begin + blockIdx.y) * st.h;
-  const int tid = threadIdx.x, lane = tid & 31, ag = lane & 7, cg = (tid >> 5) * 4 + (lane >> 3);
-  float4 S[D / 8];
-  for_state<D>(ag, S, [](int, float4& x) { x = make_float4(0.f, 0.f, 0.f, 0.f); });
+  const int tid = threadIdx.x;
+  State<D> S;
+  for_state<D>(S, [](int, int, float& x) { x = 0.f; });
   float z = 0.f;
   const int n_end = sg.begin(g + 1);
-  sum_segment<float, D>(k + base, v + base + col0, st.n, sg.begin(g), n_end, Ks, Vs, tid, ag, cg, S, z);
+  sum_segment<float, D>(k + base, v + base + col0, st.n, sg.begin(g), n_end, Ks, Vs, tid, S, z);
   float* slot = o + base + (long long)n_end * st.n + col0;  // the state before segment g + 1, once summed
-  for_state<D>(ag, S, [&](int a, float4& x) { store4(slot + (long long)a * st.n + 4 * cg, x); });
+  for_state<D>(S, [&](int a, int c, float& x) { slot[(long long)a * st.n + c] = x; });
   if (tid < D) slot[(long long)(D + tid / kW) * st.n + tid % kW] = z;
   if (blockIdx.x + blockIdx.y + blockIdx.z == 0) grid_dep_wait();
 }
@@ -416,154 +613,247 @@ __global__ void linear_prefix_kernel(float* __restrict__ o, Segs sg, Strides st,
   }
 }
 
+// A block in which a sum came out NaN: a masked weight is 0, which is nothing unless the value is infinite or NaN (0 x inf
+// = NaN), and an infinite operand's rest is NaN.  The same products with such values left out (so that what does not see them
+// keeps its bits), and the elements that see one of them, or are NaN even so, once more by plain multiply-adds.
+template <int D>
+__device__ __noinline__ void mend_block(const float* Qs, const float* Ks, const float* Vs, const float* Ps, float* Ss, float* Os,
+                                        State<D>& S, float (&acc)[2][2][4], bool more) {
+  constexpr int LD = LinT<D>::LD;
+  const Lane l = lane_of();
+  for_state<D>(S, [&](int a, int c, float& x) { Ss[a * kW + c] = x; });
+  readout<D, true>(Qs, Vs, Ps, S, acc);
+  if (l.half == 1)
+    for (int i = 0; i < 16; ++i) Os[i * 128 + (threadIdx.x & 127)] = acc[i >> 3][(i >> 2) & 1][i & 3];
+  __syncthreads();
+  if (l.half == 0)
+    for (int i = 0; i < 16; ++i) {
+      const int m = i >> 3, n = (i >> 2) & 1, e = i & 3;
+      acc[m][n][e] += Os[i * 128 + threadIdx.x];
+      const int row = 16 * m + l.g + 8 * (e >> 1), c = l.c0 + 8 * n + 2 * l.t + (e & 1);
+      bool bad = is_nan(acc[m][n][e]);
+      for (int j = 0; j <= row; ++j) bad |= !is_finite(Vs[j * kLdV + c]);
+      if (!bad) continue;
+      float x = 0.f;
+      for (int a = 0; a < D; ++a) x = fmaf(Qs[row * LD + a], Ss[a * kW + c], x);
+      for (int j = 0; j <= row; ++j) {
+        float p = Ps[row * kLdP + j];
+        if (is_nan(p)) {
+          p = 0.f;
+          for (int a = 0; a < D; ++a) p = fmaf(Qs[row * LD + a], Ks[j * LD + a], p);
+        }
+        x = fmaf(p, Vs[j * kLdV + c], x);
+      }
+      acc[m][n][e] = x;
+    }
+  if (!more) return;
+  add_outer<D, true>(Ks, Vs, S);
+  for (int n = 0; n < D / 16; ++n)
+    for (int e = 0; e < 4; ++e) {
+      const int a = l.half * (D / 2) + 8 * n + 2 * l.t + (e & 1), c = l.c0 + l.g + 8 * (e >> 1);
+      bool bad = is_nan(S[n][e]);
+      for (int j = 0; j < kC; ++j) bad |= !is_finite(Vs[j * kLdV + c]);
+      if (!bad) continue;
+      float x = Ss[a * kW + c];
+      for (int j = 0; j < kC; ++j) x = fmaf(Ks[j * LD + a], Vs[j * kLdV + c], x);
+      S[n][e] = x;
+    }
+}
+
 // Without cuts (G == 1) the state before token 0 comes from S_io; with cuts from the segment's slot (segment 0 has
 // one only when there is an initial state), or, kCluster, from S_io and the cluster's CTAs before this one.  A chain that
 // brings a state and has several slices is one cluster (G x D / kW CTAs), also when it is not cut.
-template <typename T, int D, bool kCluster>
-__global__ void __launch_bounds__(kNT)
-linear_walk_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, T* o, Segs sg, Strides st,
-                   int h_begin, int h_count, float* S_io, float* z_io, int zero_init, int after) {
-  constexpr int LD = LinT<D>::LD;
-  if (after) grid_dep_wait();  // the segments' starting states
-  grid_dep_launch();
-  extern __shared__ __align__(16) float sm[];
-  float *Qs = sm, *Ks = Qs + kC * LD, *Vs = Ks + kC * LD, *Ss = Vs + kC * kW, *Ps = Ss + D * kW, *zs = Ps + kC * kLdP,
-        *inv_s = zs + D;
-  // (a cluster's CTAs are neighbours in x: the segments of one slice, then those of the next)
-  const int g = kCluster ? blockIdx.x % sg.G : blockIdx.x / (D / kW);
-  const int col0 = (kCluster ? blockIdx.x / sg.G : blockIdx.x % (D / kW)) * kW;
-  const long long base = (long long)blockIdx.z * st.b + (long long)(h_begin + blockIdx.y) * st.h;
-  const long long sidx = (long long)blockIdx.z * h_count + blockIdx.y;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int i = lane & 7, cg = (tid >> 5) * 4 + (lane >> 3);
-  const int n_begin = sg.begin(g), n_end = sg.begin(g + 1);
+template <typename T>
+struct WalkArgs {
+  const T *q, *k, *v;
+  T* o;
+  Segs sg;
+  Strides st;
+  int h_begin, h_count;
+  float *S_io, *z_io;
+  int zero_init;
+};
 
-  float4 S[D / 8];
+template <typename T, int D, bool kCluster>
+__device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int head, int b, float* sm) {
+  constexpr int LD = LinT<D>::LD;
+  float *Qs = sm, *Ks = Qs + kC * LD, *Vs = Ks + kC * LD, *Ps = Vs + kC * kLdV, *Ss = Ps + kC * kLdP,
+        *Os = Ss + D * kW, *zs = Os + kC * kW, *inv_s = zs + D, *qz_s = inv_s + kC;
+  const Segs& sg = p.sg;
+  // (a cluster's CTAs are neighbours in x: the segments of one slice, then those of the next)
+  const int g = kCluster ? part % sg.G : part / (D / kW);
+  const int col0 = (kCluster ? part / sg.G : part % (D / kW)) * kW;
+  const long long base = (long long)b * p.st.b + (long long)(p.h_begin + head) * p.st.h;
+  const long long sidx = (long long)b * p.h_count + head;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int n_begin = sg.begin(g), n_end = sg.begin(g + 1);
+  const T *q = p.q + base, *k = p.k + base, *v = p.v + base + col0;
+  T* o = p.o + base + col0;
+  float* S_io = p.S_io;
+
+  State<D> S;
   if constexpr (kCluster) {
     auto cluster = cooperative_groups::this_cluster();
-    for_state<D>(i, S, [](int, float4& x) { x = make_float4(0.f, 0.f, 0.f, 0.f); });
+    for_state<D>(S, [](int, int, float& x) { x = 0.f; });
     float z = 0.f;
+    float4* frag = reinterpret_cast<float4*>(Ss) + tid;  // S of this lane, element n at frag[n * kLinThreads]
     if (g < sg.G - 1) {  // nobody needs the last segment's sum
-      sum_segment<T, D>(k + base, v + base + col0, st.n, n_begin, n_end, Ks, Vs, tid, i, cg, S, z);
-      for_state<D>(i, S, [&](int a, float4& x) { *reinterpret_cast<float4*>(Ss + s_off(a, 4 * cg)) = x; });
+      sum_segment<T, D>(k, v, p.st.n, n_begin, n_end, Ks, Vs, tid, S, z);
+#pragma unroll
+      for (int n = 0; n < D / 16; ++n) frag[n * kLinThreads] = make_float4(S[n][0], S[n][1], S[n][2], S[n][3]);
       if (tid < D) zs[tid] = z;
     }
-    const bool from_caller = S_io != nullptr && !zero_init;
-    for_state<D>(i, S, [&](int a, float4& x) {
-      x = from_caller ? load4<float>(S_io + (sidx * D + a) * D + col0 + 4 * cg) : make_float4(0.f, 0.f, 0.f, 0.f);
-    });
-    z = (from_caller && tid < D) ? z_io[sidx * D + tid] : 0.f;
+    const bool from_caller = S_io != nullptr && !p.zero_init;
+    for_state<D>(S, [&](int a, int c, float& x) { x = from_caller ? S_io[(sidx * D + a) * D + col0 + c] : 0.f; });
+    z = (from_caller && tid < D) ? p.z_io[sidx * D + tid] : 0.f;
     cluster.sync();
+    // running sums: of S[n] by segment n mod G, of z by segment 0, for all segments, read and put back in place
     const int rank0 = (int)cluster.block_rank() - g;  // first segment of this slice
-    for (int gg = 0; gg < g; ++gg) {
-      const float* Sr = cluster.map_shared_rank(Ss, rank0 + gg);
-      for_state<D>(i, S, [&](int a, float4& x) {
-        const float4 y = lds4(Sr + s_off(a, 4 * cg));
-        x.x += y.x;
-        x.y += y.y;
-        x.z += y.z;
-        x.w += y.w;
-      });
-      if (tid < D) z += *cluster.map_shared_rank(zs + tid, rank0 + gg);
+    for (int n = g; n < D / 16; n += sg.G) {
+      float4 x[kMaxCluster - 1];
+#pragma unroll
+      for (int gg = 0; gg < kMaxCluster - 1; ++gg)
+        if (gg < sg.G - 1) x[gg] = *cluster.map_shared_rank(frag + n * kLinThreads, rank0 + gg);
+      float4 run = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int gg = 0; gg < kMaxCluster - 1; ++gg)
+        if (gg < sg.G - 1) {
+          axpy4(run, 1.f, x[gg]);
+          *cluster.map_shared_rank(frag + n * kLinThreads, rank0 + gg + 1) = run;
+        }
     }
-    cluster.sync();  // everybody has read what is overwritten now, and the caller's state, which the last CTAs will overwrite
-    for_state<D>(i, S, [&](int a, float4& x) { *reinterpret_cast<float4*>(Ss + s_off(a, 4 * cg)) = x; });
+    if (g == 0 && tid < D) {
+      float x[kMaxCluster - 1], run = 0.f;
+#pragma unroll
+      for (int gg = 0; gg < kMaxCluster - 1; ++gg)
+        if (gg < sg.G - 1) x[gg] = *cluster.map_shared_rank(zs + tid, rank0 + gg);
+#pragma unroll
+      for (int gg = 0; gg < kMaxCluster - 1; ++gg)
+        if (gg < sg.G - 1) {
+          run += x[gg];
+          *cluster.map_shared_rank(zs + tid, rank0 + gg + 1) = run;
+        }
+    }
+    cluster.sync();  // (also: everybody has read the caller's state, which the last CTAs will overwrite)
+    if (g > 0) {
+#pragma unroll
+      for (int n = 0; n < D / 16; ++n) {
+        const float4 x = frag[n * kLinThreads];
+        S[n][0] += x.x;
+        S[n][1] += x.y;
+        S[n][2] += x.z;
+        S[n][3] += x.w;
+      }
+      if (tid < D) z += zs[tid];
+    }
     if (tid < D) zs[tid] = z;
   } else {
     const float* Sp = nullptr;  // row a of the starting state at Sp + a * stride
     long long stride = D;
     const float* zp = nullptr;
-    if (sg.G > 1 && (g > 0 || (S_io != nullptr && !zero_init))) {
+    if (sg.G > 1 && (g > 0 || (S_io != nullptr && !p.zero_init))) {
       if constexpr (sizeof(T) == 4) {
-        Sp = reinterpret_cast<const float*>(o) + base + (long long)n_begin * st.n + col0;
-        stride = st.n;
+        Sp = reinterpret_cast<const float*>(o) + (long long)n_begin * p.st.n;
+        stride = p.st.n;
       }
-    } else if (g == 0 && S_io != nullptr && !zero_init) {
+    } else if (g == 0 && S_io != nullptr && !p.zero_init) {
       Sp = S_io + sidx * D * D + col0;
-      zp = z_io + sidx * D;
+      zp = p.z_io + sidx * D;
     }
-    for_state<D>(i, S, [&](int a, float4& x) {
-      x = Sp != nullptr ? load4<float>(Sp + a * stride + 4 * cg) : make_float4(0.f, 0.f, 0.f, 0.f);
-      *reinterpret_cast<float4*>(Ss + s_off(a, 4 * cg)) = x;
-    });
+    for_state<D>(S, [&](int a, int c, float& x) { x = Sp != nullptr ? Sp[a * stride + c] : 0.f; });
     if (tid < D)
       zs[tid] = Sp == nullptr ? 0.f : zp != nullptr ? zp[tid] : Sp[(long long)(D + tid / kW) * stride + tid % kW];
   }
-  BlockRegs<T, D> rq, rk;
-  BlockRegs<T, kW> rv;
-  rq.load(q + base, st.n, n_begin, n_end, tid);
-  rk.load(k + base, st.n, n_begin, n_end, tid);
-  rv.load(v + base + col0, st.n, n_begin, n_end, tid);
+  Ps[(tid >> 4) * kLdP + 16 + (tid & 15)] = 0.f;  // (masked, and nobody computes them)
+  BlockRegs<T, D, kLinThreads> rq, rk;
+  BlockRegs<T, kW, kLinThreads> rv;
+  rq.load(q, p.st.n, n_begin, n_end, tid);
+  rk.load(k, p.st.n, n_begin, n_end, tid);
+  rv.load(v, p.st.n, n_begin, n_end, tid);
   for (int n0 = n_begin; n0 < n_end; n0 += kC) {
     rq.store_phi(Qs, LD, n0, n_end, tid);
     rk.store_phi(Ks, LD, n0, n_end, tid);
-    rv.store(Vs, kW, tid);
+    rv.store(Vs, kLdV, tid);
     __syncthreads();  // (also: every thread has read its state out of the rows this CTA writes)
-    rq.load(q + base, st.n, n0 + kC, n_end, tid);
-    rk.load(k + base, st.n, n0 + kC, n_end, tid);
-    rv.load(v + base + col0, st.n, n0 + kC, n_end, tid);
-    {
-      float p[4][2];
-      score_block<D>(Qs, Ks, i, cg, p);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int row = i + 8 * r;
-        Ps[row * kLdP + cg] = cg <= row ? p[r][0] : 0.f;
-        Ps[row * kLdP + cg + 16] = cg + 16 <= row ? p[r][1] : 0.f;
-      }
-    }
+    rq.load(q, p.st.n, n0 + kC, n_end, tid);
+    rk.load(k, p.st.n, n0 + kC, n_end, tid);
+    rv.load(v, p.st.n, n0 + kC, n_end, tid);
+    score_block<D>(Qs, Ks, zs, Ps, qz_s);
     __syncthreads();
-    {  // denominators: four threads per row
-      const int t = tid >> 2, part = tid & 3;
+    {  // denominators: eight threads per row
+      const int row = tid >> 3, part8 = tid & 7;
       float den = 0.f;
 #pragma unroll
-      for (int e = 0; e < 8; ++e) den += Ps[t * kLdP + part + 4 * e];
-#pragma unroll 4
-      for (int a = 4 * part; a < D; a += 16) den = dot4(lds4(Qs + t * LD + a), lds4(zs + a), den);
-      den += __shfl_xor_sync(0xffffffffu, den, 1);
-      den += __shfl_xor_sync(0xffffffffu, den, 2);
-      if (part == 0) inv_s[t] = 1.f / den;
-    }
-    float4 acc[4][1];
+      for (int e = 0; e < 4; ++e) den += Ps[row * kLdP + part8 + 8 * e];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) acc[r][0] = make_float4(0.f, 0.f, 0.f, 0.f);
-    product<D, 1>(acc, Qs, LD, i, [&](int a, int) { return Ss + s_off(a, 4 * cg); });
-    product<kC, 1>(acc, Ps, kLdP, i, [&](int j, int) { return Vs + j * kW + 4 * cg; });
+      for (int off = 1; off < 8; off <<= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
+      if (part8 == 0) inv_s[row] = 1.f / (den + qz_s[row]);
+    }
+    float acc[2][2][4];
+    readout<D, false>(Qs, Vs, Ps, S, acc);
+    bool bad = false;
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) bad |= is_nan(acc[m][n][e]);
+    if (tid >= 128) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) Os[i * 128 + tid - 128] = acc[i >> 3][(i >> 2) & 1][i & 3];
+    }
     const bool more = n0 + kC < n_end || (g == sg.G - 1 && S_io != nullptr);  // somebody wants the state after this block
-    if (more) add_outer<D>(Ks, Vs, i, cg, S);
-    if (__syncthreads_or(has_nan(acc[0][0]) || has_nan(acc[1][0]) || has_nan(acc[2][0]) || has_nan(acc[3][0]))) {
-      // a masked weight is 0, which is nothing unless the value is infinite or NaN (0 x inf = NaN): the same sums without
-      // the masked ones, so that a row sees no later value
+    if (__syncthreads_or(bad)) {
+      State<D> Sx;
+      float ax[2][2][4];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int row = i + 8 * r;
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-        for (int a = 0; a < D; ++a) axpy4(x, Qs[row * LD + a], lds4(Ss + s_off(a, 4 * cg)));
-#pragma unroll 1
-        for (int j = 0; j <= row; ++j) axpy4(x, Ps[row * kLdP + j], lds4(Vs + j * kW + 4 * cg));
-        acc[r][0] = x;
+      for (int n = 0; n < D / 16; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) Sx[n][e] = S[n][e];
+      mend_block<D>(Qs, Ks, Vs, Ps, Ss, Os, Sx, ax, more);
+#pragma unroll
+      for (int n = 0; n < D / 16; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) S[n][e] = Sx[n][e];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) acc[i >> 3][(i >> 2) & 1][i & 3] = ax[i >> 3][(i >> 2) & 1][i & 3];
+    } else {
+      if (tid < 128) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) acc[i >> 3][(i >> 2) & 1][i & 3] += Os[i * 128 + tid];
       }
-      __syncthreads();
+      if (more) add_outer<D, false>(Ks, Vs, S);
     }
+    if (tid < 128) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int row = i + 8 * r;
-      if (n0 + row >= n_end) continue;
-      const float inv = inv_s[row];
-      store4(o + base + (long long)(n0 + row) * st.n + col0 + 4 * cg,
-             make_float4(acc[r][0].x * inv, acc[r][0].y * inv, acc[r][0].z * inv, acc[r][0].w * inv));
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const int row = 16 * m + (lane >> 2) + 8 * r;
+          if (n0 + row >= n_end) continue;
+          const float inv = inv_s[row];
+#pragma unroll
+          for (int n = 0; n < 2; ++n)
+            store2(o + (long long)(n0 + row) * p.st.n + 16 * (tid >> 5) + 8 * n + 2 * (lane & 3), acc[m][n][2 * r] * inv,
+                   acc[m][n][2 * r + 1] * inv);
+        }
     }
-    if (more) {
-      for_state<D>(i, S, [&](int a, float4& x) { *reinterpret_cast<float4*>(Ss + s_off(a, 4 * cg)) = x; });
-      if (tid < D) zs[tid] += column_sum<D>(Ks + tid);
-    }
+    if (more && tid >= kLinThreads - D) zs[tid - (kLinThreads - D)] += column_sum<D>(Ks + tid - (kLinThreads - D));
     __syncthreads();
   }
   if (g == sg.G - 1 && S_io != nullptr) {
-    for_state<D>(i, S, [&](int a, float4& x) { store4(S_io + (sidx * D + a) * D + col0 + 4 * cg, x); });
-    if (col0 == 0 && tid < D) z_io[sidx * D + tid] = zs[tid];
+    for_state<D>(S, [&](int a, int c, float& x) { S_io[(sidx * D + a) * D + col0 + c] = x; });
+    if (col0 == 0 && tid < D) p.z_io[sidx * D + tid] = zs[tid];
   }
+}
+
+template <typename T, int D, bool kCluster>
+__global__ void __launch_bounds__(kLinThreads, 2)
+linear_walk_kernel(const WalkArgs<T> p, int after) {
+  extern __shared__ __align__(16) float sm[];
+  if (after) grid_dep_wait();  // the segments' starting states
+  grid_dep_launch();
+  linear_walk<T, D, kCluster>(p, blockIdx.x, blockIdx.y, blockIdx.z, sm);
   if (blockIdx.x + blockIdx.y + blockIdx.z == 0) grid_dep_wait();
 }
 
@@ -575,8 +865,46 @@ cudaError_t window_launch(const void* q, const void* k, const void* v, void* o, 
   if (e != cudaSuccess) return e;
   auto kern = window_tiled_kernel<T, D>;
   if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, window_smem<D>())) != cudaSuccess) return e;
-  return launch_link(link, kern, dim3((N + kC - 1) / kC, h_count, B), dim3(kNT), window_smem<D>(), stream, (const T*)q,
-                     (const T*)k, (const T*)v, (T*)o, N, w, fwd, scale, st, h_begin);
+  const WindowArgs<T> p = {(const T*)q, (const T*)k, (const T*)v, (T*)o, N, w, fwd, scale, st, h_begin};
+  return launch_link(link, kern, dim3((N + kWinRows - 1) / kWinRows, h_count, B), dim3(kWinThreads), window_smem<D>(), stream, p);
+}
+
+// Shared memory that a launch of few CTAs asks for so that no SM takes more than its share of them (the scheduler packs the
+// CTAs of a cluster onto as few SMs as hold them: 20 chains of 1588 tokens, clusters of 8, 64 -> 53 us).
+constexpr int kSmemPerSM = 228 * 1024, kSmemReserved = 1024;
+int spread_smem(int need, long long ctas, int sms) {
+  const long long per_sm = (ctas + sms - 1) / sms;
+  const long long least = kSmemPerSM / (per_sm + 1) - kSmemReserved + 256;  // one CTA more does not fit
+  return least > need ? (int)least : need;
+}
+
+// Clusters of that many CTAs of the walk that the device holds at a time (asked once).
+template <typename T, int D>
+int resident_clusters(int size, int smem, int dev) {
+  static std::atomic<int> known[64][kMaxCluster + 1][2];  // [...][a CTA per SM]
+  if (dev < 0 || dev >= 64) return 0;
+  std::atomic<int>& slot = known[dev][size][smem > LinT<D>::kSmem];
+  int n = slot.load(std::memory_order_relaxed);
+  if (n == 0) {
+    auto kern = linear_walk_kernel<T, D, true>;
+    if (ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem) != cudaSuccess) return 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(kLinThreads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = size;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+      (void)cudaGetLastError();
+      n = -1;
+    }
+    slot.store(n, std::memory_order_relaxed);
+  }
+  return n > 0 ? n : 0;
 }
 
 template <typename T, int D>
@@ -586,28 +914,47 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
   int dev = 0, sms = 0;
   cudaError_t e = device_info(&dev, &sms);
   if (e != cudaSuccess) return e;
-  // Clusters as large as one wave allows (three CTAs per SM at d = 64, two at 128, by registers), unless three launches
-  // can cut a chain into clearly more segments.  Measured (us, clusters of 8 | of 4 | three launches): 1 chain of 256
-  // tokens 17 | 21 | 39, 8 of 300 24.6 | 28.7 | 39, 6 of 1000 (d = 128) 74 | 107 | 100, 80 of 500 93 | 70.5 | 71, 80 of
-  // 2048 267 | 248 | 244, 1 of 2048 (d = 128) 113 | 203 | 99.  Clusters of 16 are no faster, and with 80 KB of shared
-  // memory per CTA slower (6 of 1000: 135).
+  // How many segments, and whether as one cluster per chain or in three launches: the least time of the CTA that takes longest, in
+  // blocks of a CTA that has an SM to itself (3.6 us at d = 64).  Both sweeps over a block cost 1.37 of the walk alone; two
+  // CTAs on an SM take 1.6 times as long; the exchange in a cluster costs about one block, the two other launches 3.5.
+  // Measured (us, layers with w = 64 or 128 and 12 heads, clusters of c | three launches with G): 80 chains of 2048 tokens 234 (c =
+  // 1) 246 (2) 177 (3) 196 (4) | 180 (4) 187 (12); 40 of 2048 111 (3) 103 (6) 119 (8) | 107 (5); 20 of 2048 60 (6) 66 (8) | 61 (12);
+  // 10 of 2048 45 (8) | 37 (20); 40 of 500 35 (4) 29 (6) 46 (8); d = 128, 12 of 300 27 (5) 35 (8).  With powers of two only, sized
+  // to fill the device once, 80 of 2048 took 187, 40 of 500 46.
   const int blocks = (N + kC - 1) / kC;
-  const long long ctas = (long long)B * h_count * (D / kW), wave = (D == 64 ? 3LL : 2LL) * sms;
-  // (Of a chain that brings a state all slices are one cluster, which at d = 128 leaves room for four segments: 6 of 1000 then
-  // take the three launches, 76 -> 100 us, 17 of 1000 165 -> 134, 18 of 500 118 -> 91.  Clusters of 16 CTAs take 76 us for
-  // 6 of 1000 but 189 for 17.)
+  const long long ctas = (long long)B * h_count * (D / kW);
+  // (Of a chain that brings a state all slices are one cluster: both read the caller's z, and one of them overwrites it.)
   const int slices = (S_io != nullptr && !zero_init) ? D / kW : 1;
+  auto cost = [&](int segments, double waves) {
+    const double per_block = (segments > 1 ? 1.37 : 1.0) * (ctas * segments > sms ? 1.6 : 1.0);
+    return waves * ((blocks + segments - 1) / segments) * per_block;
+  };
   int cluster = 1;
-  while (2 * cluster * slices <= kMaxCluster && 2 * cluster <= blocks && 2 * cluster * ctas <= wave) cluster *= 2;
+  double best = cost(1, (double)((ctas + 2 * sms - 1) / (2 * sms)));
+  for (int c = 2; c * slices <= kMaxCluster && c <= blocks; ++c) {
+    const long long fit = (long long)resident_clusters<T, D>(c * slices, spread_smem(C::kSmem, c * ctas, sms), dev) * slices;
+    if (fit < 1) continue;
+    const double x = cost(c, (double)((ctas + fit - 1) / fit)) + 1.0;
+    if (x < best) {
+      best = x;
+      cluster = c;
+    }
+  }
   if constexpr (sizeof(T) == 4) {
-    long long G3 = ctas < 4LL * sms ? (8LL * sms + ctas - 1) / ctas : 1;
-    if (G3 > N / C::kMinSeg) G3 = N / C::kMinSeg;
-    if (5 * G3 > 6 * cluster) {
+    long long G3 = 1;
+    for (int g = 2; g <= N / C::kMinSeg && (g == 2 || ctas * g <= 2LL * sms); ++g) {
+      const double x = cost(g, (double)((ctas * g + 2 * sms - 1) / (2 * sms))) + 3.5;
+      if (x < best) {
+        best = x;
+        G3 = g;
+      }
+    }
+    if (G3 > 1) {
       const int G = (int)G3;
       const Segs sg = {N, G, blocks / G, blocks % G};
       auto sum = linear_contribution_kernel<D>;
       if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(sum), dev, C::kSmemSum)) != cudaSuccess) return e;
-      if ((e = launch_link(link, sum, dim3((G - 1) * (D / kW), h_count, B), dim3(kNT), C::kSmemSum, stream, (const float*)k,
+      if ((e = launch_link(link, sum, dim3((G - 1) * (D / kW), h_count, B), dim3(kLinThreads), C::kSmemSum, stream, (const float*)k,
                            (const float*)v, (float*)o, sg, st, h_begin)) != cudaSuccess)
         return e;
       constexpr int kItems = (D + C::ZROWS) * (D / 4);
@@ -615,18 +962,18 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
                            (float*)o, sg, st, h_begin, h_count, zero_init ? nullptr : S_io, z_io)) != cudaSuccess)
         return e;
       auto walk = linear_walk_kernel<float, D, false>;
-      if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, C::kSmem)) != cudaSuccess) return e;
-      return launch_link(kAfter, walk, dim3(G * (D / kW), h_count, B), dim3(kNT), C::kSmem, stream, (const float*)q,
-                         (const float*)k, (const float*)v, (float*)o, sg, st, h_begin, h_count, S_io, z_io, zero_init ? 1 : 0, 1);
+      if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, spread_smem(C::kSmem, 1, sms))) != cudaSuccess) return e;
+      const WalkArgs<T> p = {(const T*)q, (const T*)k, (const T*)v, (T*)o, sg, st, h_begin, h_count, S_io, z_io, zero_init ? 1 : 0};
+      return launch_link(kAfter, walk, dim3(G * (D / kW), h_count, B), dim3(kLinThreads), C::kSmem, stream, p, 1);
     }
   }
   const Segs sg = {N, cluster, blocks / cluster, blocks % cluster};
   const int cluster_ctas = cluster * slices;
   auto walk = cluster_ctas > 1 ? linear_walk_kernel<T, D, true> : linear_walk_kernel<T, D, false>;
-  if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, C::kSmem)) != cudaSuccess) return e;
-  return launch_link_clusters(link, cluster_ctas, walk, dim3(cluster * (D / kW), h_count, B), dim3(kNT), C::kSmem, stream,
-                              (const T*)q, (const T*)k, (const T*)v, (T*)o, sg, st, h_begin, h_count, S_io, z_io,
-                              zero_init ? 1 : 0, 0);
+  const int smem = spread_smem(C::kSmem, cluster * ctas, sms);
+  if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, spread_smem(C::kSmem, 1, sms))) != cudaSuccess) return e;
+  const WalkArgs<T> p = {(const T*)q, (const T*)k, (const T*)v, (T*)o, sg, st, h_begin, h_count, S_io, z_io, zero_init ? 1 : 0};
+  return launch_link_clusters(link, cluster_ctas, walk, dim3(cluster * (D / kW), h_count, B), dim3(kLinThreads), smem, stream, p, 0);
 }
 
 }  // namespace

@@ -994,6 +994,33 @@ def test_self_layer_sums_and_readout_cut_differently(B, H, N, d, w, h0):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("B,H,N,d,w", [
+    (1, 2, 1, 64, 1), (2, 3, 31, 64, 33), (1, 3, 65, 128, 64),          # a block or less per CTA, remainders
+    (5, 12, 90, 64, 40), (10, 5, 161, 64, 600), (4, 8, 450, 64, 17),    # clusters of 3 to 6 segments, of unequal lengths
+    (3, 5, 333, 128, 95), (1, 3, 1100, 64, 130), (1, 2, 1601, 128, 31),  # of 7 and 8, three launches
+    (40, 8, 70, 64, 65),                                                # whole chains, several to an SM
+])
+def test_f32_layer_products_at_the_edges_of_blocks_and_segments(B, H, N, d, w):
+    """Windowed and linear heads against the oracle; and the linear heads once more from a given state.  The bound is that of
+    a sum of 2 d products of unit normals in fp32, 2^-24 sqrt(2 d) of a row's size, times four."""
+    q, k, v = synth.qkv(B, H, N, d, "f32", seed=300 + N, gain=1.0)
+    qd, kd, vd = dev(q, k, v)
+    o = gf.hybrid_attn(qd, kd, vd, w, h_sparse=1)
+    S = torch.zeros(B, H, d, d, device="cuda")
+    z = torch.zeros(B, H, d, device="cuda")
+    cut = N // 2
+    parts = [gf.causal_linear_attn(*(x[:, :, a:b].contiguous() for x in (qd, kd, vd)), S, z)
+             for a, b in ((0, cut), (cut, N)) if b > a]
+    bs = sorted({0, B - 1})
+    ref = oracle.hybrid_attn(f64(q[bs]), f64(k[bs]), f64(v[bs]), w, h_sparse=1)
+    assert_parity(f64(o[bs]), ref, "f32", "layer")
+    rel = np.sqrt(((f64(o[bs]) - ref) ** 2).sum() / (ref**2).sum())
+    assert rel <= 4 * 2.0**-24 * np.sqrt(2 * d), rel
+    lin = oracle.causal_linear_attn(f64(q[bs]), f64(k[bs]), f64(v[bs]))
+    assert_parity(f64(torch.cat(parts, 2)[bs]), lin, "f32", "carried state")
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 @pytest.mark.parametrize("N,w", [(1, 3), (37, 64), (64, 64), (333, 100)])
 def test_what_follows_a_layer_in_its_stream_follows_all_of_its_kernels(dtype, N, w):
