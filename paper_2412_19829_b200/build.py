@@ -1,4 +1,4 @@
-"""Builds libgformer.so in-tree with nvcc for sm_100a (no JIT cache, no torch extension).
+"""Builds libgformer.so in-tree with nvcc for sm_100a, and _fastcall.so beside it with g++ (no JIT cache).
 
 Usage: python -m paper_2412_19829_b200.build [--force] [--verbose]
 """
@@ -14,6 +14,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "libgformer.so")
+FASTCALL = os.path.join(HERE, "_fastcall.so")  # the binding's calls as a module (csrc/fastcall.cpp)
 SOURCES = ["api.cu", "simt_kernels.cu", "simt_tiled.cu", "tma_host.cu", "tc_window.cu", "tc_linear.cu", "tc_linear_self.cu", "noalloc.cu", "partition.cu", "tc_favor.cu"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 
@@ -30,12 +31,27 @@ def _sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(FASTCALL)):
         return True
-    t = os.path.getmtime(LIB)
-    deps = _sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
+    t = min(os.path.getmtime(LIB), os.path.getmtime(FASTCALL))
+    deps = _sources() + [os.path.join(CSRC, "fastcall.cpp")] + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     deps += [os.path.join(INCLUDE, f) for f in os.listdir(INCLUDE)]
     return any(os.path.getmtime(p) > t for p in deps)
+
+
+def _build_fastcall(out: str) -> subprocess.Popen:
+    import sysconfig
+
+    import torch
+
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc()))
+    inc = [INCLUDE, sysconfig.get_paths()["include"], os.path.join(root, "include"),
+           os.path.join(root, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}"]
+    cmd += [x for i in inc for x in ("-I", i)] + [os.path.join(CSRC, "fastcall.cpp"), "-o", out]
+    cmd += ["-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-ldl"]
+    return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -54,6 +70,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         objs.append(obj)
         procs.append((src, subprocess.Popen([nvcc, "-c", src, "-o", obj] + flags,
                                             stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+    procs.append(("fastcall.cpp", _build_fastcall(FASTCALL + f".{os.getpid()}.tmp")))
     failed = False
     for src, p in procs:
         out, _ = p.communicate()
@@ -65,6 +82,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + f".{os.getpid()}.tmp"
     subprocess.check_call([nvcc, "-shared", "-o", tmp] + objs + ARCH + ["-cudart", "static"])
     os.replace(tmp, LIB)
+    os.replace(FASTCALL + f".{os.getpid()}.tmp", FASTCALL)
     return LIB
 
 

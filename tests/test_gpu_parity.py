@@ -994,6 +994,62 @@ def test_self_layer_sums_and_readout_cut_differently(B, H, N, d, w, h0):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("dtype,layout", [("bf16", 0), ("bf16", 1), ("f32", 0)])
+def test_calls_made_natively_and_through_ctypes_are_the_same(monkeypatch, dtype, layout):
+    """Every call with usual arguments, with ones that the native module leaves to ctypes (numpy integers, a stream object, an
+    output of the caller), with a workspace that has to grow; and the errors of both."""
+    B, H, N, d, w = 2, 4, 150, 64, 40
+
+    class Ordinary:
+        def __getattr__(self, name):
+            return lambda *a: None
+
+    t = torch.float32 if dtype == "f32" else torch.bfloat16
+    q, k, v = dev(*synth.qkv(B, H, N, d, dtype, seed=5))
+    if layout:
+        q, k, v = (x.transpose(1, 2).contiguous() for x in (q, k, v))
+    W = synth.favor_projection(H - 1, d, seed=3, dtype=dtype).cuda()
+    step = [x[:, 0].contiguous() if layout else x[:, :, 0].contiguous() for x in (q, k, v)]
+
+    def calls(i):
+        gf._default_ws.clear()
+        st = gf.DecodeState(B, H, d, w, 1, t)
+        S, z = torch.zeros(B, H, d, d, device="cuda"), torch.zeros(B, H, d, device="cuda")
+        pos = torch.tensor([3, -1], device="cuda")
+        r = [gf.window_attn(q, k, v, i(w), layout=layout), gf.window_attn_self(q, k, v, w, 0.2, layout),
+             gf.hybrid_attn_self(q, k, v, w, i(1), layout=layout, stream=torch.cuda.current_stream()),
+             gf.causal_linear_attn(q, k, v, S, z, layout=layout, out=torch.empty_like(q)),
+             gf.hybrid_attn(q, k, v, w, h_sparse=1, layout=layout, W=W),
+             gf.hybrid_attn(q, k, v, w, h_sparse=1, layout=layout, state_out=st), gf.decode_step(*step, st),
+             gf.decode_step_ragged(*step, st, pos)]
+        assert st.t == N + 1
+        return r + [S, z, pos, st.S, st.z, st.k_cache, st.v_cache]
+
+    def errors():
+        small = gf.Workspace(256)
+        small.nbytes = 16
+        bad = [lambda: gf.window_attn(q.cpu(), k, v, w), lambda: gf.window_attn(q, k[:1], v, w),
+               lambda: gf.hybrid_attn(q.half(), k.half(), v.half(), w), lambda: gf.hybrid_attn(q, k, v, 0, layout=layout),
+               lambda: gf.hybrid_attn(q, k, v, w, h_sparse=1, W=W[:1], layout=layout),
+               lambda: gf.window_attn(q, k, v, w, layout=layout, ws=small), lambda: gf.window_attn(q, k, q, w, layout=layout, out=q),
+               lambda: gf.causal_linear_attn(q, k, v, layout=layout, chunk=64),
+               lambda: gf.decode_step(step[0].cpu(), *step[1:], gf.DecodeState(B, H, d, w, 1, t))]
+        got = []
+        for f in bad:
+            with pytest.raises(Exception) as e:
+                f()
+            got.append((e.type, str(e.value)))
+        return got
+
+    native, native_numpy, native_errors = calls(int), calls(np.int64), errors()
+    monkeypatch.setattr(gf, "_fast", Ordinary())
+    ordinary = calls(int)
+    for a, b, c in zip(native, native_numpy, ordinary):
+        assert torch.equal(a, c) and torch.equal(b, c)
+    assert native_errors == errors()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("B,H,N,d,w", [
     (1, 2, 1, 64, 1), (2, 3, 31, 64, 33), (1, 3, 65, 128, 64),          # a block or less per CTA, remainders
     (5, 12, 90, 64, 40), (10, 5, 161, 64, 600), (4, 8, 450, 64, 17),    # clusters of 3 to 6 segments, of unequal lengths
