@@ -67,15 +67,15 @@ int cuda_status(cudaError_t e) { return e == cudaSuccess ? GF_OK : GF_ERR_CUDA; 
 // Window heads [h_begin, h_begin+h_count) on `stream`.
 int run_window(const Tuning& tn, const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d, int w,
                float scale, int dtype, int layout, int h_begin, int h_count, WsHeader* ws,
-               cudaStream_t stream, gf::Link link, bool two_sided = false, bool hold = false) {
+               cudaStream_t stream, gf::Link link, gf::LetGo let_go, bool two_sided = false, gf::Place place = {}) {
   if (h_count <= 0) return GF_OK;
   const int w_eff = w > N ? N : w;  // keys before token 0 (or after the last one) do not exist
   const int fwd = two_sided ? w_eff - 1 : 0;
   if (!tn.force_simt && gf::tc_window_supported(N, d, w_eff, dtype))
     return cuda_status(
-        gf::launch_window_tc(q, k, v, o, B, H, N, d, w_eff, fwd, scale, layout, h_begin, h_count, ws, stream, link, hold));
+        gf::launch_window_tc(q, k, v, o, B, H, N, d, w_eff, fwd, scale, layout, h_begin, h_count, ws, stream, link, let_go));
   return cuda_status(gf::launch_window_simt(q, k, v, o, B, N, d, w_eff, fwd, scale, dtype,
-                                            gf::make_strides(layout, H, N, d), h_begin, h_count, stream, gf::kBeside));
+                                            gf::make_strides(layout, H, N, d), h_begin, h_count, stream, place));
 }
 
 // Feature map of the linear heads of one call: elu + 1 (W null), or positive random features under
@@ -103,30 +103,33 @@ int run_features(const Tuning& tn, const void* q, const void* k, int B, int H, i
   phi->fq = reinterpret_cast<uint8_t*>(ws) + phi->feat_offset;
   phi->fk = reinterpret_cast<uint8_t*>(phi->fq) + feature_bytes(B, h_count, N, d);
   return cuda_status(gf::launch_favor_features_tc(q, k, phi->W, phi->fq, phi->fk, B, H, N, d, layout, h_begin, h_count, ws,
-                                                  stream, gf::kAfter));
+                                                  stream));
 }
 
 int run_linear(const Tuning& tn, const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d, int dtype,
                int layout, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init, int max_ctas,
-               WsHeader* ws, cudaStream_t stream, gf::Link link, bool shared = false, const Phi& phi = Phi()) {
+               WsHeader* ws, cudaStream_t stream, gf::Link link, gf::LetGo let_go, bool shared = false, const Phi& phi = Phi(), gf::Place place = {}) {
   if (h_count <= 0) return GF_OK;
   if (!tn.force_simt && gf::tc_linear_supported(N, d, dtype)) {
     return cuda_status(gf::launch_linear_tc(q, k, v, o, B, H, N, d, layout, h_begin, h_count, S_io, z_io,
-                                            zero_init, tn.linear_split, max_ctas, ws, stream, link, shared, phi.fq, phi.fk));
+                                            zero_init, tn.linear_split, max_ctas, ws, stream, link, let_go, shared, phi.fq, phi.fk));
   }
   return cuda_status(gf::launch_linear_simt(q, k, v, o, B, N, d, dtype, gf::make_strides(layout, H, N, d),
-                                            h_begin, h_count, S_io, z_io, zero_init, stream, gf::kBeside, false, phi.W));
+                                            h_begin, h_count, S_io, z_io, zero_init, stream, place, false, phi.W));
 }
 
-// The first launch of every call but a decode step: zeroes the workspace header and the flags or counters of a linear kernel
-// behind it.  What follows in the call's chain of kernels (launch_link)
-// runs kAfter it or, the kernels that use no workspace and those behind one that is kAfter it, kBeside it.
+// The first launch of the calls whose kernels use the workspace: writes its header and zeroes the flags or counters of a
+// linear kernel behind it.  What follows in the call's chain of kernels (launch_link) runs kAfter it or, behind one that is
+// kAfter it, kBeside that.  The kernels that use no workspace (fp32 arithmetic) have the first of them write the header.
 // A memset and two streams with events for the two head groups, which this chain replaced, took 11 driver calls for a layer
 // instead of three and left the device idle for 2 to 4 us behind the memset and again at the end: 64 x 12 heads of 197 tokens
 // (d = 64, both directions) 33.0 -> 26.7 us, 8 x 12 of 2048 34.0 -> 32.7, 1 x 32 of 32 768 (d = 128, w = 512) 343 -> 336.
+gf::Place first_of_call(const Tuning& tn, void* ws, bool last) {
+  return {(uint4*)ws, (unsigned int)tn.wait_kcycles, (unsigned int)tn.drop_flag, last};
+}
+constexpr gf::Place kLastOfCall = {nullptr, 0, 0, 1};
 int clear_ws(const Tuning& tn, void* ws, cudaStream_t stream, size_t flag_bytes = 0) {
-  return cuda_status(gf::launch_clear_ws(ws, sizeof(WsHeader) + flag_bytes, (unsigned int)tn.wait_kcycles,
-                                         (unsigned int)tn.drop_flag, stream));
+  return cuda_status(gf::launch_clear_ws(first_of_call(tn, ws, false), sizeof(WsHeader) + flag_bytes, stream));
 }
 
 // How the tensor-core kernel of the causal linear heads will run a call's chains: max_ctas as for launch_linear_tc, bytes of
@@ -278,9 +281,10 @@ int gformer_window_attn(const void* q, const void* k, const void* v, void* o, in
   if (rc != GF_OK) return rc;
   if (!(scale > 0.f)) scale = 1.0f / sqrtf((float)d);
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  rc = clear_ws(tn, ws, stream);
-  if (rc != GF_OK) return rc;
-  return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream, gf::kAfter);
+  const bool tc = !tn.force_simt && gf::tc_window_supported(N, d, w, dtype);
+  if (tc && (rc = clear_ws(tn, ws, stream)) != GF_OK) return rc;
+  return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream, gf::kAfter, gf::kAtEnd,
+                    false, first_of_call(tn, ws, true));
 }
 
 int gformer_window_attn_self(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
@@ -294,9 +298,10 @@ int gformer_window_attn_self(const void* q, const void* k, const void* v, void* 
   if (rc != GF_OK) return rc;
   if (!(scale > 0.f)) scale = 1.0f / sqrtf((float)d);
   cudaStream_t stream = (cudaStream_t)cuda_stream;
-  rc = clear_ws(tn, ws, stream);
-  if (rc != GF_OK) return rc;
-  return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream, gf::kAfter, true);
+  const bool tc = !tn.force_simt && gf::tc_window_supported(N, d, w, dtype);
+  if (tc && (rc = clear_ws(tn, ws, stream)) != GF_OK) return rc;
+  return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream, gf::kAfter, gf::kAtEnd,
+                    true, first_of_call(tn, ws, true));
 }
 
 int gformer_hybrid_attn_self(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
@@ -323,18 +328,20 @@ int gformer_hybrid_attn_self_w(const void* q, const void* k, const void* v, void
   if (!(scale > 0.f)) scale = 1.0f / sqrtf((float)d);
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   const bool tc_linear = !tn.force_simt && gf::tc_linear_supported(N, d, dtype);
-  rc = clear_ws(tn, ws, stream, tc_linear ? gf::linear_self_count_bytes(B * (H - h_sparse)) : 0);
-  if (rc != GF_OK) return rc;
+  if (tc_linear && (rc = clear_ws(tn, ws, stream, gf::linear_self_count_bytes(B * (H - h_sparse)))) != GF_OK) return rc;
   Phi fm;
   fm.W = W;
   fm.feat_offset = feat_offset;
   if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, h_sparse, H - h_sparse, (WsHeader*)ws, stream, &fm)) != GF_OK)
     return rc;
   if (h_sparse == H)
-    return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream, gf::kAfter, true);
+    return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, H, (WsHeader*)ws, stream, gf::kAfter, gf::kAtEnd,
+                      true, first_of_call(tn, ws, true));
   int wrc = GF_OK;  // of the windowed heads: on the SMs that the linear heads leave idle, and between their kernels
-  auto window = [&]() -> cudaError_t {
-    wrc = run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, stream, gf::kBeside, true);
+  auto window = [&](gf::LetGo let_go) -> cudaError_t {
+    if (h_sparse == 0) return cudaSuccess;
+    wrc = run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, stream, gf::kBeside, let_go, true,
+                     kLastOfCall);
     return wrc == GF_OK ? cudaSuccess : cudaErrorUnknown;
   };
   if (tc_linear) {
@@ -344,8 +351,8 @@ int gformer_hybrid_attn_self_w(const void* q, const void* k, const void* v, void
                                                sizeof(WsHeader), stream, window, window_us, fm.fq, fm.fk));
   } else {  // fp32 storage (or the CUDA-core knob): token by token, a summing sweep and a readout sweep
     rc = cuda_status(gf::launch_linear_simt(q, k, v, o, B, N, d, dtype, gf::make_strides(layout, H, N, d), h_sparse,
-                                            H - h_sparse, nullptr, nullptr, true, stream, gf::kBeside, true, W));
-    if (rc == GF_OK) (void)window();
+                                            H - h_sparse, nullptr, nullptr, true, stream, first_of_call(tn, ws, h_sparse == 0), true, W));
+    if (rc == GF_OK) (void)window(gf::kAtEnd);
   }
   return wrc != GF_OK ? wrc : rc;
 }
@@ -377,10 +384,11 @@ int gformer_causal_linear_attn_w(const void* q, const void* k, const void* v, vo
   int max_ctas = 0;
   size_t flags = 0;
   if ((rc = plan_linear(tn, B * H, N, d, dtype, false, stream, &max_ctas, &flags, &order)) != GF_OK) return rc;
-  if ((rc = clear_ws(tn, ws, stream, flags)) != GF_OK) return rc;
+  const bool tc = !tn.force_simt && gf::tc_linear_supported(N, d, dtype);
+  if (tc && (rc = clear_ws(tn, ws, stream, flags)) != GF_OK) return rc;
   if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, 0, H, (WsHeader*)ws, stream, &fm)) != GF_OK) return rc;
   if ((rc = run_linear(tn, q, k, v, o, B, H, N, d, dtype, layout, 0, H, S_io, z_io, false, max_ctas, (WsHeader*)ws, stream,
-                       gf::kAfter, false, fm)) != GF_OK)
+                       gf::kAfter, gf::kAtEnd, false, fm, first_of_call(tn, ws, true))) != GF_OK)
     return rc;
   return cuda_status(order.leave());
 }
@@ -431,31 +439,47 @@ int gformer_hybrid_attn_w(const void* q, const void* k, const void* v, void* o, 
   int max_ctas = 0;
   size_t flags = 0;
   if ((rc = plan_linear(tn, B * h_lin, N, d, dtype, both, stream, &max_ctas, &flags, &order)) != GF_OK) return rc;
-  if ((rc = clear_ws(tn, ws, stream, flags)) != GF_OK) return rc;
+  const bool tc = !tn.force_simt && gf::tc_linear_supported(N, d, dtype);
+  const gf::Strides st = gf::make_strides(layout, H, N, d);
+  const bool layer = both && !tc && W == nullptr;  // the fp32-arithmetic kernels take both head groups in one launch
+  if (tc && (rc = clear_ws(tn, ws, stream, flags)) != GF_OK) return rc;
   if ((rc = run_features(tn, q, k, B, H, N, d, dtype, layout, h_sparse, h_lin, (WsHeader*)ws, stream, &fm)) != GF_OK) return rc;
-  auto linear = [&](gf::Link link) {
+  auto linear = [&](gf::Link link, gf::LetGo let_go) {
     return run_linear(tn, q, k, v, o, B, H, N, d, dtype, layout, h_sparse, h_lin, S_out, z_out, true, max_ctas, (WsHeader*)ws,
-                      stream, link, both, fm);
+                      stream, link, let_go, both, fm, first_of_call(tn, ws, let_go == gf::kAtEnd));
   };
-  auto window = [&](gf::Link link, bool hold) {
-    return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, stream, link, false, hold);
+  auto window = [&](gf::Link link, gf::LetGo let_go) {
+    return run_window(tn, q, k, v, o, B, H, N, d, w, scale, dtype, layout, 0, h_sparse, (WsHeader*)ws, stream, link, let_go, false,
+                      h_lin > 0 ? kLastOfCall : first_of_call(tn, ws, let_go == gf::kAtEnd));
   };
   // Behind a pre-pass of random features the windowed heads come first and fill its tail, and the linear heads theirs (us, after
   // the linear heads and ahead of them: 32 heads of 32 768 tokens, d = 128, 461 and 444; 8 x 8 of 3217, d = 64, 62.0 and 57.9;
   // 32 x 12 of 1024 87.8 and 86.1; without features ahead of them is slower, 8 x 12 of 2048 32.6 and 39.6).
   const bool window_first = both && fm.fq != nullptr;
-  if (window_first) {
-    if ((rc = window(gf::kBeside, true)) != GF_OK) return rc;  // (it lets go of the linear heads when the features are complete)
-    if ((rc = linear(gf::kBeside)) != GF_OK) return rc;
-  } else if ((rc = linear(gf::kAfter)) != GF_OK) {
-    return rc;
+  const bool ring = state_out && h_sparse > 0;
+  auto export_ring = [&]() {
+    return ring ? cuda_status(gf::launch_export_ring(k, v, state_out->k_cache, state_out->v_cache, B, N, d, w, dtype, st, h_sparse,
+                                                     stream))
+                : GF_OK;
+  };
+  if (layer) {
+    if ((rc = cuda_status(gf::launch_layer_tiled(q, k, v, o, B, N, d, w < N ? w : N, scale, dtype, st, h_sparse, h_lin, S_out, z_out,
+                                                 stream, first_of_call(tn, ws, !ring)))) != GF_OK ||
+        (rc = export_ring()) != GF_OK)
+      return rc;
+  } else if (window_first) {
+    // (the windowed heads let go of the linear ones when the features are complete)
+    if ((rc = window(gf::kBeside, gf::kWhenPreviousDone)) != GF_OK ||
+        (rc = linear(gf::kBeside, ring ? gf::kAtStart : gf::kAtEnd)) != GF_OK || (rc = export_ring()) != GF_OK)
+      return rc;
+  } else if (h_lin > 0) {
+    if ((rc = linear(gf::kAfter, both ? gf::kAtStart : gf::kAtEnd)) != GF_OK || (rc = export_ring()) != GF_OK ||
+        (both && (rc = window(gf::kBeside, gf::kAtEnd)) != GF_OK))
+      return rc;
+  } else {
+    // (windowed heads alone wait for the cleared header themselves, and the export runs beside them)
+    if ((rc = window(gf::kAfter, ring ? gf::kAtStart : gf::kAtEnd)) != GF_OK || (rc = export_ring()) != GF_OK) return rc;
   }
-  if (state_out && (rc = cuda_status(gf::launch_export_ring(k, v, state_out->k_cache, state_out->v_cache, B, N, d, w, dtype,
-                                                            gf::make_strides(layout, H, N, d), h_sparse, stream,
-                                                            gf::kBeside))) != GF_OK)
-    return rc;
-  // (with windowed heads alone nothing before them has waited for the cleared header)
-  if (!window_first && (rc = window(h_lin > 0 ? gf::kBeside : gf::kAfter, false)) != GF_OK) return rc;
   if ((rc = cuda_status(order.leave())) != GF_OK) return rc;
   if (state_out) state_out->t = N;
   return GF_OK;

@@ -4,7 +4,6 @@
 // bidirectional layer's sums, positive random features), and the memory-bound decode step and ring export, which have
 // no dense contraction worth a tensor core.  Plain data-parallel kernels: no inter-CTA communication, no spin waits.
 #include <cooperative_groups.h>
-#include <stddef.h>
 
 #include "common.cuh"
 
@@ -48,7 +47,7 @@ __global__ void __launch_bounds__(256)
 linear_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                    T* __restrict__ o, int N, Strides st, int h_begin, int h_count,
                    float* __restrict__ S_io, float* __restrict__ z_io, int zero_init, int global_sum,
-                   const T* __restrict__ W /* [h_count, D, D] or null: elu + 1 */) {
+                   const T* __restrict__ W /* [h_count, D, D] or null: elu + 1 */, Place place) {
   constexpr int TB = 16;
   constexpr int AR = D / 8;
   __shared__ float qs[TB][D];
@@ -58,7 +57,7 @@ linear_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
   __shared__ float red[TB][8][33];
   __shared__ float redden[TB][8];
 
-  grid_dep_launch();
+  begin(place);
   const int slice = blockIdx.x, hl = blockIdx.y, b = blockIdx.z;
   const int h = h_begin + hl;
   const long long base = (long long)b * st.b + (long long)h * st.h;
@@ -331,6 +330,7 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
   __shared__ float gm[GW], gl[GW];
   __shared__ __align__(16) float part[GW][D];  // GW >= G
 
+  grid_dep_wait();  // (nothing is read or written before the kernel before this one is complete)
   // the windowed heads of the whole batch come first: they take longest, so none of them should start late
   const int tid = threadIdx.x, id = blockIdx.x, n_win = (int)(gridDim.x / (unsigned)H) * h_sparse;
   int h, b;
@@ -437,6 +437,7 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
       gm[gw] = m;
       gl[gw] = l;
     }
+    grid_dep_launch();
     __syncthreads();
     if (tid < D) {
       float mx = -INFINITY, sum = 0.f, lsum = 0.f;
@@ -530,6 +531,7 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
       }
     }
     *reinterpret_cast<float4*>(&part[grp][4 * c4]) = acc;
+    grid_dep_launch();
     __syncthreads();
     if (tid < D) {
       float sum = 0.f, den = 0.f;
@@ -545,11 +547,11 @@ decode_step_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
 template <typename T>
 cudaError_t linear_dispatch(const void* q, const void* k, const void* v, void* o, int B, int N, int d,
                             Strides st, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
-                            bool global_sum, cudaStream_t stream, Link link, const void* W) {
-  return launch_link_clusters(link, S_io != nullptr && !zero_init ? d / 32 : 1,
+                            bool global_sum, cudaStream_t stream, Place place, const void* W) {
+  return launch_link_clusters(S_io != nullptr && !zero_init ? d / 32 : 1,
                               d == 64 ? linear_simt_kernel<T, 64> : linear_simt_kernel<T, 128>, dim3(d / 32, h_count, B),
                               dim3(256), 0, stream, (const T*)q, (const T*)k, (const T*)v, (T*)o, N, st, h_begin, h_count, S_io,
-                              z_io, zero_init ? 1 : 0, global_sum ? 1 : 0, (const T*)W);
+                              z_io, zero_init ? 1 : 0, global_sum ? 1 : 0, (const T*)W, place);
 }
 
 template <typename T>
@@ -566,58 +568,50 @@ cudaError_t decode_dispatch(const void* q, const void* k, const void* v, void* o
   auto* kern = d == 128                          ? decode_step_kernel<T, 128, 4, 4>
                : (long long)B * H <= 4LL * sms ? decode_step_kernel<T, 64, 4, 4>
                                                  : decode_step_kernel<T, 64, 6, 2>;
-  kern<<<(unsigned)(B * H), 256, 0, stream>>>((const T*)q, (const T*)k, (const T*)v, (T*)o, (T*)kc, (T*)vc, S, z, t, t_seq,
-                                              H, w, h_sparse, scale, (const T*)W);
-  note_launch();
-  return cudaGetLastError();
+  return launch_link(kern, dim3((unsigned)(B * H)), dim3(256), 0, stream, (const T*)q, (const T*)k, (const T*)v, (T*)o,
+                     (T*)kc, (T*)vc, S, z, t, t_seq, H, w, h_sparse, scale, (const T*)W);
 }
 
 }  // namespace
 
 cudaError_t launch_linear_simt(const void* q, const void* k, const void* v, void* o, int B, int N, int d,
                                int dtype, Strides st, int h_begin, int h_count, float* S_io, float* z_io,
-                               bool zero_init, cudaStream_t stream, Link link, bool global_sum, const void* W) {
+                               bool zero_init, cudaStream_t stream, Place place, bool global_sum, const void* W) {
   if (h_count <= 0 || B <= 0) return cudaSuccess;
   if (!global_sum && W == nullptr)
-    return launch_linear_tiled(q, k, v, o, B, N, d, dtype, st, h_begin, h_count, S_io, z_io, zero_init, stream, link);
+    return launch_linear_tiled(q, k, v, o, B, N, d, dtype, st, h_begin, h_count, S_io, z_io, zero_init, stream, place);
   if (dtype == GF_F32)
     return linear_dispatch<float>(q, k, v, o, B, N, d, st, h_begin, h_count, S_io, z_io, zero_init, global_sum,
-                                  stream, link, W);
+                                  stream, place, W);
   return linear_dispatch<__nv_bfloat16>(q, k, v, o, B, N, d, st, h_begin, h_count, S_io, z_io, zero_init, global_sum,
-                                        stream, link, W);
+                                        stream, place, W);
 }
 
 cudaError_t launch_export_ring(const void* k, const void* v, void* k_cache, void* v_cache, int B, int N, int d,
-                               int w, int dtype, Strides st, int h_sparse, cudaStream_t stream, Link link) {
+                               int w, int dtype, Strides st, int h_sparse, cudaStream_t stream) {
   if (h_sparse <= 0 || B <= 0) return cudaSuccess;
   const int wn = N < w ? N : w, per16 = dtype == GF_F32 ? 4 : 8;  // elements of 16 bytes
   const long long total = (long long)B * h_sparse * wn * (d / per16);
   // (64 GB of keys)
   if (total > 0xffffffffLL - 2 * kExportThreads) return cudaErrorInvalidValue;
   const Strides st16 = {st.b / per16, st.h / per16, st.n / per16};
-  return launch_link(link, export_ring_kernel, dim3((unsigned)((total + 2 * kExportThreads - 1) / (2 * kExportThreads))),
+  return launch_link(export_ring_kernel, dim3((unsigned)((total + 2 * kExportThreads - 1) / (2 * kExportThreads))),
                      dim3(kExportThreads), 0, stream, (const uint4*)k, (const uint4*)v, (uint4*)k_cache, (uint4*)v_cache, N,
                      d / per16, w, wn, st16, h_sparse, (unsigned)total);
 }
 
 namespace {
-__global__ void clear_ws_kernel(uint4* ws, unsigned int n16, unsigned int wait_kcycles, unsigned int drop_flag) {
-  grid_dep_launch();
+__global__ void clear_ws_kernel(Place place, unsigned int n16) {
+  begin(place);
   const unsigned int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n16) return;
-  uint4 x = make_uint4(0u, 0u, 0u, 0u);
-  if (i == 0) x.w = wait_kcycles;  // WsHeader::wait_kcycles
-  if (i == 1) x.x = drop_flag;     // WsHeader::drop_flag
-  ws[i] = x;
+  if (i >= sizeof(WsHeader) / 16 && i < n16) place.ws[i] = make_uint4(0u, 0u, 0u, 0u);
 }
-static_assert(offsetof(WsHeader, wait_kcycles) == 12 && offsetof(WsHeader, drop_flag) == 16, "what the kernel above writes");
 }  // namespace
 
-cudaError_t launch_clear_ws(void* ws, size_t bytes, unsigned int wait_kcycles, unsigned int drop_flag, cudaStream_t stream) {
+cudaError_t launch_clear_ws(Place place, size_t bytes, cudaStream_t stream) {
   const size_t n16 = bytes / 16;
   if (n16 > 0x7fffffffu) return cudaErrorInvalidValue;
-  return launch_link(kFirst, clear_ws_kernel, dim3((unsigned)((n16 + 255) / 256)), dim3(256), 0, stream, (uint4*)ws,
-                     (unsigned)n16, wait_kcycles, drop_flag);
+  return launch_link(clear_ws_kernel, dim3((unsigned)((n16 + 255) / 256)), dim3(256), 0, stream, place, (unsigned)n16);
 }
 
 cudaError_t launch_decode_step(const void* q, const void* k, const void* v, void* o, void* k_cache,

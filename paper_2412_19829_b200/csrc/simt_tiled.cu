@@ -16,6 +16,7 @@
 #include <cooperative_groups.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -364,10 +365,11 @@ __device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, in
 
 template <typename T, int D>
 __global__ void __launch_bounds__(kWinThreads, D == 64 ? 2 : 1)
-window_tiled_kernel(const WindowArgs<T> p) {
+window_tiled_kernel(const WindowArgs<T> p, Place place) {
   extern __shared__ __align__(16) float sm[];
-  grid_dep_launch();
+  begin(place);
   window_tile<T, D>(p, blockIdx.x, blockIdx.y, blockIdx.z, sm);
+  grid_dep_launch();
   if (blockIdx.x + blockIdx.y + blockIdx.z == 0) grid_dep_wait();
 }
 
@@ -560,9 +562,9 @@ __device__ __forceinline__ void sum_segment(const T* k, const T* v, long long st
 template <int D>
 __global__ void __launch_bounds__(kLinThreads, 2)
 linear_contribution_kernel(const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ o, Segs sg,
-                           Strides st, int h_begin) {
+                           Strides st, int h_begin, Place place) {
   extern __shared__ __align__(16) float sm[];
-  grid_dep_launch();
+  begin(place);
   float *Ks = sm, *Vs = Ks + kC * LinT<D>::LD;
   const int g = blockIdx.x / (D / kW), col0 = (blockIdx.x % (D / kW)) * kW;
   const long long base = (long long)blockIdx.z * st.b + (long long)(h_begin + blockIdx.y) * st.h;
@@ -691,6 +693,13 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
   T* o = p.o + base + col0;
   float* S_io = p.S_io;
 
+  BlockRegs<T, D, kLinThreads> rq, rk;
+  BlockRegs<T, kW, kLinThreads> rv;
+  auto load_first = [&]() {
+    rq.load(q, p.st.n, n_begin, n_end, tid);
+    rk.load(k, p.st.n, n_begin, n_end, tid);
+    rv.load(v, p.st.n, n_begin, n_end, tid);
+  };
   State<D> S;
   if constexpr (kCluster) {
     auto cluster = cooperative_groups::this_cluster();
@@ -703,6 +712,7 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
       for (int n = 0; n < D / 16; ++n) frag[n * kLinThreads] = make_float4(S[n][0], S[n][1], S[n][2], S[n][3]);
       if (tid < D) zs[tid] = z;
     }
+    load_first();  // (under way while the sums are exchanged)
     const bool from_caller = S_io != nullptr && !p.zero_init;
     for_state<D>(S, [&](int a, int c, float& x) { x = from_caller ? S_io[(sidx * D + a) * D + col0 + c] : 0.f; });
     z = (from_caller && tid < D) ? p.z_io[sidx * D + tid] : 0.f;
@@ -748,6 +758,7 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
     }
     if (tid < D) zs[tid] = z;
   } else {
+    load_first();
     const float* Sp = nullptr;  // row a of the starting state at Sp + a * stride
     long long stride = D;
     const float* zp = nullptr;
@@ -765,11 +776,6 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
       zs[tid] = Sp == nullptr ? 0.f : zp != nullptr ? zp[tid] : Sp[(long long)(D + tid / kW) * stride + tid % kW];
   }
   Ps[(tid >> 4) * kLdP + 16 + (tid & 15)] = 0.f;  // (masked, and nobody computes them)
-  BlockRegs<T, D, kLinThreads> rq, rk;
-  BlockRegs<T, kW, kLinThreads> rv;
-  rq.load(q, p.st.n, n_begin, n_end, tid);
-  rk.load(k, p.st.n, n_begin, n_end, tid);
-  rv.load(v, p.st.n, n_begin, n_end, tid);
   for (int n0 = n_begin; n0 < n_end; n0 += kC) {
     rq.store_phi(Qs, LD, n0, n_end, tid);
     rk.store_phi(Ks, LD, n0, n_end, tid);
@@ -849,24 +855,24 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
 
 template <typename T, int D, bool kCluster>
 __global__ void __launch_bounds__(kLinThreads, 2)
-linear_walk_kernel(const WalkArgs<T> p, int after) {
+linear_walk_kernel(const WalkArgs<T> p, int after, Place place) {
   extern __shared__ __align__(16) float sm[];
   if (after) grid_dep_wait();  // the segments' starting states
-  grid_dep_launch();
+  begin(place);
   linear_walk<T, D, kCluster>(p, blockIdx.x, blockIdx.y, blockIdx.z, sm);
+  grid_dep_launch();
   if (blockIdx.x + blockIdx.y + blockIdx.z == 0) grid_dep_wait();
 }
 
 template <typename T, int D>
-cudaError_t window_launch(const void* q, const void* k, const void* v, void* o, int B, int N, int w, int fwd, float scale,
-                          Strides st, int h_begin, int h_count, cudaStream_t stream, Link link) {
+cudaError_t window_launch(const WindowArgs<T>& p, int B, int h_count, cudaStream_t stream, Place place) {
   int dev = 0, sms = 0;
   cudaError_t e = device_info(&dev, &sms);
   if (e != cudaSuccess) return e;
   auto kern = window_tiled_kernel<T, D>;
   if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, window_smem<D>())) != cudaSuccess) return e;
-  const WindowArgs<T> p = {(const T*)q, (const T*)k, (const T*)v, (T*)o, N, w, fwd, scale, st, h_begin};
-  return launch_link(link, kern, dim3((N + kWinRows - 1) / kWinRows, h_count, B), dim3(kWinThreads), window_smem<D>(), stream, p);
+  return launch_link(kern, dim3((p.N + kWinRows - 1) / kWinRows, h_count, B), dim3(kWinThreads),
+                     window_smem<D>(), stream, p, place);
 }
 
 // Shared memory that a launch of few CTAs asks for so that no SM takes more than its share of them (the scheduler packs the
@@ -907,13 +913,14 @@ int resident_clusters(int size, int smem, int dev) {
   return n > 0 ? n : 0;
 }
 
+// Segments per chain: as a cluster, or (three > 1) in three launches.
+struct LinearPlan {
+  int cluster, slices, three;
+  long long ctas;  // of one segment per chain
+};
 template <typename T, int D>
-cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, int B, int N, Strides st, int h_begin,
-                          int h_count, float* S_io, float* z_io, bool zero_init, cudaStream_t stream, Link link) {
+LinearPlan linear_plan(int B, int N, int h_count, bool brings_state, int dev, int sms) {
   using C = LinT<D>;
-  int dev = 0, sms = 0;
-  cudaError_t e = device_info(&dev, &sms);
-  if (e != cudaSuccess) return e;
   // How many segments, and whether as one cluster per chain or in three launches: the least time of the CTA that takes longest, in
   // blocks of a CTA that has an SM to itself (3.6 us at d = 64).  Both sweeps over a block cost 1.37 of the walk alone; two
   // CTAs on an SM take 1.6 times as long; the exchange in a cluster costs about one block, the two other launches 3.5.
@@ -924,12 +931,12 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
   const int blocks = (N + kC - 1) / kC;
   const long long ctas = (long long)B * h_count * (D / kW);
   // (Of a chain that brings a state all slices are one cluster: both read the caller's z, and one of them overwrites it.)
-  const int slices = (S_io != nullptr && !zero_init) ? D / kW : 1;
+  const int slices = brings_state ? D / kW : 1;
   auto cost = [&](int segments, double waves) {
     const double per_block = (segments > 1 ? 1.37 : 1.0) * (ctas * segments > sms ? 1.6 : 1.0);
     return waves * ((blocks + segments - 1) / segments) * per_block;
   };
-  int cluster = 1;
+  int cluster = 1, G3 = 1;
   double best = cost(1, (double)((ctas + 2 * sms - 1) / (2 * sms)));
   for (int c = 2; c * slices <= kMaxCluster && c <= blocks; ++c) {
     const long long fit = (long long)resident_clusters<T, D>(c * slices, spread_smem(C::kSmem, c * ctas, sms), dev) * slices;
@@ -941,7 +948,6 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
     }
   }
   if constexpr (sizeof(T) == 4) {
-    long long G3 = 1;
     for (int g = 2; g <= N / C::kMinSeg && (g == 2 || ctas * g <= 2LL * sms); ++g) {
       const double x = cost(g, (double)((ctas * g + 2 * sms - 1) / (2 * sms))) + 3.5;
       if (x < best) {
@@ -949,51 +955,131 @@ cudaError_t linear_launch(const void* q, const void* k, const void* v, void* o, 
         G3 = g;
       }
     }
-    if (G3 > 1) {
-      const int G = (int)G3;
-      const Segs sg = {N, G, blocks / G, blocks % G};
+  }
+  return {cluster, slices, G3, ctas};
+}
+
+template <typename T, int D>
+cudaError_t linear_launch(const LinearPlan& plan, WalkArgs<T> p, int B, int N, int dev, int sms, cudaStream_t stream, Place place) {
+  using C = LinT<D>;
+  cudaError_t e;
+  const int blocks = (N + kC - 1) / kC;
+  if constexpr (sizeof(T) == 4) {
+    if (plan.three > 1) {
+      const int G = plan.three;
+      const Segs sg = p.sg = {N, G, blocks / G, blocks % G};
       auto sum = linear_contribution_kernel<D>;
       if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(sum), dev, C::kSmemSum)) != cudaSuccess) return e;
-      if ((e = launch_link(link, sum, dim3((G - 1) * (D / kW), h_count, B), dim3(kLinThreads), C::kSmemSum, stream, (const float*)k,
-                           (const float*)v, (float*)o, sg, st, h_begin)) != cudaSuccess)
+      if ((e = launch_link(sum, dim3((G - 1) * (D / kW), p.h_count, B), dim3(kLinThreads), C::kSmemSum, stream, p.k, p.v, p.o,
+                           sg, p.st, p.h_begin, Place{place.ws, place.wait_kcycles, place.drop_flag, 0})) != cudaSuccess)
         return e;
       constexpr int kItems = (D + C::ZROWS) * (D / 4);
-      if ((e = launch_link(kAfter, linear_prefix_kernel<D>, dim3((kItems + 127) / 128, h_count, B), dim3(128), 0, stream,
-                           (float*)o, sg, st, h_begin, h_count, zero_init ? nullptr : S_io, z_io)) != cudaSuccess)
+      if ((e = launch_link(linear_prefix_kernel<D>, dim3((kItems + 127) / 128, p.h_count, B), dim3(128), 0, stream, p.o, sg,
+                           p.st, p.h_begin, p.h_count, p.zero_init ? nullptr : p.S_io, p.z_io)) != cudaSuccess)
         return e;
       auto walk = linear_walk_kernel<float, D, false>;
       if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, spread_smem(C::kSmem, 1, sms))) != cudaSuccess) return e;
-      const WalkArgs<T> p = {(const T*)q, (const T*)k, (const T*)v, (T*)o, sg, st, h_begin, h_count, S_io, z_io, zero_init ? 1 : 0};
-      return launch_link(kAfter, walk, dim3(G * (D / kW), h_count, B), dim3(kLinThreads), C::kSmem, stream, p, 1);
+      return launch_link(walk, dim3(G * (D / kW), p.h_count, B), dim3(kLinThreads), C::kSmem, stream, p, 1, Place{nullptr, 0, 0, place.last});
     }
   }
-  const Segs sg = {N, cluster, blocks / cluster, blocks % cluster};
-  const int cluster_ctas = cluster * slices;
+  p.sg = {N, plan.cluster, blocks / plan.cluster, blocks % plan.cluster};
+  const int cluster_ctas = plan.cluster * plan.slices;
   auto walk = cluster_ctas > 1 ? linear_walk_kernel<T, D, true> : linear_walk_kernel<T, D, false>;
-  const int smem = spread_smem(C::kSmem, cluster * ctas, sms);
+  const int smem = spread_smem(C::kSmem, plan.cluster * plan.ctas, sms);
   if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(walk), dev, spread_smem(C::kSmem, 1, sms))) != cudaSuccess) return e;
-  const WalkArgs<T> p = {(const T*)q, (const T*)k, (const T*)v, (T*)o, sg, st, h_begin, h_count, S_io, z_io, zero_init ? 1 : 0};
-  return launch_link_clusters(link, cluster_ctas, walk, dim3(cluster * (D / kW), h_count, B), dim3(kLinThreads), smem, stream, p, 0);
+  return launch_link_clusters(cluster_ctas, walk, dim3(plan.cluster * (D / kW), p.h_count, B), dim3(kLinThreads), smem, stream, p,
+                              0, place);
+}
+
+// Both head groups in one launch: first the CTAs of the linear heads, `parts` per chain, then those of the windowed heads.
+template <typename T, int D, bool kCluster>
+__global__ void __launch_bounds__(kLinThreads, D == 64 ? 2 : 1)
+layer_kernel(const WalkArgs<T> lp, const WindowArgs<T> wp, int parts, int n_lin, int h_sparse, int n_win, Place place) {
+  static_assert(kLinThreads == kWinThreads, "one block size for both");
+  extern __shared__ __align__(16) float sm[];
+  begin(place);
+  const int id = blockIdx.x;
+  if (id < n_lin) {
+    const int chain = id / parts, b = chain / lp.h_count;
+    linear_walk<T, D, kCluster>(lp, id - chain * parts, chain - b * lp.h_count, b, sm);
+  } else if (id - n_lin < n_win) {  // (the grid is a multiple of the cluster size)
+    const int tiles = (wp.N + kWinRows - 1) / kWinRows, row = (id - n_lin) / tiles, b = row / h_sparse;
+    window_tile<T, D>(wp, id - n_lin - row * tiles, row - b * h_sparse, b, sm);
+  }
+  grid_dep_launch();
+}
+
+template <typename T, int D>
+cudaError_t layer_launch(WalkArgs<T> lp, const WindowArgs<T>& wp, int B, int h_sparse, cudaStream_t stream, Place place) {
+  using C = LinT<D>;
+  int dev = 0, sms = 0;
+  cudaError_t e = device_info(&dev, &sms);
+  if (e != cudaSuccess) return e;
+  const int N = wp.N;
+  const LinearPlan plan = linear_plan<T, D>(B, N, lp.h_count, false, dev, sms);
+  const long long n_lin = plan.ctas * plan.cluster, n_win = (long long)B * h_sparse * ((N + kWinRows - 1) / kWinRows);
+  // One launch for both unless the linear heads take three, or the device does not hold all CTAs at a time (two per SM, at d =
+  // 128, by the windowed heads' registers, one; us, one launch and two: 1 x 2 heads of 1030 tokens, d = 128, 44.6 and 51.5, 1 x 8 of
+  // 64 14.3 and 16.4; but 8 x 12 of 2048, d = 64, 189 and 181, 32 x 12 of 1024 330 and 321).
+  if (plan.three > 1 || n_lin + n_win > (D == 64 ? 2LL : 1LL) * sms) {
+    const Place first = {place.ws, place.wait_kcycles, place.drop_flag, 0};
+    if ((e = linear_launch<T, D>(plan, lp, B, N, dev, sms, stream, first)) != cudaSuccess) return e;
+    return window_launch<T, D>(wp, B, h_sparse, stream, Place{nullptr, 0, 0, place.last});
+  }
+  const int blocks = (N + kC - 1) / kC;
+  lp.sg = {N, plan.cluster, blocks / plan.cluster, blocks % plan.cluster};
+  auto kern = plan.cluster > 1 ? layer_kernel<T, D, true> : layer_kernel<T, D, false>;
+  constexpr int kNeed = C::kSmem > window_smem<D>() ? C::kSmem : window_smem<D>();
+  if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, spread_smem(kNeed, 1, sms))) != cudaSuccess) return e;
+  const long long grid = (n_lin + n_win + plan.cluster - 1) / plan.cluster * plan.cluster;
+  return launch_link_clusters(plan.cluster, kern, dim3((unsigned)grid), dim3(kLinThreads),
+                              spread_smem(kNeed, grid, sms), stream, lp, wp, plan.cluster * (D / kW), (int)n_lin, h_sparse,
+                              (int)n_win, place);
+}
+
+template <typename F>
+cudaError_t dispatch(int dtype, int d, F f) {
+  if (dtype == GF_F32) return d == 64 ? f(float(), std::integral_constant<int, 64>()) : f(float(), std::integral_constant<int, 128>());
+  return d == 64 ? f(__nv_bfloat16(), std::integral_constant<int, 64>()) : f(__nv_bfloat16(), std::integral_constant<int, 128>());
 }
 
 }  // namespace
 
 cudaError_t launch_window_simt(const void* q, const void* k, const void* v, void* o, int B, int N, int d, int w, int fwd,
-                               float scale, int dtype, Strides st, int h_begin, int h_count, cudaStream_t stream,
-                               Link link) {
+                               float scale, int dtype, Strides st, int h_begin, int h_count, cudaStream_t stream, Place place) {
   if (h_count <= 0 || B <= 0) return cudaSuccess;
-  auto* f = dtype == GF_F32 ? (d == 64 ? window_launch<float, 64> : window_launch<float, 128>)
-                            : (d == 64 ? window_launch<__nv_bfloat16, 64> : window_launch<__nv_bfloat16, 128>);
-  return f(q, k, v, o, B, N, w, fwd, scale, st, h_begin, h_count, stream, link);
+  return dispatch(dtype, d, [&](auto t, auto dd) {
+    using T = decltype(t);
+    const WindowArgs<T> p = {(const T*)q, (const T*)k, (const T*)v, (T*)o, N, w, fwd, scale, st, h_begin};
+    return window_launch<T, decltype(dd)::value>(p, B, h_count, stream, place);
+  });
 }
 
 cudaError_t launch_linear_tiled(const void* q, const void* k, const void* v, void* o, int B, int N, int d, int dtype,
                                 Strides st, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
-                                cudaStream_t stream, Link link) {
+                                cudaStream_t stream, Place place) {
   if (h_count <= 0 || B <= 0) return cudaSuccess;
-  auto* f = dtype == GF_F32 ? (d == 64 ? linear_launch<float, 64> : linear_launch<float, 128>)
-                            : (d == 64 ? linear_launch<__nv_bfloat16, 64> : linear_launch<__nv_bfloat16, 128>);
-  return f(q, k, v, o, B, N, st, h_begin, h_count, S_io, z_io, zero_init, stream, link);
+  int dev = 0, sms = 0;
+  const cudaError_t e = device_info(&dev, &sms);
+  if (e != cudaSuccess) return e;
+  return dispatch(dtype, d, [&](auto t, auto dd) {
+    using T = decltype(t);
+    constexpr int D = decltype(dd)::value;
+    const WalkArgs<T> p = {(const T*)q, (const T*)k, (const T*)v, (T*)o, Segs{}, st, h_begin, h_count, S_io, z_io, zero_init ? 1 : 0};
+    const LinearPlan plan = linear_plan<T, D>(B, N, h_count, S_io != nullptr && !zero_init, dev, sms);
+    return linear_launch<T, D>(plan, p, B, N, dev, sms, stream, place);
+  });
+}
+
+cudaError_t launch_layer_tiled(const void* q, const void* k, const void* v, void* o, int B, int N, int d, int w, float scale,
+                               int dtype, Strides st, int h_sparse, int h_lin, float* S_io, float* z_io, cudaStream_t stream,
+                               Place place) {
+  return dispatch(dtype, d, [&](auto t, auto dd) {
+    using T = decltype(t);
+    const WalkArgs<T> lp = {(const T*)q, (const T*)k, (const T*)v, (T*)o, Segs{}, st, h_sparse, h_lin, S_io, z_io, 1};
+    const WindowArgs<T> wp = {(const T*)q, (const T*)k, (const T*)v, (T*)o, N, w, 0, scale, st, 0};
+    return layer_launch<T, decltype(dd)::value>(lp, wp, B, h_sparse, stream, place);
+  });
 }
 
 }  // namespace gf

@@ -242,7 +242,7 @@ favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__
 
 cudaError_t launch_favor_features_tc(const void* q, const void* k, const void* W, void* fq, void* fk, int B, int H,
                                      int N, int d, int layout, int h_begin, int h_count, WsHeader* ws,
-                                     cudaStream_t stream, Link link) {
+                                     cudaStream_t stream) {
   if (h_count <= 0) return cudaSuccess;
   CUtensorMap mxq, mxk, mw, mfq, mfk;
   if (!make_qkv_tensor_map(&mxq, q, B, H, N, d, layout, 128) || !make_qkv_tensor_map(&mxk, k, B, H, N, d, layout, 128) ||
@@ -264,7 +264,7 @@ cudaError_t launch_favor_features_tc(const void* q, const void* k, const void* W
     if (err == cudaSuccess) err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem);
     if (err != cudaSuccess) return err;
     const unsigned grid = (unsigned)(total < sms ? total : sms);
-    return launch_link(link, kern, dim3(grid), dim3(kFavorThreads), smem, stream, mxq, mxk, mw, mfq, mfk, p);
+    return launch_link(kern, dim3(grid), dim3(kFavorThreads), smem, stream, mxq, mxk, mw, mfq, mfk, p);
   };
   return d == 64 ? launch(favor_tc_kernel<64>, FavorCfg<64>::kBytes) : launch(favor_tc_kernel<128>, FavorCfg<128>::kBytes);
 }

@@ -118,6 +118,7 @@ struct LinParams {
   float* z_io;           // [B, h_count, D] or null
   int zero_init;
   int beside;            // the kernel before this one in the stream may still be running (Link::kBeside)
+  LetGo let_go;
   unsigned int* status;  // two words: status, where
   unsigned int* flags;   // [nchains * G] x kFlagStride: 1 once the segment's inclusive state is in `prefix`
   float* prefix;         // [nchains * G][D*D + D]
@@ -489,7 +490,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
   if (!p.beside) grid_dep_wait();
-  grid_dep_launch();
+  if (p.let_go == kAtStart) grid_dep_launch();
 
   // Every role walks the same item list and keeps the same running counters: ta = K tiles of pass
   // A so far (slot = ta % KA, phase = ta / KA), nq = pass-C chunks so far (K slot = nq % KS, phase =
@@ -569,6 +570,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         }
         ++n_items;
       }
+      if (p.let_go == kAtEnd) grid_dep_launch();
     }
   } else if (warp == 1) {
     // ================================================================ MMA issuer
@@ -1439,7 +1441,7 @@ cudaError_t CutChainOrder::leave() {
 
 cudaError_t launch_linear_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                              int layout, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
-                             int split, int max_ctas, WsHeader* ws, cudaStream_t stream, Link link, bool shared,
+                             int split, int max_ctas, WsHeader* ws, cudaStream_t stream, Link link, LetGo let_go, bool shared,
                              const void* fq, const void* fk) {
   if (h_count <= 0) return cudaSuccess;
   // fq, fk: feature tensors [B, h_count, N, d] that stand in for Q and K (feature map: identity)
@@ -1477,7 +1479,8 @@ cudaError_t launch_linear_tc(const void* q, const void* k, const void* v, void* 
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, (int)smem);
     if (err != cudaSuccess) return err;
     p.beside = link == kBeside;
-    err = launch_link(link, kern, dim3(p.nitems < sms ? p.nitems : sms), dim3(kThreads), smem, stream, mq, mk, mv, mo, p);
+    p.let_go = p.chain0 + p.nchains < nchains ? kAtStart : let_go;
+    err = launch_link(kern, dim3(p.nitems < sms ? p.nitems : sms), dim3(kThreads), smem, stream, mq, mk, mv, mo, p);
     link = kBeside;  // a second launch depends on nothing that the first one does
     return err;
   };

@@ -353,7 +353,6 @@ linear_self_readout_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
-  grid_dep_launch();
 
   // Running counters shared by all roles: nq = chunks so far (Q slot, phi(Q) slot and O buffer
   // nq & 1, phase nq >> 1; staging buffer phase nq), ni = items so far.
@@ -373,6 +372,7 @@ linear_self_readout_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
                              pol);
         }
       }
+      grid_dep_launch();
     }
   } else if (warp == 1) {
     if (elect_one()) {
@@ -963,9 +963,9 @@ size_t linear_self_workspace_bytes(int nchains, int N, int d) {
 
 cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                                   int layout, int h_begin, int h_count, WsHeader* ws, size_t scratch_offset,
-                                  cudaStream_t stream, const std::function<cudaError_t()>& beside, double beside_us, const void* fq,
+                                  cudaStream_t stream, const std::function<cudaError_t(LetGo)>& beside, double beside_us, const void* fq,
                                   const void* fk) {
-  if (h_count <= 0) return beside();
+  if (h_count <= 0) return beside(kAtEnd);
   // fq, fk: feature tensors [B, h_count, N, d] that stand in for Q and K (feature map: identity)
   const bool features = fq != nullptr;
   CUtensorMap mq, mk, mv, mo;
@@ -1005,18 +1005,18 @@ cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, v
   if (whole) {
     auto kern = features ? linear_self_whole_kernel<true> : linear_self_whole_kernel<false>;
     if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, WholeCfg::kBytes)) != cudaSuccess) return e;
-    e = launch_link(kAfter, kern, grid, dim3(WholeCfg::kThreads), WholeCfg::kBytes, stream, mq, mk, mv, mo, p);
-    return e == cudaSuccess ? beside() : e;
+    e = launch_link(kern, grid, dim3(WholeCfg::kThreads), WholeCfg::kBytes, stream, mq, mk, mv, mo, p);
+    return e == cudaSuccess ? beside(kAtEnd) : e;
   }
   auto launch_red = [&](auto kern, int smem, int threads) -> cudaError_t {
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem);
     if (err != cudaSuccess) return err;
-    return launch_link(kAfter, kern, grid, dim3(threads), smem, stream, mk, mv, p);
+    return launch_link(kern, grid, dim3(threads), smem, stream, mk, mv, p);
   };
   auto launch_out = [&](auto kern, int smem, int threads) -> cudaError_t {
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem);
     if (err != cudaSuccess) return err;
-    return launch_link(kBeside, kern, grid, dim3(threads), smem, stream, mq, mo, p);
+    return launch_link(kern, grid, dim3(threads), smem, stream, mq, mo, p);
   };
   if (features)
     e = (d == 64) ? launch_red(linear_self_reduce_kernel<64, true>, RedCfg<64>::kBytes, RedCfg<64>::kThreads)
@@ -1027,8 +1027,8 @@ cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, v
   if (e != cudaSuccess) return e;
   // The windowed heads between the two: they start on the SMs that the first kernel leaves, and the readout on those that they
   // leave.
-  if ((e = beside()) != cudaSuccess) return e;
-  if (p.G > 1 && (e = launch_link(kBeside, linear_self_sum_kernel, dim3(p.sum_blocks, p.nchains), dim3(kSumThreads), 0, stream, p,
+  if ((e = beside(kAtStart)) != cudaSuccess) return e;
+  if (p.G > 1 && (e = launch_link(linear_self_sum_kernel, dim3(p.sum_blocks, p.nchains), dim3(kSumThreads), 0, stream, p,
                                   state_floats)) != cudaSuccess)
     return e;
   p.totals_of_one = p.G == 1;

@@ -90,7 +90,7 @@ struct WinParams {
   unsigned int* status;
   unsigned int* ticket;  // zero at launch; units beyond the first one of every CTA come from here
   int beside;            // the kernel before this one in the stream may still be running (Link::kBeside)
-  int hold;              // the next kernel may only start when the one before this is complete
+  LetGo let_go;
 };
 
 // A wait that first polls the barrier for a few microseconds (a thread parked in try_wait takes a
@@ -200,7 +200,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   tc_fence_after_sync();
   const uint32_t tmem = ctl->tmem_base;
   if (!p.beside) grid_dep_wait();
-  if (!p.hold) grid_dep_launch();
+  if (p.let_go == kAtStart) grid_dep_launch();
 
   auto decode = [&](int4 u) {
     Unit x;
@@ -271,6 +271,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         ++nu;
         u = u_next;
       }
+      if (p.let_go == kAtEnd) grid_dep_launch();
     }
   } else if (warp == kWarpIo) {
     // ------------------------------------------------------------ Q loads and output stores
@@ -297,7 +298,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       load_next();
       load_next();
       load_next();
-      if (p.hold) {
+      if (p.let_go == kWhenPreviousDone) {
         grid_dep_wait();
         grid_dep_launch();
       }
@@ -605,7 +606,7 @@ bool tc_window_supported(int N, int d, int w, int dtype) {
 
 cudaError_t launch_window_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
                              int w, int fwd, float scale, int layout, int h_begin, int h_count, WsHeader* ws,
-                             cudaStream_t stream, Link link, bool hold) {
+                             cudaStream_t stream, Link link, LetGo let_go) {
   if (h_count <= 0) return cudaSuccess;
   CUtensorMap mq, mk, mv, mo;
   if (!make_qkv_tensor_map(&mq, q, B, H, N, d, layout, 128) || !make_qkv_tensor_map(&mk, k, B, H, N, d, layout, 64) ||
@@ -628,7 +629,7 @@ cudaError_t launch_window_tc(const void* q, const void* k, const void* v, void* 
   p.status = &ws->status;
   p.ticket = &ws->ticket;  // zeroed with the workspace header by the caller
   p.beside = link == kBeside;
-  p.hold = hold;
+  p.let_go = let_go;
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = device_info(&dev, &sms)) != cudaSuccess) return e;
@@ -638,7 +639,7 @@ cudaError_t launch_window_tc(const void* q, const void* k, const void* v, void* 
   auto launch = [&](auto kern, int smem) -> cudaError_t {
     cudaError_t err = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, smem);
     if (err != cudaSuccess) return err;
-    return launch_link(link, kern, grid, dim3(kThreads), smem, stream, mq, mk, mv, mo, p);
+    return launch_link(kern, grid, dim3(kThreads), smem, stream, mq, mk, mv, mo, p);
   };
   if (d == 64)
     return fwd > 0 ? launch(window_tc_kernel<64, true>, WinSmem<64>::kBytes)

@@ -994,6 +994,58 @@ def test_self_layer_sums_and_readout_cut_differently(B, H, N, d, w, h0):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_calls_between_other_work_of_a_stream(dtype):
+    """Inputs written by copies, fills and kernels right before a call, outputs read right behind it, layers, decoding and other
+    work in turn, another stream joined in between: eagerly and replayed from a graph the bits of calls made one by one."""
+    B, H, N, d, w, h0 = 2, 6, 300, 64, 50, 2
+    t = torch.float32 if dtype == "f32" else torch.bfloat16
+    src = [dev(*synth.qkv(B, H, N, d, dtype, seed=s)) for s in range(4)]
+    step = [[x[:, :, 7].contiguous() for x in s] for s in src]
+    q, k, v = (torch.empty_like(src[0][0]) for _ in range(3))
+    qs, ks, vs = (torch.empty_like(step[0][0]) for _ in range(3))
+    st = gf.DecodeState(B, H, d, w, h0, t)
+    pos = torch.zeros(B, dtype=torch.int64, device="cuda")
+    ws = gf.Workspace.for_problem(B, H, N, d, w, 0, gf.GF_F32 if dtype == "f32" else gf.GF_BF16)
+    side = torch.cuda.Stream()
+    calls = [lambda: gf.hybrid_attn(q, k, v, w, h_sparse=h0, ws=ws, state_out=st), lambda: gf.decode_step_ragged(qs, ks, vs, st, pos),
+             lambda: gf.hybrid_attn_self(q, k, v, w, h_sparse=h0, ws=ws), lambda: gf.window_attn(q, k, v, w, ws=ws),
+             lambda: gf.decode_step_ragged(qs, ks, vs, st, pos), lambda: gf.causal_linear_attn(q, k, v, ws=ws)]
+
+    def run(between):
+        outs = []
+        pos.fill_(N)
+        for i, f in enumerate(calls):
+            for a, b in zip((q, k, v, qs, ks, vs), [*src[i % 4], *step[i % 4]]):
+                a.copy_(b) if i % 2 else torch.mul(b, 1, out=a)
+            if i == 3:  # v of this call comes from another stream
+                side.wait_stream(torch.cuda.current_stream())
+                with torch.cuda.stream(side):
+                    v.copy_(src[0][2])
+                torch.cuda.current_stream().wait_stream(side)
+            between()
+            o = f()
+            outs.append(o.clone())
+            if i % 3 == 0:
+                o.zero_()
+        return outs + [x.clone() for x in (st.k_cache, st.v_cache, st.S, st.z, pos)]
+
+    want = run(torch.cuda.synchronize)
+    for got in (run(lambda: None), run(lambda: None)):
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        got = run(lambda: None)
+    for _ in range(2):
+        for x in got:
+            x.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("dtype,layout", [("bf16", 0), ("bf16", 1), ("f32", 0)])
 def test_calls_made_natively_and_through_ctypes_are_the_same(monkeypatch, dtype, layout):
     """Every call with usual arguments, with ones that the native module leaves to ctypes (numpy integers, a stream object, an
