@@ -83,8 +83,8 @@ static_assert(sizeof(WinCtl) <= 640 && alignof(WinCtl) <= 16, "control block");
 static_assert(WinSmem<128>::kBytes <= 227 * 1024, "shared memory of one SM");
 
 struct WinParams {
-  int N, w, tiles_back;  // tiles_back = number of key tiles before the diagonal one
-  int fwd, tiles_fwd;    // keys after the query it may see (0: causal; w - 1: two-sided) and the tiles they span
+  int N, w, nkh;  // nkh: half tiles of keys
+  int fwd;        // keys after the query it may see (0: causal; w - 1: two-sided)
   float scale_log2;
   int h_begin, h_count, nqt, npair, total;  // work units: (batch, head, pair of query tiles), pair fastest
   unsigned int* status;
@@ -126,13 +126,17 @@ __device__ __forceinline__ void publish(uint32_t* counter, uint32_t value) {
   *reinterpret_cast<volatile uint32_t*>(counter) = value;
 }
 
-// A unit: query tiles qtA (and qtA + 1 when nt == 2); tile x walks the key tiles f[x] .. l[x].
+// A unit: query tiles qtA (and qtA + 1 when nt == 2); tile x walks the half tiles of 64 keys f[x] .. l[x], those in which one of
+// its rows sees a key.  (In whole key tiles a window of 32 or 64 keys took four half tiles a tile instead of three, two-sided
+// six instead of four: 64 x 3 heads of 4096 tokens, d = 64, w = 32 101 and 92 us, 4 x 13 of 3000, d = 128, w = 50 38.7 and 35.3,
+// 13 of 10 000, d = 64, w = 300 36.6 and 35.0; no difference for multiples of 128.)
 struct Unit {
   int h, b, qtA, nt;
   int f[2], l[2];
   // half tiles of tile x: number `off` of the unit's half tiles on, n_sub of them
-  __device__ __forceinline__ int off(int x) const { return 2 * (f[x] - f[0]); }
-  __device__ __forceinline__ int n_sub(int x) const { return x < nt ? 2 * (l[x] - f[x] + 1) : 0; }
+  __device__ __forceinline__ int off(int x) const { return f[x] - f[0]; }
+  __device__ __forceinline__ int n_sub(int x) const { return x < nt ? l[x] - f[x] + 1 : 0; }
+  __device__ __forceinline__ int n_half() const { return (nt == 2 ? l[1] : l[0]) - f[0] + 1; }
 };
 
 template <int D, bool kTwoSided>
@@ -211,9 +215,9 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
 #pragma unroll
     for (int t = 0; t < 2; ++t) {
       const int qt = x.qtA + t;
-      x.f[t] = (qt - p.tiles_back) > 0 ? (qt - p.tiles_back) : 0;
-      // kTwoSided: the tiles after the diagonal one that the window reaches, up to the sequence end
-      x.l[t] = !kTwoSided ? qt : ((qt + p.tiles_fwd) < p.nqt ? (qt + p.tiles_fwd) : p.nqt - 1);
+      const int first = (qt * 128 - p.w + 1) >> 6, last = (kTwoSided ? qt * 128 + 127 + p.fwd : qt * 128 + 127) >> 6;
+      x.f[t] = first > 0 ? first : 0;
+      x.l[t] = last < p.nkh ? last : p.nkh - 1;  // (up to the sequence end)
     }
     return x;
   };
@@ -236,12 +240,11 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         // draw the next ticket now; its value is needed once this unit's first loads are out
         const unsigned int t_next = atomicAdd(p.ticket, 1u);
         int4 u_next = make_int4(-1, 0, 0, 0);
-        const int g0 = x.f[0], g1 = x.nt == 2 ? x.l[1] : x.l[0];
         // A slot is released by two arrivals.  For a stream that has no use for a half tile the producer arrives itself,
         // so that the stream need not wait until it has landed.
-        const int off1 = x.off(1), n0 = x.n_sub(0), n1 = x.n_sub(1);
-        for (int hg = 2 * g0; hg <= 2 * g1 + 1; ++hg, ++kt) {  // kt counts half tiles here
-          const int m = hg - 2 * g0;
+        const int off1 = x.off(1), n0 = x.n_sub(0), n1 = x.n_sub(1), n_half = x.n_half();
+        for (int m = 0; m < n_half; ++m, ++kt) {  // kt counts half tiles here
+          const int hg = x.f[0] + m;
           const bool unused = m >= n0 || m < off1 || m >= off1 + n1;  // by one of the streams
           const uint32_t slot = kt % ST, use = kt / ST;
           if (use >= 1 && !mbar_wait(&ctl->k_empty[slot], (use - 1) & 1, p.status, 10)) { ok = false; break; }
@@ -256,7 +259,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
             tma_load_4d(sV + slot * SM::kHalf + c * 8192, &mv, &ctl->v_full[slot], c * 64, hg * 64, x.h, x.b);
           if (unused) mbar_arrive(&ctl->v_empty[slot]);
           publish(&ctl->v_issued, kt + 1);
-          if (hg == 2 * g0) {  // the other roles learn of the next unit early (its Q is requested ahead)
+          if (m == 0) {  // the other roles learn of the next unit early (its Q is requested ahead)
             if (t_next < (unsigned int)(p.total - (int)gridDim.x)) u_next = split((int)(gridDim.x + t_next));
             const uint32_t use_next = (nu + 1) / kUnitRing;
             if (use_next >= 1 && !mbar_wait(&ctl->unit_read[(nu + 1) % kUnitRing], (use_next - 1) & 1, p.status, 12)) {
@@ -326,7 +329,7 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
   } else if (warp == kWarpMma || warp == kWarpMma + 1) {
     // ------------------------------------------------------------ MMA issuers
     // One issuing thread per query tile of the pair ("stream").  A stream's products are, in order,
-    // S(0), S(1), then P V(j) followed by S(j + 2): S buffer j & 1 is free again once P V(j) has been
+    // S(0), S(1), then P V(j) followed by S(j + 2): the S buffer of j is free again once P V(j) has been
     // issued, because the tensor core runs one thread's products in issue order.  The two streams
     // meet only in the ring: a half tile goes back to the producer when both streams are done
     // with it (or the producer has arrived for a stream that has no use for it), and stream 1, whose window starts one key
@@ -353,14 +356,14 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
           if (u.x < 0) break;
           unit_read(nu);
           const Unit x = decode(u);
-          const uint32_t n_half = 2 * (uint32_t)((x.nt == 2 ? x.l[1] : x.l[0]) - x.f[0] + 1);
+          const uint32_t n_half = (uint32_t)x.n_half();
           const int n_sub = x.n_sub(t);
           const uint32_t rbase = kt + (t ? (uint32_t)x.off(1) : 0u);  // ring number of the stream's first half tile
           const uint32_t qbuf = (qn + t) % 3;
           const uint64_t dq = umma_smem_desc(aX + qbuf * SM::kTile, 16, 1024);
           for (int m = 0; m < n_sub + 2 && n_sub > 0; ++m) {
             if (m >= 2) {  // O += P V of half tile jj
-              const int jj = m - 2, half = jj & 1;
+              const int jj = m - 2, half = (sub + jj) & 1;
               const uint32_t n = rbase + (uint32_t)jj, slot = n % ST;
               if (!landed(&ctl->v_issued, ctl->v_full, n, 23)) return;
               if (!mbar_wait_hot(&ctl->p_full[t][half], ((sub + jj) >> 1) & 1, p.status, 22)) return;
@@ -376,8 +379,8 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
               umma_commit(&ctl->pv_done[t]);
               if (jj == n_sub - 1) umma_commit(&ctl->o_full[t]);
             }
-            if (m < n_sub) {  // S of half tile m into S buffer m & 1
-              const int half = m & 1;
+            if (m < n_sub) {  // S of half tile m into the S buffer that PV(m - 2), or the tile before, has left
+              const int half = (sub + m) & 1;
               const uint32_t n = rbase + (uint32_t)m, slot = n % ST;
               if (t == 1) {  // bounded: stream 0's next S must lie behind this half tile
                 if (*front <= n) {
@@ -442,13 +445,13 @@ window_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
       if (t >= x.nt) continue;
       const int i0 = (x.qtA + t) * 128, i = i0 + r;
       const int f_t = t ? x.f[1] : x.f[0], l_t = t ? x.l[1] : x.l[0];  // (no run-time index: the unit stays in registers)
-      const int n_sub = 2 * (l_t - f_t + 1);
+      const int n_sub = l_t - f_t + 1;
       const int i_first = i0 + quarter * 32;  // the warp's first row
       float m_ref = -INFINITY;  // reference maximum the stored O and l are relative to (same in both halves)
       float l = 0.f;            // sum over this thread's columns
-      for (int j = 0; j < n_sub; ++j, ++sub) {
-        const int half = j & 1;  // which 64 keys of the key tile; also the S buffer
-        const int j0 = (f_t + (j >> 1)) * 128 + half * 64 + hh * 32;  // first key of this thread's 32 columns
+      int half = sub & 1;       // the S buffer: half tiles take turns, also from one query tile to the next
+      for (int j = 0; j < n_sub; ++j, ++sub, half ^= 1) {
+        const int j0 = (f_t + j) * 64 + hh * 32;  // first key of this thread's 32 columns
         const uint32_t tS = tmem + t * 128 + half * 64 + hh * 32 + lane_off;
         // valid key columns of this row among its 32: [lo, hi]; over the warp's 32 rows lo and hi move
         // by 31, so the block is classified per warp: nothing visible (costs nothing), all visible to
@@ -615,9 +618,8 @@ cudaError_t launch_window_tc(const void* q, const void* k, const void* v, void* 
   WinParams p;
   p.N = N;
   p.w = w;
-  p.tiles_back = (w - 1 + 127) / 128;
+  p.nkh = (N + 63) / 64;
   p.fwd = fwd;
-  p.tiles_fwd = (fwd + 127) / 128;
   p.scale_log2 = scale * kLog2e;
   p.h_begin = h_begin;
   p.h_count = h_count;

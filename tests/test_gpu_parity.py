@@ -994,6 +994,22 @@ def test_self_layer_sums_and_readout_cut_differently(B, H, N, d, w, h0):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("N", [1, 63, 65, 128, 193, 300, 577, 1000])
+def test_windows_that_start_or_end_in_either_half_of_a_key_tile(N, d):
+    """Odd and even numbers of half tiles of keys per query tile, one-sided and two-sided, several units per CTA."""
+    B, H = 40, 4
+    q, k, v = synth.qkv(B, H, N, d, "bf16", seed=600 + N)
+    qd, kd, vd = dev(q, k, v)
+    for w in (1, 2, 33, 64, 65, 66, 128, 129, 193, 194, 321):
+        if w > N + 64:
+            continue
+        for f, ref in ((gf.window_attn, oracle.window_attn), (gf.window_attn_self, oracle.window_attn_self)):
+            o = f(qd, kd, vd, w)
+            assert_parity(f64(o[-1:]), ref(f64(q[-1:]), f64(k[-1:]), f64(v[-1:]), w), "bf16", f"{f.__name__} N={N} w={w} d={d}")
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("dtype", ["bf16", "f32"])
 def test_calls_between_other_work_of_a_stream(dtype):
     """Inputs written by copies, fills and kernels right before a call, outputs read right behind it, layers, decoding and other
