@@ -241,7 +241,7 @@ __device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, in
       for (int n = 0; n < 4; ++n)
 #pragma unroll
         for (int e = 0; e < 4; ++e) s[n][e] = 0.f;
-#pragma unroll 1
+#pragma unroll(D == 64 ? NT / 2 : 1)  // (212 -> 208 us for 96 chains of 2048; d = 128 has no registers left: 470, and 492 unrolled)
       for (int kk = 0; kk < NT; kk += 2) {
         Split a[2][4];
         rows_a(a[0], Qs + (16 * warp + g) * LD + 8 * kk + 2 * t, 8 * LD);
@@ -435,7 +435,7 @@ template <int D, bool kSane>
 __device__ __forceinline__ void add_outer(const float* Ks, const float* Vs, State<D>& S) {
   constexpr int LD = LinT<D>::LD;
   const Lane l = lane_of();
-#pragma unroll 2
+#pragma unroll(D == 64 ? 4 : 2)
   for (int kk = 0; kk < kC / 8; ++kk) {
     const float *v = Vs + (8 * kk + l.t) * kLdV + l.c0 + l.g, *k = Ks + (8 * kk + l.t) * LD + l.half * (D / 2) + l.g;
     const Split a[4] = {split_value<kSane>(v[0]), split_value<kSane>(v[8]), split_value<kSane>(v[4 * kLdV]),
@@ -482,15 +482,15 @@ __device__ __forceinline__ void readout(const float* Qs, const float* Vs, const 
     }
   }
 }
-// The six tiles of P that are not all masked, 16 rows x 8 keys each, by six warps; phi(Q) z by the other two.
+// The six tiles of P that are not all masked, 16 rows x 8 keys each, by six warps ...
 template <int D>
-__device__ __forceinline__ void score_block(const float* Qs, const float* Ks, const float* zs, float* Ps, float* qz_s) {
+__device__ __forceinline__ void score_block(const float* Qs, const float* Ks, float* Ps) {
   constexpr int LD = LinT<D>::LD;
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, warp = threadIdx.x >> 5;
   if (warp < 6) {
     const int m = warp < 2 ? 0 : 1, n = warp < 2 ? warp : warp - 2;
     float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};  // (two sums: half the chain)
-#pragma unroll 4
+#pragma unroll(D == 64 ? 8 : 4)
     for (int kk = 0; kk < D / 8; ++kk) {
       Split a[4], b0, b1;
       lds_split2(b0, b1, Ks + (8 * n + g) * LD + 8 * kk + 2 * t);
@@ -503,7 +503,13 @@ __device__ __forceinline__ void score_block(const float* Qs, const float* Ks, co
       store2(Ps + row * kLdP + key, key <= row ? s[0][2 * r] + s[1][2 * r] : 0.f,
              key + 1 <= row ? s[0][2 * r + 1] + s[1][2 * r + 1] : 0.f);
     }
-  } else {
+  }
+}
+// ... and phi(Q) z by the other two.
+template <int D>
+__device__ __forceinline__ void dot_z(const float* Qs, const float* zs, float* qz_s) {
+  constexpr int LD = LinT<D>::LD;
+  if (threadIdx.x >= 192) {
     const int row = (threadIdx.x - 192) >> 1, part = threadIdx.x & 1;
     float d[2] = {0.f, 0.f};
 #pragma unroll 4
@@ -700,6 +706,17 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
     rk.load(k, p.st.n, n_begin, n_end, tid);
     rv.load(v, p.st.n, n_begin, n_end, tid);
   };
+  // phi(Q), phi(K) and V of the block at n0 into shared memory, the next block's on their way
+  auto store_block = [&](int n0) {
+    rq.store_phi(Qs, LD, n0, n_end, tid);
+    rk.store_phi(Ks, LD, n0, n_end, tid);
+    rv.store(Vs, kLdV, tid);
+    __syncthreads();  // (also: every thread has read its state out of the rows this CTA writes)
+    rq.load(q, p.st.n, n0 + kC, n_end, tid);
+    rk.load(k, p.st.n, n0 + kC, n_end, tid);
+    rv.load(v, p.st.n, n0 + kC, n_end, tid);
+  };
+  Ps[(tid >> 4) * kLdP + 16 + (tid & 15)] = 0.f;  // (masked, and nobody computes them)
   State<D> S;
   if constexpr (kCluster) {
     auto cluster = cooperative_groups::this_cluster();
@@ -712,11 +729,16 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
       for (int n = 0; n < D / 16; ++n) frag[n * kLinThreads] = make_float4(S[n][0], S[n][1], S[n][2], S[n][3]);
       if (tid < D) zs[tid] = z;
     }
-    load_first();  // (under way while the sums are exchanged)
+    load_first();
     const bool from_caller = S_io != nullptr && !p.zero_init;
     for_state<D>(S, [&](int a, int c, float& x) { x = from_caller ? S_io[(sidx * D + a) * D + col0 + c] : 0.f; });
     z = (from_caller && tid < D) ? p.z_io[sidx * D + tid] : 0.f;
-    cluster.sync();
+    // the first block's scores while the sums of the others arrive (a layer of 8 x 12 chains of 300 tokens 35.5 -> 34.1 us,
+    // one of 256 9.4 -> 9.0)
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    store_block(n_begin);
+    score_block<D>(Qs, Ks, Ps);
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     // running sums: of S[n] by segment n mod G, of z by segment 0, for all segments, read and put back in place
     const int rank0 = (int)cluster.block_rank() - g;  // first segment of this slice
     for (int n = g; n < D / 16; n += sg.G) {
@@ -757,6 +779,7 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
       if (tid < D) z += zs[tid];
     }
     if (tid < D) zs[tid] = z;
+    __syncthreads();
   } else {
     load_first();
     const float* Sp = nullptr;  // row a of the starting state at Sp + a * stride
@@ -775,16 +798,12 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
     if (tid < D)
       zs[tid] = Sp == nullptr ? 0.f : zp != nullptr ? zp[tid] : Sp[(long long)(D + tid / kW) * stride + tid % kW];
   }
-  Ps[(tid >> 4) * kLdP + 16 + (tid & 15)] = 0.f;  // (masked, and nobody computes them)
   for (int n0 = n_begin; n0 < n_end; n0 += kC) {
-    rq.store_phi(Qs, LD, n0, n_end, tid);
-    rk.store_phi(Ks, LD, n0, n_end, tid);
-    rv.store(Vs, kLdV, tid);
-    __syncthreads();  // (also: every thread has read its state out of the rows this CTA writes)
-    rq.load(q, p.st.n, n0 + kC, n_end, tid);
-    rk.load(k, p.st.n, n0 + kC, n_end, tid);
-    rv.load(v, p.st.n, n0 + kC, n_end, tid);
-    score_block<D>(Qs, Ks, zs, Ps, qz_s);
+    if (!kCluster || n0 > n_begin) {
+      store_block(n0);
+      score_block<D>(Qs, Ks, Ps);
+    }
+    dot_z<D>(Qs, zs, qz_s);
     __syncthreads();
     {  // denominators: eight threads per row
       const int row = tid >> 3, part8 = tid & 7;
