@@ -305,7 +305,10 @@ struct OutCfg {
   static constexpr int kSb = 2 * kTile;   // bf16 totals [D rows][D columns] in 64-column boxes ...
   static constexpr int kZb = kSb + D * D * 2;  // ... followed by one more box: columns 0, 1 = hi(z), lo(z)
   static constexpr int kStage = kZb + kSbBox;  // two output tiles staged for the TMA store
-  static constexpr int kBytes = kStage + 2 * kTile + 1024;
+  // One CTA per SM, also at d = 64, where the tiles take 81 KB: its launch comes early, and CTAs that found room beside another
+  // one's (of either kernel: both take all of the tensor memory) waited for it while other SMs stood idle (160 chains of 4096
+  // tokens with random features: 74 us, 43 with this).
+  static constexpr int kTiles = kStage + 2 * kTile + 1024, kBytes = kTiles > 120 * 1024 ? kTiles : 120 * 1024;
   static constexpr int kAcc = D + 16;
   static constexpr uint32_t tQ = 0, tO = D;  // phi(Q): 2 x D/2 columns; O | den: 2 x (D + 16)
   static constexpr int kThreads = 15 * 32;
