@@ -940,17 +940,30 @@ int self_sum_segments(int nchains, int nch, int d, double beside_us) {
   return best_g;
 }
 
-// Whether whole chains go through linear_self_whole_kernel: its ceil(chains / CTAs) rounds of a whole chain each against
-// the three launches, whose work is spread evenly but costs a sixth more per chunk (its two halves do not run side by
-// side) and about nine chunks' time in launches and start-up.  Measured (us, whole | three launches): where the rule takes
-// whole chains 128 of 1024 tokens 20.5 | 30.8, 160 of 1024 29.2 | 41.0, 310 of 2048 74 | 89, 260 of 4096 110 | 126, 24 of 197
-// 10.3 | 19.7; where it takes three launches 40 of 2048 30.8 | 26.7, 160 of 4096 94.1 | 90.1, 160 of 8192 175 | 157, 150 of
-// 16 384 333 | 279.  It errs where the last round is thin or the chains are short: 160 of 2048 51.1 | 59.4, 200 of 4096
-// 97 | 101, 300 of 4096 139 | 152, all three in three launches.
-bool self_whole(int nchains, int nch, int d, int sms) {
+// Whether whole chains go through linear_self_whole_kernel, by estimates of both forms in microseconds, within 8 % of what was
+// measured over 20 to 640 chains of 1024 to 8192 tokens.
+// Whole: while a CTA reads one chain out it sums up its next, so R rounds of chains are R + 1 phases of nch chunks each; a chunk
+// takes 0.72 where few CTAs are at work, 0.92 where each has one chain in hand and 1.5, HBM's pace, where each has two.
+// Three launches: 1.83 a chunk of both passes, spread evenly, with one more chunk per segment, and 10 for their starts;
+// behind a pre-pass of random features 5 more and 0.15 a chunk.
+// Windowed heads add what they take of the whole device (beside_us); behind whole chains less what the SMs without a chain in the
+// last round leave idle, and up to 8 for coming late.
+// us, whole | three: where the rule takes whole chains 128 of 1024 tokens 20.5 | 30.8, 160 of 2048 48.2 | 50.5, 300 of 2048 69.7 |
+// 77.2, 448 of 4096 187 | 210, with windowed heads of w = 128 160 of 4096 96.7 | 106, 320 of 4096 166 | 204; where it takes three
+// launches 40 of 1536 22.4 | 17.6, 100 of 4096 55.6 | 53.4, 160 of 4096 90.5 | 76.4, 220 of 8192 192 | 186.
+bool self_whole(int nchains, int nch, int d, int sms, double beside_us, bool features) {
   if (d != WholeCfg::D) return false;
-  const double rounds = (double)((nchains + sms - 1) / sms) * nch;
-  return rounds <= 1.17 * nchains * nch / sms + 9.0;
+  const int rounds = (nchains + sms - 1) / sms, last = nchains - (rounds - 1) * sms;
+  auto chunk_us = [&](int streams) {  // (chains being summed up and chains being read out)
+    const double x = (double)streams / sms;
+    return x <= 1.0 ? 0.72 + 0.2 * x * x : 0.92 + 0.58 * (x - 1.0);
+  };
+  double whole = 5.0 + 2.0 * nch * chunk_us(last);
+  if (rounds > 1) whole = 5.0 + nch * (chunk_us(sms) + (rounds - 2) * chunk_us(2 * sms) + chunk_us(sms + last) + chunk_us(last));
+  const double work = (double)nchains * (nch + self_segments(nchains, nch)) / sms;
+  const double three = 10.0 + 1.83 * work + (features ? 5.0 + 0.15 * work : 0.0);
+  const double idle = (1.0 - (double)last / sms) * nch * chunk_us(last) * (rounds > 1 ? 1 : 2), late = 0.4 * beside_us;
+  return whole + (beside_us > idle ? beside_us - idle : 0.0) + (late < 8.0 ? late : 8.0) <= three + beside_us;
 }
 
 }  // namespace
@@ -988,7 +1001,7 @@ cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, v
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = device_info(&dev, &sms)) != cudaSuccess) return e;
-  const bool whole = self_whole(p.nchains, p.nch, d, sms);
+  const bool whole = self_whole(p.nchains, p.nch, d, sms, beside_us, features);
   auto cut = [&](int G) {
     p.G = G;
     p.seg_base = p.nch / G;

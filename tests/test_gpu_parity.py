@@ -1561,6 +1561,24 @@ def test_self_linear_heads_whole_chains(B, H, N, d, favor):
     assert_parity(f64(o[:, hs]), ref, "bf16", f"whole chains B={B} H={H} N={N} d={d}")
 
 
+@pytest.mark.parametrize("bnhd,favor", [(False, False), (True, False), (False, True)])
+@pytest.mark.parametrize("B,H,N,w,h0", [(80, 3, 1999, 33, 1), (20, 3, 1501, 33, 1), (18, 7, 2500, 900, 2), (3, 9, 4001, 64, 2)])
+def test_self_layer_of_some_rounds_of_chains(B, H, N, w, h0, bnhd, favor):
+    """More chains than CTAs with a thin last round, a few long ones, windowed heads that outlast them: whichever form the
+    size takes, the last batch row against the oracle and two calls alike."""
+    q, k, v = synth.qkv(B, H, N, 64, "bf16", seed=990 + N)
+    W = _proj(H - h0, 64, "bf16", 5) if favor else None
+    lay, args = gf.GF_BHND, dev(q, k, v)
+    if bnhd:
+        lay, args = gf.GF_BNHD, [x.transpose(1, 2).contiguous() for x in args]
+    run = lambda: gf.hybrid_attn_self(*args, w, h_sparse=h0, layout=lay, W=W.cuda() if favor else None)  # noqa: E731
+    o, again = run(), run()
+    assert torch.equal(o, again)
+    o = o[-1:].transpose(1, 2) if bnhd else o[-1:]
+    ref = oracle.hybrid_attn_self(f64(q[-1:]), f64(k[-1:]), f64(v[-1:]), w, h_sparse=h0, **({"W": f64(W)} if favor else {}))
+    assert_parity(f64(o), ref, "bf16", f"self layer B={B} H={H} N={N} bnhd={bnhd} favor={favor}")
+
+
 # ------------------------------------------------------------------ decode: both forms of the kernel, partial rounds of slots
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("B,H,d,w,h0,t0", [(1, 2, 64, 1, 1, 0), (1, 3, 128, 129, 2, 40), (2, 4, 64, 600, 2, 599), (2, 4, 64, 600, 2, 2000),
