@@ -157,7 +157,7 @@ favor_tc_kernel(const __grid_constant__ CUtensorMap mxq, const __grid_constant__
         const uint32_t s = n % NX;
         if (!mbar_wait(&staged[s], (n / NX) & 1, p.status, 905)) break;
         for (int c = 0; c < D / 64; ++c)
-          tma_store_4d(x.is_k ? &mfk : &mfq, sm + s * C::kTile + c * 16384, c * 64, x.i0, p.h_begin + x.hl, x.b);
+          tma_store_4d(x.is_k ? &mfk : &mfq, sm + s * C::kTile + c * 16384, c * 64, x.i0, x.hl, x.b);
         tma_store_commit();
         tma_store_wait_read<1>();  // the one before has been read out
         if (n >= 1) mbar_arrive(&x_free[(n - 1) % NX]);
@@ -246,8 +246,8 @@ cudaError_t launch_favor_features_tc(const void* q, const void* k, const void* W
   if (h_count <= 0) return cudaSuccess;
   CUtensorMap mxq, mxk, mw, mfq, mfk;
   if (!make_qkv_tensor_map(&mxq, q, B, H, N, d, layout, 128) || !make_qkv_tensor_map(&mxk, k, B, H, N, d, layout, 128) ||
-      !make_feature_tensor_map(&mfq, fq, B, H, N, d, h_begin, h_count, 128) ||
-      !make_feature_tensor_map(&mfk, fk, B, H, N, d, h_begin, h_count, 128) ||
+      !make_qkv_tensor_map(&mfq, fq, B, h_count, N, d, GF_BHND, 128) ||
+      !make_qkv_tensor_map(&mfk, fk, B, h_count, N, d, GF_BHND, 128) ||
       !make_qkv_tensor_map(&mw, W, 1, h_count, d, d, GF_BHND, d))  // [1, heads, d features, d inputs]: box of d rows
     return cudaErrorInvalidValue;
   FavorParams p;

@@ -541,7 +541,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
               if (!ok) break;
               mbar_arrive_expect_tx(&bar.ka_full[sa], C::kTile);
               for (int x = 0; x < D / 64; ++x)
-                tma_load_4d_hint(a_kslot(sa) + x * C::kBoxBytes, &mk, &bar.ka_full[sa], x * 64, n0, it.h, it.b,
+                tma_load_4d_hint(a_kslot(sa) + x * C::kBoxBytes, &mk, &bar.ka_full[sa], x * 64, n0, kId ? it.hl : it.h, it.b,
                                  kPark ? pol_stream : pol_keep);
               ++iss_a[sa];
               ++ta;
@@ -553,7 +553,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
               mbar_arrive_expect_tx(&bar.k_full[sc], C::kTile);
               for (int x = 0; x < D / 64; ++x)  // the phi(K) tile parked in the output rows, or K itself
                 tma_load_4d_hint(sK + sc * C::kTile + x * C::kBoxBytes, kPark ? &mo : &mk, &bar.k_full[sc], x * 64, n0,
-                                 it.h, it.b, pol_stream);
+                                 kId ? it.hl : it.h, it.b, pol_stream);
               ++iss_c[sc];
               ++nq;
             }
@@ -872,7 +872,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
     auto request_q = [&](int slot, const LinItem& w_it, int w_j) {
       mbar_arrive_expect_tx(&bar.q_full[slot], C::kTile);
       for (int x = 0; x < D / 64; ++x)
-        tma_load_4d_hint(q_box(slot, x), &mq, &bar.q_full[slot], x * 64, (w_it.c_begin + w_j) * 128, w_it.h, w_it.b,
+        tma_load_4d_hint(q_box(slot, x), &mq, &bar.q_full[slot], x * 64, (w_it.c_begin + w_j) * 128, kId ? w_it.hl : w_it.h, w_it.b,
                          l2_policy_evict_first());
     };
     if (tid == 6 * 32 && (int)blockIdx.x < p.nitems) {
@@ -880,7 +880,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
         const LinItem first = decode_item<D, kDirect>(p, blockIdx.x);
         mbar_arrive_expect_tx(&bar.q_full[0], C::kTile);
         for (int x = 0; x < D / 64; ++x)
-          tma_load_4d_hint(q_box(0, x), &mq, &bar.q_full[0], x * 64, first.c_begin * 128, first.h, first.b,
+          tma_load_4d_hint(q_box(0, x), &mq, &bar.q_full[0], x * 64, first.c_begin * 128, kId ? first.hl : first.h, first.b,
                            l2_policy_evict_first());
       } else {
         int w_item = blockIdx.x, w_j = 0;
@@ -1074,7 +1074,7 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__
                     fence_proxy_async_smem();
                     mbar_arrive_expect_tx(&bar.q_full[0], C::kTile);
                     for (int x = 0; x < D / 64; ++x)
-                      tma_load_4d_hint(q_box(0, x), &mq, &bar.q_full[0], x * 64, n_chunk * 128, nx.h, nx.b,
+                      tma_load_4d_hint(q_box(0, x), &mq, &bar.q_full[0], x * 64, n_chunk * 128, kId ? nx.hl : nx.h, nx.b,
                                        l2_policy_evict_first());
                   }
                 }
@@ -1444,11 +1444,12 @@ cudaError_t launch_linear_tc(const void* q, const void* k, const void* v, void* 
                              int split, int max_ctas, WsHeader* ws, cudaStream_t stream, Link link, LetGo let_go, bool shared,
                              const void* fq, const void* fk) {
   if (h_count <= 0) return cudaSuccess;
-  // fq, fk: feature tensors [B, h_count, N, d] that stand in for Q and K (feature map: identity)
+  // fq, fk: feature tensors [B, h_count, N, d] that stand in for Q and K (feature map: identity);
+  // their heads are counted from the first linear one
   const bool features = fq != nullptr;
   CUtensorMap mq, mk, mv, mo;
-  if (features ? (!make_feature_tensor_map(&mq, fq, B, H, N, d, h_begin, h_count, 128) ||
-                  !make_feature_tensor_map(&mk, fk, B, H, N, d, h_begin, h_count, 128))
+  if (features ? (!make_qkv_tensor_map(&mq, fq, B, h_count, N, d, GF_BHND, 128) ||
+                  !make_qkv_tensor_map(&mk, fk, B, h_count, N, d, GF_BHND, 128))
                : (!make_qkv_tensor_map(&mq, q, B, H, N, d, layout, 128) ||
                   !make_qkv_tensor_map(&mk, k, B, H, N, d, layout, 128)))
     return cudaErrorInvalidValue;

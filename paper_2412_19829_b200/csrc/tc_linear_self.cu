@@ -63,7 +63,7 @@ __device__ __forceinline__ bool wait_count(const unsigned int* counter, unsigned
 }
 
 struct SelfItem {
-  int chain, g, b, h, c_begin, nC;
+  int chain, g, b, hl, h, c_begin, nC;
 };
 
 __device__ __forceinline__ SelfItem self_item(const SelfParams& p, int item) {
@@ -71,7 +71,8 @@ __device__ __forceinline__ SelfItem self_item(const SelfParams& p, int item) {
   it.chain = item / p.G;
   it.g = item - it.chain * p.G;
   it.b = it.chain / p.h_count;
-  it.h = p.h_begin + (it.chain - it.b * p.h_count);
+  it.hl = it.chain - it.b * p.h_count;
+  it.h = p.h_begin + it.hl;
   it.c_begin = it.g * p.seg_base + (it.g < p.seg_rem ? it.g : p.seg_rem);
   it.nC = p.seg_base + (it.g < p.seg_rem ? 1 : 0);
   return it;
@@ -161,7 +162,7 @@ linear_self_reduce_kernel(const __grid_constant__ CUtensorMap mk, const __grid_c
           if (nk >= KS && !mbar_wait(&k_free[sk], ((nk / KS) + 1) & 1, p.status, 700)) { ok = false; break; }
           mbar_arrive_expect_tx(&k_full[sk], C::kTile);
           for (int x = 0; x < D / 64; ++x)
-            tma_load_4d_hint(sK + sk * C::kTile + x * kBox, &mk, &k_full[sk], x * 64, n0, it.h, it.b, pol);
+            tma_load_4d_hint(sK + sk * C::kTile + x * kBox, &mk, &k_full[sk], x * 64, n0, kId ? it.hl : it.h, it.b, pol);
           ++nk;
           if (nv >= VS && !mbar_wait(&v_free[sv], ((nv / VS) + 1) & 1, p.status, 701)) { ok = false; break; }
           mbar_arrive_expect_tx(&v_full[sv], C::kTile);
@@ -371,7 +372,7 @@ linear_self_readout_kernel(const __grid_constant__ CUtensorMap mq, const __grid_
           if (nq >= 2 && !mbar_wait(&q_free[s], ((nq >> 1) + 1) & 1, p.status, 800)) { ok = false; break; }
           mbar_arrive_expect_tx(&q_full[s], C::kTile);
           for (int x = 0; x < D / 64; ++x)
-            tma_load_4d_hint(sQ + s * C::kTile + x * kBox, &mq, &q_full[s], x * 64, (it.c_begin + j) * 128, it.h, it.b,
+            tma_load_4d_hint(sQ + s * C::kTile + x * kBox, &mq, &q_full[s], x * 64, (it.c_begin + j) * 128, kId ? it.hl : it.h, it.b,
                              pol);
         }
       }
@@ -659,7 +660,7 @@ linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_co
             const uint32_t sk = n % KS, sv = n % VS;
             if (n >= KS && !mbar_wait(&k_free[sk], ((n / KS) + 1) & 1, p.status, 900)) { ok = false; break; }
             mbar_arrive_expect_tx(&k_full[sk], C::kTile);
-            tma_load_4d_hint(sm + C::kK + sk * C::kTile, &mk, &k_full[sk], 0, j * 128, it.h, it.b, pol);
+            tma_load_4d_hint(sm + C::kK + sk * C::kTile, &mk, &k_full[sk], 0, j * 128, kId ? it.hl : it.h, it.b, pol);
             if (n >= VS && !mbar_wait(&v_free[sv], ((n / VS) + 1) & 1, p.status, 901)) { ok = false; break; }
             mbar_arrive_expect_tx(&v_full[sv], C::kTile);
             tma_load_4d_hint(sm + sv * kBox, &mv, &v_full[sv], 0, j * 128, it.h, it.b, pol);
@@ -667,7 +668,7 @@ linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_co
             const uint32_t s = n & 1;
             if (n >= 2 && !mbar_wait(&q_free[s], ((n >> 1) + 1) & 1, p.status, 902)) { ok = false; break; }
             mbar_arrive_expect_tx(&q_full[s], C::kTile);
-            tma_load_4d_hint(sm + C::kQ + s * C::kTile, &mq, &q_full[s], 0, j * 128, it.h, it.b, pol);
+            tma_load_4d_hint(sm + C::kQ + s * C::kTile, &mq, &q_full[s], 0, j * 128, kId ? it.hl : it.h, it.b, pol);
           }
         }
       }
@@ -982,11 +983,12 @@ cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, v
                                   cudaStream_t stream, const std::function<cudaError_t(LetGo)>& beside, double beside_us, const void* fq,
                                   const void* fk) {
   if (h_count <= 0) return beside(kAtEnd);
-  // fq, fk: feature tensors [B, h_count, N, d] that stand in for Q and K (feature map: identity)
+  // fq, fk: feature tensors [B, h_count, N, d] that stand in for Q and K (feature map: identity);
+  // their heads are counted from the first linear one
   const bool features = fq != nullptr;
   CUtensorMap mq, mk, mv, mo;
-  if (features ? (!make_feature_tensor_map(&mq, fq, B, H, N, d, h_begin, h_count, 128) ||
-                  !make_feature_tensor_map(&mk, fk, B, H, N, d, h_begin, h_count, 128))
+  if (features ? (!make_qkv_tensor_map(&mq, fq, B, h_count, N, d, GF_BHND, 128) ||
+                  !make_qkv_tensor_map(&mk, fk, B, h_count, N, d, GF_BHND, 128))
                : (!make_qkv_tensor_map(&mq, q, B, H, N, d, layout, 128) ||
                   !make_qkv_tensor_map(&mk, k, B, H, N, d, layout, 128)))
     return cudaErrorInvalidValue;
