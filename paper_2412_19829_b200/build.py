@@ -63,26 +63,29 @@ def build(force: bool = False, verbose: bool = False) -> str:
     flags = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC] + ARCH
     if verbose:
         flags += ["-Xptxas", "-v"]
-    procs = []
-    objs = []
-    for src in _sources():
-        obj = os.path.join(objdir, os.path.basename(src)[:-3] + ".o")
-        objs.append(obj)
-        procs.append((src, subprocess.Popen([nvcc, "-c", src, "-o", obj] + flags,
-                                            stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
-    procs.append(("fastcall.cpp", _build_fastcall(FASTCALL + f".{os.getpid()}.tmp")))
-    failed = False
-    for src, p in procs:
-        out, _ = p.communicate()
-        if out.strip() and (verbose or p.returncode != 0):
-            print(out, file=sys.stderr)
-        failed |= p.returncode != 0
-    if failed:
-        raise RuntimeError("nvcc failed")
-    tmp = LIB + f".{os.getpid()}.tmp"
-    subprocess.check_call([nvcc, "-shared", "-o", tmp] + objs + ARCH + ["-cudart", "static"])
-    os.replace(tmp, LIB)
-    os.replace(FASTCALL + f".{os.getpid()}.tmp", FASTCALL)
+    objs = [os.path.join(objdir, os.path.basename(src)[:-3] + ".o") for src in _sources()]
+    # (linked beside the objects, which git ignores, and moved into place when complete)
+    lib_tmp, fast_tmp = (os.path.join(objdir, f"{os.path.basename(x)}.{os.getpid()}.tmp") for x in (LIB, FASTCALL))
+    try:
+        procs = [(src, subprocess.Popen([nvcc, "-c", src, "-o", obj] + flags,
+                                        stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True))
+                 for src, obj in zip(_sources(), objs)]
+        procs.append(("fastcall.cpp", _build_fastcall(fast_tmp)))
+        failed = False
+        for src, p in procs:
+            out, _ = p.communicate()
+            if out.strip() and (verbose or p.returncode != 0):
+                print(out, file=sys.stderr)
+            failed |= p.returncode != 0
+        if failed:
+            raise RuntimeError("nvcc failed")
+        subprocess.check_call([nvcc, "-shared", "-o", lib_tmp] + objs + ARCH + ["-cudart", "static"])
+        os.replace(lib_tmp, LIB)
+        os.replace(fast_tmp, FASTCALL)
+    finally:
+        for x in (lib_tmp, fast_tmp):
+            if os.path.exists(x):
+                os.remove(x)
     return LIB
 
 
