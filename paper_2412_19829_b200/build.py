@@ -30,13 +30,29 @@ def _sources():
     return [os.path.join(CSRC, s) for s in SOURCES if os.path.exists(os.path.join(CSRC, s))]
 
 
+def _older(target: str, deps) -> bool:
+    return not os.path.exists(target) or any(os.path.getmtime(p) > os.path.getmtime(target) for p in deps)
+
+
 def _stale() -> bool:
-    if not (os.path.exists(LIB) and os.path.exists(FASTCALL)):
-        return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(FASTCALL))
-    deps = _sources() + [os.path.join(CSRC, "fastcall.cpp")] + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
-    deps += [os.path.join(INCLUDE, f) for f in os.listdir(INCLUDE)]
-    return any(os.path.getmtime(p) > t for p in deps)
+    headers = [os.path.join(INCLUDE, f) for f in os.listdir(INCLUDE)]
+    return (_older(LIB, _sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))] + headers)
+            or _older(FASTCALL, [os.path.join(CSRC, "fastcall.cpp")] + headers) or _fastcall_built_for() != fastcall_target())
+
+
+def fastcall_target() -> str:
+    """What the module is built against, which it is no good without."""
+    import torch
+
+    return f"{sys.implementation.cache_tag}, torch {torch.__version__}"
+
+
+def _fastcall_built_for() -> str:
+    try:
+        with open(os.path.join(HERE, "build", "_fastcall.target")) as f:
+            return f.read()
+    except OSError:
+        return ""
 
 
 def _build_fastcall(out: str) -> subprocess.Popen:
@@ -48,7 +64,8 @@ def _build_fastcall(out: str) -> subprocess.Popen:
     cuda = os.path.dirname(os.path.dirname(_nvcc()))
     inc = [INCLUDE, sysconfig.get_paths()["include"], os.path.join(root, "include"),
            os.path.join(root, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
-    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}"]
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           f'-DGF_BUILT_FOR="{fastcall_target()}"']
     cmd += [x for i in inc for x in ("-I", i)] + [os.path.join(CSRC, "fastcall.cpp"), "-o", out]
     cmd += ["-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda", "-ldl"]
     return subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
@@ -70,18 +87,28 @@ def build(force: bool = False, verbose: bool = False) -> str:
         procs = [(src, subprocess.Popen([nvcc, "-c", src, "-o", obj] + flags,
                                         stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True))
                  for src, obj in zip(_sources(), objs)]
-        procs.append(("fastcall.cpp", _build_fastcall(fast_tmp)))
+        # The library needs neither torch nor g++, and binding.py does without the module.
+        try:
+            fast = _build_fastcall(fast_tmp)
+        except (ImportError, OSError) as e:
+            fast = None
+            print(f"_fastcall.so not built: {e}", file=sys.stderr)
         failed = False
-        for src, p in procs:
+        for src, p in procs + ([("fastcall.cpp", fast)] if fast else []):
             out, _ = p.communicate()
             if out.strip() and (verbose or p.returncode != 0):
                 print(out, file=sys.stderr)
-            failed |= p.returncode != 0
+            failed |= p.returncode != 0 and p is not fast
         if failed:
             raise RuntimeError("nvcc failed")
         subprocess.check_call([nvcc, "-shared", "-o", lib_tmp] + objs + ARCH + ["-cudart", "static"])
         os.replace(lib_tmp, LIB)
-        os.replace(fast_tmp, FASTCALL)
+        if fast is not None and fast.returncode == 0:
+            os.replace(fast_tmp, FASTCALL)
+            with open(os.path.join(objdir, "_fastcall.target"), "w") as f:
+                f.write(fastcall_target())
+        elif os.path.exists(FASTCALL):  # (made for another library)
+            os.remove(FASTCALL)
     finally:
         for x in (lib_tmp, fast_tmp):
             if os.path.exists(x):

@@ -266,5 +266,7 @@ PyMODINIT_FUNC PyInit__fastcall(void) {
     PyErr_SetString(PyExc_ImportError, "libgformer.so beside _fastcall.so cannot be loaded, or is older than it");
     return nullptr;
   }
-  return PyModule_Create(&module);
+  PyObject* m = PyModule_Create(&module);
+  if (m != nullptr && PyModule_AddStringConstant(m, "built_for", GF_BUILT_FOR) != 0) Py_CLEAR(m);
+  return m;
 }

@@ -1,10 +1,14 @@
 """The build's host logic, with compilers that only pretend: what it leaves behind and what it goes on without."""
+import importlib
 import os
 import stat
 import sys
+import types
 
 import pytest
+import torch
 
+from paper_2412_19829_b200 import binding as gf
 from paper_2412_19829_b200 import build as gf_build
 
 FAKE = """#!{python}
@@ -60,3 +64,41 @@ def test_a_build_puts_both_files_in_place(tree):
     assert gf_build.build(force=True) == gf_build.LIB
     assert os.path.exists(gf_build.LIB) and os.path.exists(gf_build.FASTCALL) and _left_behind(root) == []
     assert not gf_build._stale()
+
+
+def test_the_library_is_built_where_the_module_of_the_binding_cannot_be(tree):
+    tree()
+    gf_build.build(force=True)
+    root = tree("fastcall.cpp")
+    assert gf_build.build(force=True) == gf_build.LIB
+    assert os.path.exists(gf_build.LIB) and _left_behind(root) == []
+    assert not os.path.exists(gf_build.FASTCALL)  # (no module of an earlier library beside this one)
+    assert gf_build._stale()
+
+
+def test_a_module_built_for_another_torch_is_stale(tree, monkeypatch):
+    tree()
+    gf_build.build(force=True)
+    assert not gf_build._stale()
+    monkeypatch.setattr(torch, "__version__", "9.9.9")
+    assert gf_build._stale()
+
+
+@pytest.mark.parametrize("case", ["missing", "other torch"])
+def test_calls_go_through_ctypes_where_the_module_cannot_be_used(case, monkeypatch):
+    real = importlib.import_module
+
+    def fake(name, package=None):
+        if name != "._fastcall":
+            return real(name, package)
+        if case == "missing":
+            raise ImportError("no module")
+        return types.SimpleNamespace(built_for="another")
+
+    monkeypatch.setattr(gf, "_fast", None)
+    monkeypatch.setattr(importlib, "import_module", fake)
+    x = torch.zeros(1, 1, 4, 64)
+    with pytest.warns(UserWarning, match="through ctypes"), pytest.raises(ValueError, match="CUDA tensors"):
+        gf.window_attn(x, x, x, 4)
+    with pytest.raises(ValueError, match="CUDA tensors"):
+        gf.hybrid_attn(x, x, x, 4)
