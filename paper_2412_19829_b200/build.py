@@ -15,7 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "libgformer.so")
 FASTCALL = os.path.join(HERE, "_fastcall.so")  # the binding's calls as a module (csrc/fastcall.cpp)
-SOURCES = ["api.cu", "simt_kernels.cu", "simt_tiled.cu", "tma_host.cu", "tc_window.cu", "tc_linear.cu", "tc_linear_self.cu", "noalloc.cu", "partition.cu", "tc_favor.cu"]
+SOURCES = ["api.cu", "simt_kernels.cu", "simt_tiled.cu", "tma_host.cu", "host_state.cu", "tc_window.cu", "tc_linear.cu", "tc_linear_self.cu", "noalloc.cu", "partition.cu", "tc_favor.cu"]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 
 

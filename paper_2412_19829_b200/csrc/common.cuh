@@ -11,6 +11,7 @@
 #include <mutex>
 
 #include "gformer.h"
+#include "host_state.h"
 
 namespace gf {
 
@@ -134,8 +135,6 @@ cudaError_t launch_decode_step(const void* q, const void* k, const void* v, void
 
 // The current device and its SM count (asked of the driver once per device).
 cudaError_t device_info(int* dev, int* sms);
-// cudaFuncAttributeMaxDynamicSharedMemorySize of a kernel, set once per kernel and device.
-cudaError_t ensure_dynamic_smem(const void* kernel, int dev, int bytes);
 
 // ---- tensor-core (tcgen05 / TMEM / TMA) path: bf16 storage, d in {64,128}.
 bool tc_window_supported(int N, int d, int w, int dtype);

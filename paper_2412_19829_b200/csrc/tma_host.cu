@@ -2,7 +2,6 @@
 #include <string.h>
 
 #include <mutex>
-#include <vector>
 
 #include "common.cuh"
 #include "sm100.cuh"
@@ -34,25 +33,6 @@ cudaError_t device_info(int* dev, int* sms) {
     cached[*dev] = n;
   }
   *sms = n;
-  return cudaSuccess;
-}
-
-cudaError_t ensure_dynamic_smem(const void* kernel, int dev, int bytes) {
-  struct Done {
-    const void* kernel;
-    int dev, bytes;
-  };
-  static std::mutex mu;
-  static std::vector<Done> done;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    for (const Done& x : done)
-      if (x.kernel == kernel && x.dev == dev && x.bytes >= bytes) return cudaSuccess;
-  }
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e != cudaSuccess) return e;
-  std::lock_guard<std::mutex> lock(mu);
-  done.push_back(Done{kernel, dev, bytes});
   return cudaSuccess;
 }
 
