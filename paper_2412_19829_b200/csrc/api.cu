@@ -423,6 +423,7 @@ int gformer_hybrid_attn_w(const void* q, const void* k, const void* v, void* o, 
     if (h_sparse > 0 && (!s->k_cache || !s->v_cache || !aligned16(s->k_cache) || !aligned16(s->v_cache)))
       return GF_ERR_INVALID_ARG;
     if (h_lin > 0 && (!s->S || !s->z || !aligned16(s->S) || !aligned16(s->z))) return GF_ERR_INVALID_ARG;
+    if (h_sparse > 0 && !gf::export_ring_fits(B, N, d, w, dtype, h_sparse)) return GF_ERR_CUDA;
   }
   rc = check_ws(ws, ws_bytes, workspace_bytes(tn, B, H, N, d, h_sparse, dtype, phi, &fm.feat_offset));
   if (rc != GF_OK) return rc;

@@ -8,7 +8,6 @@
 #include <stdint.h>
 
 #include <functional>
-#include <mutex>
 
 #include "gformer.h"
 #include "host_state.h"
@@ -124,6 +123,7 @@ cudaError_t launch_linear_tiled(const void* q, const void* k, const void* v, voi
 cudaError_t launch_layer_tiled(const void* q, const void* k, const void* v, void* o, int B, int N, int d, int w, float scale,
                                int dtype, Strides st, int h_sparse, int h_lin, float* S_io, float* z_io, cudaStream_t stream,
                                Place place);
+bool export_ring_fits(int B, int N, int d, int w, int dtype, int h_sparse);
 cudaError_t launch_export_ring(const void* k, const void* v, void* k_cache, void* v_cache, int B, int N, int d,
                                int w, int dtype, Strides st, int h_sparse, cudaStream_t stream);  // kBeside
 // t_seq == nullptr: every sequence is at position t; else sequence b is at t_seq[b] (device array,
@@ -171,22 +171,6 @@ cudaError_t launch_linear_tc(const void* q, const void* k, const void* v, void* 
                              int layout, int h_begin, int h_count, float* S_io, float* z_io, bool zero_init,
                              int split, int max_ctas, WsHeader* ws, cudaStream_t stream, Link link, LetGo let_go, bool shared = false,
                              const void* fq = nullptr, const void* fk = nullptr);
-// The CTAs of a cut-chain launch wait for one another, so two such kernels must not share the SMs: each could hold some of
-// them while its own unplaced CTAs wait for the rest.  Per device the calls that have one are therefore chained by an event:
-// such a call starts only when the previous one, from whatever stream or host thread, has finished.  (Not inside a stream
-// capture, where an outside event cannot be waited for: there the order of the caller's graphs applies.)  Entered ahead
-// of the call's first launch and left behind its last one, because an event between two kernels would part their chain.
-class CutChainOrder {
- public:
-  cudaError_t enter(int dev, cudaStream_t stream);
-  cudaError_t leave();  // records the event
-
- private:
-  std::unique_lock<std::mutex> lock_;
-  int dev_ = 0;
-  cudaStream_t stream_ = nullptr;
-};
-
 // Positive random features phi_W of Q and K of heads [h_begin, h_begin + h_count) (bf16 storage) into the
 // contiguous bf16 tensors fq, fk [B, h_count, N, d]; W: [h_count, d, d] bf16, row a of a head's matrix is
 // its projection vector w_a.  With fq, fk given, the two linear-attention launchers read them in place

@@ -587,13 +587,18 @@ cudaError_t launch_linear_simt(const void* q, const void* k, const void* v, void
                                         stream, place, W);
 }
 
+// (32-bit indices of 16-byte pieces: 64 GB of keys)
+bool export_ring_fits(int B, int N, int d, int w, int dtype, int h_sparse) {
+  const long long rows = (long long)B * h_sparse * (N < w ? N : w);
+  return rows * (d / (dtype == GF_F32 ? 4 : 8)) <= 0xffffffffLL - 2 * kExportThreads;
+}
+
 cudaError_t launch_export_ring(const void* k, const void* v, void* k_cache, void* v_cache, int B, int N, int d,
                                int w, int dtype, Strides st, int h_sparse, cudaStream_t stream) {
   if (h_sparse <= 0 || B <= 0) return cudaSuccess;
   const int wn = N < w ? N : w, per16 = dtype == GF_F32 ? 4 : 8;  // elements of 16 bytes
   const long long total = (long long)B * h_sparse * wn * (d / per16);
-  // (64 GB of keys)
-  if (total > 0xffffffffLL - 2 * kExportThreads) return cudaErrorInvalidValue;
+  if (!export_ring_fits(B, N, d, w, dtype, h_sparse)) return cudaErrorInvalidValue;
   const Strides st16 = {st.b / per16, st.h / per16, st.n / per16};
   return launch_link(export_ring_kernel, dim3((unsigned)((total + 2 * kExportThreads - 1) / (2 * kExportThreads))),
                      dim3(kExportThreads), 0, stream, (const uint4*)k, (const uint4*)v, (uint4*)k_cache, (uint4*)v_cache, N,

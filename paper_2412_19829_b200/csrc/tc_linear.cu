@@ -50,7 +50,6 @@
 // no parking and no hand-over; the phi warps transform each K tile in place one chunk ahead of
 // the chunk pipeline (four K slots at D = 64).
 // Every wait is bounded; on expiry the kernel records a status word and drains.
-#include <mutex>
 #include <type_traits>
 
 #include "common.cuh"
@@ -1414,29 +1413,6 @@ size_t linear_tc_flag_bytes(int nchains, int N, int split) {
 size_t linear_tc_workspace_bytes(int nchains, int N, int d, int split) {
   return linear_tc_flag_bytes(nchains, N, split) +
          (size_t)plan_slots_max(nchains, N, split) * ((size_t)128 * d + d) * sizeof(float);
-}
-
-namespace {
-std::mutex g_cut_mutex;
-cudaEvent_t g_cut_last[64] = {};  // per device: behind the last call that has a cut-chain launch
-}  // namespace
-
-cudaError_t CutChainOrder::enter(int dev, cudaStream_t stream) {
-  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-  cudaError_t e = cudaStreamIsCapturing(stream, &capturing);
-  if (e != cudaSuccess || capturing != cudaStreamCaptureStatusNone) return e;
-  lock_ = std::unique_lock<std::mutex>(g_cut_mutex);
-  dev_ = dev;
-  stream_ = stream;
-  cudaEvent_t& ev = g_cut_last[dev];
-  return ev == nullptr ? cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) : cudaStreamWaitEvent(stream, ev, 0);
-}
-
-cudaError_t CutChainOrder::leave() {
-  if (!lock_.owns_lock()) return cudaSuccess;
-  const cudaError_t e = cudaEventRecord(g_cut_last[dev_], stream_);
-  lock_.unlock();
-  return e;
 }
 
 cudaError_t launch_linear_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,
