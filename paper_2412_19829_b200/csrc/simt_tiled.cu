@@ -903,12 +903,15 @@ int spread_smem(int need, long long ctas, int sms) {
   return least > need ? (int)least : need;
 }
 
-// Clusters of that many CTAs of the walk that the device holds at a time (asked once).
+// Clusters of that many CTAs of the walk that the device holds at a time (asked once for each number of CTAs that the shared
+// memory asked for leaves an SM).
 template <typename T, int D>
 int resident_clusters(int size, int smem, int dev) {
-  static std::atomic<int> known[64][kMaxCluster + 1][2];  // [...][a CTA per SM]
+  constexpr int kMost = 4;  // (of the CTAs with the least shared memory)
+  static_assert(kSmemPerSM / (LinT<D>::kSmem + kSmemReserved) <= kMost, "a slot for each number");
+  static std::atomic<int> known[64][kMaxCluster + 1][kMost + 1];
   if (dev < 0 || dev >= 64) return 0;
-  std::atomic<int>& slot = known[dev][size][smem > LinT<D>::kSmem];
+  std::atomic<int>& slot = known[dev][size][kSmemPerSM / (smem + kSmemReserved)];
   int n = slot.load(std::memory_order_relaxed);
   if (n == 0) {
     auto kern = linear_walk_kernel<T, D, true>;
@@ -923,11 +926,12 @@ int resident_clusters(int size, int smem, int dev) {
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+    if (e != cudaSuccess) {
       (void)cudaGetLastError();
-      n = -1;
+      return 0;
     }
-    slot.store(n, std::memory_order_relaxed);
+    slot.store(n > 0 ? n : -1, std::memory_order_relaxed);
   }
   return n > 0 ? n : 0;
 }

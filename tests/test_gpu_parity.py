@@ -1,5 +1,9 @@
 """GPU parity: libgformer (through the C ABI binding) against the fp64 oracle, element by
 element on the same seeded, storage-rounded inputs."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -1163,6 +1167,29 @@ def test_what_follows_a_layer_in_its_stream_follows_all_of_its_kernels(dtype, N,
         for ring, x in ((got[i][1], sets[i % 3][1]), (got[i][2], sets[i % 3][2])):
             for j in range(N - n, N):
                 assert torch.equal(ring[:, :, j % w], x[:, :h0, j])
+
+
+# chains, tokens: clusters with one, two and three CTAs to an SM, and three launches
+F32_PLANS = [(1, 256), (40, 1024), (40, 500), (30, 500), (50, 512), (80, 2048)]
+
+
+@pytest.mark.gpu
+def test_f32_linear_heads_are_planned_by_the_call_alone():
+    """The same bits and as many launches whatever sizes the process has seen before."""
+    program = """
+import sys, hashlib, torch
+from paper_2412_19829_b200 import binding as gf
+for c, n in eval(sys.argv[1]):
+    x = [torch.randn(1, c, n, 64, generator=torch.Generator().manual_seed(i + n)).cuda() for i in range(3)]
+    before = gf.launch_count()
+    o = gf.causal_linear_attn(*x)
+    print(c, n, gf.launch_count() - before, hashlib.sha1(o.cpu().numpy().tobytes()).hexdigest())
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    seen = [set(subprocess.check_output([sys.executable, "-c", program, repr(plans)], cwd=root, text=True).splitlines())
+            for plans in (F32_PLANS, F32_PLANS[::-1], F32_PLANS[1:2], F32_PLANS[2:3])]
+    assert len(seen[0]) == len(F32_PLANS)
+    assert seen[0] == seen[1] and seen[2] < seen[0] and seen[3] < seen[0]
 
 
 # ----------------------------------------------------------------------------- head partition (Algorithm 2)
