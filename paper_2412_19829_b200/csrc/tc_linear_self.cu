@@ -975,7 +975,11 @@ size_t linear_self_count_bytes(int nchains) { return ((size_t)nchains * 2 * size
 size_t linear_self_workspace_bytes(int nchains, int N, int d) {
   const int nch = (N + 127) / 128;
   const size_t state = ((size_t)d * d + d) * sizeof(float);
-  return linear_self_count_bytes(nchains) + (size_t)nchains * (self_segments(nchains, nch) + 1) * state;
+  const int G = self_segments(nchains, nch);
+  // One segment: its sum is the total, and the counters take less than the room that totals would (what fits the fixed
+  // scratch of the allocation-free call depends on this: 252 chains of up to 512 tokens, d = 64).
+  if (G == 1) return 2 * (size_t)nchains * state;
+  return linear_self_count_bytes(nchains) + (size_t)nchains * (G + 1) * state;
 }
 
 cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, void* o, int B, int H, int N, int d,

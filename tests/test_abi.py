@@ -76,6 +76,12 @@ def test_workspace_covers_every_plan():
     assert auto >= fixed
 
 
+@pytest.mark.parametrize("chains,N,d", [(252, 512, 64), (252, 1, 64), (63, 512, 128)])
+def test_calls_at_the_limit_of_the_allocation_free_scratch(chains, N, d):
+    """8 MiB hold two states of d * (d + 1) floats per chain of one segment, and have to go on doing so."""
+    assert gf.workspace_bytes(1, chains, N, d, 1, 0, gf.GF_BF16) <= 8 << 20
+
+
 def _state_scratch(chains, segments, d):
     # per segment: one 128-byte flag line and one published state (S: 128 x d floats, z: d floats)
     return 256 + chains * segments * (128 + (128 * d + d) * 4)
