@@ -2,8 +2,9 @@
 // tcgen05 kernels are switched off).
 //
 // The products run on the tensor cores as mma.sync with tf32 operands, each operand split in two (x = hi + lo, hi rounded to
-// tf32's 11 bits, lo the exact rest, of which at most the last bit is dropped): hi hi + hi lo + lo hi, what is left out is
-// 2^-24 of a product.  The tensor core rounds towards zero when it adds to an accumulator, so no sum runs through it: the 8 products of
+// tf32's 11 bits, lo the exact rest, of which the tensor core reads 11 bits: a quarter of all operands lose their last one):
+// hi hi + hi lo + lo hi, at most 2^-21.1 of a product away from it, 2^-23.7 in the mean square.  Sums of many terms come out nearer
+// than with FFMA, which rounds after each; those of fewer than kFewKeys stay FFMA's.  The tensor core rounds towards zero when it adds to an accumulator, so no sum runs through it: the 8 products of
 // an instruction (windowed heads: of two) start from zero and are added to the running sum on the CUDA cores, rounded to
 // nearest.  Against 64 bits (2 x 12 heads of 2048 tokens, d = 64, w = 128; relative error, windowed and linear heads) that is
 // 2.0e-7 and 1.1e-7, all sums in the accumulators 1.2e-6 and 1.1e-6, FFMA products 3.1e-7 and 1.5e-7.  (tcgen05.mma, four times
@@ -153,15 +154,19 @@ constexpr int kWinRows = 64, kWinGroup = 128, kWinThreads = 2 * kWinGroup;
 template <int D>
 constexpr int window_smem() { return (kWinRows * (D + 8) + 2 * kC * (D + 8) + 2 * kC * (D + 4)) * 4; }
 
-// Masked keys have weight 0 in the products above, which is nothing unless their value is infinite or NaN (0 x inf = NaN), and
-// an infinite operand's rest is NaN: the output row of query i once more, by the four lanes that share it, over the keys it
-// sees and no others.
-template <typename T, int D>
+// The output row of query i with FFMA products, by the four lanes that share it, over the keys it sees and no others.
+// For rows in which a sum came out NaN: masked keys have weight 0 in the products above, which is nothing unless their value
+// is infinite or NaN (0 x inf = NaN), and an infinite operand's rest is NaN.  And, kShort, for those of so few keys that the
+// errors of split operands do not average out: one key, whose value comes out as it is, and windows of fewer than kFewKeys (relative
+// error of split operands at d = 64, FFMA's = 1: w = 2 1.21, 4 1.05, 8 0.91; us, 8 x 12 heads of 2048 tokens, w = 4 split 120, so 68).
+constexpr int kFewKeys = 6;
+template <typename T, int D, bool kShort>
 __device__ __noinline__ void window_row(const T* q, const T* k, const T* v, T* o, int i, int j_begin, int j_end, float scale,
                                         long long stride, int part, unsigned int quad) {
+  constexpr int kAhead = kShort ? kFewKeys - 2 : 1, kCols = kShort ? D / 16 : 1;
   auto score = [&](int j) {
     float s = 0.f;
-#pragma unroll 1
+#pragma unroll(kCols)
     for (int c = 0; c < D / 16; ++c)
       s = dot4(load4<T>(q + i * stride + 4 * (part + 4 * c)), load4<T>(k + j * stride + 4 * (part + 4 * c)), s);
     s += __shfl_xor_sync(quad, s, 1);
@@ -169,13 +174,13 @@ __device__ __noinline__ void window_row(const T* q, const T* k, const T* v, T* o
     return s * scale;
   };
   float m = -INFINITY, l = 0.f;
-#pragma unroll 1
+#pragma unroll(kAhead)
   for (int j = j_begin; j < j_end; ++j) m = fmaxf(m, score(j));
   const float ref = m == -INFINITY ? 0.f : m;
   float4 acc[D / 16];
 #pragma unroll
   for (int c = 0; c < D / 16; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
+#pragma unroll(kAhead)
   for (int j = j_begin; j < j_end; ++j) {
     const float p = expf(score(j) - ref);
     l += p;
@@ -198,6 +203,13 @@ struct WindowArgs {
 };
 
 template <typename T, int D>
+__device__ __forceinline__ void window_short_tile(const WindowArgs<T>& p, int tile, int head, int b) {
+  const long long base = (long long)b * p.st.b + (long long)(p.h_begin + head) * p.st.h;
+  if (const int i = tile * kWinRows + (int)threadIdx.x / 4; i < p.N)
+    window_row<T, D, true>(p.q + base, p.k + base, p.v + base, p.o + base, i, max(i - p.w + 1, 0), min(i + p.fwd, p.N - 1) + 1, p.scale,
+                           p.st.n, threadIdx.x & 3, 0xfu << (threadIdx.x & 28));
+}
+template <typename T, int D>
 __device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, int head, int b, float* sm) {
   constexpr int LD = D + 8, LDV = D + 4, NT = D / 8;
   const int group = threadIdx.x / kWinGroup, tid = threadIdx.x % kWinGroup, lane = tid & 31, warp = tid >> 5;
@@ -207,6 +219,10 @@ __device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, in
   const int i0 = tile * kWinRows;
   const int g = lane >> 2, t = lane & 3;
   const int iw = i0 + 16 * warp;  // the warp's first row
+  auto short_row = [&](int i) {
+    window_row<T, D, true>(p.q + base, p.k + base, p.v + base, p.o + base, i, max(i - p.w + 1, 0), min(i + p.fwd, N - 1) + 1, p.scale,
+                           p.st.n, t, 0xfu << (lane & 28));
+  };
   auto sync_group = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kWinGroup) : "memory"); };
 
   const int jlo = max(i0 - p.w + 1, 0) + kC * group, jhi = min(min(i0 + kWinRows, N) - 1 + p.fwd, N - 1);
@@ -334,7 +350,11 @@ __device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, in
     }
   }
   __syncthreads();
-  if (group == 1) return;
+  const int one = p.fwd == 0 ? 0 : -1;  // the row that sees one key
+  if (group == 1) {
+    if (i0 == one && tid < 4) short_row(one);
+    return;
+  }
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int i = iw + g + 8 * r;
@@ -350,14 +370,14 @@ __device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, in
 #pragma unroll
     for (int n = 0; n < NT; ++n) {
       bad |= is_nan(acc[n][2 * r]) || is_nan(acc[n][2 * r + 1]);
-      if (i < N)
+      if (i < N && i != one)
         store2(p.o + base + (long long)i * p.st.n + 8 * n + 2 * t, acc[n][2 * r] * inv, acc[n][2 * r + 1] * inv);
     }
     const unsigned int quad = 0xfu << (lane & 28);
-    if ((__ballot_sync(0xffffffffu, bad) & quad) != 0u && i < N) {
+    if ((__ballot_sync(0xffffffffu, bad) & quad) != 0u && i < N && i != one) {
       __syncwarp(quad);  // (the row's stores above come first)
-      window_row<T, D>(p.q + base, p.k + base, p.v + base, p.o + base, i, max(i - p.w + 1, 0), min(i + p.fwd, N - 1) + 1, p.scale,
-                       p.st.n, t, quad);
+      window_row<T, D, false>(p.q + base, p.k + base, p.v + base, p.o + base, i, max(i - p.w + 1, 0), min(i + p.fwd, N - 1) + 1,
+                              p.scale, p.st.n, t, quad);
     }
     __syncwarp();
   }
@@ -368,7 +388,8 @@ __global__ void __launch_bounds__(kWinThreads, D == 64 ? 2 : 1)
 window_tiled_kernel(const WindowArgs<T> p, Place place) {
   extern __shared__ __align__(16) float sm[];
   begin(place);
-  window_tile<T, D>(p, blockIdx.x, blockIdx.y, blockIdx.z, sm);
+  if (p.w < kFewKeys) window_short_tile<T, D>(p, blockIdx.x, blockIdx.y, blockIdx.z);
+  else window_tile<T, D>(p, blockIdx.x, blockIdx.y, blockIdx.z, sm);
   grid_dep_launch();
   if (blockIdx.x + blockIdx.y + blockIdx.z == 0) grid_dep_wait();
 }
@@ -798,6 +819,16 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
     if (tid < D)
       zs[tid] = Sp == nullptr ? 0.f : zp != nullptr ? zp[tid] : Sp[(long long)(D + tid / kW) * stride + tid % kW];
   }
+  // Whether the chain starts from nothing, so that its first rows see few keys: kept in a column of P that nobody uses.
+  if (g == 0) {
+    bool any = false;
+    if (S_io != nullptr && !p.zero_init) {
+      any = tid < D && zs[tid] != 0.f;
+      for_state<D>(S, [&](int, int, float& x) { any |= x != 0.f; });
+      any = __syncthreads_or(any);
+    }
+    if (tid == 0) Ps[kC] = any ? 0.f : 1.f;
+  }
   for (int n0 = n_begin; n0 < n_end; n0 += kC) {
     if (!kCluster || n0 > n_begin) {
       store_block(n0);
@@ -862,6 +893,18 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
             store2(o + (long long)(n0 + row) * p.st.n + 16 * (tid >> 5) + 8 * n + 2 * (lane & 3), acc[m][n][2 * r] * inv,
                    acc[m][n][2 * r + 1] * inv);
         }
+    }
+    // Rows that see fewer than kFewKeys keys, with FFMA products, over what was just stored (largest error of chains of 64 to 2048
+    // tokens, d = 64, FFMA's = 1: 1.39 without this, 0.73 with it; 0.2 us of a chain).
+    if (n0 == 0 && Ps[kC] != 0.f) {
+      __syncthreads();
+      if (const int row = tid >> 4, c = 4 * (tid & 15); row < kFewKeys - 1 && row < n_end) {
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        for (int j = 0; j <= row; ++j) axpy4(x, Ps[row * kLdP + j], lds4(Vs + j * kLdV + c));
+        const float inv = inv_s[row];
+        store4(o + (long long)row * p.st.n + c, make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv));
+      }
     }
     if (more && tid >= kLinThreads - D) zs[tid - (kLinThreads - D)] += column_sum<D>(Ks + tid - (kLinThreads - D));
     __syncthreads();
@@ -1027,7 +1070,8 @@ layer_kernel(const WalkArgs<T> lp, const WindowArgs<T> wp, int parts, int n_lin,
     linear_walk<T, D, kCluster>(lp, id - chain * parts, chain - b * lp.h_count, b, sm);
   } else if (id - n_lin < n_win) {  // (the grid is a multiple of the cluster size)
     const int tiles = (wp.N + kWinRows - 1) / kWinRows, row = (id - n_lin) / tiles, b = row / h_sparse;
-    window_tile<T, D>(wp, id - n_lin - row * tiles, row - b * h_sparse, b, sm);
+    if (wp.w < kFewKeys) window_short_tile<T, D>(wp, id - n_lin - row * tiles, row - b * h_sparse, b);
+    else window_tile<T, D>(wp, id - n_lin - row * tiles, row - b * h_sparse, b, sm);
   }
   grid_dep_launch();
 }

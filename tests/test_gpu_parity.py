@@ -1192,6 +1192,30 @@ for c, n in eval(sys.argv[1]):
     assert seen[0] == seen[1] and seen[2] < seen[0] and seen[3] < seen[0]
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("N", [1, 5, 70, 200])
+def test_f32_rows_that_see_one_key_or_few(N, d):
+    """One key: a windowed head gives its value as it is, a linear one after three roundings (a product, a reciprocal, a product).
+    A few: the bound of test_f32_layer_products_at_the_edges_of_blocks_and_segments."""
+    B, H = 4, 6
+    q, k, v = synth.qkv(B, H, N, d, "f32", seed=17 + N, gain=1.0)
+    qd, kd, vd = dev(q, k, v)
+    for attn in (gf.window_attn, gf.window_attn_self):
+        assert torch.equal(attn(qd, kd, vd, 1), vd)
+        for w in (2, 5, 6):
+            o, ref = f64(attn(qd, kd, vd, w)), (oracle.window_attn_self if attn is gf.window_attn_self else oracle.window_attn)(
+                f64(q), f64(k), f64(v), w)
+            assert np.sqrt(((o - ref) ** 2).sum() / (ref**2).sum()) <= 4 * 2.0**-24 * np.sqrt(2 * d)
+    S, z = torch.zeros(B, H, d, d, device="cuda"), torch.zeros(B, H, d, device="cuda")
+    layer = gf.hybrid_attn(qd, kd, vd, 40, h_sparse=2)
+    assert torch.equal(gf.window_attn(qd, kd, vd, 40)[:, :, 0], vd[:, :, 0])
+    assert torch.equal(layer[:, :2, 0], vd[:, :2, 0])
+    for o in (gf.causal_linear_attn(qd, kd, vd), gf.causal_linear_attn(qd, kd, vd, S, z), layer[:, 2:]):
+        first = vd[:, -o.shape[1]:, 0]
+        assert ((o[:, :, 0] - first).abs().double() <= 3.01 * 2.0**-24 * first.abs().double()).all()
+
+
 # ----------------------------------------------------------------------------- head partition (Algorithm 2)
 @pytest.mark.gpu
 def test_measured_partition_balances_the_two_head_kinds():
