@@ -549,6 +549,32 @@ __device__ __forceinline__ float column_sum(const float* col) {
   return (s[0] + s[1]) + (s[2] + s[3]);
 }
 
+// Below 2^-112 tf32 has fewer than 11 bits for the rest of an operand.  Features are that small under inputs of -77.6, their
+// products sooner, and what comes out is a quotient, in which the size of all features cancels: of rows whose denominators, and
+// segments whose feature sums, are all under kLow the products are FFMA's.  (Above it such operands are lost beside the others.  Values
+// below 2^-112 keep an error of 2^-136.)  Error beside FFMA's with keys around -84, d = 64: 11 times without this, equal with it.  Such
+// blocks take five times as long; the question costs the others 0.5 to 1.5 % (8 x 12 heads of 2048 tokens 170 -> 172 us).
+constexpr float kLow = 0x1p-84f;
+
+// S += phi(K)^T V with FFMA products
+template <int D>
+__device__ __forceinline__ void add_outer_ffma(const float* Ks, const float* Vs, State<D>& S) {
+  const Lane l = lane_of();
+  const float *k = Ks + l.half * (D / 2) + 2 * l.t, *v = Vs + l.c0 + l.g;
+#pragma unroll 1
+  for (int j = 0; j < kC; ++j, k += LinT<D>::LD, v += kLdV) {
+    const float v0 = v[0], v1 = v[8];
+#pragma unroll
+    for (int n = 0; n < D / 16; ++n) {
+      const float2 x = lds2(k + 8 * n);
+      S[n][0] = fmaf(x.x, v0, S[n][0]);
+      S[n][1] = fmaf(x.y, v0, S[n][1]);
+      S[n][2] = fmaf(x.x, v1, S[n][2]);
+      S[n][3] = fmaf(x.y, v1, S[n][3]);
+    }
+  }
+}
+
 // Adds tokens [n_begin, n_end) to S = 0 and z = 0 (thread tid < D: feature tid).
 template <typename T, int D>
 __device__ __forceinline__ void sum_segment(const T* k, const T* v, long long stride, int n_begin, int n_end, float* Ks,
@@ -557,6 +583,7 @@ __device__ __forceinline__ void sum_segment(const T* k, const T* v, long long st
   BlockRegs<T, kW, kLinThreads> rv;
   rk.load(k, stride, n_begin, n_end, tid);
   rv.load(v, stride, n_begin, n_end, tid);
+  int big = 0;  // some feature's sum is not under kLow
   for (int n0 = n_begin; n0 < n_end; n0 += kC) {
     rk.store_phi(Ks, LinT<D>::LD, n0, n_end, tid);
     rv.store(Vs, kLdV, tid);
@@ -565,7 +592,19 @@ __device__ __forceinline__ void sum_segment(const T* k, const T* v, long long st
     rv.load(v, stride, n0 + kC, n_end, tid);
     add_outer<D, false>(Ks, Vs, S);
     if (tid < D) z += column_sum<D>(Ks + tid);
-    __syncthreads();
+    big = __syncthreads_or(tid < D && !(z < kLow));
+  }
+  if (!big && __syncthreads_or(tid < D && z > 0.f)) {
+    for_state<D>(S, [](int, int, float& x) { x = 0.f; });
+    for (int n0 = n_begin; n0 < n_end; n0 += kC) {
+      rk.load(k, stride, n0, n_end, tid);
+      rv.load(v, stride, n0, n_end, tid);
+      rk.store_phi(Ks, LinT<D>::LD, n0, n_end, tid);
+      rv.store(Vs, kLdV, tid);
+      __syncthreads();
+      add_outer_ffma<D>(Ks, Vs, S);
+      __syncthreads();
+    }
   }
   // (an infinite operand's rest is NaN)
   bool bad = false;
@@ -640,6 +679,48 @@ __global__ void linear_prefix_kernel(float* __restrict__ o, Segs sg, Strides st,
         store4(slot + (long long)sg.begin(g0 + e) * st.n, run);
       }
   }
+}
+
+// 1 / (row sums of P + phi(Q) z), eight threads per row.  Whether the thread has found one under kLow (past the end they are 0)
+__device__ __forceinline__ bool invert_denominators(const float* Ps, const float* qz_s, float* inv_s) {
+  const int row = threadIdx.x >> 3, part8 = threadIdx.x & 7;
+  float den = 0.f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) den += Ps[row * kLdP + part8 + 8 * e];
+#pragma unroll
+  for (int off = 1; off < 8; off <<= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
+  den += qz_s[row];
+  if (part8 == 0) inv_s[row] = 1.f / den;
+  return den > 0.f && den < kLow;
+}
+
+// A block with a row whose denominator is under kLow: all of it with FFMA products.
+template <int D>
+__device__ __noinline__ void low_block(const float* Qs, const float* Ks, const float* Vs, float* Ps, float* Ss, const float* qz_s,
+                                       float* inv_s, State<D>& S, float (&acc)[2][2][4], bool more) {
+  constexpr int LD = LinT<D>::LD;
+  const Lane l = lane_of();
+  for_state<D>(S, [&](int a, int c, float& x) { Ss[a * kW + c] = x; });
+  for (int e = 0; e < 4; ++e) {
+    const int row = threadIdx.x >> 3, key = (threadIdx.x & 7) + 8 * e;
+    float x = 0.f;
+    if (key <= row)
+      for (int a = 0; a < D; a += 4) x = dot4(lds4(Qs + row * LD + a), lds4(Ks + key * LD + a), x);
+    Ps[row * kLdP + key] = x;
+  }
+  __syncthreads();
+  (void)invert_denominators(Ps, qz_s, inv_s);
+  if (l.half == 0)
+    for (int i = 0; i < 16; ++i) {
+      const int m = i >> 3, n = (i >> 2) & 1, e = i & 3;
+      const int row = 16 * m + l.g + 8 * (e >> 1), c = l.c0 + 8 * n + 2 * l.t + (e & 1);
+      float x = 0.f;
+      for (int a = 0; a < D; ++a) x = fmaf(Qs[row * LD + a], Ss[a * kW + c], x);
+      for (int j = 0; j <= row; ++j) x = fmaf(Ps[row * kLdP + j], Vs[j * kLdV + c], x);
+      acc[m][n][e] = x;
+    }
+  if (more) add_outer_ffma<D>(Ks, Vs, S);
+  __syncthreads();
 }
 
 // A block in which a sum came out NaN: a masked weight is 0, which is nothing unless the value is infinite or NaN (0 x inf
@@ -836,18 +917,10 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
     }
     dot_z<D>(Qs, zs, qz_s);
     __syncthreads();
-    {  // denominators: eight threads per row
-      const int row = tid >> 3, part8 = tid & 7;
-      float den = 0.f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) den += Ps[row * kLdP + part8 + 8 * e];
-#pragma unroll
-      for (int off = 1; off < 8; off <<= 1) den += __shfl_xor_sync(0xffffffffu, den, off);
-      if (part8 == 0) inv_s[row] = 1.f / (den + qz_s[row]);
-    }
+    const bool low = invert_denominators(Ps, qz_s, inv_s);
     float acc[2][2][4];
     readout<D, false>(Qs, Vs, Ps, S, acc);
-    bool bad = false;
+    bool bad = low;
 #pragma unroll
     for (int m = 0; m < 2; ++m)
 #pragma unroll
@@ -866,7 +939,8 @@ __device__ __forceinline__ void linear_walk(const WalkArgs<T>& p, int part, int 
       for (int n = 0; n < D / 16; ++n)
 #pragma unroll
         for (int e = 0; e < 4; ++e) Sx[n][e] = S[n][e];
-      mend_block<D>(Qs, Ks, Vs, Ps, Ss, Os, Sx, ax, more);
+      if (__syncthreads_or(low)) low_block<D>(Qs, Ks, Vs, Ps, Ss, qz_s, inv_s, Sx, ax, more);
+      else mend_block<D>(Qs, Ks, Vs, Ps, Ss, Os, Sx, ax, more);
 #pragma unroll
       for (int n = 0; n < D / 16; ++n)
 #pragma unroll

@@ -1216,6 +1216,27 @@ def test_f32_rows_that_see_one_key_or_few(N, d):
         assert ((o[:, :, 0] - first).abs().double() <= 3.01 * 2.0**-24 * first.abs().double()).all()
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("shift_q,shift_k", [(0, -84), (-84, 0), (-43, -43)])
+@pytest.mark.parametrize("B,H,N,d", [(2, 3, 200, 64), (40, 8, 70, 64), (1, 2, 4000, 64), (1, 2, 1601, 128)])
+def test_f32_linear_heads_whose_features_are_all_tiny(B, H, N, d, shift_q, shift_k):
+    """phi = exp of inputs far below zero, 2^-121 in the mean: their size cancels in the output, whose error stays that of other
+    inputs (the bound of test_f32_layer_products_at_the_edges_of_blocks_and_segments)."""
+    q, k, v = synth.qkv(B, H, N, d, "f32", seed=23 + N, gain=1.0)
+    q, k = q + shift_q, k + shift_k
+    qd, kd, vd = dev(q, k, v)
+    S, z = torch.zeros(B, H, d, d, device="cuda"), torch.zeros(B, H, d, device="cuda")
+    cut = N // 3
+    carried = torch.cat([gf.causal_linear_attn(*(x[:, :, a:b].contiguous() for x in (qd, kd, vd)), S, z)
+                         for a, b in ((0, cut), (cut, N))], 2)
+    bs = sorted({0, B - 1})
+    S_ref, z_ref = np.zeros((len(bs), H, d, d)), np.zeros((len(bs), H, d))
+    ref = oracle.causal_linear_attn(f64(q[bs]), f64(k[bs]), f64(v[bs]), S_ref, z_ref)
+    for got, want in ((gf.causal_linear_attn(qd, kd, vd), ref), (carried, ref), (S, S_ref), (z, z_ref)):
+        err = f64(got[bs]) - want
+        assert np.sqrt((err**2).sum() / (want**2).sum()) <= 4 * 2.0**-24 * np.sqrt(2 * d)
+
+
 # ----------------------------------------------------------------------------- head partition (Algorithm 2)
 @pytest.mark.gpu
 def test_measured_partition_balances_the_two_head_kinds():
