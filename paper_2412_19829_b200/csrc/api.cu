@@ -347,7 +347,9 @@ int gformer_hybrid_attn_self_w(const void* q, const void* k, const void* v, void
   if (tc_linear) {
     // (half tiles of 64 keys, 0.6 us each on an SM: tc_window.cu)
     const int tiles = (N + 127) / 128, seen = 2 * (((w < N ? w : N) + 126) / 128) + 1;  // (key tiles that a query tile sees)
-    const double window_us = 1.0 * B * h_sparse * tiles * (seen < tiles ? seen : tiles) / 148.0;
+    int dev = 0, sms = 0;
+    if (gf::device_info(&dev, &sms) != cudaSuccess) return GF_ERR_CUDA;
+    const double window_us = 1.0 * B * h_sparse * tiles * (seen < tiles ? seen : tiles) / sms;
     rc = cuda_status(gf::launch_linear_self_tc(q, k, v, o, B, H, N, d, layout, h_sparse, H - h_sparse, (WsHeader*)ws,
                                                sizeof(WsHeader), stream, window, window_us, fm.fq, fm.fk));
   } else {  // fp32 storage (or the CUDA-core knob): token by token, a summing sweep and a readout sweep

@@ -922,15 +922,15 @@ int self_segments(int nchains, int nch) {
 // Segments that the sums are formed in, at most self_segments.  Where windowed heads run behind the first launch (beside_us)
 // they fill the SMs that it leaves idle, so that only what they do not fill counts, in microseconds, beside the work itself; more segments
 // are more slots to add up, beside the windowed heads at 0.7 TB/s.
-int self_sum_segments(int nchains, int nch, int d, double beside_us) {
+int self_sum_segments(int nchains, int nch, int d, int sms, double beside_us) {
   const int g_max = self_segments(nchains, nch);
   if (beside_us <= 0.0) return g_max;
   const double chunk_us = d == 128 ? 1.5 : 0.8, state = ((double)d * d + d) * sizeof(float);
   int best_g = 1;
   double best = 1e300;
   for (int g = 1; g <= g_max; ++g) {
-    const double rounds = (double)(((long long)nchains * g + 147) / 148);
-    const double work = nchains * (double)(nch + g) / 148 * chunk_us, span = rounds * ((nch + g - 1) / g + 1) * chunk_us;
+    const double rounds = (double)(((long long)nchains * g + sms - 1) / sms);
+    const double work = nchains * (double)(nch + g) / sms * chunk_us, span = rounds * ((nch + g - 1) / g + 1) * chunk_us;
     const double idle = span - work - beside_us, sum = g > 1 ? 1.0 + nchains * g * state / 0.7e6 - 0.7 * beside_us : 0.0;
     const double cost = work + (idle > 0.0 ? idle : 0.0) + (g > 1 ? (sum > 1.0 ? sum : 1.0) : 0.0);
     if (cost < best) {
@@ -1015,7 +1015,7 @@ cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, v
     p.nitems = p.nchains * G;
     return dim3(p.nitems < sms ? p.nitems : sms);
   };
-  dim3 grid = cut(whole ? 1 : self_sum_segments(p.nchains, p.nch, d, beside_us));
+  dim3 grid = cut(whole ? 1 : self_sum_segments(p.nchains, p.nch, d, sms, beside_us));
   const int state_floats = d * d + d;
   uint8_t* scratch = reinterpret_cast<uint8_t*>(ws) + scratch_offset;
   p.summed = reinterpret_cast<unsigned int*>(scratch);
