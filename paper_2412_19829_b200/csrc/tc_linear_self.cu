@@ -40,6 +40,7 @@ struct SelfParams {
   unsigned int *summed, *totalled;
   unsigned int sum_blocks;
   int totals_of_one;  // the sums were formed in one segment per chain: no totals
+  LetGo let_go;       // of the kernel for whole chains
 };
 constexpr int kSumThreads = 64;
 
@@ -643,7 +644,7 @@ linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_co
   tc_fence_after_sync();
   const uint32_t tmem = tmem_base_s;
   grid_dep_wait();
-  grid_dep_launch();
+  if (p.let_go == kAtStart) grid_dep_launch();
 
   // Every role walks the chains blockIdx.x, blockIdx.x + gridDim.x, ... (an item is a whole chain) and keeps the same
   // running counters: n = chunks so far, c = chains so far.
@@ -672,6 +673,7 @@ linear_self_whole_kernel(const __grid_constant__ CUtensorMap mq, const __grid_co
           }
         }
       }
+      if (!kv && p.let_go == kAtEnd) grid_dep_launch();
     }
   } else if (warp == 1) {
     if (elect_one()) {
@@ -1024,6 +1026,7 @@ cudaError_t launch_linear_self_tc(const void* q, const void* k, const void* v, v
   p.partial = reinterpret_cast<float*>(scratch + linear_self_count_bytes(p.nchains));
   p.total = p.G == 1 ? p.partial : p.partial + (size_t)p.nitems * state_floats;  // one segment: its sum is the total
   p.status = &ws->status;
+  p.let_go = h_begin > 0 ? kAtStart : kAtEnd;  // (the windowed heads, where there are any, run beside it)
   if (whole) {
     auto kern = features ? linear_self_whole_kernel<true> : linear_self_whole_kernel<false>;
     if ((e = ensure_dynamic_smem(reinterpret_cast<const void*>(kern), dev, WholeCfg::kBytes)) != cudaSuccess) return e;
