@@ -352,7 +352,7 @@ int gformer_hybrid_attn_self_w(const void* q, const void* k, const void* v, void
     const double window_us = 1.0 * B * h_sparse * tiles * (seen < tiles ? seen : tiles) / sms;
     rc = cuda_status(gf::launch_linear_self_tc(q, k, v, o, B, H, N, d, layout, h_sparse, H - h_sparse, (WsHeader*)ws,
                                                sizeof(WsHeader), stream, window, window_us, fm.fq, fm.fk));
-  } else {  // fp32 storage (or the CUDA-core knob): token by token, a summing sweep and a readout sweep
+  } else {  // fp32 storage (or GF_TUNE_FORCE_SIMT): token by token, a summing sweep and a readout sweep
     rc = cuda_status(gf::launch_linear_simt(q, k, v, o, B, N, d, dtype, gf::make_strides(layout, H, N, d), h_sparse,
                                             H - h_sparse, nullptr, nullptr, true, stream, first_of_call(tn, ws, h_sparse == 0), true, W));
     if (rc == GF_OK) (void)window(gf::kAtEnd);

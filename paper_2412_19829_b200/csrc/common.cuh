@@ -102,7 +102,7 @@ struct Place {
 // call whose kernels use it.
 cudaError_t launch_clear_ws(Place place, size_t bytes, cudaStream_t stream);
 
-// ---- SIMT (CUDA-core, fp32 arithmetic) path: any w, d in {64,128}, f32 or bf16 storage.
+// ---- fp32 arithmetic (split tf32 products by mma.sync, or FFMA): any w, d in {64,128}, f32 or bf16 storage.
 // Heads [h_begin, h_begin + h_count) of the [B, H, N, d] tensors are processed.
 // fwd: keys after the query it may see: 0 = the causal window, w - 1 = the two-sided window |i - j| < w.
 cudaError_t launch_window_simt(const void* q, const void* k, const void* v, void* o, int B, int N, int d,

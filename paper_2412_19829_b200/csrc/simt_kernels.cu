@@ -1,6 +1,6 @@
-// CUDA-core (fp32 arithmetic) kernels of libgformer.
+// FFMA kernels (fp32 arithmetic) of libgformer.
 //
-// The linear heads of fp32 tensors where neither the tensor-core kernels nor the register-tiled ones apply (the
+// The linear heads of fp32 tensors where neither the tcgen05 kernels nor those of split tf32 products apply (the
 // bidirectional layer's sums, positive random features), and the memory-bound decode step and ring export, which have
 // no dense contraction worth a tensor core.  Plain data-parallel kernels: no inter-CTA communication, no spin waits.
 #include <cooperative_groups.h>

@@ -10,9 +10,9 @@
 // 2.0e-7 and 1.1e-7, all sums in the accumulators 1.2e-6 and 1.1e-6, FFMA products 3.1e-7 and 1.5e-7.  (tcgen05.mma, four times
 // as fast, could only add up in its accumulators.)
 // Register-tiled FFMA products, which this replaced, were bound by shared memory (us, before and now): 8 x 12 heads of 2048
-// tokens, d = 64, windowed (w = 128) 296 and 214, linear 240 and 173; d = 128 548 and 469, 843 and 698; the layer with 2
-// windowed heads 246 and 181.  What bounds these is the issue of instructions and their latency: 1600 a warp for a block of 32
-// tokens, a quarter of them splitting operands, at 55 % of the issue slots; tensor pipe 38 %.  Not faster: operands split once
+// tokens, d = 64, windowed (w = 128) 296 and 209, linear 240 and 172; d = 128 548 and 472, 843 and 686; the layer with 2
+// windowed heads 246 and 171.  What bounds these is the latency of their instructions and the issue of them: 1400 a warp for a block of 32
+// tokens, a quarter of them splitting operands, at 49 % of the issue slots (windowed 48 %); tensor pipe 36 % (42 %).  Not faster: operands split once
 // and kept as pairs in shared memory (10 to 25 % slower), cvt.rna (8 %), the three products of a split apart (3 %).
 #include <cooperative_groups.h>
 

@@ -1113,7 +1113,29 @@ def test_calls_made_natively_and_through_ctypes_are_the_same(monkeypatch, dtype,
             got.append((e.type, str(e.value)))
         return got
 
-    native, native_numpy, native_errors = calls(int), calls(np.int64), errors()
+    answers = []
+
+    class Recorder:
+        def __init__(self, module):
+            self.module = module
+
+        def __getattr__(self, name):
+            def call(*args):
+                r = getattr(self.module, name)(*args)
+                answers.append((name, type(r)))
+                return r
+            return call
+
+    monkeypatch.setattr(gf, "_fast", Recorder(gf._fastcall()))
+    calls(int)  # (the default workspace is large enough from here on)
+    answers.clear()
+    native = calls(int)
+    assert {name for name, r in answers if r is torch.Tensor} == {"window_attn", "hybrid_attn_self", "causal_linear_attn",
+                                                                   "hybrid_attn", "decode_step"}
+    assert all(r is torch.Tensor for _, r in answers)
+    answers.clear()
+    native_numpy, native_errors = calls(np.int64), errors()
+    assert answers[0] == ("window_attn", type(None)) and answers[2] == ("hybrid_attn_self", type(None))
     monkeypatch.setattr(gf, "_fast", Ordinary())
     ordinary = calls(int)
     for a, b, c in zip(native, native_numpy, ordinary):
