@@ -10,7 +10,7 @@
 // 2.0e-7 and 1.1e-7, all sums in the accumulators 1.2e-6 and 1.1e-6, FFMA products 3.1e-7 and 1.5e-7.  (tcgen05.mma, four times
 // as fast, could only add up in its accumulators.)
 // Register-tiled FFMA products, which this replaced, were bound by shared memory (us, before and now): 8 x 12 heads of 2048
-// tokens, d = 64, windowed (w = 128) 296 and 209, linear 240 and 172; d = 128 548 and 472, 843 and 686; the layer with 2
+// tokens, d = 64, windowed (w = 128) 296 and 212, linear 240 and 172; d = 128 548 and 470, 843 and 686; the layer with 2
 // windowed heads 246 and 171.  What bounds these is the latency of their instructions and the issue of them: 1400 a warp for a block of 32
 // tokens, a quarter of them splitting operands, at 49 % of the issue slots (windowed 48 %); tensor pipe 36 % (42 %).  Not faster: operands split once
 // and kept as pairs in shared memory (10 to 25 % slower), cvt.rna (8 %), the three products of a split apart (3 %).
@@ -156,8 +156,8 @@ constexpr int window_smem() { return (kWinRows * (D + 8) + 2 * kC * (D + 8) + 2 
 
 // The output row of query i with FFMA products, by the four lanes that share it, over the keys it sees and no others.
 // For rows in which a sum came out NaN: masked keys have weight 0 in the products above, which is nothing unless their value
-// is infinite or NaN (0 x inf = NaN), and an infinite operand's rest is NaN.  And, kShort, for those of so few keys that the
-// errors of split operands do not average out: one key, whose value comes out as it is, and windows of fewer than kFewKeys (relative
+// is infinite or NaN (0 x inf = NaN), and an infinite operand's rest is NaN.  And, kShort, for windows of fewer than kFewKeys keys, in
+// which the errors of split operands do not average out (relative
 // error of split operands at d = 64, FFMA's = 1: w = 2 1.21, 4 1.05, 8 0.91; us, 8 x 12 heads of 2048 tokens, w = 4 split 120, so 68).
 constexpr int kFewKeys = 6;
 template <typename T, int D, bool kShort>
@@ -202,6 +202,26 @@ struct WindowArgs {
   int h_begin;
 };
 
+// The causal row that sees one key, over what the tile has stored: that key's value as it is, NaN unless the score is finite.  By a warp
+// of the group that has no part in the tile's end, and behind the tile, since anything within it cost other tiles 1 to 4 %.
+template <typename T, int D>
+__device__ __noinline__ void window_first_row(const T* q, const T* k, const T* v, T* o, float scale) {
+  const int lane = (int)threadIdx.x - kWinGroup;
+  const bool part = lane >= 0 && 4 * lane < D;
+  float4 value = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (lane >= 0 && lane < 32) {
+    float s = 0.f;
+    if (part) {
+      value = load4<T>(v + 4 * lane);
+      s = dot4(load4<T>(q + 4 * lane), load4<T>(k + 4 * lane), 0.f);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (!is_finite(s * scale)) value = make_float4(NAN, NAN, NAN, NAN);
+  }
+  __syncthreads();
+  if (part) store4(o + 4 * lane, value);
+}
 template <typename T, int D>
 __device__ __forceinline__ void window_short_tile(const WindowArgs<T>& p, int tile, int head, int b) {
   const long long base = (long long)b * p.st.b + (long long)(p.h_begin + head) * p.st.h;
@@ -219,10 +239,6 @@ __device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, in
   const int i0 = tile * kWinRows;
   const int g = lane >> 2, t = lane & 3;
   const int iw = i0 + 16 * warp;  // the warp's first row
-  auto short_row = [&](int i) {
-    window_row<T, D, true>(p.q + base, p.k + base, p.v + base, p.o + base, i, max(i - p.w + 1, 0), min(i + p.fwd, N - 1) + 1, p.scale,
-                           p.st.n, t, 0xfu << (lane & 28));
-  };
   auto sync_group = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kWinGroup) : "memory"); };
 
   const int jlo = max(i0 - p.w + 1, 0) + kC * group, jhi = min(min(i0 + kWinRows, N) - 1 + p.fwd, N - 1);
@@ -350,11 +366,7 @@ __device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, in
     }
   }
   __syncthreads();
-  const int one = p.fwd == 0 ? 0 : -1;  // the row that sees one key
-  if (group == 1) {
-    if (i0 == one && tid < 4) short_row(one);
-    return;
-  }
+  if (group == 1) return;
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int i = iw + g + 8 * r;
@@ -370,11 +382,11 @@ __device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, in
 #pragma unroll
     for (int n = 0; n < NT; ++n) {
       bad |= is_nan(acc[n][2 * r]) || is_nan(acc[n][2 * r + 1]);
-      if (i < N && i != one)
+      if (i < N)
         store2(p.o + base + (long long)i * p.st.n + 8 * n + 2 * t, acc[n][2 * r] * inv, acc[n][2 * r + 1] * inv);
     }
     const unsigned int quad = 0xfu << (lane & 28);
-    if ((__ballot_sync(0xffffffffu, bad) & quad) != 0u && i < N && i != one) {
+    if ((__ballot_sync(0xffffffffu, bad) & quad) != 0u && i < N) {
       __syncwarp(quad);  // (the row's stores above come first)
       window_row<T, D, false>(p.q + base, p.k + base, p.v + base, p.o + base, i, max(i - p.w + 1, 0), min(i + p.fwd, N - 1) + 1,
                               p.scale, p.st.n, t, quad);
@@ -384,12 +396,24 @@ __device__ __forceinline__ void window_tile(const WindowArgs<T>& p, int tile, in
 }
 
 template <typename T, int D>
+__device__ __forceinline__ void any_window_tile(const WindowArgs<T>& p, int tile, int head, int b, float* sm) {
+  if (p.w < kFewKeys) {
+    window_short_tile<T, D>(p, tile, head, b);
+    return;
+  }
+  window_tile<T, D>(p, tile, head, b, sm);
+  if (tile == 0 && p.fwd == 0) {
+    const long long base = (long long)b * p.st.b + (long long)(p.h_begin + head) * p.st.h;
+    window_first_row<T, D>(p.q + base, p.k + base, p.v + base, p.o + base, p.scale);
+  }
+}
+
+template <typename T, int D>
 __global__ void __launch_bounds__(kWinThreads, D == 64 ? 2 : 1)
 window_tiled_kernel(const WindowArgs<T> p, Place place) {
   extern __shared__ __align__(16) float sm[];
   begin(place);
-  if (p.w < kFewKeys) window_short_tile<T, D>(p, blockIdx.x, blockIdx.y, blockIdx.z);
-  else window_tile<T, D>(p, blockIdx.x, blockIdx.y, blockIdx.z, sm);
+  any_window_tile<T, D>(p, blockIdx.x, blockIdx.y, blockIdx.z, sm);
   grid_dep_launch();
   if (blockIdx.x + blockIdx.y + blockIdx.z == 0) grid_dep_wait();
 }
@@ -1144,8 +1168,7 @@ layer_kernel(const WalkArgs<T> lp, const WindowArgs<T> wp, int parts, int n_lin,
     linear_walk<T, D, kCluster>(lp, id - chain * parts, chain - b * lp.h_count, b, sm);
   } else if (id - n_lin < n_win) {  // (the grid is a multiple of the cluster size)
     const int tiles = (wp.N + kWinRows - 1) / kWinRows, row = (id - n_lin) / tiles, b = row / h_sparse;
-    if (wp.w < kFewKeys) window_short_tile<T, D>(wp, id - n_lin - row * tiles, row - b * h_sparse, b);
-    else window_tile<T, D>(wp, id - n_lin - row * tiles, row - b * h_sparse, b, sm);
+    any_window_tile<T, D>(wp, id - n_lin - row * tiles, row - b * h_sparse, b, sm);
   }
   grid_dep_launch();
 }
